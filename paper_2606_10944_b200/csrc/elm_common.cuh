@@ -110,6 +110,10 @@ __device__ __forceinline__ int64_t checked_row(int64_t row, int64_t n, int *stat
     return row;
 }
 
+// Entries per problem of the per-pair arrays (running shifts, decay factors): room for n / 2 pairs, a multiple of 4 so
+// that every problem's row starts on a 16-byte boundary whatever n is (the Gram kernel reads it with vector loads).
+__host__ __device__ __forceinline__ int64_t pair_stride(int64_t n) { return (n / 2 + 3) & ~(int64_t)3; }
+
 // Philox4x32-10 (Salmon et al., SC'11), first output word only.
 __host__ __device__ __forceinline__ uint32_t philox4x32_10_word0(uint32_t c0, uint32_t c1, uint32_t c2,
                                                                  uint32_t c3, uint32_t k0, uint32_t k1)

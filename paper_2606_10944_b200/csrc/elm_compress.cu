@@ -17,8 +17,8 @@ CompressLayout compress_layout(const elm_params *p)
     L.cnorm = take(BH * n * ts);
     L.cur = take(BH * n * 4);
     L.nxt = take(BH * n * 4);
-    L.Mpair = take(BH * (n / 2 + 1) * ts);
-    L.rdecay = take(BH * (n / 2 + 1) * ts);
+    L.Mpair = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
+    L.rdecay = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
     L.F_stride = n_out * n_out;
     L.F = take(p->m > 0 ? BH * L.F_stride * ts : 0);
     L.wide = take(p->dtype == ELM_E4M3 ? 2 * BH * n * (size_t)p->d * 2 : 0);

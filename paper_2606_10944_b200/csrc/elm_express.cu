@@ -133,13 +133,13 @@ static ExpressLayout express_layout(const elm_params *p, int mbar = 0, bool pref
     L.listB = take(BH * n * 4);
     L.E = take(BH * n * 4);                // every point list is [BH][n]-strided, like the lists of elm_compress
     L.T1 = take(BH * n * 4);
-    L.Mpair = take(BH * (n / 2 + 1) * ts);
-    L.rdecay = take(BH * (n / 2 + 1) * ts);
+    L.Mpair = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
+    L.rdecay = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
     L.F_stride = 4 * n_out * n_out;        // the first halving of E is one call of 2 n_out pairs
     L.F = take(BH * L.F_stride * ts);
     L.E2 = take(BH * n * 4);
-    L.Mpair2 = take(BH * (n / 2 + 1) * ts);       // (indexed with the problem stride n / 2, like Mpair)
-    L.rdecay2 = take(BH * (n / 2 + 1) * ts);
+    L.Mpair2 = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);       // (indexed with the problem stride of Mpair)
+    L.rdecay2 = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
     L.F2 = take(BH * L.F_stride * ts);
     L.levels = L.ep_idx = L.ep_w = L.ep_birth = L.ep_death = L.ep_blk = L.ws_attend = L.ep_cap = L.ep_pad = L.ep_stride = 0;
     L.ws_attend_stride = L.lse = 0;

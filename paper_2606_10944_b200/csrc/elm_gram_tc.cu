@@ -140,10 +140,10 @@ gram_tc_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restr
     }
     if (tid < TP) {
         const int64_t jc = JC + tid;
-        misc->colshift[tid] = jc < Ptotal ? Mpair[(int64_t)p * (n / 2) + jc] * LOG2E : 0.f;
+        misc->colshift[tid] = jc < Ptotal ? Mpair[(int64_t)p * pair_stride(n) + jc] * LOG2E : 0.f;
         if (wk.fused) {
             // everything the in-tile walk needs from global memory, fetched while the tile is built
-            misc->rdec[tid] = jc < Ptotal ? wk.rdecay[(int64_t)p * (n / 2) + jc] : 1.f;
+            misc->rdec[tid] = jc < Ptotal ? wk.rdecay[(int64_t)p * pair_stride(n) + jc] : 1.f;
             uint32_t cgroup, ccode;
             call_counter((int)(jc / P), wk.level, cgroup, ccode);
             misc->unif[tid] = halving_uniform<float>(wk.seed, (uint32_t)(jc % P), cgroup, ccode, (uint32_t)p + wk.pbase);
@@ -461,8 +461,8 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
             // running shifts of this thread's 32 pair columns (in log2 units), fetched while the MMAs run
             float sh[32];
             {
-                // 32 consecutive floats, 128-byte aligned (n / 2 and JC are multiples of 32)
-                const float4 *mp = reinterpret_cast<const float4 *>(Mpair + (int64_t)p * (n / 2) + JC + ch * 32);
+                // 32 consecutive floats, 16-byte aligned (the rows' stride is a multiple of 4, JC of 32)
+                const float4 *mp = reinterpret_cast<const float4 *>(Mpair + (int64_t)p * pair_stride(n) + JC + ch * 32);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const float4 v = __ldg(mp + i);

@@ -125,8 +125,8 @@ static __global__ void __launch_bounds__(1024) level_prep_kernel(const T *__rest
         T excl = lane == 0 ? before : (before > prev_lane ? before : prev_lane);
         T M = inc > before ? inc : before;
         if (i < P) {
-            Mpair[(int64_t)p * (n / 2) + base + i] = M;
-            rdecay[(int64_t)p * (n / 2) + base + i] = (i == 0) ? (T)1 : (T)exp(-(double)(M - excl) * 0.5);
+            Mpair[(int64_t)p * pair_stride(n) + base + i] = M;
+            rdecay[(int64_t)p * pair_stride(n) + base + i] = (i == 0) ? (T)1 : (T)exp(-(double)(M - excl) * 0.5);
         }
         T tot = carry;
         for (int w = 0; w < nwarp; ++w) tot = tot > warp_tot[w] ? tot : warp_tot[w];
@@ -230,7 +230,7 @@ static __global__ void __launch_bounds__(256) gram_simt_kernel(const Tin *__rest
     for (int cp = 0; cp < 2; ++cp) {
         const int64_t jc = JC + 2 * tx + cp;
         if (jc >= Ptotal) continue;
-        const T M = Mpair[(int64_t)p * (n / 2) + jc];
+        const T M = Mpair[(int64_t)p * pair_stride(n) + jc];
         const int64_t gc = jc / P;
 #pragma unroll
         for (int rp = 0; rp < 2; ++rp) {
@@ -384,7 +384,7 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
         alpha_s[i] = 0;
         const T d = Fg[(int64_t)i * P + i];
         b_s[i] = sqrt(d > 0 ? d : (T)0);
-        r_s[i] = rdecay[(int64_t)p * (n / 2) + base + i];
+        r_s[i] = rdecay[(int64_t)p * pair_stride(n) + base + i];
         U_s[i] = halving_uniform<T>(seed, (uint32_t)i, cgroup, ccode, (uint32_t)p + pbase);
     }
     if (warp <= 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -524,7 +524,7 @@ static __global__ void __launch_bounds__(256) walk_warp_kernel(const T *__restri
     const int64_t base = (int64_t)g * P;
     T bmax = 0;
     const bool live = lane < P;
-    const T r = live ? rdecay[(int64_t)p * (n / 2) + base + lane] : (T)1;
+    const T r = live ? rdecay[(int64_t)p * pair_stride(n) + base + lane] : (T)1;
     uint32_t cgroup, ccode;
     call_counter(g, lvl, cgroup, ccode);
     const T U = halving_uniform<T>(seed, (uint32_t)lane, cgroup, ccode, (uint32_t)p + pbase);

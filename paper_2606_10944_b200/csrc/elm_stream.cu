@@ -23,8 +23,8 @@ static StreamLayout stream_layout(const elm_params *p, int mbar)
     L.E = take(BH * n * 4);                    // every point list is [BH][n_kv]-strided, like the lists of elm_compress
     L.T1 = take(BH * n * 4);
     L.S = take((size_t)(mbar + 1) * BH * n * 4);
-    L.Mpair = take(BH * (n / 2 + 1) * ts);
-    L.rdecay = take(BH * (n / 2 + 1) * ts);
+    L.Mpair = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
+    L.rdecay = take(BH * (size_t)(pair_stride((int64_t)n) + 1) * ts);
     L.F_stride = 4 * n_out * n_out;
     L.F = take(BH * L.F_stride * ts);
     L.ep_cap = 6 * n_out + 1;                  // Theorem 1's cache bound, plus the token itself
@@ -267,8 +267,8 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
                 c1.V = V + (int64_t)pi * n * p->d;
                 c1.vmax_bits = c.vmax_bits + pi;
                 c1.cnorm = c.cnorm + (int64_t)pi * n;
-                c1.Mpair = c.Mpair + (int64_t)pi * (n / 2);
-                c1.rdecay = c.rdecay + (int64_t)pi * (n / 2);
+                c1.Mpair = c.Mpair + (int64_t)pi * pair_stride(n);
+                c1.rdecay = c.rdecay + (int64_t)pi * pair_stride(n);
                 c1.F = c.F + (int64_t)pi * c.F_stride;
                 c1.pbase = (uint32_t)pi;
                 for (int i = 0; i < q && call_due[i]; ++i) {

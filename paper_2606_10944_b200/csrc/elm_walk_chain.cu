@@ -245,7 +245,7 @@ walk_chain_kernel(const __grid_constant__ CUtensorMap mapF, const T *__restrict_
             if (i < col0 + W) ball_s[i] = sqrt(dv[q] > 0 ? dv[q] : (T)0);
         }
     }
-    for (int i = threadIdx.x; i < col0 + W; i += nthr) rall_s[i] = rdecay[(int64_t)p * (n / 2) + base + i];
+    for (int i = threadIdx.x; i < col0 + W; i += nthr) rall_s[i] = rdecay[(int64_t)p * pair_stride(n) + base + i];
     uint32_t cgroup, ccode;
     call_counter(g, lvl, cgroup, ccode);
     for (int i = threadIdx.x; i < W; i += nthr) {

@@ -134,3 +134,16 @@ def test_ragged_rejects_bad_sizes():
         elm.compress_ragged(K, K, 3, 3, n_sink=30, n_window=30)
     with pytest.raises(elm.ElmError):
         elm.compress_ragged(K, K, 1, 6)                       # level-0 stretches below one pair
+
+
+@pytest.mark.parametrize("n", [20002, 20005, 20007])
+def test_ragged_lengths_that_are_no_multiple_of_eight(n):
+    """Calls of 64 and more pairs of the second problem on: the per-pair arrays' rows start 16-byte aligned whatever
+    n is (tensor-core Gram, vector loads).  Same cache as the fp64 mode up to decisions within rounding distance."""
+    wl = WORKLOADS["cfg5"].scaled(n=n, kv_heads=3, q_heads=3, n_q=8)
+    _, K, V = generate(wl, seed=78)
+    a, wa = elm.compress_ragged(K.cuda(), V.cuda(), 8, 7, 32, 32, seed=5, precision="fp32")
+    b, wb = elm.compress_ragged(K.cuda(), V.cuda(), 8, 7, 32, 32, seed=5, precision="fp64")
+    torch.cuda.synchronize()
+    assert torch.equal(wa, wb)
+    assert (a != b).float().mean().item() <= 0.02
