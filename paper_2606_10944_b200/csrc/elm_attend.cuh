@@ -80,4 +80,18 @@ bool attend_decode_applies(const elm_params *p);
 int attend_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int n_core,
                   const elm_params *p, void *O, unsigned char *ws, cudaStream_t st, bool timed);
 
+// The same for many tokens of a streaming run in one launch.  Window i holds the tokens tok0[i] .. tok0[i + 1] - 1 of
+// the launch (tok0[0] = 0); its list starts at entry off[i] of every problem's row of idx / w (row stride
+// list_stride), and its j-th token sees the first seen0[i] + j entries.  Q and O are [tokens][batch][q_heads][1][d].
+// Applies when the longest list a token sees has n_core entries and attend_decode_windows_apply says so; a token's
+// output is then the one attend_decode computes for it.
+constexpr int DECODE_MAX_WINDOWS = 32;
+struct DecodeWindows {
+    int32_t n;
+    int32_t tok0[DECODE_MAX_WINDOWS + 1], seen0[DECODE_MAX_WINDOWS], off[DECODE_MAX_WINDOWS];
+};
+bool attend_decode_windows_apply(const elm_params *p, int n_core);
+int attend_decode_windows(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
+                          const DecodeWindows &win, const elm_params *p, void *O, int *status, cudaStream_t st);
+
 }  // namespace elm

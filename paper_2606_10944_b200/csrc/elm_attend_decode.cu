@@ -1,167 +1,476 @@
 // Weighted attention over a coreset for a few queries per head (decode: one new token, or a handful):
 //   O[j,:] = sum_c w_c exp(<q_j,k_c>/sqrt(d)) v_c / sum_c w_c exp(<q_j,k_c>/sqrt(d))      Eq. (def:att_approx)
 // With so few queries the work is reading each coreset row of K and V once: HBM-bound, and far too
-// small for the tile kernels.  The list of an attention problem is split over `splits` CTAs; all
-// query heads that share the KV head (and all their query rows: G vectors in total, G <= 8) are
-// processed together, so a row is read once for the whole group.  Rows are read through the index
-// list straight from K and V (no gathered copy).  A warp takes one list entry at a time, a lane owns
-// D/32 consecutive dimensions: the dot products are finished with warp shuffles, the softmax is kept
-// online per query (running maximum, denominator, accumulator), the warps of a CTA and then the
-// CTAs of a problem are combined through the usual (max, denominator, accumulator) merge.
-// fp32 arithmetic on fp32 or bf16 inputs.
+// small for the tile kernels.  All query heads that share the KV head (and all their query rows: G vectors
+// in total, G <= 8) are processed together, so a row is read once for the whole group.  Rows are read through
+// the index list straight from K and V (no gathered copy).  fp32 arithmetic on fp32 or bf16 inputs.
+//
+// A warp takes a tile of 32 list entries (16 when a row is 512 bytes): the tile's K and V rows come to shared memory
+// by asynchronous copies (the next tile's keys are requested as soon as this tile's logits are formed, its values
+// behind this tile's), eight lanes share a key row, and their partial dot products are reduced AND distributed in
+// one butterfly, so that a lane ends with finished logits of its own - 14 shuffles per 16 entries of four queries
+// where a butterfly that leaves every sum in every lane needs 20 per entry.  The softmax of a tile is one entry per
+// lane; for the values a lane owns one 16-byte chunk of the row.  The instruction count per entry is what decides
+// here: the version with one entry per warp at a time and the softmax repeated in every lane issued about 120
+// instructions per entry of four bf16 queries (this one about 45) and took 68.0 us for 4 x 8 problems of 5193 entries
+// (86 MB), bound by issue; now 20.0 us (4.3 TB/s).  8 problems of 2048 entries: 8.0 -> 6.6 us, latency of the chain row
+// number -> row -> softmax -> merge.
+//
+// The list of an attention problem is split over CTAs.  elm_attend: over as many as the SMs can hold, which leave
+// partial results (maximum, denominator, accumulator) in the workspace for decode_merge_kernel.  A single token of a
+// streaming run: over the CTAs of a thread-block cluster, which hand each other their partial results through
+// distributed shared memory.  Many tokens of a streaming run in one launch (DecodeWindows: a token sees a prefix of its
+// window's list): a CTA takes as many neighbouring tokens as fit the G query vectors and walks the parts of the list
+// one after the other - the same parts, tiles and merges in the same order as the cluster's, so a token's output is the
+// same bit for bit whichever launch computes it.
 #include <math.h>
+
+#include <type_traits>
 
 #include "elm_attend.cuh"
 #include "elm_common.cuh"
+#include "elm_sm100.cuh"
 
 namespace elm {
 namespace {
 
-constexpr int DEC_WARPS = 8;
+using sm100::add2;
+using sm100::fma2;
+using sm100::mul2;
+using sm100::pack2;
+using sm100::smem_u32;
+using sm100::unpack2;
+
+constexpr int DEC_WARPS = 4;
 constexpr int DEC_GMAX = 8;
-constexpr int DEC_UNR = 4;             // list entries a warp has in flight
+constexpr int DEC_MAX_CLUSTER = 16;
 
-template <int DPL> __device__ __forceinline__ void load_dims(const float *p, float (&x)[DPL])
+template <typename Tin, int D, int G> struct DecodeCfg {
+    static constexpr int RB = D * (int)sizeof(Tin);              // bytes per row
+    static constexpr int EPC = 16 / (int)sizeof(Tin);            // elements per 16-byte chunk
+    static constexpr int NC = RB / 16;                           // chunks per row: 8, 16 or 32
+    static constexpr int CH = NC / 8;                            // chunks of a key row per lane (eight lanes share a row)
+    static constexpr int TILE = RB > 256 ? 16 : 32;              // entries per warp tile
+    static constexpr int UB = G == 8 ? 2 : 4;                    // entries whose dot products a lane forms at a time
+    static constexpr int NV = UB * G;                            // partial sums per lane: 4, 8 or 16
+    static constexpr int EPI = 32 / NC;                          // entries a warp takes at a time in the value pass
+    static constexpr int TILE_BYTES = TILE * RB;
+    // shared memory: per warp a K tile, a V tile and the tile's logits; the scaled queries; what the cluster sends
+    static constexpr int OFF_SC = DEC_WARPS * 2 * TILE_BYTES;
+    static constexpr int OFF_Q = OFF_SC + DEC_WARPS * 32 * G * 4;
+    static constexpr int OFF_ML = OFF_Q + G * D * 4;             // [DEC_WARPS][G][2]
+    static constexpr int OFF_RML = OFF_ML + DEC_WARPS * G * 2 * 4;      // [DEC_MAX_CLUSTER][G][2]
+    // [ranks][slice] with slice = ceil(G D / ranks): at most G D + DEC_MAX_CLUSTER floats
+    static constexpr int OFF_RECV = OFF_RML + DEC_MAX_CLUSTER * G * 2 * 4;
+    static constexpr int TOTAL = OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4;
+};
+
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool live)
 {
-    if constexpr (DPL == 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-    } else {
-        const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
-        x[0] = v.x; x[1] = v.y;
-    }
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
 }
-template <int DPL> __device__ __forceinline__ void load_dims(const __nv_bfloat16 *p, float (&x)[DPL])
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// the elements of a 16-byte chunk as packed pairs of floats
+__device__ __forceinline__ void chunk_pairs(const uint4 &x, uint64_t (&f)[4], const __nv_bfloat16 *)
 {
-    if constexpr (DPL == 4) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
-        x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xffff0000u);
-        x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xffff0000u);
-    } else {
-        const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(p));
-        x[0] = __uint_as_float(v << 16); x[1] = __uint_as_float(v & 0xffff0000u);
-    }
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+}
+__device__ __forceinline__ void chunk_pairs(const uint4 &x, uint64_t (&f)[2], const float *)
+{
+    f[0] = pack2(__uint_as_float(x.x), __uint_as_float(x.y));
+    f[1] = pack2(__uint_as_float(x.z), __uint_as_float(x.w));
 }
 
-// partial results: part[problem][split][g][D + 2] = accumulator (D), running maximum, denominator
-template <typename Tin, int D, int G>
-__global__ void __launch_bounds__(DEC_WARPS * 32)
-decode_partial_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *__restrict__ V,
-                      const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int n_core, int q_heads,
-                      int kv_heads, int n_q, int groups /* live query vectors <= G */, int chunk, float *__restrict__ part,
-                      int *__restrict__ status)
+// folds a part's (maximum, denominator, accumulator) into the running ones
+__device__ __forceinline__ void merge_part(float &M, float &den, float &acc, float m, float d, float x)
 {
-    constexpr int DPL = D / 32;
-    __shared__ float sm_o[DEC_WARPS][G][D];
-    __shared__ float sm_ml[DEC_WARPS][G][2];
+    const float Mn = fmaxf(M, m);
+    const float a = M == -INFINITY ? 0.f : exp2f(M - Mn), b = m == -INFINITY ? 0.f : exp2f(m - Mn);
+    den = fmaf(b, d, __fmul_rn(den, a));
+    acc = fmaf(b, x, __fmul_rn(acc, a));
+    M = Mn;
+}
+
+// DEC_TOKENS: which tokens a CTA takes
+struct DecodeGroups {
+    int32_t per_group;                             // tokens per CTA: a power of two, at most 8
+    int32_t g0[DECODE_MAX_WINDOWS + 1];            // groups of the windows before
+};
+
+// How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp, at most `cap` parts.
+// Depends on n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
+__host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entries, int tile, int cap, int &parts, int &chunk)
+{
+    const int len = (n_core + 127) / 128 * 128;
+    const int t = (len + 2 * cta_entries - 1) / (2 * cta_entries);
+    parts = t < 1 ? 1 : (t < cap ? t : cap);
+    chunk = ((len + parts - 1) / parts + tile - 1) / tile * tile;
+}
+
+// grid (splits, problems); partial results part[problem][split][g][D + 2] = accumulator (D), maximum, denominator
+constexpr int DEC_SPLIT = 0;
+// grid (cluster size, problems), one token: rank r of the cluster takes the r-th part of the list
+constexpr int DEC_CLUSTER = 1;
+// grid (token groups, problems): neighbouring tokens, part after part
+constexpr int DEC_TOKENS = 2;
+
+template <typename Tin, int D, int G, int MODE>
+__global__ void __launch_bounds__(DEC_WARPS * 32, 3)
+decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *__restrict__ V,
+              const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int64_t list_stride, int q_heads,
+              int kv_heads, int n_q, int per_token /* query vectors of a token */, const __grid_constant__ DecodeWindows win,
+              const __grid_constant__ DecodeGroups grp, int cap, Tin *__restrict__ O, float *__restrict__ part,
+              int *__restrict__ status)
+{
+    using C = DecodeCfg<Tin, D, G>;
+    constexpr int TILE = C::TILE, NC = C::NC, CH = C::CH, EPC = C::EPC, UB = C::UB, NV = C::NV, EPI = C::EPI;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char *kt = smem + warp * 2 * C::TILE_BYTES, *vt = kt + C::TILE_BYTES;
+    float *sc = reinterpret_cast<float *>(smem + C::OFF_SC) + warp * 32 * G;      // [entry][g] logits, then probabilities
+    float *qs = reinterpret_cast<float *>(smem + C::OFF_Q);
+    float *ml = reinterpret_cast<float *>(smem + C::OFF_ML);
+    float *recv = reinterpret_cast<float *>(smem + C::OFF_RECV), *rml = reinterpret_cast<float *>(smem + C::OFF_RML);
     // (launched with programmatic stream serialization: resident before the kernel in front of it has finished;
-    // nothing is read before this point)
+    // nothing is read or written before this point)
     cudaGridDependencySynchronize();
-    const int prob = blockIdx.y, split = blockIdx.x, splits = gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = prob / kv_heads, kvh = prob % kv_heads, rep = q_heads / kv_heads;
-    const float scale = 1.4426950408889634f / sqrtf((float)D);
-
-    // query vector g = (head within the group) * n_q + row
-    float q[G][DPL];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-#pragma unroll
-        for (int i = 0; i < DPL; ++i) q[g][i] = 0.f;
-        if (g < groups) {
-            const int h = kvh * rep + g / n_q, r = g % n_q;
-            load_dims<DPL>(Q + (((int64_t)b * q_heads + h) * n_q + r) * D + lane * DPL, q[g]);
-#pragma unroll
-            for (int i = 0; i < DPL; ++i) q[g][i] *= scale;
-        }
+    if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const int prob = blockIdx.y, rank = MODE == DEC_TOKENS ? 0 : blockIdx.x;
+#ifndef ELM_BOUNDS_CHECK
+    // this path has no bounded waits and (in this build) no row checks: its status word reads 0 - written here
+    // rather than by a memset of its own
+    if (tid == 0 && prob == 0 && blockIdx.x == 0) *status = 0;
+#endif
+    // the tokens: z0 .. z0 + tokens - 1 of the launch, the first of which sees seen0 entries, the next one more, ...
+    int wi = 0, z0 = 0, tokens = 1, seen0 = win.seen0[0];
+    if constexpr (MODE == DEC_TOKENS) {
+        while (wi + 1 < win.n && (int)blockIdx.x >= grp.g0[wi + 1]) ++wi;
+        // group k of a window: the tokens that see (k0 + k) per_group + 1 .. (k0 + k + 1) per_group entries
+        const int first = ((win.seen0[wi] - 1) / grp.per_group + ((int)blockIdx.x - grp.g0[wi])) * grp.per_group + 1;
+        const int last_seen = win.seen0[wi] + (win.tok0[wi + 1] - win.tok0[wi]) - 1;
+        seen0 = first > win.seen0[wi] ? first : win.seen0[wi];
+        const int end = first + grp.per_group - 1 < last_seen ? first + grp.per_group - 1 : last_seen;
+        tokens = end - seen0 + 1;
+        z0 = win.tok0[wi] + (seen0 - win.seen0[wi]);
     }
-    float m[G], l[G], o[G][DPL];
+    const int n_core = seen0 + tokens - 1;                         // what the last token sees
+    const int groups = tokens * per_token;                         // live query vectors
+    int parts, chunk;
+    if constexpr (MODE == DEC_SPLIT) {
+        // whole tiles per part, so that only the end of the list leaves a tile partly filled
+        parts = gridDim.x;
+        chunk = ((n_core + parts - 1) / parts + TILE - 1) / TILE * TILE;
+    } else {
+        decode_parts(n_core, DEC_WARPS * TILE, TILE, cap, parts, chunk);
+    }
+    const int b = prob / kv_heads, kvh = prob % kv_heads, rep = q_heads / kv_heads;
+    const int32_t *ip = idx + (int64_t)prob * list_stride + win.off[wi];
+    const float *wp = w + (int64_t)prob * list_stride + win.off[wi];
+    const Tin *Kp = K + (int64_t)prob * n * D, *Vp = V + (int64_t)prob * n * D;
+    // offset of query vector g's row in Q and O: token g / per_token, in it (head within the group) * n_q + row
+    auto q_row = [&](int g) -> int64_t {
+        const int64_t z = z0 + g / per_token;
+        const int in = g % per_token;
+        return (((z * (gridDim.y / kv_heads) + b) * q_heads + kvh * rep + in / n_q) * n_q + in % n_q) * D;
+    };
+    int c0, c1 = 0;                                                // the part being worked on
+
+    // row number and log2 weight of the tile's entry `lane`
+    int32_t row = 0, row_next = 0;
+    float lw = 0.f, lw_next = 0.f;
+    auto fetch_entries = [&](int t0) {
+        row_next = 0;
+        lw_next = -INFINITY;
+        if (lane < TILE && t0 + lane < c1) {
+            row_next = (int32_t)checked_row(__ldg(ip + t0 + lane), n, status);
+            lw_next = __ldg(wp + t0 + lane);
+        }
+    };
+    // the rows of a tile, chunk by chunk: chunk q = lane + 32 i of the tile lies in entry q / NC.  Entries past the end
+    // read as zeros, so that nothing they might hold meets their zero probability.
+    auto copy_rows = [&](unsigned char *dst, const Tin *X, int32_t rows, int t0) {
+        const uint32_t d0 = smem_u32(dst);
+#pragma unroll
+        for (int i = 0; i < TILE / EPI; ++i) {
+            const int e = lane / NC + i * EPI;
+            const int64_t r = __shfl_sync(0xffffffffu, rows, e);
+            cp_async16_zfill(d0 + (lane + 32 * i) * 16, X + r * D + (lane % NC) * EPC, t0 + e < c1);
+        }
+        cp_async_commit();
+    };
+    // the query vectors, scaled; laid out so that the eight lanes of a key row read
+    // 128 contiguous bytes: [g][chunk / 8][16-byte half][chunk % 8][4]
+    const float scale = 1.4426950408889634f / sqrtf((float)D);
+    for (int i = tid; i < G * D; i += DEC_WARPS * 32) {
+        const int g = i / D, dim = i % D, ck = dim / EPC, in = dim % EPC;
+        float x = 0.f;
+        if (g < groups) x = load_as<float>(Q, q_row(g) + dim) * scale;
+        qs[(((g * CH + ck / 8) * (EPC / 4) + in / 4) * 8 + ck % 8) * 4 + in % 4] = x;
+    }
+    if constexpr (MODE == DEC_TOKENS) {
+        for (int i = tid; i < G * D; i += DEC_WARPS * 32) recv[i] = 0.f;       // (each element stays with its thread)
+        if (tid < G) { rml[tid * 2] = -INFINITY; rml[tid * 2 + 1] = 0.f; }
+    }
+    // what query vector g sees of the list (DEC_TOKENS: its token's prefix)
+    auto limit = [&](int g) { return MODE == DEC_TOKENS ? seen0 + g / per_token : n_core; };
+    const int gl = lane >> 3, sub = lane & 7;
+
+    for (int pt = rank; pt < (MODE == DEC_TOKENS ? parts : rank + 1); ++pt) {
+    c0 = pt * chunk < n_core ? pt * chunk : n_core;
+    c1 = pt < parts ? (c0 + chunk < n_core ? c0 + chunk : n_core) : c0;
+    int t0 = c0 + warp * TILE;
+    fetch_entries(t0);
+    row = row_next;
+    lw = log2f(lw_next);
+    // (the queries are laid out / the merge of the part before has read the tiles)
+    __syncthreads();
+    if (t0 < c1) {
+        copy_rows(kt, Kp, row, t0);
+        copy_rows(vt, Vp, row, t0);
+        fetch_entries(t0 + DEC_WARPS * TILE);
+    }
+    float m[G], l[G];
+    uint64_t o[G][EPC / 2];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         m[g] = -INFINITY;
         l[g] = 0.f;
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) o[g][i] = 0.f;
+        for (int i = 0; i < EPC / 2; ++i) o[g][i] = 0;
     }
-    const int c0 = split * chunk, c1 = c0 + chunk < n_core ? c0 + chunk : n_core;
-    const int32_t *ip = idx + (int64_t)prob * n_core;
-    const float *wp = w + (int64_t)prob * n_core;
-    const Tin *Kp = K + (int64_t)prob * n * D, *Vp = V + (int64_t)prob * n * D;
-    // DEC_UNR entries per warp at a time: their row numbers, then all their K and V rows are requested
-    // before the first one is used, so that several rows per warp are in flight (the kernel has
-    // nothing to hide the memory latency with but its own loads)
-    int32_t myrow = 0;
-    float mylw = 0.f;
-    auto fetch_entries = [&](int e0) {                                   // lane j < DEC_UNR: entry e0 + j
-        myrow = 0;
-        mylw = 0.f;
-        if (lane < DEC_UNR && e0 + lane < c1) {
-            myrow = (int32_t)checked_row(__ldg(ip + e0 + lane), n, status);
-            mylw = log2f(__ldg(wp + e0 + lane));
+    for (; t0 < c1; t0 += DEC_WARPS * TILE) {
+        const bool more = t0 + DEC_WARPS * TILE < c1;
+        // ---- logits: entry gl + 4 u of the tile by the eight lanes of group gl ----
+        cp_async_wait<1>();                                        // the keys (the values are the newer group)
+        __syncwarp();
+#pragma unroll
+        for (int ub = 0; ub < TILE / 4 / UB; ++ub) {
+            uint64_t acc[UB][G];
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+#pragma unroll
+                for (int g = 0; g < G; ++g) acc[u][g] = 0;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                uint64_t kf[UB][EPC / 2];
+#pragma unroll
+                for (int u = 0; u < UB; ++u) {
+                    const int e = gl + 4 * (ub * UB + u);
+                    chunk_pairs(*reinterpret_cast<const uint4 *>(kt + (e * NC + c * 8 + sub) * 16), kf[u], (const Tin *)nullptr);
+                }
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+#pragma unroll
+                    for (int h = 0; h < EPC / 4; ++h) {
+                        const float4 q4 = *reinterpret_cast<const float4 *>(qs + (((g * CH + c) * (EPC / 4) + h) * 8 + sub) * 4);
+                        const uint64_t qa = pack2(q4.x, q4.y), qb = pack2(q4.z, q4.w);
+#pragma unroll
+                        for (int u = 0; u < UB; ++u) acc[u][g] = fma2(kf[u][2 * h + 1], qb, fma2(kf[u][2 * h], qa, acc[u][g]));
+                    }
+                }
+            }
+            // reduce over the eight lanes and leave each with its share of the NV sums
+            float v[NV];
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    float lo, hi;
+                    unpack2(acc[u][g], lo, hi);
+                    v[u * G + g] = lo + hi;
+                }
+            int base = 0;
+            {
+                int cnt = NV;
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) {
+                    if (cnt >= 2) {
+                        const bool up = (sub & off) != 0;
+                        cnt >>= 1;
+#pragma unroll
+                        for (int i = 0; i < NV / 2; ++i) {
+                            if (i < cnt) {
+                                const float send = up ? v[i] : v[i + cnt], keep = up ? v[i + cnt] : v[i];
+                                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                            }
+                        }
+                        base += up ? cnt : 0;
+                    } else {
+                        v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+                    }
+                }
+            }
+            constexpr int LEFT = NV >= 8 ? NV / 8 : 1;             // finished sums in this lane
+#pragma unroll
+            for (int i = 0; i < LEFT; ++i) {
+                const int j = base + i, u = j / G, g = j % G;
+                sc[(gl + 4 * (ub * UB + u)) * G + g] = v[i];
+            }
         }
-    };
-    fetch_entries(c0 + warp * DEC_UNR);
-    for (int e0 = c0 + warp * DEC_UNR; e0 < c1; e0 += DEC_WARPS * DEC_UNR) {
-        float k[DEC_UNR][DPL], v[DEC_UNR][DPL], lw[DEC_UNR];
+        __syncwarp();
+        const int32_t row_ahead = row_next;
+        const float lw_ahead = lw_next;
+        if (more) copy_rows(kt, Kp, row_ahead, t0 + DEC_WARPS * TILE);
+        // ---- softmax of the tile, one entry per lane ----
+        float alpha[G];
 #pragma unroll
-        for (int j = 0; j < DEC_UNR; ++j) {
-            const int64_t row = __shfl_sync(0xffffffffu, myrow, j);
-            lw[j] = __shfl_sync(0xffffffffu, mylw, j);
-            load_dims<DPL>(Kp + row * D + lane * DPL, k[j]);            // (row 0 for entries past the end: unused)
-            load_dims<DPL>(Vp + row * D + lane * DPL, v[j]);
+        for (int g = 0; g < G; ++g) {
+            const bool live = lane < TILE && t0 + lane < (MODE == DEC_TOKENS ? min(c1, limit(g)) : c1);
+            const float s = live ? sc[lane * G + g] + lw : -INFINITY;            // base-2 logit
+            float mx = s;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            mx = fmaxf(m[g], mx);
+            const float ref = mx == -INFINITY ? 0.f : mx;
+            alpha[g] = exp2f(m[g] - ref);                                        // exp2f(-inf) = 0 on the first tile
+            const float pw = live ? exp2f(s - ref) : 0.f;
+            l[g] = fmaf(l[g], alpha[g], pw);
+            m[g] = mx;
+            sc[lane * G + g] = pw;
         }
-        fetch_entries(e0 + DEC_WARPS * DEC_UNR);                         // the next batch's row numbers, behind the rows
 #pragma unroll
-        for (int j = 0; j < DEC_UNR; ++j) {
-            if (e0 + j >= c1) break;
-            float s[G];
+        for (int g = 0; g < G; ++g) {
+            const uint64_t a2 = pack2(alpha[g], alpha[g]);
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                float a = 0.f;
+            for (int i = 0; i < EPC / 2; ++i) o[g][i] = mul2(o[g][i], a2);
+        }
+        // ---- values: lane owns chunk lane % NC of a row, EPI entries at a time ----
+        if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
+        else cp_async_wait<0>();
+        __syncwarp();
+        const int filled = c1 - t0 < TILE ? c1 - t0 : TILE;
+#pragma unroll 4
+        for (int i = 0; i < TILE / EPI; ++i) {
+            if (i * EPI >= filled) break;
+            const int e = i * EPI + lane / NC;
+            uint64_t vf[EPC / 2];
+            chunk_pairs(*reinterpret_cast<const uint4 *>(vt + (lane + 32 * i) * 16), vf, (const Tin *)nullptr);
+            float pe[G];
+            if constexpr (G >= 4) {
 #pragma unroll
-                for (int i = 0; i < DPL; ++i) a = fmaf(q[g][i], k[j][i], a);
-                s[g] = a;
+                for (int g = 0; g < G; g += 4) {
+                    const float4 p4 = *reinterpret_cast<const float4 *>(sc + e * G + g);
+                    pe[g] = p4.x; pe[g + 1] = p4.y; pe[g + 2] = p4.z; pe[g + 3] = p4.w;
+                }
+            } else {
+#pragma unroll
+                for (int g = 0; g < G; ++g) pe[g] = sc[e * G + g];
             }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-                for (int g = 0; g < G; ++g) s[g] += __shfl_xor_sync(0xffffffffu, s[g], off);
-#pragma unroll
             for (int g = 0; g < G; ++g) {
-                const float sg = s[g] + lw[j];                               // base-2 logit
-                const float mn = fmaxf(m[g], sg);
-                const float a = exp2f(m[g] - mn), pw = exp2f(sg - mn);       // exp2f(-inf) = 0 on the first entry
-                l[g] = l[g] * a + pw;
+                // (an entry behind the token's own must not meet its zero probability: it might be infinite)
+                if (MODE == DEC_TOKENS && t0 + TILE > seen0 && t0 + e >= limit(g)) continue;
+                const uint64_t p2 = pack2(pe[g], pe[g]);
 #pragma unroll
-                for (int i = 0; i < DPL; ++i) o[g][i] = o[g][i] * a + pw * v[j][i];
-                m[g] = mn;
+                for (int j = 0; j < EPC / 2; ++j) o[g][j] = fma2(p2, vf[j], o[g][j]);
             }
         }
+        __syncwarp();
+        if (more) {
+            copy_rows(vt, Vp, row_ahead, t0 + DEC_WARPS * TILE);
+            lw = log2f(lw_ahead);
+            fetch_entries(t0 + 2 * DEC_WARPS * TILE);
+        }
     }
-    // combine the warps of the CTA
+
+    // ---- the warp's partial result, over its own K tile ----
+    float *po = reinterpret_cast<float *>(kt);                     // [g][D]
 #pragma unroll
     for (int g = 0; g < G; ++g) {
+        float ls = l[g];
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) sm_o[warp][g][lane * DPL + i] = o[g][i];
-        if (lane == 0) { sm_ml[warp][g][0] = m[g]; sm_ml[warp][g][1] = l[g]; }
+        for (int off = 16; off > 0; off >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, off);
+        if (lane == 0) {
+            ml[(warp * G + g) * 2] = m[g];
+            ml[(warp * G + g) * 2 + 1] = ls;
+        }
+#pragma unroll
+        for (int i = 0; i < EPC / 2; ++i) {
+            float x, y;
+            unpack2(o[g][i], x, y);
+#pragma unroll
+            for (int off = NC; off < 32; off <<= 1) {
+                x += __shfl_xor_sync(0xffffffffu, x, off);
+                y += __shfl_xor_sync(0xffffffffu, y, off);
+            }
+            if (lane < NC) *reinterpret_cast<float2 *>(po + g * D + lane * EPC + 2 * i) = make_float2(x, y);
+        }
     }
     __syncthreads();
-    float *out = part + (((int64_t)prob * splits + split) * G) * (D + 2);
-    for (int t = threadIdx.x; t < G * D; t += DEC_WARPS * 32) {
-        const int g = t / D, d = t % D;
-        float M = -INFINITY;
+    // ---- the part's result: to the workspace, to the cluster rank that finishes this slice of the output, or merged
+    // into what the parts before left ----
+    const int slice = (G * D + parts - 1) / parts;
+    // every CTA of the cluster is running (its shared memory may be written) once this wait is over
+    if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    auto remote = [&](const float *mine, int to) -> uint32_t {
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(to));
+        return a;
+    };
+    if (pt < parts) {
+        for (int i = tid; i < G * D; i += DEC_WARPS * 32) {
+            const int g = i / D;
+            float M = -INFINITY;
 #pragma unroll
-        for (int wv = 0; wv < DEC_WARPS; ++wv) M = fmaxf(M, sm_ml[wv][g][0]);
-        float acc = 0.f, den = 0.f;
+            for (int wv = 0; wv < DEC_WARPS; ++wv) M = fmaxf(M, ml[(wv * G + g) * 2]);
+            float acc = 0.f, den = 0.f;
 #pragma unroll
-        for (int wv = 0; wv < DEC_WARPS; ++wv) {
-            const float mw = sm_ml[wv][g][0];
-            const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
-            acc += f * sm_o[wv][g][d];
-            den += f * sm_ml[wv][g][1];
+            for (int wv = 0; wv < DEC_WARPS; ++wv) {
+                const float mw = ml[(wv * G + g) * 2];
+                const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
+                acc = fmaf(f, reinterpret_cast<const float *>(smem + wv * 2 * C::TILE_BYTES)[i], acc);
+                den = fmaf(f, ml[(wv * G + g) * 2 + 1], den);
+            }
+            if constexpr (MODE == DEC_CLUSTER) {
+                const int to = i / slice;
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(recv + rank * slice + i - to * slice, to)), "f"(acc) : "memory");
+                if (i % D < parts) {                               // (parts <= 16 <= D: one thread per (g, rank))
+                    const uint32_t a = remote(rml + (rank * G + g) * 2, i % D);
+                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(M) : "memory");
+                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a + 4), "f"(den) : "memory");
+                }
+            } else if constexpr (MODE == DEC_TOKENS) {
+                // (running maximum and denominator in two buffers, part pt reading one and writing the other)
+                const float *was = rml + ((pt & 1) * G + g) * 2;
+                float Mr = was[0], dr = was[1], ar = recv[i];
+                merge_part(Mr, dr, ar, M, den, acc);
+                recv[i] = ar;
+                if (i % D == 0) {
+                    float *now = rml + (((pt + 1) & 1) * G + g) * 2;
+                    now[0] = Mr;
+                    now[1] = dr;
+                }
+            } else {
+                float *out = part + (((int64_t)prob * gridDim.x + rank) * G + g) * (D + 2);
+                out[i % D] = acc;
+                if (i % D == 0) { out[D] = M; out[D + 1] = den; }
+            }
         }
-        out[g * (D + 2) + d] = acc;
-        if (d == 0) { out[g * (D + 2) + D] = M; out[g * (D + 2) + D + 1] = den; }
+    }
+    if constexpr (MODE == DEC_CLUSTER) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        const int i1 = (rank + 1) * slice < G * D ? (rank + 1) * slice : G * D;
+        if (rank < parts) {
+            for (int i = rank * slice + tid; i < i1; i += DEC_WARPS * 32) {
+                const int g = i / D;
+                if (g >= groups) break;
+                float M = -INFINITY, den = 0.f, acc = 0.f;
+                for (int r = 0; r < parts; ++r)
+                    merge_part(M, den, acc, rml[(r * G + g) * 2], rml[(r * G + g) * 2 + 1], recv[r * slice + i - rank * slice]);
+                store_from(O, q_row(g) + i % D, acc / den);
+            }
+        }
+    }
+    }
+    if constexpr (MODE == DEC_TOKENS) {
+        __syncthreads();
+        for (int i = tid; i < groups * D; i += DEC_WARPS * 32)
+            store_from(O, q_row(i / D) + i % D, recv[i] / rml[((parts & 1) * G + i / D) * 2 + 1]);
     }
 }
 
@@ -172,17 +481,12 @@ decode_partial_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, cons
 constexpr int DEC_MAX_SPLITS = 256;
 template <typename Tin, int D, int G>
 __global__ void __launch_bounds__(D) decode_merge_kernel(const float *__restrict__ part, int splits, int q_heads, int kv_heads,
-                                                         int n_q, Tin *__restrict__ O, int *__restrict__ status)
+                                                         int n_q, Tin *__restrict__ O)
 {
     __shared__ float sf[DEC_MAX_SPLITS];
     __shared__ float red[2][D / 32];
     const int prob = blockIdx.y, g = blockIdx.x, d = threadIdx.x;
     const int warp = d >> 5, lane = d & 31;
-#ifndef ELM_BOUNDS_CHECK
-    // this path has no bounded waits and (in this build) no row checks: its status word reads 0 - written here
-    // rather than by a memset of its own, which would be a third of a decode step's launches
-    if (prob == 0 && g == 0 && d == 0) *status = 0;
-#endif
     const int b = prob / kv_heads, kvh = prob % kv_heads, rep = q_heads / kv_heads;
     const float *p = part + ((int64_t)prob * splits * G + g) * (D + 2);
     // launched with programmatic stream serialization: the CTAs of this kernel are resident while the partial
@@ -240,51 +544,117 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float *__restrict
     store_from(O, (((int64_t)b * q_heads + h) * n_q + r) * D + d, acc / den);
 }
 
-template <typename Tin, int D, int G>
-int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, const float *w, int n_core,
-                  const elm_params *p, Tin *O, float *part, int *status, int splits, int groups, cudaStream_t st)
+// Streaming tokens: most parts of a list - a power of two, so that three CTAs per SM (what shared memory allows) hold
+// one token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
+// most SMs idle is left to the form with partial results in the workspace.
+static int decode_cap(int problems)
 {
+    const int most = 3 * device_sm_count() / problems;
+    int cap = DEC_MAX_CLUSTER;
+    while (cap > 1 && cap > most) cap >>= 1;
+    return cap;
+}
+template <typename Tin, int D, int G> bool decode_clustered(int n_core, int problems)
+{
+    const int cap = decode_cap(problems), entries = DEC_WARPS * DecodeCfg<Tin, D, G>::TILE;
+    return n_core <= 8 * entries * cap || problems * cap >= device_sm_count();
+}
+
+// win set: streaming tokens (G counts the query vectors of a CTA: of one token, or of several when the launch holds
+// more than one); else the list of elm_attend, n_core entries long
+template <typename Tin, int D, int G>
+int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
+                  const DecodeWindows *win, const elm_params *p, Tin *O, float *part, size_t part_room, int *status, int per_token,
+                  cudaStream_t st)
+{
+    using C = DecodeCfg<Tin, D, G>;
     const int problems = p->batch * p->kv_heads;
-    const int chunk = (n_core + splits - 1) / splits;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)splits, (unsigned)problems);
-        cfg.blockDim = dim3(DEC_WARPS * 32);
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int64_t n_kv = p->n_kv;
-        int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
-        ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_kernel<Tin, D, G>, Q, K, V, idx, w, n_kv, n_core, q_heads, kv_heads,
-                                        n_q, groups, chunk, part, status));
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(DEC_WARPS * 32);
+    cfg.dynamicSmemBytes = C::TOTAL;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const int64_t n_kv = p->n_kv;
+    const int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
+    DecodeGroups grp = {};
+    if (win) {
+        const int cap = decode_cap(problems), tokens = win->tok0[win->n];
+        auto kern = tokens == 1 ? decode_kernel<Tin, D, G, DEC_CLUSTER> : decode_kernel<Tin, D, G, DEC_TOKENS>;
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::TOTAL));
+        if (tokens == 1) {
+            int parts, chunk, size = 1;
+            decode_parts(win->seen0[0], DEC_WARPS * C::TILE, C::TILE, cap, parts, chunk);
+            while (size < parts) size <<= 1;
+            if (size > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            attr[1].id = cudaLaunchAttributeClusterDimension;
+            attr[1].val.clusterDim.x = (unsigned)size;
+            attr[1].val.clusterDim.y = 1;
+            attr[1].val.clusterDim.z = 1;
+            cfg.numAttrs = 2;
+            cfg.gridDim = dim3((unsigned)size, (unsigned)problems);
+        } else {
+            grp.per_group = 1;
+            while (grp.per_group * 2 * per_token <= G) grp.per_group *= 2;
+            for (int i = 0; i < win->n; ++i) {
+                const int last = win->seen0[i] + (win->tok0[i + 1] - win->tok0[i]) - 1;
+                grp.g0[i + 1] = grp.g0[i] + (last - 1) / grp.per_group - (win->seen0[i] - 1) / grp.per_group + 1;
+            }
+            cfg.gridDim = dim3((unsigned)grp.g0[win->n], (unsigned)problems);
+        }
+        ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, *win, grp,
+                                        cap, O, (float *)nullptr, status));
+        count_launches(1);
+        return cuda_status(cudaGetLastError());
     }
-    {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)groups, (unsigned)problems);
-        cfg.blockDim = dim3(D);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const float *part_c = part;
-        int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
-        ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_merge_kernel<Tin, D, G>, part_c, splits, q_heads, kv_heads, n_q, O, status));
-    }
+    DecodeWindows whole = {};
+    whole.n = 1;
+    whole.tok0[1] = 1;
+    whole.seen0[0] = n_core;
+    // as many CTAs as are resident at once, but at least one tile per warp
+    int splits = (n_core + DEC_WARPS * C::TILE - 1) / (DEC_WARPS * C::TILE);
+    const int wanted = 3 * device_sm_count() / problems;
+    if (splits > wanted) splits = wanted < 1 ? 1 : wanted;
+    const size_t most = part_room / ((size_t)problems * G * (D + 2) * sizeof(float));
+    if ((size_t)splits > most) splits = (int)most;
+    if (splits > DEC_MAX_SPLITS) splits = DEC_MAX_SPLITS;
+    if (splits < 1) return ELM_ERR_WORKSPACE;
+    auto kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
+    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::TOTAL));
+    cfg.gridDim = dim3((unsigned)splits, (unsigned)problems);
+    ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, whole, grp, 0, O,
+                                    part, status));
+    cfg.gridDim = dim3((unsigned)per_token, (unsigned)problems);
+    cfg.blockDim = dim3(D);
+    cfg.dynamicSmemBytes = 0;
+    const float *part_c = part;
+    ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_merge_kernel<Tin, D, G>, part_c, splits, q_heads, kv_heads, n_q, O));
     count_launches(2);
     return cuda_status(cudaGetLastError());
 }
 
-template <typename Tin, int D>
-int dispatch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, const float *w, int n_core,
-                    const elm_params *p, Tin *O, float *part, int *status, int splits, int groups, cudaStream_t st)
+// Calls `f` with the compile-time query count that covers `groups`
+template <typename F> int with_groups(int groups, F f)
 {
-    if (groups <= 1) return launch_decode<Tin, D, 1>(Q, K, V, idx, w, n_core, p, O, part, status, splits, groups, st);
-    if (groups <= 2) return launch_decode<Tin, D, 2>(Q, K, V, idx, w, n_core, p, O, part, status, splits, groups, st);
-    if (groups <= 4) return launch_decode<Tin, D, 4>(Q, K, V, idx, w, n_core, p, O, part, status, splits, groups, st);
-    return launch_decode<Tin, D, 8>(Q, K, V, idx, w, n_core, p, O, part, status, splits, groups, st);
+    if (groups <= 1) return f(std::integral_constant<int, 1>());
+    if (groups <= 2) return f(std::integral_constant<int, 2>());
+    if (groups <= 4) return f(std::integral_constant<int, 4>());
+    return f(std::integral_constant<int, 8>());
+}
+template <typename Tin>
+int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
+                    const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
+{
+    const int per_token = (p->q_heads / p->kv_heads) * p->n_q;
+    return with_groups(win && win->tok0[win->n] > 1 ? DEC_GMAX : per_token, [&](auto G) {
+        const Tin *q = (const Tin *)Q, *k = (const Tin *)K, *v = (const Tin *)V;
+        constexpr int g = decltype(G)::value;
+        return p->d == 64 ? launch_decode<Tin, 64, g>(q, k, v, idx, w, list_stride, n_core, win, p, (Tin *)O, part, part_room, status, per_token, st)
+                          : launch_decode<Tin, 128, g>(q, k, v, idx, w, list_stride, n_core, win, p, (Tin *)O, part, part_room, status, per_token, st);
+    });
 }
 
 }  // namespace
@@ -296,42 +666,43 @@ bool attend_decode_applies(const elm_params *p)
     return groups <= DEC_GMAX;
 }
 
+bool attend_decode_windows_apply(const elm_params *p, int n_core)
+{
+    if (!attend_decode_applies(p) || p->n_q != 1 || (p->dtype != ELM_F32 && p->dtype != ELM_BF16)) return false;
+    const int problems = p->batch * p->kv_heads;
+    // (a tile's entries do not depend on the number of query vectors)
+    if (p->dtype == ELM_F32)
+        return p->d == 64 ? decode_clustered<float, 64, 1>(n_core, problems) : decode_clustered<float, 128, 1>(n_core, problems);
+    return p->d == 64 ? decode_clustered<__nv_bfloat16, 64, 1>(n_core, problems) : decode_clustered<__nv_bfloat16, 128, 1>(n_core, problems);
+}
+
+int attend_decode_windows(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
+                          const DecodeWindows &win, const elm_params *p, void *O, int *status, cudaStream_t st)
+{
+    StageTimer t(ELM_STAGE_ATTEND, st, 1);
+#ifdef ELM_BOUNDS_CHECK
+    ELM_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
+#endif
+    return p->dtype == ELM_F32 ? dispatch_decode<float>(Q, K, V, idx, w, list_stride, 0, &win, p, O, nullptr, 0, status, st)
+                               : dispatch_decode<__nv_bfloat16>(Q, K, V, idx, w, list_stride, 0, &win, p, O, nullptr, 0, status, st);
+}
+
 int attend_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int n_core,
                   const elm_params *p, void *O, unsigned char *ws, cudaStream_t st, bool timed)
 {
     const AttendLayout L = attend_layout(p, n_core);
     const int problems = p->batch * p->kv_heads;
-    const int groups = (p->q_heads / p->kv_heads) * p->n_q;
-    const int G = groups <= 1 ? 1 : groups <= 2 ? 2 : groups <= 4 ? 4 : 8;
     // the partial results live where the other paths keep their gathered operands
-    const size_t room = L.bias - L.Kc;
-    const size_t per_split = (size_t)problems * G * (p->d + 2) * sizeof(float);
-    // enough CTAs for about two per SM, but at least one batch of entries per warp
-    const int sm_count = device_sm_count();
-    int splits = (n_core + DEC_WARPS * DEC_UNR - 1) / (DEC_WARPS * DEC_UNR);
-    // (3, 4, 6, 8 per SM were measured: 27 / 24 / 24 / 24 us at 2048 entries and 52 / 49 / 53 / 58 us at 12288 against 22 / 43)
-    const int wanted = (2 * sm_count + problems - 1) / problems;
-    if (splits > wanted) splits = wanted;
-    const int most = (int)(room / per_split);
-    if (splits > most) splits = most;
-    if (splits > 256) splits = 256;
-    if (splits < 1) return ELM_ERR_WORKSPACE;
     float *part = reinterpret_cast<float *>(ws + L.Kc);
+    const size_t room = L.bias - L.Kc;
     int *status = reinterpret_cast<int *>(ws + L.flags) + problems;
     StageTimer t(timed ? ELM_STAGE_ATTEND : -1, st, 2);
 #ifdef ELM_BOUNDS_CHECK
-    // the partial kernel reports bad row numbers through the status word
+    // bad row numbers are reported through the status word
     ELM_CUDA_TRY(cudaMemsetAsync(ws + L.flags, 0, sizeof(int) * (size_t)(problems + 1), st));
 #endif
-    if (p->dtype == ELM_F32) {
-        const float *q = (const float *)Q, *k = (const float *)K, *v = (const float *)V;
-        return p->d == 64 ? dispatch_decode<float, 64>(q, k, v, idx, w, n_core, p, (float *)O, part, status, splits, groups, st)
-                          : dispatch_decode<float, 128>(q, k, v, idx, w, n_core, p, (float *)O, part, status, splits, groups, st);
-    }
-    typedef __nv_bfloat16 bf;
-    const bf *q = (const bf *)Q, *k = (const bf *)K, *v = (const bf *)V;
-    return p->d == 64 ? dispatch_decode<bf, 64>(q, k, v, idx, w, n_core, p, (bf *)O, part, status, splits, groups, st)
-                      : dispatch_decode<bf, 128>(q, k, v, idx, w, n_core, p, (bf *)O, part, status, splits, groups, st);
+    return p->dtype == ELM_F32 ? dispatch_decode<float>(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st)
+                               : dispatch_decode<__nv_bfloat16>(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st);
 }
 
 }  // namespace elm
