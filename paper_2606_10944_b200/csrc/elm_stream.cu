@@ -8,6 +8,7 @@
 namespace elm {
 struct StreamLayout {
     size_t vmax_bits, cnorm, E, T1, S, Mpair, rdecay, F, F_stride, ep_idx, ep_w, ws_attend, ep_cap, total;
+    size_t win_idx, win_w, win_cap;            // the lists of the windows of one attention launch (stream_steps_impl)
 };
 static StreamLayout stream_layout(const elm_params *p, int mbar)
 {
@@ -33,6 +34,12 @@ static StreamLayout stream_layout(const elm_params *p, int mbar)
     elm_params one = *p;
     one.n_q = 1;
     L.ws_attend = take(attend_layout(&one, (int32_t)L.ep_cap).total);
+    // room for up to 16 of the longest lists, less when they are so long that 32 MB would not hold them
+    size_t lists = ((size_t)32 << 20) / (BH * L.ep_cap * 8);
+    lists = lists < 1 ? 1 : (lists > 16 ? 16 : lists);
+    L.win_cap = lists * L.ep_cap;
+    L.win_idx = take(BH * L.win_cap * 4);
+    L.win_w = take(BH * L.win_cap * 4);
     L.total = off;
     return L;
 }
@@ -53,17 +60,17 @@ __global__ void append_kernel(int32_t *__restrict__ list, int64_t stride, int64_
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < problems) list[(int64_t)p * stride + pos] = value;
 }
-// build_list_kernel and, in the same launch, list[p][pos] = value for every problem p: the token's own entry into E
-// or S_0 (Express.update), which lies behind the entries the pieces read.  A decode step is a handful of
-// microsecond-sized launches, so each one saved shows.
+// build_list_kernel and, in the same launch, list[p][pos + j] = value + j for j < count and every problem p: the
+// tokens' own entries into E or S_0 (Express.update), which lie behind the entries the pieces read.  A decode step is
+// a handful of microsecond-sized launches, so each one saved shows.
 __global__ void build_list_append_kernel(ListPieces pc, int64_t src_stride, int32_t *__restrict__ idx, float *__restrict__ w,
-                                         int64_t cap, int32_t *__restrict__ list, int64_t pos, int32_t value)
+                                         int64_t cap, int32_t *__restrict__ list, int64_t pos, int32_t value, int count)
 {
     // (launched with programmatic stream serialization; nothing is read or written before this point)
     cudaGridDependencySynchronize();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t pr = blockIdx.y;
-    if (i == 0) list[pr * src_stride + pos] = value;
+    if (i < count) list[pr * src_stride + pos + i] = value + i;
     if (i >= pc.dst_off[pc.n]) return;
     int k = 0;
     while (i >= pc.dst_off[k + 1]) ++k;
@@ -72,9 +79,10 @@ __global__ void build_list_append_kernel(ListPieces pc, int64_t src_stride, int3
     w[pr * cap + i] = pc.w[k];
 }
 
-// wtd_cache() of Algorithm 1 (+ the token t itself when t >= 0) as list pieces
+// wtd_cache() of Algorithm 1 (+ the `tokens` tokens from t on when t >= 0) as list pieces.  newest_last: E first and
+// S_0 last, so that as long as no Halve call comes due the list of the next token is this one with one more entry.
 static void stream_pieces(const elm_stream *s, const int64_t *n_S, const StreamLayout &L, unsigned char *ws,
-                          const elm_params *p, int64_t t, ListPieces &pc)
+                          const elm_params *p, int64_t t, ListPieces &pc, bool newest_last = false, int64_t tokens = 1)
 {
     const size_t BH = (size_t)p->batch * p->kv_heads;
     int32_t *S = reinterpret_cast<int32_t *>(ws + L.S);
@@ -86,9 +94,13 @@ static void stream_pieces(const elm_stream *s, const int64_t *n_S, const StreamL
         at += (int32_t)count;
         ++k;
     };
-    for (int i = 0; i <= s->q; ++i) piece(S + (size_t)i * BH * p->n_kv, 0, n_S[i], (float)ldexp(1.0, i - s->q));
-    piece(reinterpret_cast<int32_t *>(ws + L.E), 0, s->n_E, 1.f);
-    if (t >= 0) piece(nullptr, t, 1, (float)ldexp(1.0, -s->q));          // the token enters S_0
+    if (newest_last) piece(reinterpret_cast<int32_t *>(ws + L.E), 0, s->n_E, 1.f);
+    for (int j = 0; j <= s->q; ++j) {
+        const int i = newest_last ? s->q - j : j;
+        piece(S + (size_t)i * BH * p->n_kv, 0, n_S[i], (float)ldexp(1.0, i - s->q));
+    }
+    if (!newest_last) piece(reinterpret_cast<int32_t *>(ws + L.E), 0, s->n_E, 1.f);
+    if (t >= 0) piece(nullptr, t, tokens, (float)ldexp(1.0, -s->q));     // the token enters S_0
     pc.dst_off[k] = at;
     pc.n = k;
 }
@@ -157,9 +169,26 @@ static bool stratum_state(const elm_stream *s, int64_t n_out, StratumDraw &dr, i
     return true;
 }
 
+// Status word of the attention launches over cluster-split lists (elm_attend's place for the longest list).
+static int *stream_attend_status(const elm_params *p, const StreamLayout &L, unsigned char *ws)
+{
+    return reinterpret_cast<int *>(ws + L.ws_attend + attend_layout(p, (int32_t)L.ep_cap).flags) + p->batch * p->kv_heads;
+}
+
+// Windows of a streaming run whose lists have been built and whose attention has not been launched yet.
+struct PendingWindows {
+    DecodeWindows win = {};
+    int64_t entries = 0;                    // list entries per problem
+    const void *Q = nullptr;                // of the first pending token
+    void *O = nullptr;
+};
+
+// One step of W tokens (W > 1, with `pend`: tokens of one window - nothing but appends happens between them, so the
+// list of each is a prefix of the list of the last; the list is built and the attention left to the launch that takes
+// all pending windows).  Without `pend`, one token, attended at once.
 template <typename Tin, typename T>
 static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin *V, const elm_params *p, Tin *O,
-                            unsigned char *ws, cudaStream_t st)
+                            unsigned char *ws, cudaStream_t st, int64_t W = 1, PendingWindows *pend = nullptr)
 {
     const StreamLayout L = stream_layout(p, s->mbar);
     const int BH = p->batch * p->kv_heads;
@@ -182,9 +211,11 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
     int32_t *S = reinterpret_cast<int32_t *>(ws + L.S);
     auto Slist = [&](int i) { return S + (size_t)i * BH * n; };
     auto blocks = [](int64_t count) { return (unsigned)((count + 255) / 256); };
-    if (t >= s->n_known) {
-        // a token that was not there at init: its key norm, and v_max grows with it
-        prepass_kernel<Tin, T><<<dim3(1, (unsigned)BH), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, T1, t, t + 1);
+    if (t + W > s->n_known) {
+        // tokens that were not there at init: their key norms, and v_max grows with them (it is read by the Halve
+        // calls alone, which come behind the last token of a window)
+        const int64_t from = t > s->n_known ? t : s->n_known;
+        prepass_kernel<Tin, T><<<dim3(blocks(t + W - from), (unsigned)BH), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, T1, from, t + W);
         count_launches(1);
         ELM_CUDA_TRY(cudaGetLastError());
     }
@@ -197,10 +228,10 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
     bool appended = false;
     {
         ListPieces pc = {};
-        stream_pieces(s, s->n_S, L, ws, p, t, pc);
+        stream_pieces(s, s->n_S, L, ws, p, t, pc, !sub, W);
         int total = pc.dst_off[pc.n];
-        int32_t *ep_idx = reinterpret_cast<int32_t *>(ws + L.ep_idx);
-        float *ep_w = reinterpret_cast<float *>(ws + L.ep_w);
+        int32_t *ep_idx = pend ? reinterpret_cast<int32_t *>(ws + L.win_idx) + pend->entries : reinterpret_cast<int32_t *>(ws + L.ep_idx);
+        float *ep_w = pend ? reinterpret_cast<float *>(ws + L.win_w) + pend->entries : reinterpret_cast<float *>(ws + L.ep_w);
         if (sub && dr.o > 0) {
             // some problems have taken this stratum's update already
             ListPieces pb = {};
@@ -209,29 +240,38 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
             if ((size_t)total > L.ep_cap) return ELM_ERR_WORKSPACE;
             build_list_choice_kernel<<<dim3(blocks(total), (unsigned)BH), 256, 0, st>>>(pc, pb, dr, n, ep_idx, ep_w, total);
         } else if (!sub) {
-            // the token's entry into E (exact phase) or S_0 rides along (the bookkeeping follows below)
+            // the tokens' entries into E (exact phase) or S_0 ride along (the bookkeeping follows below)
             int32_t *list = s->n + 1 <= n_out ? E : Slist(0);
             const int64_t pos = s->n + 1 <= n_out ? s->n_E : s->n_S[0];
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(blocks(total), (unsigned)BH);
-            cfg.blockDim = dim3(256);
-            cfg.stream = st;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            const int64_t cap = total;
-            const int32_t value = (int32_t)t;
-            ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, build_list_append_kernel, pc, n, ep_idx, ep_w, cap, list, pos, value));
+            ELM_CUDA_TRY(launch_after(build_list_append_kernel, dim3(blocks(total), (unsigned)BH), dim3(256), 0, st, pc, n, ep_idx,
+                                      ep_w, pend ? (int64_t)L.win_cap : (int64_t)total, list, pos, (int32_t)t, (int)W));
             appended = true;
         } else {
             build_list_kernel<<<dim3(blocks(total), (unsigned)BH), 256, 0, st>>>(pc, n, ep_idx, ep_w, total);
         }
         count_launches(1);
         ELM_CUDA_TRY(cudaGetLastError());
-        const int rc = attend_enqueue(Q, K, V, ep_idx, ep_w, total, p, O, ws + L.ws_attend, st);
-        if (rc != ELM_OK) return rc;
+        if (pend) {
+            DecodeWindows &dw = pend->win;
+            if (dw.n == 0) { pend->Q = Q; pend->O = O; }
+            dw.off[dw.n] = (int32_t)pend->entries;
+            dw.seen0[dw.n] = total - (int32_t)W + 1;
+            dw.tok0[dw.n + 1] = dw.tok0[dw.n] + (int32_t)W;
+            ++dw.n;
+            pend->entries += total;
+        } else {
+            int rc;
+            if (!sub && attend_decode_windows_apply(p, total)) {
+                DecodeWindows dw = {};
+                dw.n = 1;
+                dw.tok0[1] = 1;
+                dw.seen0[0] = total;
+                rc = attend_decode_windows(Q, K, V, ep_idx, ep_w, total, dw, p, O, stream_attend_status(p, L, ws), st);
+            } else {
+                rc = attend_enqueue(Q, K, V, ep_idx, ep_w, total, p, O, ws + L.ws_attend, st);
+            }
+            if (rc != ELM_OK) return rc;
+        }
     }
     // ---- Algorithm 1: Express.update ----
     auto append = [&](int32_t *list, int64_t pos) {
@@ -240,13 +280,13 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
         count_launches(1);
         return cuda_status(cudaGetLastError());
     };
-    s->n += 1;
+    s->n += W;
     if (s->n <= n_out) {                                                   // exact phase
         const int rc = append(E, s->n_E);
-        s->n_E += 1;
+        s->n_E += W;
         return rc;
     }
-    s->ell += 1;                                                           // thin phase: Compress2.update
+    s->ell += W;                                                           // thin phase: Compress2.update
     if (sub) {
         // Subsample: only the problems whose draw is this token take the update now; the counters in *s
         // move on when the stratum ends
@@ -292,7 +332,7 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
         const int q = s->q;
         int rc = append(Slist(0), s->n_S[0]);
         if (rc != ELM_OK) return rc;
-        s->n_S[0] += 1;
+        s->n_S[0] += W;
         const double dm = kh_express_delta(p->delta, s->m);
         for (int i = 0; i < q; ++i) {
             const int64_t thresh = ((n_out << q) << i) >> (2 * (q - 1));  // n_in 2^i / 4^(q-1)
@@ -331,6 +371,68 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
         for (int i = 0; i < 16; ++i) { s->n_S[i] = 0; s->calls[i] = 0; }
     }
     return ELM_OK;
+}
+
+// Tokens from the next one on, at most `limit`, between which nothing but appends to E or S_0 happens: up to the one
+// that completes the exact phase, fills a level-0 Halve call's input, or ends a segment.
+static int64_t stream_window(const elm_stream *s, const elm_params *p, int64_t limit)
+{
+    const int64_t n_out = (int64_t)1 << p->log2_nout;
+    int64_t W = limit;
+    auto at_most = [&](int64_t v) { if (v < W) W = v; };
+    at_most((int64_t)p->n_kv - s->n);
+    if (s->n < n_out) {
+        at_most(n_out - s->n);
+    } else {
+        at_most((n_out << s->m) - s->ell);
+        if (s->q >= 1) at_most(((n_out << s->q) >> (2 * (s->q - 1))) - s->n_S[0]);
+    }
+    return W < 1 ? 1 : W;
+}
+
+// n_tokens tokens, window by window: the list, the prepass and the Halve calls of a window are enqueued as its tokens
+// would have them, and the attention of many windows' tokens is one launch of the decode kernel - a list built for a window is
+// not touched by what comes behind it, so the launch may wait.  2496 tokens of 32 query / 8 KV heads, n_out = 256, bf16: 1.93 ms
+// (attention 1.61 in one launch, the chain of 8 Halve calls and 10 lists 0.3) against 32.8 ms token by token (four to
+// five launches of 2 - 5 us each).
+template <typename Tin, typename T>
+static int stream_steps_impl(elm_stream *s, int64_t n_tokens, const Tin *Q, const Tin *K, const Tin *V, const elm_params *p, Tin *O,
+                             unsigned char *ws, cudaStream_t st)
+{
+    const StreamLayout L = stream_layout(p, s->mbar);
+    const int64_t row = (int64_t)p->batch * p->q_heads * p->d;
+    const int64_t n_out = (int64_t)1 << p->log2_nout;
+    PendingWindows pend;
+    auto flush = [&]() -> int {
+        if (pend.win.n == 0) return ELM_OK;
+        const int rc = attend_decode_windows(pend.Q, K, V, reinterpret_cast<int32_t *>(ws + L.win_idx), reinterpret_cast<float *>(ws + L.win_w),
+                                             (int64_t)L.win_cap, pend.win, p, pend.O, stream_attend_status(p, L, ws), st);
+        pend = PendingWindows();
+        return rc;
+    };
+    for (int64_t i = 0; i < n_tokens;) {
+        const Tin *q = Q + i * row;
+        Tin *o = O + i * row;
+        const int64_t W = stream_window(s, p, n_tokens - i < 32768 ? n_tokens - i : 32768);
+        int64_t len = s->n_E + W;                                          // the list of the window's last token
+        for (int k = 0; k <= s->q; ++k) len += s->n_S[k];
+        // (a phase with Subsample: the problems take their updates at different tokens - one step at a time)
+        const bool sub = s->m > s->mbar && s->n >= n_out;
+        const bool together = n_tokens > 1 && !sub && s->n < p->n_kv && len <= (int64_t)L.win_cap && attend_decode_windows_apply(p, (int)len);
+        if (!together || pend.win.n == DECODE_MAX_WINDOWS || pend.entries + len > (int64_t)L.win_cap ||
+            pend.win.tok0[pend.win.n] + W > 65535) {
+            const int rc = flush();
+            if (rc != ELM_OK) return rc;
+        }
+        const int rc = together ? stream_step_impl<Tin, T>(s, q, K, V, p, o, ws, st, W, &pend)
+                                : stream_step_impl<Tin, T>(s, q, K, V, p, o, ws, st);
+        if (rc != ELM_OK) {
+            const int rf = flush();                                        // the steps before it stay enqueued
+            return rf != ELM_OK ? rf : rc;
+        }
+        i += together ? W : 1;
+    }
+    return flush();
 }
 }  // namespace elm
 
@@ -386,15 +488,14 @@ extern "C" int elm_stream_init(elm_stream *s, const void *K, const void *V, int6
     return ELM_OK;
 }
 
-extern "C" int elm_stream_step(elm_stream *s, const void *Q_t, const void *K, const void *V, const elm_params *params,
-                               void *O_t, void *workspace, size_t workspace_bytes, void *stream)
+namespace elm {
+static int stream_steps_checked(elm_stream *s, int32_t n_tokens, const void *Q, const void *K, const void *V, const elm_params *params,
+                                void *O, void *workspace, size_t workspace_bytes, void *stream)
 {
-    using namespace elm;
-    if (!s || !params) return ELM_ERR_NULL;
     const int rc = validate_stream(params, s->mbar);
     if (rc != ELM_OK) return rc;
-    if (!Q_t || !K || !V || !O_t || !workspace) return ELM_ERR_NULL;
-    if (((uintptr_t)Q_t | (uintptr_t)K | (uintptr_t)V | (uintptr_t)O_t) & 15) return ELM_ERR_ALIGN;
+    if (!Q || !K || !V || !O || !workspace) return ELM_ERR_NULL;
+    if (((uintptr_t)Q | (uintptr_t)K | (uintptr_t)V | (uintptr_t)O) & 15) return ELM_ERR_ALIGN;
     if ((uintptr_t)workspace & 255) return ELM_ERR_ALIGN;
     if (workspace_bytes < stream_layout(params, s->mbar).total) return ELM_ERR_WORKSPACE;
     unsigned char *ws = (unsigned char *)workspace;
@@ -402,11 +503,19 @@ extern "C" int elm_stream_step(elm_stream *s, const void *Q_t, const void *K, co
     const bool det = params->precision == ELM_PREC_FP64_DET;
     typedef __nv_bfloat16 bf;
     if (params->dtype == ELM_F32) {
-        return det ? stream_step_impl<float, double>(s, (const float *)Q_t, (const float *)K, (const float *)V, params, (float *)O_t, ws, st)
-                   : stream_step_impl<float, float>(s, (const float *)Q_t, (const float *)K, (const float *)V, params, (float *)O_t, ws, st);
+        return det ? stream_steps_impl<float, double>(s, n_tokens, (const float *)Q, (const float *)K, (const float *)V, params, (float *)O, ws, st)
+                   : stream_steps_impl<float, float>(s, n_tokens, (const float *)Q, (const float *)K, (const float *)V, params, (float *)O, ws, st);
     }
-    return det ? stream_step_impl<bf, double>(s, (const bf *)Q_t, (const bf *)K, (const bf *)V, params, (bf *)O_t, ws, st)
-               : stream_step_impl<bf, float>(s, (const bf *)Q_t, (const bf *)K, (const bf *)V, params, (bf *)O_t, ws, st);
+    return det ? stream_steps_impl<bf, double>(s, n_tokens, (const bf *)Q, (const bf *)K, (const bf *)V, params, (bf *)O, ws, st)
+               : stream_steps_impl<bf, float>(s, n_tokens, (const bf *)Q, (const bf *)K, (const bf *)V, params, (bf *)O, ws, st);
+}
+}  // namespace elm
+
+extern "C" int elm_stream_step(elm_stream *s, const void *Q_t, const void *K, const void *V, const elm_params *params,
+                               void *O_t, void *workspace, size_t workspace_bytes, void *stream)
+{
+    if (!s || !params) return ELM_ERR_NULL;
+    return elm::stream_steps_checked(s, 1, Q_t, K, V, params, O_t, workspace, workspace_bytes, stream);
 }
 
 extern "C" int elm_stream_steps(elm_stream *s, int32_t n_tokens, const void *Q_T, const void *K, const void *V,
@@ -414,15 +523,11 @@ extern "C" int elm_stream_steps(elm_stream *s, int32_t n_tokens, const void *Q_T
 {
     if (!s || !params) return ELM_ERR_NULL;
     if (n_tokens < 0) return ELM_ERR_SHAPE;
-    if (n_tokens > 0 && (!Q_T || !O_T)) return ELM_ERR_NULL;
+    if (n_tokens == 0) return ELM_OK;
+    if (!Q_T || !O_T) return ELM_ERR_NULL;
     const size_t per_token = (size_t)params->batch * params->q_heads * params->d * elm::elt_bytes(params->dtype);
     if (per_token & 15) return ELM_ERR_ALIGN;
-    for (int32_t i = 0; i < n_tokens; ++i) {
-        const int rc = elm_stream_step(s, (const unsigned char *)Q_T + (size_t)i * per_token, K, V, params,
-                                       (unsigned char *)O_T + (size_t)i * per_token, workspace, workspace_bytes, stream);
-        if (rc != ELM_OK) return rc;
-    }
-    return ELM_OK;
+    return elm::stream_steps_checked(s, n_tokens, Q_T, K, V, params, O_T, workspace, workspace_bytes, stream);
 }
 
 extern "C" int elm_stream_cache(const elm_stream *s, const elm_params *params, int32_t *idx_out, float *w_out,

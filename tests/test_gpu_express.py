@@ -281,3 +281,30 @@ def test_stream_steps_in_one_call_equal_single_steps():
     ia, wa = a.cache()
     ib, wb = b.cache()
     assert torch.equal(ia, ib) and torch.equal(wa, wb)
+
+
+@pytest.mark.parametrize("dtype,d,hq,hkv,batch,log2_nout,mbar,n,cuts", [
+    ("bf16", 128, 8, 2, 1, 6, 4, 900, (1, 63, 64, 257, 258, 900)),   # windows of 64, 16 tokens; two tokens per CTA
+    ("bf16", 64, 3, 1, 2, 5, 1, 333, (332,)),                        # three query heads per KV head: two tokens per CTA
+    ("f32", 128, 2, 2, 1, 7, 5, 1100, (500,)),                       # 512-byte rows, eight tokens per CTA
+    ("f32", 64, 8, 1, 1, 5, 3, 300, ()),                             # eight query heads per KV head: one token per CTA
+])
+def test_stream_steps_in_windows_equal_single_steps(dtype, d, hq, hkv, batch, log2_nout, mbar, n, cuts):
+    """Tokens attended together (lists longer than one part, several windows per launch, windows cut by the calls'
+    ends) get the outputs of single steps bit for bit, and the same cache; a value that only later tokens see may be
+    infinite."""
+    wl = WORKLOADS["cfg2"].scaled(batch=batch, q_heads=hq, kv_heads=hkv, n=n, n_q=n, d=d, dtype=dtype)
+    Q, K, V = generate(wl, seed=5, want_q=True)
+    V[:, :, n - 1, 0] = float("inf")
+    Qd, Kd, Vd = Q.cuda(), K.cuda(), V.cuda()
+    a = elm.Stream(Kd, Vd, hq, log2_nout, mbar, seed=9, n_known=n // 2)
+    one = torch.stack([a.step(Qd[:, :, t:t + 1, :].contiguous()) for t in range(n)])
+    b = elm.Stream(Kd, Vd, hq, log2_nout, mbar, seed=9, n_known=n // 2)
+    q_T = Qd.permute(2, 0, 1, 3).unsqueeze(3).contiguous()
+    edges = [0, *cuts, n]
+    many = torch.cat([b.steps(q_T[lo:hi]) for lo, hi in zip(edges, edges[1:]) if hi > lo])
+    torch.cuda.synchronize()
+    assert torch.isfinite(many[:n - 1].float()).all() and not torch.isfinite(many[n - 1].float()).all()
+    assert torch.equal(one[:n - 1], many[:n - 1]) and torch.equal(one[n - 1].nan_to_num(), many[n - 1].nan_to_num())
+    for x, y in zip(a.cache(), b.cache()):
+        assert torch.equal(x, y)
