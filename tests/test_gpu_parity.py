@@ -296,3 +296,24 @@ def test_stage_profile_of_the_attention_stage_only():
     for stage in ("prepass", "level_prep", "gram", "walk", "emit"):
         assert prof[stage][0] == 0.0 and prof[stage][1] >= 1
     assert torch.equal(idx, idx0) and torch.equal(w, w0) and torch.equal(O, O0)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_q,n_core", [(9, 1), (63, 63), (64, 65), (65, 64), (130, 200)])
+def test_attend_f32_edges_of_tiles(d, n_q, n_core):
+    """fp32 inputs in fp32 mode, blocks of 64 queries x 64 points: partly filled tiles, unequal weights, grouped heads."""
+    wl = WORKLOADS["cfg2"].scaled(batch=2, q_heads=4, kv_heads=2, n=512, n_q=n_q, d=d, dtype="f32")
+    err, tol = _attend_case(wl, "fp32", weights="random", n_core=n_core)
+    assert err <= tol
+
+
+@pytest.mark.parametrize("d,log2_nout,m", [(64, 6, 6), (128, 7, 4), (128, 6, 6)])
+def test_compress_f32_inputs_select_what_the_fp64_mode_selects(d, log2_nout, m):
+    """fp32 Gram tiles of 64 x 64 points: calls of 1 ... 256 pairs (several calls per tile, several tiles per call); the
+    decisions differ from the fp64 mode's only within rounding distance of their probabilities."""
+    wl = WORKLOADS["cfg2"].scaled(batch=1, q_heads=3, kv_heads=3, n=1 << (log2_nout + m), n_q=8, d=d, dtype="f32")
+    _, K, V = generate(wl, seed=41)
+    a, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp32")
+    b, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp64")
+    torch.cuda.synchronize()
+    assert (a != b).float().mean().item() <= 0.02
