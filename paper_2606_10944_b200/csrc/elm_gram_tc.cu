@@ -6,7 +6,7 @@
 // into the 128-byte-swizzled K-major layout tcgen05.mma reads (rows are never copied in HBM).
 // Two accumulators in TMEM hold K K^T and V V^T; the epilogue applies the exponential, the
 // product and the +/- pair combination F[j,i] = G[2j,2i] - G[2j,2i+1] - G[2j+1,2i] + G[2j+1,2i+1]
-// (Algorithm A.1's <f_j, f_i>) and stores only j <= i within one Halve call.
+// (Algorithm A.1's <f_j, f_i>; of use for j <= i within one Halve call).
 #include <math.h>
 
 #include "elm_common.cuh"
@@ -23,28 +23,34 @@ constexpr int TP = 64;            // pairs per tile side
 constexpr int TR = 128;           // points per tile side
 constexpr int NTHREADS = 256;
 constexpr uint32_t TMEM_COLS = 256;
+constexpr int FS_LD = 68;         // row stride of the shared-memory pair Gram of a fused tile (floats)
 
-// Shared memory holds ONE pair of operand tiles (row points, column points): the keys first, then,
-// once K K^T has been consumed, the values in the same place.  64 KB (d = 128) lets two CTAs share
-// an SM, so one CTA's gather overlaps the other's MMAs and epilogue.
+// Shared memory of the kernel that walks its tiles itself: the tile's keys, its values, its pair Gram.  92 KB (d = 128)
+// let two CTAs share an SM.
 template <int D> struct Smem {
     static constexpr int KH = D / 64;
     static constexpr int OPERAND = TR * D * 2;                 // one 128-row operand tile, bytes
-    static constexpr int OFF_A = 0, OFF_B = OPERAND;
+    static constexpr int OFF_K = 0, OFF_V = OPERAND;
     static constexpr int OFF_MISC = 2 * OPERAND;
-    static constexpr int TOTAL = OFF_MISC + 2048 + 1024;       // misc block + alignment slack
+    static constexpr int OFF_F = OFF_MISC + 3072;
+    // The block walker reads 32 rows and 64 columns from a call's corner whatever the call's size (and ignores what lies
+    // outside): from call 3 of 16 pairs on, row 48 + 31, column 48 + 63.
+    static constexpr int F_BYTES = ((48 + 31) * FS_LD + 48 + 64) * 4;
+    static constexpr int TOTAL = OFF_F + F_BYTES + 1024;       // + alignment slack
 };
 
+struct TileMisc {
+    float colshift[TP];          // M of each pair column, in log2 units
+    float rdec[TP], unif[TP];    // the walk's decay factor and uniform of each pair of the tile
+    int32_t rows[TR];
+};
 struct Misc {
-    uint64_t mma_done[2];        // K K^T done, V V^T done
+    uint64_t mma_done;
     uint32_t tmem_base;
     uint32_t pad;
-    float colshift[TP];          // M of each pair column, in log2 units
-    float rdec[TP], unif[TP];    // fused walk: decay factor and uniform of each pair of the tile
-    int32_t rowsA[TR], rowsB[TR];
+    TileMisc tile[2];            // this tile's and the next one's
 };
-
-constexpr int FS_LD = 68;         // row stride of the shared-memory pair Gram of a fused tile (floats)
+static_assert(sizeof(Misc) <= 3072, "the misc block's share of shared memory");
 
 // Halving walk (Algorithm A.1) of the calls that lie inside one 64-pair tile, on the tile's pair
 // Gram in shared memory: warp w walks call w of the tile (P = 16, 32 or 64 pairs per call) in blocks
@@ -97,12 +103,18 @@ __device__ __forceinline__ void gather_operand(unsigned char *dst, const __nv_bf
     }
 }
 
+// Levels whose calls are smaller than a tile (P < 64 pairs; a tile holds 64 / P whole calls or the level's last ones):
+// row points = column points, and the calls are walked on the tile's pair Gram without it leaving shared memory.
+// Persistent, two CTAs per SM, bound by the latency of a tile's stages (row numbers, gather, MMAs, epilogue, walk): the
+// row numbers and everything else a tile needs from global memory are fetched while the tile before is multiplied, and
+// its rows are gathered while that one's epilogue and walk run.  64 problems x 8192 points, d = 128: 16 pairs a
+// call 116 -> 83 us, 32 pairs 57 -> 42 us against one CTA per tile (HBM floor of the first: 41 us).
 template <int D>
 __global__ void __launch_bounds__(NTHREADS, 2)
-gram_tc_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
-               const int32_t *__restrict__ cur, const float *__restrict__ Mpair,
-               const unsigned *__restrict__ vmax_bits, int64_t n, int P, int64_t Ptotal,
-               float *__restrict__ F, int64_t F_stride, int *__restrict__ status, WalkArgs wk)
+gram_walk_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
+                 const int32_t *__restrict__ cur, const float *__restrict__ Mpair,
+                 const unsigned *__restrict__ vmax_bits, int64_t n, int P, int64_t Ptotal, int tiles_per_problem, int total_tiles,
+                 int *__restrict__ status, WalkArgs wk)
 {
     cudaGridDependencySynchronize();           // launched with programmatic stream serialization (launch_after)
     using SM = Smem<D>;
@@ -110,114 +122,86 @@ gram_tc_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restr
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     Misc *misc = reinterpret_cast<Misc *>(smem + SM::OFF_MISC);
+    float *Fs = reinterpret_cast<float *>(smem + SM::OFF_F);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int p = blockIdx.y;
 
     if (*reinterpret_cast<volatile int *>(status) != 0) return;
-
-    int64_t JR, JC;
-    if (P >= TP) {
-        const int Tg = P / TP, ntri = Tg * (Tg + 1) / 2;
-        const int g = blockIdx.x / ntri, local = blockIdx.x % ntri;
-        int tc = (int)((sqrtf(8.f * (float)local + 1.f) - 1.f) * 0.5f);
-        while ((tc + 1) * (tc + 2) / 2 <= local) ++tc;
-        while (tc * (tc + 1) / 2 > local) --tc;
-        const int tr = local - tc * (tc + 1) / 2;
-        JR = (int64_t)g * P + tr * TP;
-        JC = (int64_t)g * P + tc * TP;
-    } else {
-        JR = JC = (int64_t)blockIdx.x * TP;
-    }
-    const bool diagonal = JR == JC;
-    const int32_t *curp = cur + (int64_t)p * n;
     const float LOG2E = 1.4426950408889634f;
-    if (tid < TR) {
-        const int64_t pt = 2 * JR + tid;
-        misc->rowsA[tid] = pt < 2 * Ptotal ? curp[pt] : 0;
-    } else {
-        const int64_t pt = 2 * JC + (tid - TR);
-        misc->rowsB[tid - TR] = pt < 2 * Ptotal ? curp[pt] : 0;
-    }
-    if (tid < TP) {
-        const int64_t jc = JC + tid;
-        misc->colshift[tid] = jc < Ptotal ? Mpair[(int64_t)p * pair_stride(n) + jc] * LOG2E : 0.f;
-        if (wk.fused) {
-            // everything the in-tile walk needs from global memory, fetched while the tile is built
-            misc->rdec[tid] = jc < Ptotal ? wk.rdecay[(int64_t)p * pair_stride(n) + jc] : 1.f;
+    // what tile `it` needs from global memory besides its rows: row numbers, running shifts, decay factors, uniforms
+    auto fetch_misc = [&](int it, TileMisc &m) {
+        const int p = it / tiles_per_problem;
+        const int64_t JR = (int64_t)(it % tiles_per_problem) * TP;
+        if (tid < TR) {
+            const int64_t pt = 2 * JR + tid;
+            m.rows[tid] = pt < 2 * Ptotal ? __ldg(cur + (int64_t)p * n + pt) : 0;
+        } else if (tid < TR + TP) {
+            const int i = tid - TR;
+            const int64_t jc = JR + i;
+            m.colshift[i] = jc < Ptotal ? __ldg(Mpair + (int64_t)p * pair_stride(n) + jc) * LOG2E : 0.f;
+            m.rdec[i] = jc < Ptotal ? __ldg(wk.rdecay + (int64_t)p * pair_stride(n) + jc) : 1.f;
+        } else {
+            const int i = tid - TR - TP;
+            const int64_t jc = JR + i;
             uint32_t cgroup, ccode;
             call_counter((int)(jc / P), wk.level, cgroup, ccode);
-            misc->unif[tid] = halving_uniform<float>(wk.seed, (uint32_t)(jc % P), cgroup, ccode, (uint32_t)p + wk.pbase);
+            m.unif[i] = halving_uniform<float>(wk.seed, (uint32_t)(jc % P), cgroup, ccode, (uint32_t)p + wk.pbase);
         }
-    }
+    };
+    auto gather = [&](int it, const TileMisc &m) {
+        const int64_t first = (int64_t)(it / tiles_per_problem) * n * D;
+        gather_operand<D>(smem + SM::OFF_K, K + first, m.rows, tid);
+        gather_operand<D>(smem + SM::OFF_V, V + first, m.rows, tid);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     if (tid == 0) {
-        mbar_init(&misc->mma_done[0], 1);
-        mbar_init(&misc->mma_done[1], 1);
+        mbar_init(&misc->mma_done, 1);
         fence_barrier_init();
     }
     if (warp == 1) tmem_alloc(&misc->tmem_base, TMEM_COLS);
+    if ((int)blockIdx.x < total_tiles) fetch_misc(blockIdx.x, misc->tile[0]);
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = misc->tmem_base;
+    if ((int)blockIdx.x < total_tiles) gather(blockIdx.x, misc->tile[0]);
 
-    const __nv_bfloat16 *Kp = K + (int64_t)p * n * D;
-    const __nv_bfloat16 *Vp = V + (int64_t)p * n * D;
     constexpr uint32_t IDESC = umma_idesc_bf16(TR, TR);
-    const uint32_t sA = smem_u32(smem + SM::OFF_A);
-    const uint32_t sB = smem_u32(smem + SM::OFF_B);
-    uint32_t tmem = 0;
+    const uint32_t sK = smem_u32(smem + SM::OFF_K), sV = smem_u32(smem + SM::OFF_V);
+    const int r = (warp & 3) * 32 + lane;                     // epilogue: point row in the tile = TMEM lane
+    const int ch = warp >> 2;                                 // and column half
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch * 64;
+    const float qscale = LOG2E / sqrtf((float)D);
     bool ok = true;
-    auto issue = [&](int acc, uint32_t a_addr, uint32_t b_addr) {     // one 128 x 128 x D product into accumulator `acc`
-#pragma unroll
-        for (int kh = 0; kh < KH; ++kh)
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ss(tmem + acc * 128, umma_desc_k128(a_addr + kh * (TR * 128) + ks * 32),
-                       umma_desc_k128(b_addr + kh * (TR * 128) + ks * 32), IDESC, (kh | ks) != 0);
-    };
-    auto publish = [&]() {                                            // make the gathered tiles visible to the MMAs
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    int k = 0;
+    for (int it = blockIdx.x; it < total_tiles; it += gridDim.x, ++k) {
+        const TileMisc &m = misc->tile[k & 1];
+        const int p = it / tiles_per_problem;
+        const int64_t JR = (int64_t)(it % tiles_per_problem) * TP;
+        const bool more = it + (int)gridDim.x < total_tiles;
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         fence_proxy_async();
         tc_fence_before();
-        __syncthreads();
+        __syncthreads();                                      // rows gathered; the tile before is walked
         tc_fence_after();
-        tmem = misc->tmem_base;
-    };
-    if (diagonal) {
-        // row points = column points: keys in the first slot, values in the second, one gather round
-        gather_operand<D>(smem + SM::OFF_A, Kp, misc->rowsA, tid);
-        gather_operand<D>(smem + SM::OFF_B, Vp, misc->rowsA, tid);
-        publish();
         if (tid == 0) {
-            const uint32_t sV = smem_u32(smem + SM::OFF_B);
-            issue(0, sA, sA);
-            issue(1, sV, sV);
-            tc_commit(&misc->mma_done[1]);
-        }
-        ok = mbar_wait(&misc->mma_done[1], 0);
-    } else {
 #pragma unroll
-        for (int phase = 0; phase < 2; ++phase) {              // 0: keys -> K K^T, 1: values -> V V^T
-            const __nv_bfloat16 *X = phase == 0 ? Kp : Vp;
-            gather_operand<D>(smem + SM::OFF_A, X, misc->rowsA, tid);
-            gather_operand<D>(smem + SM::OFF_B, X, misc->rowsB, tid);
-            publish();
-            if (tid == 0) {
-                issue(phase, sA, sB);
-                tc_commit(&misc->mma_done[phase]);
-            }
-            // the operand tiles are reused by the next phase only after the MMAs have read them
-            ok = ok && mbar_wait(&misc->mma_done[phase], 0);
+            for (int op = 0; op < 2; ++op)
+#pragma unroll
+                for (int kh = 0; kh < KH; ++kh)
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks) {
+                        const uint64_t d = umma_desc_k128((op == 0 ? sK : sV) + kh * (TR * 128) + ks * 32);
+                        mma_ss(tmem + op * 128, d, d, IDESC, (kh | ks) != 0);
+                    }
+            tc_commit(&misc->mma_done);
         }
-    }
-
-    // epilogue: warp w owns TMEM lanes 32 (w % 4) .. +31 (tile rows) and the column half w / 4
-    if (ok) {
-        tc_fence_after();
-        const int r = (warp & 3) * 32 + lane;                 // point row in the tile
-        const int ch = warp >> 2;                             // columns [64 ch, 64 ch + 64)
-        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch * 64;
+        if (more) fetch_misc(it + gridDim.x, misc->tile[(k + 1) & 1]);
         const float vm = __uint_as_float(vmax_bits[p]);
         const float vm2 = vm * vm;
-        const float qscale = LOG2E / sqrtf((float)D);
+        ok = mbar_wait(&misc->mma_done, (uint32_t)k & 1u);
+        if (__syncthreads_or(!ok)) { ok = false; break; }     // (and the next tile's row numbers are there)
+        tc_fence_after();
+        if (more) gather(it + gridDim.x, misc->tile[(k + 1) & 1]);
         float h[32];                                          // G[r,2i] - G[r,2i+1] for the 32 pair columns
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -227,7 +211,7 @@ gram_tc_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restr
             tmem_wait_ld();
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-                const float sh = misc->colshift[ch * 32 + q * 16 + (c >> 1)];
+                const float sh = m.colshift[ch * 32 + q * 16 + (c >> 1)];
                 float e0 = fmaf(__uint_as_float(kk[c]), qscale, -sh);
                 float e1 = fmaf(__uint_as_float(kk[c + 1]), qscale, -sh);
                 float g0 = e0 < -115.f ? 0.f : fast_exp2(e0) * (__uint_as_float(vv[c]) + vm2);
@@ -238,43 +222,30 @@ gram_tc_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restr
         // pair rows are adjacent lanes: the even lane finishes pair columns 0..15 of its 32, the odd
         // lane columns 16..31
         const bool odd = lane & 1;
-        float f[16];
+        float *Fr = Fs + (r >> 1) * FS_LD + ch * 32 + (odd ? 16 : 0);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float send = odd ? h[i] : h[i + 16];
-            const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
-            f[i] = odd ? recv - h[i + 16] : h[i] - recv;
-        }
-        const int64_t jr = JR + (r >> 1);
-        const int64_t jc0 = JC + ch * 32 + (odd ? 16 : 0);
-        if (wk.fused) {
-            // calls of at most 64 pairs lie inside this (diagonal) tile: keep the pair Gram in shared
-            // memory (over the operand tiles, which the MMAs have finished reading) and walk here
-            float *Fs = reinterpret_cast<float *>(smem + SM::OFF_A);
+        for (int i = 0; i < 16; i += 4) {
+            float f[4];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) Fs[(r >> 1) * FS_LD + ch * 32 + (odd ? 16 : 0) + i] = f[i];
-        } else {
-            float *Fp = F + (int64_t)p * F_stride;
-            if (jr < Ptotal) {
-                const int64_t gr = jr / P;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int64_t jc = jc0 + i;
-                    if (jc < Ptotal && jr <= jc && jc / P == gr) Fp[jr * P + (jc - gr * P)] = f[i];
-                }
+            for (int j = 0; j < 4; ++j) {
+                const float send = odd ? h[i + j] : h[i + j + 16];
+                const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
+                f[j] = odd ? recv - h[i + j + 16] : h[i + j] - recv;
             }
+            *reinterpret_cast<float4 *>(Fr + i) = make_float4(f[0], f[1], f[2], f[3]);
         }
-    } else if (lane == 0) {
-        atomicExch(status, 4);
+        tc_fence_before();
+        __syncthreads();
+        walk_in_tile(Fs, m.rdec, m.unif, p, JR, P, Ptotal, n, cur, wk, warp, lane);
     }
+    if (!ok && lane == 0) atomicExch(status, 4);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
-    if (wk.fused && ok) walk_in_tile(reinterpret_cast<float *>(smem + SM::OFF_A),
-                                     misc->rdec, misc->unif, p, JR, P, Ptotal, n, cur, wk, warp, lane);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -535,10 +506,11 @@ static int launch(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const elm_para
     } else {
         tiles = (Ptotal + TP - 1) / TP;
     }
-    if (P > TP || (P == TP && !wk.fused)) {
-        // calls that span several tiles: persistent, pipelined kernel, one CTA per SM
-        const int sm_count = device_sm_count();
-        const int64_t total = tiles * BH;
+    const int sm_count = device_sm_count();
+    const int64_t total = tiles * BH;
+    if (total > 0x7fffffff / 2) return ELM_ERR_SHAPE;
+    if (!wk.fused) {
+        // calls that fill whole tiles: persistent, pipelined kernel, one CTA per SM
         const int grid = (int)(total < sm_count ? total : sm_count);
         auto pk = gram_tc_persistent_kernel<D>;
         ELM_CUDA_TRY(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, PSmem<D>::TOTAL));
@@ -547,10 +519,11 @@ static int launch(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const elm_para
         count_launches(1);
         return cuda_status(cudaGetLastError());
     }
-    auto kern = gram_tc_kernel<D>;
+    auto kern = gram_walk_kernel<D>;
     ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::TOTAL));
-    ELM_CUDA_TRY(launch_after(kern, dim3((unsigned)tiles, (unsigned)BH), dim3(NTHREADS), (size_t)Smem<D>::TOTAL, st, K, V, cur, Mpair, vmax_bits,
-                              p->n_kv, P, Ptotal, F, F_stride, status, wk));
+    const int grid = (int)(total < 2 * sm_count ? total : 2 * sm_count);
+    ELM_CUDA_TRY(launch_after(kern, dim3((unsigned)grid), dim3(NTHREADS), (size_t)Smem<D>::TOTAL, st, K, V, cur, Mpair, vmax_bits,
+                              p->n_kv, P, Ptotal, (int)tiles, (int)total, status, wk));
     count_launches(1);
     return cuda_status(cudaGetLastError());
 }

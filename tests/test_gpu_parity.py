@@ -317,3 +317,17 @@ def test_compress_f32_inputs_select_what_the_fp64_mode_selects(d, log2_nout, m):
     b, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp64")
     torch.cuda.synchronize()
     assert (a != b).float().mean().item() <= 0.02
+
+
+@pytest.mark.parametrize("d,kv_heads,n,log2_nout,m", [
+    (128, 8, 8192, 8, 5),       # calls of 16, 32, 64, 128, 256 pairs; more tiles than resident CTAs
+    (64, 3, 2048, 7, 4),        # calls of 32 pairs and more, few tiles
+])
+def test_compress_bf16_small_calls_select_what_the_fp64_mode_selects(d, kv_heads, n, log2_nout, m):
+    """Tiles that hold several calls and walk them themselves; running shifts by a warp per call."""
+    wl = WORKLOADS["cfg3"].scaled(batch=1, q_heads=kv_heads, kv_heads=kv_heads, n=n, n_q=8, d=d, dtype="bf16")
+    _, K, V = generate(wl, seed=43)
+    a, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp32")
+    b, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp64")
+    torch.cuda.synchronize()
+    assert (a != b).float().mean().item() <= 0.02
