@@ -507,13 +507,20 @@ __device__ __forceinline__ void load4(const double *p, double (&f)[4])
 //              blocks c and c+1, so block c+1's scores are complete when block c ends; fp64: one
 //              vote per pair on the diagonal tile (c, c) after adding block c-1's contribution
 //              from the cross tile (c-1, c).
-//   warp 1     copies the tiles the walker needs for block c+1 (asynchronous copies).
+//   warp 1     copies the tiles the walker needs (asynchronous copies) AHEAD blocks before it needs them; DEEP: also
+//              the next block's thresholds.
 //   warps 2..  the updaters fold block c-1 into the scores of all columns from block c+1 on, one
 //              block behind the walker.  The rows of a block are streamed through two shared-memory
 //              panels with asynchronous copies; F does not depend on the decisions, so the first
 //              panel of the next round is already in flight when its swap mask becomes known.
 // One __syncthreads per block separates the iterations.
-template <typename T>
+// DEEP (fp32, calls of 256 pairs and more): a block takes about 1000 cycles, less than a copy from L2 or HBM, so tiles
+// are requested three blocks ahead and panels two.  Shorter calls hide the latency behind each other instead: shared
+// memory for twice as many CTAs per SM.  Clock stamps of a call of 512 pairs showed the walker (1600 cycles a block)
+// waiting for the copying warp (3300) and the updaters (4000), most of it divisions by the number of chunks in a row;
+// without those, with a thread per column, the thresholds moved and the copies ahead a block takes about 2700.  128 calls
+// of 512 pairs: 37.7 -> 25.4 us, 512 calls of 256 pairs: 40.5 -> 31.9 us.
+template <typename T, bool DEEP>
 static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restrict__ F, int64_t F_stride,
                                                        const T *__restrict__ rdecay,
                                                        const int32_t *__restrict__ cur,
@@ -524,15 +531,17 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
     cudaGridDependencySynchronize();           // launched with programmatic stream serialization (launch_after)
     constexpr int PW = 2048 / sizeof(T);                             // panel width in columns (64 KB / 2 buffers... per 32 rows)
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *tiles = reinterpret_cast<T *>(smem_raw);                      // [2][2][32][32]: buffer, (diag, cross)
-    T *alpha_s = tiles + 4 * 1024;                                   // [P] scores from finished rounds
+    constexpr int AHEAD = DEEP ? 3 : 1;                              // blocks between a tile's request and its use
+    constexpr int TB = AHEAD + 1, PB = DEEP ? 3 : 2;                 // tile buffers, panel buffers
+    T *tiles = reinterpret_cast<T *>(smem_raw);                      // [TB][2][32][32]: buffer, (diag, cross)
+    T *alpha_s = tiles + TB * 2048;                                  // [P] scores from finished rounds
     T *b_s = alpha_s + P;                                            // [P]
     T *r_s = b_s + P;                                                // [P]
     T *U_s = r_s + P;                                                // [P]
-    T *a32_s = U_s + P;                                              // [32] the walker's scores of the block
-    T *panels = a32_s + 32;                                          // [2][32][pw_alloc]
+    T *a32_s = U_s + P;                                              // [2][32] thresholds of a block (DEEP)
+    T *panels = a32_s + 64;                                          // [PB][32][pw_alloc]
     const int pw_alloc = P - 64 < PW ? (P - 64 > 0 ? P - 64 : 32) : PW;
-    uint32_t *mask_s = reinterpret_cast<uint32_t *>(panels + 2 * 32 * pw_alloc);   // [P/32] swap masks
+    uint32_t *mask_s = reinterpret_cast<uint32_t *>(panels + PB * 32 * pw_alloc);  // [P/32] swap masks
     const int p = blockIdx.y, g = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nthr = blockDim.x;
@@ -551,17 +560,29 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
     };
     // fp32: rows of a block x the columns of that block and of the next one, [32][64]
     auto copy_tile64 = [&](T *dst, int r0) {
-        const int ncols = P - r0 < 64 ? P - r0 : 64, cpr = ncols / CH;
-        for (int q = lane; q < 32 * cpr; q += 32) {
-            const int t = q / cpr, k = q % cpr;
-            cp_async16(dst + t * 64 + k * CH, Fg + (int64_t)(r0 + t) * P + r0 + k * CH);
+        // (constant shapes: a division by a variable per chunk cost this warp 3000 cycles a block, twice what the walker takes)
+        if (P - r0 >= 64) {
+#pragma unroll
+            for (int q = 0; q < 2 * CPR; ++q) {
+                const int t = (lane + 32 * q) / (2 * CPR), k = (lane + 32 * q) % (2 * CPR);
+                cp_async16(dst + t * 64 + k * CH, Fg + (int64_t)(r0 + t) * P + r0 + k * CH);
+            }
+        } else {                                                     // the last block: its own 32 columns
+#pragma unroll
+            for (int q = 0; q < CPR; ++q) {
+                const int t = (lane + 32 * q) / CPR, k = (lane + 32 * q) % CPR;
+                cp_async16(dst + t * 64 + k * CH, Fg + (int64_t)(r0 + t) * P + r0 + k * CH);
+            }
         }
     };
     constexpr bool WARP_WALK = std::is_same<T, float>::value;
     if (warp == (nthr > 32 ? 1 : 0)) {
-        if constexpr (WARP_WALK) copy_tile64(tiles, 0);
-        else copy_tile(tiles, 0, 0);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        // (a group is committed for every block, past the end an empty one, so that the waits below count blocks)
+        for (int c = 0; c < AHEAD; ++c) {
+            if constexpr (WARP_WALK) { if (c < nb) copy_tile64(tiles + c * 2048, 32 * c); }
+            else copy_tile(tiles, 0, 0);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
     }
     uint32_t cgroup, ccode;
     call_counter(g, lvl, cgroup, ccode);
@@ -572,42 +593,62 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
         r_s[i] = rdecay[(int64_t)p * pair_stride(n) + base + i];
         U_s[i] = halving_uniform<T>(seed, (uint32_t)i, cgroup, ccode, (uint32_t)p + pbase);
     }
-    if (warp <= 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (warp <= 1) asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
 
     // ---- updater streaming state ----
     const int NU = nthr - 64;                                        // updater threads (warps 2..)
     const int u = threadIdx.x - 64;
     // panel `pi` of round `r` (rows of block r): columns [32 (r + 2) + pi * PW, ...)
     auto panels_of = [&](int r) { const int cols = P - 32 * (r + 2); return cols > 0 ? (cols + PW - 1) / PW : 0; };
-    auto issue_panel = [&](int r, int pi, int buf) {
+    // the panels in the order they are used, each into the next of the PB buffers; past the last one an empty group
+    int next_r = 0, next_pi = 0, next_buf = 0;
+    auto issue_panel = [&]() {
+        const int r = next_r, pi = next_pi, buf = next_buf;
+        if (panels_of(r) == 0) {                                     // (rounds have fewer columns the later they are)
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            return;
+        }
+        if (++next_pi == panels_of(r)) { next_pi = 0; ++next_r; }
+        if (++next_buf == PB) next_buf = 0;
         const int col0 = 32 * (r + 2) + pi * PW;
         const int pw = P - col0 < PW ? P - col0 : PW;
         const int cpr = pw / CH;
         const T *rows = Fg + (int64_t)(32 * r) * P + col0;
         T *dst = panels + (size_t)buf * 32 * pw_alloc;
-        for (int q = u; q < 32 * cpr; q += NU) {
-            const int t = q / cpr, k = q % cpr;
-            cp_async16(dst + t * pw_alloc + k * CH, rows + (int64_t)t * P + k * CH);
-        }
+        // a warp takes a row at a time
+        for (int t = warp - 2; t < 32; t += NU >> 5)
+            for (int k = lane; k < cpr; k += 32) cp_async16(dst + t * pw_alloc + k * CH, rows + (int64_t)t * P + k * CH);
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    int stream = 0;                                                  // panels consumed so far (buffer parity)
-    if (warp >= 2 && panels_of(0) > 0) issue_panel(0, 0, 0);
+    int buf = 0;                                                     // buffer of the next panel to be used
+    if (warp >= 2)
+        for (int i = 0; i < PB - 1; ++i) issue_panel();
     __syncthreads();
 
     T bmax = 0;
     float dn = 0.f;                                                  // fp32 walker: the next block's scores from the current block
+    // thresholds do not depend on decisions: in long calls the copying warp has those of the next block ready (380 cycles
+    // off the walker; in short ones the barrier in front costs more than that)
+    auto thresholds = [&](int c) {
+        if constexpr (DEEP) a32_s[(c & 1) * 32 + lane] = walk_block_thresholds(b_s[32 * c + lane], r_s[32 * c + lane], bmax, logfac, lane);
+    };
+    if constexpr (DEEP) {
+        if (warp == 1) thresholds(0);
+        __syncthreads();
+    }
     for (int c = 0; c < nb; ++c) {
         const int i0 = 32 * c;
-        T *tdiag = tiles + (c & 1) * 2048, *tcross = tdiag + 1024;
-        T *ndiag = tiles + ((c + 1) & 1) * 2048, *ncross = ndiag + 1024;
+        T *tdiag = tiles + (c % TB) * 2048, *tcross = tdiag + 1024;
+        T *ndiag = tiles + ((c + AHEAD) % TB) * 2048, *ncross = ndiag + 1024;      // block c + AHEAD's; block c - 1's before
         if (warp == 0) {
             if constexpr (WARP_WALK) {
                 // the previous block folded its decisions into this block's scores as it went (dn)
-                const float a = walk_block_thresholds(b_s[i0 + lane], r_s[i0 + lane], bmax, logfac, lane);
+                float a;
+                if constexpr (DEEP) a = a32_s[(c & 1) * 32 + lane];
+                else a = walk_block_thresholds(b_s[i0 + lane], r_s[i0 + lane], bmax, logfac, lane);
                 const float d = walk_sign_score(alpha_s[i0 + lane] + dn, a, U_s[i0 + lane]);
                 dn = 0.f;
-                const uint32_t swaps = walk_block_warp(tiles + (c & 1) * 2048, 64, d, dn, lane);
+                const uint32_t swaps = walk_block_warp(tdiag, 64, d, dn, lane);
                 if (lane == 0) mask_s[c] = swaps;
             } else {
                 T alpha = alpha_s[i0 + lane];
@@ -627,29 +668,26 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
                 if (lane == 0) mask_s[c] = swaps;
             }
         } else if (warp == 1) {
-            if (c + 1 < nb) {
+            if (c + AHEAD < nb) {
                 if constexpr (WARP_WALK) {
-                    copy_tile64(tiles + ((c + 1) & 1) * 2048, i0 + 32);
+                    copy_tile64(ndiag, i0 + 32 * AHEAD);
                 } else {
+                    static_assert(WARP_WALK || AHEAD == 1, "the cross tile is block c's with block c + 1's columns");
                     copy_tile(ndiag, i0 + 32, i0 + 32);
                     copy_tile(ncross, i0, i0 + 32);
                 }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
+            if (c + 1 < nb) thresholds(c + 1);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");       // block c + 1's tile is there
         } else if (c > 0) {
             // round r = c-1: rows of block r into every column from block r+2 on
             const int r = c - 1;
             const uint32_t pm = mask_s[r];
             const int np = panels_of(r);
-            for (int pi = 0; pi < np; ++pi, ++stream) {
-                const int buf = stream & 1;
-                bool issued = true;
-                if (pi + 1 < np) issue_panel(r, pi + 1, buf ^ 1);
-                else if (panels_of(c) > 0) issue_panel(c, 0, buf ^ 1);       // first panel of the next round
-                else issued = false;
-                if (issued) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                else asm volatile("cp.async.wait_group 0;" ::: "memory");
+            for (int pi = 0; pi < np; ++pi) {
+                issue_panel();                                       // into the buffer of the panel used before this one
+                asm volatile("cp.async.wait_group %0;" ::"n"(PB - 1) : "memory");
                 asm volatile("bar.sync 1, %0;" ::"r"(NU) : "memory");
                 const int col0 = 32 * (r + 2) + pi * PW;
                 const int pw = P - col0 < PW ? P - col0 : PW;
@@ -663,6 +701,7 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
                     }
                     alpha_s[col0 + j] += acc;
                 }
+                if (++buf == PB) buf = 0;
                 asm volatile("bar.sync 1, %0;" ::"r"(NU) : "memory");
             }
         }
@@ -675,6 +714,8 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
         out[(int64_t)p * out_stride + base + i] = cur[(int64_t)p * n + 2 * (base + i) + sw];
     }
 }
+
+constexpr int WALK_DEEP_MIN_PAIRS = 256;
 
 // Smallest call (in pairs) that goes to the chain kernel of elm_walk_chain.cu.  From about a
 // thousand pairs on, a call is worth a cluster of CTAs; below that one CTA per call (walk_cta_kernel)
@@ -843,15 +884,22 @@ static int run_halve_level(const LevelCtx<Tin, T> &c, const int32_t *cur, int32_
         if (chain_rc == ELM_OK) {
             // launched by walk_chain
         } else if (P >= 32) {
-            // walker warp + tile-copy warp + updaters (one per two pairs, at most 512 threads)
-            int upd = P / 2;
+            // walker warp + tile-copy warp + updaters: a thread per column of long calls (at most 512), per two of the
+            // others, which share the SM (64 and 128 pairs, a thread per column: 52 and 44 us against 42 and 34)
+            int upd = P >= WALK_DEEP_MIN_PAIRS ? P : P / 2;
             upd = upd < 32 ? 32 : (upd > 512 ? 512 : upd);
             const int threads = P == 32 ? 32 : 64 + upd;
             constexpr int PW = 2048 / sizeof(T);
             const int pw_alloc = P - 64 < PW ? (P - 64 > 0 ? P - 64 : 32) : PW;
-            const size_t smem = (size_t)(4 * 1024 + 4 * P + 32 + 2 * 32 * pw_alloc) * sizeof(T) + (size_t)(P / 32) * 4;
+            auto smem_for = [&](int tb, int pb) {
+                return (size_t)(tb * 2048 + 4 * P + 64 + pb * 32 * pw_alloc) * sizeof(T) + (size_t)(P / 32) * 4;
+            };
+            const bool deep = std::is_same<T, float>::value && P >= WALK_DEEP_MIN_PAIRS && smem_for(4, 3) <= 227 * 1024;
+            const size_t smem = deep ? smem_for(4, 3) : smem_for(2, 2);
             if (smem > 227 * 1024) return ELM_ERR_SHAPE;               // a call this long needs the chain kernel
-            auto kern = walk_cta_kernel<T>;
+            auto kern = walk_cta_kernel<T, false>;
+            if constexpr (std::is_same<T, float>::value)
+                if (deep) kern = walk_cta_kernel<T, true>;
             ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             ELM_CUDA_TRY(launch_after(kern, dim3((unsigned)groups, (unsigned)BH), dim3(threads), smem, st,
                                       c.F, c.F_stride, c.rdecay, cur, out, out_stride, n, P, lvl, c.seed, logfac, c.pbase));
