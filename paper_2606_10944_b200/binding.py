@@ -117,10 +117,11 @@ def _check(rc: int, what: str):
 
 
 def _require_cuda(*tensors):
-    if not torch.cuda.is_available():
-        raise ElmError("no CUDA device: the library has no CPU fallback")
     for t in tensors:
         if not t.is_cuda or not t.is_contiguous():
+            # (asked only now: a CUDA tensor answers it, and the question costs more than a kernel launch)
+            if not torch.cuda.is_available():
+                raise ElmError("no CUDA device: the library has no CPU fallback")
             raise ElmError("tensors must be contiguous CUDA tensors")
 
 
@@ -135,7 +136,8 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the current device's current stream, without a torch.cuda.Stream object made for every call
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def make_params(batch, q_heads, kv_heads, n_kv, n_q, d, log2_nout, m, dtype_code, precision="fp32",
