@@ -118,12 +118,22 @@ __global__ void __launch_bounds__(256) gather_tc_kernel(const __nv_bfloat16 *__r
     const float w0 = w[(int64_t)p * n_core];
     bool differs = false;
     // rows move in 16-byte chunks: lanes 0 .. CH-1 the key row (straight to Kc), lanes 16 .. 16+CH-1 the
-    // value row (to shared memory, to be written transposed)
-    for (int r = warp; r < GATHER_COLS; r += 8) {
-        const int c = c0 + r;
+    // value row (to shared memory, to be written transposed).  A warp's eight row numbers and weights are fetched by eight
+    // lanes, then its rows four at a time: one after the other, number and row, they were sixteen dependent reads.
+    // Four launches of a prefill of 131072 tokens: 562 -> 499 us.
+    int32_t row_mine = 0;
+    float w_mine = 0.f;
+    if (lane < GATHER_COLS / 8 && c0 + warp + 8 * lane < n_core) {
+        row_mine = (int32_t)checked_row(idx[(int64_t)p * n_core + c0 + warp + 8 * lane], n, nonuniform + gridDim.y);
+        w_mine = w[(int64_t)p * n_core + c0 + warp + 8 * lane];
+    }
+    const int chunk = lane & 15;
+#pragma unroll 4
+    for (int i = 0; i < GATHER_COLS / 8; ++i) {
+        const int r = warp + 8 * i, c = c0 + r;
         const bool ok = c < n_core;
-        const int64_t row = ok ? checked_row(idx[(int64_t)p * n_core + c], n, nonuniform + gridDim.y) : 0;
-        const int chunk = lane & 15;
+        const int64_t row = __shfl_sync(0xffffffffu, row_mine, i);
+        const float wc = __shfl_sync(0xffffffffu, w_mine, i);
         if constexpr (E4M3) {
             // a row is D bytes = D / 16 chunks
             const unsigned char *K8 = reinterpret_cast<const unsigned char *>(K), *V8 = reinterpret_cast<const unsigned char *>(V);
@@ -153,7 +163,6 @@ __global__ void __launch_bounds__(256) gather_tc_kernel(const __nv_bfloat16 *__r
             }
         }
         if (lane < 16) {
-            const float wc = ok ? w[(int64_t)p * n_core + c] : 0.f;
             // in the logits' own units (they are multiplied by scale_log2 later); -1e30 hides a padded column
             const float x = ok ? log2f(wc) * inv_scale_log2 : -1e30f;
             const __nv_bfloat16 hi = __float2bfloat16(x);
