@@ -382,6 +382,11 @@ int elm_debug_set(int32_t what, int64_t value);
 int elm_debug_round_check(const elm_params *params, int32_t mbar, int32_t r, uint64_t seed, int64_t *missing,
                           int64_t *listed_blocks, int64_t *needed_blocks, int64_t *partly_blocks);
 
+/* How elm_attend with these params and a list of n_core entries lays out a decode call (fp32 mode, at most 8 query
+ * vectors per KV head; else ELM_ERR_SHAPE): the CTAs it launches, and how many of them the current device holds at
+ * once.  For tests. */
+int elm_debug_decode_grid(const elm_params *params, int32_t n_core, int32_t *ctas, int32_t *resident);
+
 /* Kernels launched by this library since it was loaded (all calls, all stages). */
 int64_t elm_launch_count(void);
 

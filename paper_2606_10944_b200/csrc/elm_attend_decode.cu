@@ -44,6 +44,14 @@ using sm100::unpack2;
 constexpr int DEC_WARPS = 4;
 constexpr int DEC_GMAX = 8;
 constexpr int DEC_MAX_CLUSTER = 16;
+constexpr int DEC_CTAS = 3;                                      // CTAs per SM the kernel is compiled for
+
+// grid (splits, problems); partial results part[problem][split][g][D + 2] = accumulator (D), maximum, denominator
+constexpr int DEC_SPLIT = 0;
+// grid (cluster size, problems), one token: rank r of the cluster takes the r-th part of the list
+constexpr int DEC_CLUSTER = 1;
+// grid (token groups, problems): neighbouring tokens, part after part
+constexpr int DEC_TOKENS = 2;
 
 template <typename Tin, int D, int G> struct DecodeCfg {
     static constexpr int RB = D * (int)sizeof(Tin);              // bytes per row
@@ -55,14 +63,25 @@ template <typename Tin, int D, int G> struct DecodeCfg {
     static constexpr int NV = UB * G;                            // partial sums per lane: 4, 8 or 16
     static constexpr int EPI = 32 / NC;                          // entries a warp takes at a time in the value pass
     static constexpr int TILE_BYTES = TILE * RB;
-    // shared memory: per warp a K tile, a V tile and the tile's logits; the scaled queries; what the cluster sends
+    // shared memory: per warp a K tile, a V tile and the tile's logits; the scaled queries; what a form needs besides
     static constexpr int OFF_SC = DEC_WARPS * 2 * TILE_BYTES;
     static constexpr int OFF_Q = OFF_SC + DEC_WARPS * 32 * G * 4;
     static constexpr int OFF_ML = OFF_Q + G * D * 4;             // [DEC_WARPS][G][2]
-    static constexpr int OFF_RML = OFF_ML + DEC_WARPS * G * 2 * 4;      // [DEC_MAX_CLUSTER][G][2]
-    // [ranks][slice] with slice = ceil(G D / ranks): at most G D + DEC_MAX_CLUSTER floats
+    // DEC_CLUSTER: what the other ranks send, [DEC_MAX_CLUSTER][G][2] and [ranks][slice] with slice = ceil(G D / ranks),
+    // at most G D + DEC_MAX_CLUSTER floats.  DEC_TOKENS: the running maxima and denominators, [2][G][2].
+    static constexpr int OFF_RML = OFF_ML + DEC_WARPS * G * 2 * 4;
     static constexpr int OFF_RECV = OFF_RML + DEC_MAX_CLUSTER * G * 2 * 4;
-    static constexpr int TOTAL = OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4;
+    template <int MODE> static constexpr int total()
+    {
+        return MODE == DEC_SPLIT ? OFF_RML : MODE == DEC_TOKENS ? OFF_RML + 2 * G * 2 * 4 : OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4;
+    }
+    // CTAs an SM holds: of 228 KB shared memory the system takes 1 KB per CTA; registers are kept to what three leave
+    // (launch bounds).  DEC_SPLIT and DEC_TOKENS always get three; DEC_CLUSTER two at G = 8 and D = 128 (79 KB), where
+    // two against three cost 1.2 times the time (8 problems x 5193 entries, split form: 24.0 against 20.0 us).
+    template <int MODE> static constexpr int ctas_per_sm()
+    {
+        return 228 * 1024 / (total<MODE>() + 1024) < DEC_CTAS ? 228 * 1024 / (total<MODE>() + 1024) : DEC_CTAS;
+    }
 };
 
 __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool live)
@@ -111,15 +130,8 @@ __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entrie
     chunk = ((len + parts - 1) / parts + tile - 1) / tile * tile;
 }
 
-// grid (splits, problems); partial results part[problem][split][g][D + 2] = accumulator (D), maximum, denominator
-constexpr int DEC_SPLIT = 0;
-// grid (cluster size, problems), one token: rank r of the cluster takes the r-th part of the list
-constexpr int DEC_CLUSTER = 1;
-// grid (token groups, problems): neighbouring tokens, part after part
-constexpr int DEC_TOKENS = 2;
-
 template <typename Tin, int D, int G, int MODE>
-__global__ void __launch_bounds__(DEC_WARPS * 32, 3)
+__global__ void __launch_bounds__(DEC_WARPS * 32, DEC_CTAS)
 decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *__restrict__ V,
               const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int64_t list_stride, int q_heads,
               int kv_heads, int n_q, int per_token /* query vectors of a token */, const __grid_constant__ DecodeWindows win,
@@ -211,8 +223,12 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         if (g < groups) x = load_as<float>(Q, q_row(g) + dim) * scale;
         qs[(((g * CH + ck / 8) * (EPC / 4) + in / 4) * 8 + ck % 8) * 4 + in % 4] = x;
     }
+    // DEC_TOKENS: the running accumulators, element tid + 128 k of [g][D]
+    constexpr int EPT = (G * D + DEC_WARPS * 32 - 1) / (DEC_WARPS * 32);
+    float run[MODE == DEC_TOKENS ? EPT : 1];
     if constexpr (MODE == DEC_TOKENS) {
-        for (int i = tid; i < G * D; i += DEC_WARPS * 32) recv[i] = 0.f;       // (each element stays with its thread)
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) run[k] = 0.f;
         if (tid < G) { rml[tid * 2] = -INFINITY; rml[tid * 2 + 1] = 0.f; }
     }
     // what query vector g sees of the list (DEC_TOKENS: its token's prefix)
@@ -412,7 +428,10 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         return a;
     };
     if (pt < parts) {
-        for (int i = tid; i < G * D; i += DEC_WARPS * 32) {
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            const int i = tid + k * DEC_WARPS * 32;
+            if (i >= G * D) break;
             const int g = i / D;
             float M = -INFINITY;
 #pragma unroll
@@ -436,9 +455,8 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
             } else if constexpr (MODE == DEC_TOKENS) {
                 // (running maximum and denominator in two buffers, part pt reading one and writing the other)
                 const float *was = rml + ((pt & 1) * G + g) * 2;
-                float Mr = was[0], dr = was[1], ar = recv[i];
-                merge_part(Mr, dr, ar, M, den, acc);
-                recv[i] = ar;
+                float Mr = was[0], dr = was[1];
+                merge_part(Mr, dr, run[k], M, den, acc);
                 if (i % D == 0) {
                     float *now = rml + (((pt + 1) & 1) * G + g) * 2;
                     now[0] = Mr;
@@ -469,8 +487,11 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
     }
     if constexpr (MODE == DEC_TOKENS) {
         __syncthreads();
-        for (int i = tid; i < groups * D; i += DEC_WARPS * 32)
-            store_from(O, q_row(i / D) + i % D, recv[i] / rml[((parts & 1) * G + i / D) * 2 + 1]);
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            const int i = tid + k * DEC_WARPS * 32;
+            if (i < groups * D) store_from(O, q_row(i / D) + i % D, run[k] / rml[((parts & 1) * G + i / D) * 2 + 1]);
+        }
     }
 }
 
@@ -544,20 +565,46 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float *__restrict
     store_from(O, (((int64_t)b * q_heads + h) * n_q + r) * D + d, acc / den);
 }
 
-// Streaming tokens: most parts of a list - a power of two, so that three CTAs per SM (what shared memory allows) hold
-// one token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
-// most SMs idle is left to the form with partial results in the workspace.
-static int decode_cap(int problems)
+// Calls `f` with the compile-time query count that covers `groups`
+template <typename F> auto with_groups(int groups, F f)
 {
-    const int most = 3 * device_sm_count() / problems;
+    if (groups <= 1) return f(std::integral_constant<int, 1>());
+    if (groups <= 2) return f(std::integral_constant<int, 2>());
+    if (groups <= 4) return f(std::integral_constant<int, 4>());
+    return f(std::integral_constant<int, 8>());
+}
+
+// Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
+// token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
+// most SMs idle is left to the form with partial results in the workspace.
+template <typename Tin, int D> int decode_cap(int problems, int per_token)
+{
+    const int ctas = with_groups(per_token, [](auto G) { return DecodeCfg<Tin, D, decltype(G)::value>::template ctas_per_sm<DEC_CLUSTER>(); });
+    const int most = ctas * device_sm_count() / problems;
     int cap = DEC_MAX_CLUSTER;
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
 }
-template <typename Tin, int D, int G> bool decode_clustered(int n_core, int problems)
+template <typename Tin, int D> bool decode_clustered(int n_core, int problems, int per_token)
 {
-    const int cap = decode_cap(problems), entries = DEC_WARPS * DecodeCfg<Tin, D, G>::TILE;
+    // (a tile's entries do not depend on the number of query vectors)
+    const int cap = decode_cap<Tin, D>(problems, per_token), entries = DEC_WARPS * DecodeCfg<Tin, D, 1>::TILE;
     return n_core <= 8 * entries * cap || problems * cap >= device_sm_count();
+}
+
+// How many CTAs per problem elm_attend's list is split over: as many as are resident at once, but at least one tile
+// per warp, and no more partial results than the workspace has room for.
+template <typename Tin, int D, int G> int decode_splits(int n_core, int problems, size_t part_room)
+{
+    using C = DecodeCfg<Tin, D, G>;
+    static_assert(C::template ctas_per_sm<DEC_SPLIT>() == DEC_CTAS && C::template ctas_per_sm<DEC_TOKENS>() == DEC_CTAS,
+                  "shared memory for as many CTAs as there are registers for");
+    int splits = (n_core + DEC_WARPS * C::TILE - 1) / (DEC_WARPS * C::TILE);
+    const int wanted = C::template ctas_per_sm<DEC_SPLIT>() * device_sm_count() / problems;
+    if (splits > wanted) splits = wanted < 1 ? 1 : wanted;
+    const size_t most = part_room / ((size_t)problems * G * (D + 2) * sizeof(float));
+    if ((size_t)splits > most) splits = (int)most;
+    return splits > DEC_MAX_SPLITS ? DEC_MAX_SPLITS : splits;
 }
 
 // win set: streaming tokens (G counts the query vectors of a CTA: of one token, or of several when the launch holds
@@ -574,7 +621,6 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(DEC_WARPS * 32);
-    cfg.dynamicSmemBytes = C::TOTAL;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -582,9 +628,16 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     const int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
     DecodeGroups grp = {};
     if (win) {
-        const int cap = decode_cap(problems), tokens = win->tok0[win->n];
-        auto kern = tokens == 1 ? decode_kernel<Tin, D, G, DEC_CLUSTER> : decode_kernel<Tin, D, G, DEC_TOKENS>;
-        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::TOTAL));
+        const int cap = decode_cap<Tin, D>(problems, per_token), tokens = win->tok0[win->n];
+        auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
+        cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
+        if constexpr (G == DEC_GMAX) {                             // (what dispatch_decode gives launches of several tokens)
+            if (tokens > 1) {
+                kern = decode_kernel<Tin, D, G, DEC_TOKENS>;
+                cfg.dynamicSmemBytes = C::template total<DEC_TOKENS>();
+            }
+        }
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
         if (tokens == 1) {
             int parts, chunk, size = 1;
             decode_parts(win->seen0[0], DEC_WARPS * C::TILE, C::TILE, cap, parts, chunk);
@@ -614,16 +667,11 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     whole.n = 1;
     whole.tok0[1] = 1;
     whole.seen0[0] = n_core;
-    // as many CTAs as are resident at once, but at least one tile per warp
-    int splits = (n_core + DEC_WARPS * C::TILE - 1) / (DEC_WARPS * C::TILE);
-    const int wanted = 3 * device_sm_count() / problems;
-    if (splits > wanted) splits = wanted < 1 ? 1 : wanted;
-    const size_t most = part_room / ((size_t)problems * G * (D + 2) * sizeof(float));
-    if ((size_t)splits > most) splits = (int)most;
-    if (splits > DEC_MAX_SPLITS) splits = DEC_MAX_SPLITS;
+    const int splits = decode_splits<Tin, D, G>(n_core, problems, part_room);
     if (splits < 1) return ELM_ERR_WORKSPACE;
     auto kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
-    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::TOTAL));
+    cfg.dynamicSmemBytes = C::template total<DEC_SPLIT>();
+    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
     cfg.gridDim = dim3((unsigned)splits, (unsigned)problems);
     ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, whole, grp, 0, O,
                                     part, status));
@@ -636,14 +684,6 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     return cuda_status(cudaGetLastError());
 }
 
-// Calls `f` with the compile-time query count that covers `groups`
-template <typename F> int with_groups(int groups, F f)
-{
-    if (groups <= 1) return f(std::integral_constant<int, 1>());
-    if (groups <= 2) return f(std::integral_constant<int, 2>());
-    if (groups <= 4) return f(std::integral_constant<int, 4>());
-    return f(std::integral_constant<int, 8>());
-}
 template <typename Tin>
 int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
                     const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
@@ -669,12 +709,28 @@ bool attend_decode_applies(const elm_params *p)
 bool attend_decode_windows_apply(const elm_params *p, int n_core)
 {
     if (!attend_decode_applies(p) || p->n_q != 1 || (p->dtype != ELM_F32 && p->dtype != ELM_BF16)) return false;
-    const int problems = p->batch * p->kv_heads;
-    // (a tile's entries do not depend on the number of query vectors)
+    const int problems = p->batch * p->kv_heads, per_token = p->q_heads / p->kv_heads;
     if (p->dtype == ELM_F32)
-        return p->d == 64 ? decode_clustered<float, 64, 1>(n_core, problems) : decode_clustered<float, 128, 1>(n_core, problems);
-    return p->d == 64 ? decode_clustered<__nv_bfloat16, 64, 1>(n_core, problems) : decode_clustered<__nv_bfloat16, 128, 1>(n_core, problems);
+        return p->d == 64 ? decode_clustered<float, 64>(n_core, problems, per_token) : decode_clustered<float, 128>(n_core, problems, per_token);
+    return p->d == 64 ? decode_clustered<__nv_bfloat16, 64>(n_core, problems, per_token)
+                      : decode_clustered<__nv_bfloat16, 128>(n_core, problems, per_token);
 }
+
+namespace {
+template <typename Tin, int D, int G> int decode_grid(const elm_params *p, int n_core, int32_t *ctas, int32_t *resident)
+{
+    using C = DecodeCfg<Tin, D, G>;
+    const int problems = p->batch * p->kv_heads, smem = C::template total<DEC_SPLIT>();
+    const AttendLayout L = attend_layout(p, n_core);
+    auto kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
+    int per_sm = 0;
+    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ELM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DEC_WARPS * 32, (size_t)smem));
+    *ctas = decode_splits<Tin, D, G>(n_core, problems, L.bias - L.Kc) * problems;
+    *resident = per_sm * device_sm_count();
+    return ELM_OK;
+}
+}  // namespace
 
 int attend_decode_windows(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
                           const DecodeWindows &win, const elm_params *p, void *O, int *status, cudaStream_t st)
@@ -706,3 +762,19 @@ int attend_decode(const void *Q, const void *K, const void *V, const int32_t *id
 }
 
 }  // namespace elm
+
+extern "C" int elm_debug_decode_grid(const elm_params *params, int32_t n_core, int32_t *ctas, int32_t *resident)
+{
+    using namespace elm;
+    if (!params || !ctas || !resident) return ELM_ERR_NULL;
+    const int rc = validate_attend_params(params);
+    if (rc != ELM_OK) return rc;
+    if (n_core < 1 || n_core > params->n_kv || !attend_decode_applies(params)) return ELM_ERR_SHAPE;
+    return with_groups((params->q_heads / params->kv_heads) * params->n_q, [&](auto G) {
+        constexpr int g = decltype(G)::value;
+        if (params->dtype == ELM_F32)
+            return params->d == 64 ? decode_grid<float, 64, g>(params, n_core, ctas, resident) : decode_grid<float, 128, g>(params, n_core, ctas, resident);
+        return params->d == 64 ? decode_grid<__nv_bfloat16, 64, g>(params, n_core, ctas, resident)
+                               : decode_grid<__nv_bfloat16, 128, g>(params, n_core, ctas, resident);
+    });
+}
