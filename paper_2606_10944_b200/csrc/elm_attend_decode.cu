@@ -17,12 +17,11 @@
 // number -> row -> softmax -> merge.
 //
 // The list of an attention problem is split over CTAs.  elm_attend: over as many as the SMs can hold, which leave
-// partial results (maximum, denominator, accumulator) in the workspace for decode_merge_kernel.  A single token of a
-// streaming run: over the CTAs of a thread-block cluster, which hand each other their partial results through
-// distributed shared memory.  Many tokens of a streaming run in one launch (DecodeWindows: a token sees a prefix of its
-// window's list): a CTA takes as many neighbouring tokens as fit the G query vectors and walks the parts of the list
-// one after the other - the same parts, tiles and merges in the same order as the cluster's, so a token's output is the
-// same bit for bit whichever launch computes it.
+// partial results (maximum, denominator, accumulator) in the workspace for decode_merge_kernel.  Tokens of a streaming
+// run (DecodeWindows: a token sees a prefix of its window's list): each over the CTAs of a thread-block cluster, which
+// hand each other their partial results through distributed shared memory, or, once there are tokens enough to fill the
+// SMs, by one CTA that walks the parts of the list one after the other (decode_form) - the same parts, tiles and merges
+// in the same order as the cluster's, so a token's output is the same bit for bit whichever launch computes it.
 #include <math.h>
 
 #include <type_traits>
@@ -43,15 +42,18 @@ using sm100::unpack2;
 
 constexpr int DEC_WARPS = 4;
 constexpr int DEC_GMAX = 8;
+constexpr int DEC_GSERIAL = 4;         // fewest query vectors of a CTA that walks the parts of a list one after the other
 constexpr int DEC_MAX_CLUSTER = 16;
 constexpr int DEC_CTAS = 3;                                      // CTAs per SM the kernel is compiled for
 
 // grid (splits, problems); partial results part[problem][split][g][D + 2] = accumulator (D), maximum, denominator
 constexpr int DEC_SPLIT = 0;
-// grid (cluster size, problems), one token: rank r of the cluster takes the r-th part of the list
+// grid (tokens x cluster size, problems): rank r of a token's cluster takes the r-th part of its list
 constexpr int DEC_CLUSTER = 1;
-// grid (token groups, problems): neighbouring tokens, part after part
+// grid (tokens, problems): a token's parts one after the other
 constexpr int DEC_TOKENS = 2;
+// grid (groups, problems): the same for neighbouring tokens whose query vectors fit G together
+constexpr int DEC_NEIGHBOURS = 3;
 
 template <typename Tin, int D, int G> struct DecodeCfg {
     static constexpr int RB = D * (int)sizeof(Tin);              // bytes per row
@@ -68,12 +70,12 @@ template <typename Tin, int D, int G> struct DecodeCfg {
     static constexpr int OFF_Q = OFF_SC + DEC_WARPS * 32 * G * 4;
     static constexpr int OFF_ML = OFF_Q + G * D * 4;             // [DEC_WARPS][G][2]
     // DEC_CLUSTER: what the other ranks send, [DEC_MAX_CLUSTER][G][2] and [ranks][slice] with slice = ceil(G D / ranks),
-    // at most G D + DEC_MAX_CLUSTER floats.  DEC_TOKENS: the running maxima and denominators, [2][G][2].
+    // at most G D + DEC_MAX_CLUSTER floats.  DEC_TOKENS, DEC_NEIGHBOURS: the running maxima and denominators, [2][G][2].
     static constexpr int OFF_RML = OFF_ML + DEC_WARPS * G * 2 * 4;
     static constexpr int OFF_RECV = OFF_RML + DEC_MAX_CLUSTER * G * 2 * 4;
     template <int MODE> static constexpr int total()
     {
-        return MODE == DEC_SPLIT ? OFF_RML : MODE == DEC_TOKENS ? OFF_RML + 2 * G * 2 * 4 : OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4;
+        return MODE == DEC_SPLIT ? OFF_RML : MODE == DEC_CLUSTER ? OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4 : OFF_RML + 2 * G * 2 * 4;
     }
     // CTAs an SM holds: of 228 KB shared memory the system takes 1 KB per CTA; registers are kept to what three leave
     // (launch bounds).  DEC_SPLIT and DEC_TOKENS always get three; DEC_CLUSTER two at G = 8 and D = 128 (79 KB), where
@@ -114,9 +116,10 @@ __device__ __forceinline__ void merge_part(float &M, float &den, float &acc, flo
     M = Mn;
 }
 
-// DEC_TOKENS: which tokens a CTA takes
+// The groups of tokens of a streaming launch
 struct DecodeGroups {
-    int32_t per_group;                             // tokens per CTA: a power of two, at most 8
+    int32_t cluster;                               // CTAs per group
+    int32_t per_group;                             // tokens per group: a power of two, 1 but in DEC_NEIGHBOURS
     int32_t g0[DECODE_MAX_WINDOWS + 1];            // groups of the windows before
 };
 
@@ -151,7 +154,9 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
     // nothing is read or written before this point)
     cudaGridDependencySynchronize();
     if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    const int prob = blockIdx.y, rank = MODE == DEC_TOKENS ? 0 : blockIdx.x;
+    constexpr bool SERIAL = MODE == DEC_TOKENS || MODE == DEC_NEIGHBOURS;
+    const int prob = blockIdx.y, group = MODE == DEC_SPLIT ? 0 : (int)blockIdx.x / grp.cluster;
+    const int rank = (int)blockIdx.x - group * grp.cluster;
 #ifndef ELM_BOUNDS_CHECK
     // this path has no bounded waits and (in this build) no row checks: its status word reads 0 - written here
     // rather than by a memset of its own
@@ -159,10 +164,10 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
 #endif
     // the tokens: z0 .. z0 + tokens - 1 of the launch, the first of which sees seen0 entries, the next one more, ...
     int wi = 0, z0 = 0, tokens = 1, seen0 = win.seen0[0];
-    if constexpr (MODE == DEC_TOKENS) {
-        while (wi + 1 < win.n && (int)blockIdx.x >= grp.g0[wi + 1]) ++wi;
+    if constexpr (MODE != DEC_SPLIT) {
+        while (wi + 1 < win.n && group >= grp.g0[wi + 1]) ++wi;
         // group k of a window: the tokens that see (k0 + k) per_group + 1 .. (k0 + k + 1) per_group entries
-        const int first = ((win.seen0[wi] - 1) / grp.per_group + ((int)blockIdx.x - grp.g0[wi])) * grp.per_group + 1;
+        const int first = ((win.seen0[wi] - 1) / grp.per_group + (group - grp.g0[wi])) * grp.per_group + 1;
         const int last_seen = win.seen0[wi] + (win.tok0[wi + 1] - win.tok0[wi]) - 1;
         seen0 = first > win.seen0[wi] ? first : win.seen0[wi];
         const int end = first + grp.per_group - 1 < last_seen ? first + grp.per_group - 1 : last_seen;
@@ -223,19 +228,19 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         if (g < groups) x = load_as<float>(Q, q_row(g) + dim) * scale;
         qs[(((g * CH + ck / 8) * (EPC / 4) + in / 4) * 8 + ck % 8) * 4 + in % 4] = x;
     }
-    // DEC_TOKENS: the running accumulators, element tid + 128 k of [g][D]
+    // SERIAL: the running accumulators, element tid + 128 k of [g][D]
     constexpr int EPT = (G * D + DEC_WARPS * 32 - 1) / (DEC_WARPS * 32);
-    float run[MODE == DEC_TOKENS ? EPT : 1];
-    if constexpr (MODE == DEC_TOKENS) {
+    float run[SERIAL ? EPT : 1];
+    if constexpr (SERIAL) {
 #pragma unroll
         for (int k = 0; k < EPT; ++k) run[k] = 0.f;
         if (tid < G) { rml[tid * 2] = -INFINITY; rml[tid * 2 + 1] = 0.f; }
     }
-    // what query vector g sees of the list (DEC_TOKENS: its token's prefix)
-    auto limit = [&](int g) { return MODE == DEC_TOKENS ? seen0 + g / per_token : n_core; };
+    // what query vector g sees of the list: its token's prefix
+    auto limit = [&](int g) { return MODE == DEC_NEIGHBOURS ? seen0 + g / per_token : n_core; };
     const int gl = lane >> 3, sub = lane & 7;
 
-    for (int pt = rank; pt < (MODE == DEC_TOKENS ? parts : rank + 1); ++pt) {
+    for (int pt = rank; pt < (SERIAL ? parts : rank + 1); ++pt) {
     c0 = pt * chunk < n_core ? pt * chunk : n_core;
     c1 = pt < parts ? (c0 + chunk < n_core ? c0 + chunk : n_core) : c0;
     int t0 = c0 + warp * TILE;
@@ -335,7 +340,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         float alpha[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const bool live = lane < TILE && t0 + lane < (MODE == DEC_TOKENS ? min(c1, limit(g)) : c1);
+            const bool live = lane < TILE && t0 + lane < (MODE == DEC_NEIGHBOURS ? min(c1, limit(g)) : c1);
             const float s = live ? sc[lane * G + g] + lw : -INFINITY;            // base-2 logit
             float mx = s;
 #pragma unroll
@@ -379,7 +384,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 // (an entry behind the token's own must not meet its zero probability: it might be infinite)
-                if (MODE == DEC_TOKENS && t0 + TILE > seen0 && t0 + e >= limit(g)) continue;
+                if (MODE == DEC_NEIGHBOURS && t0 + TILE > seen0 && t0 + e >= limit(g)) continue;
                 const uint64_t p2 = pack2(pe[g], pe[g]);
 #pragma unroll
                 for (int j = 0; j < EPC / 2; ++j) o[g][j] = fma2(p2, vf[j], o[g][j]);
@@ -452,7 +457,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
                     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(M) : "memory");
                     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a + 4), "f"(den) : "memory");
                 }
-            } else if constexpr (MODE == DEC_TOKENS) {
+            } else if constexpr (SERIAL) {
                 // (running maximum and denominator in two buffers, part pt reading one and writing the other)
                 const float *was = rml + ((pt & 1) * G + g) * 2;
                 float Mr = was[0], dr = was[1];
@@ -485,7 +490,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         }
     }
     }
-    if constexpr (MODE == DEC_TOKENS) {
+    if constexpr (SERIAL) {
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
@@ -607,12 +612,42 @@ template <typename Tin, int D, int G> int decode_splits(int n_core, int problems
     return splits > DEC_MAX_SPLITS ? DEC_MAX_SPLITS : splits;
 }
 
-// win set: streaming tokens (G counts the query vectors of a CTA: of one token, or of several when the launch holds
-// more than one); else the list of elm_attend, n_core entries long
+// How a launch of streaming tokens is laid out: query vectors per group, tokens per group, CTAs per group's cluster (0:
+// one CTA per group, part after part).
+struct DecodeForm {
+    int32_t vectors, per_group, cluster;
+};
+template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, int problems, int per_token)
+{
+    constexpr int TILE = DecodeCfg<Tin, D, 1>::TILE;               // (does not depend on the number of query vectors)
+    int longest = 0, parts, chunk, size = 1;
+    for (int i = 0; i < win.n; ++i) {
+        const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
+        longest = last > longest ? last : longest;
+    }
+    decode_parts(longest, DEC_WARPS * TILE, TILE, decode_cap<Tin, D>(problems, per_token), parts, chunk);
+    while (size < parts) size <<= 1;
+    const int64_t tokens = win.tok0[win.n];
+    if (tokens == 1) return {per_token, 1, size};
+    // tokens that share a CTA when it walks the parts itself
+    int per_group = 1;
+    while (per_group * 2 * per_token <= DEC_GSERIAL) per_group *= 2;
+    const int vectors = per_token > DEC_GSERIAL ? DEC_GMAX : DEC_GSERIAL;
+    // Clusters spread a token over the SMs and are never slower than the tokens one by one (6144 entries, 8 KV heads of 4
+    // query heads, bf16: 2 tokens 23 us, 8 tokens 68 us, one token 18 us).  Walking part after part saves their barriers
+    // and merges but takes as long as one CTA needs for a whole list (137 us), so it pays from about one token per SM on
+    // (16 tokens of 8 heads: 119 us in clusters, 137 walked; 32 tokens: 224 against 185; 64: 431 against 345), from two
+    // on when its CTAs take several tokens (1 query head per KV head: 32 tokens 147 against 171, 64 tokens 282 against
+    // 172).  A list of one part needs no merge at all.
+    const bool serial = tokens * problems >= (per_group > 1 ? 2 : 1) * device_sm_count() || (parts == 1 && per_group == 1);
+    return serial ? DecodeForm{vectors, per_group, 0} : DecodeForm{per_token, 1, size};
+}
+
+// win set: streaming tokens, laid out as `form` says; else the list of elm_attend, n_core entries long
 template <typename Tin, int D, int G>
 int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
-                  const DecodeWindows *win, const elm_params *p, Tin *O, float *part, size_t part_room, int *status, int per_token,
-                  cudaStream_t st)
+                  const DecodeWindows *win, DecodeForm form, const elm_params *p, Tin *O, float *part, size_t part_room, int *status,
+                  int per_token, cudaStream_t st)
 {
     using C = DecodeCfg<Tin, D, G>;
     const int problems = p->batch * p->kv_heads;
@@ -628,36 +663,31 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     const int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
     DecodeGroups grp = {};
     if (win) {
-        const int cap = decode_cap<Tin, D>(problems, per_token), tokens = win->tok0[win->n];
+        const int cap = decode_cap<Tin, D>(problems, per_token);
+        grp.per_group = form.per_group;
+        for (int i = 0; i < win->n; ++i) {
+            const int last = win->seen0[i] + (win->tok0[i + 1] - win->tok0[i]) - 1;
+            grp.g0[i + 1] = grp.g0[i] + (last - 1) / grp.per_group - (win->seen0[i] - 1) / grp.per_group + 1;
+        }
         auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
         cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
-        if constexpr (G == DEC_GMAX) {                             // (what dispatch_decode gives launches of several tokens)
-            if (tokens > 1) {
+        if constexpr (G >= DEC_GSERIAL) {
+            if (form.cluster == 0) {
                 kern = decode_kernel<Tin, D, G, DEC_TOKENS>;
+                if constexpr (G == DEC_GSERIAL)
+                    if (form.per_group > 1) kern = decode_kernel<Tin, D, G, DEC_NEIGHBOURS>;
                 cfg.dynamicSmemBytes = C::template total<DEC_TOKENS>();
             }
         }
+        grp.cluster = form.cluster ? form.cluster : 1;
         ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
-        if (tokens == 1) {
-            int parts, chunk, size = 1;
-            decode_parts(win->seen0[0], DEC_WARPS * C::TILE, C::TILE, cap, parts, chunk);
-            while (size < parts) size <<= 1;
-            if (size > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            attr[1].id = cudaLaunchAttributeClusterDimension;
-            attr[1].val.clusterDim.x = (unsigned)size;
-            attr[1].val.clusterDim.y = 1;
-            attr[1].val.clusterDim.z = 1;
-            cfg.numAttrs = 2;
-            cfg.gridDim = dim3((unsigned)size, (unsigned)problems);
-        } else {
-            grp.per_group = 1;
-            while (grp.per_group * 2 * per_token <= G) grp.per_group *= 2;
-            for (int i = 0; i < win->n; ++i) {
-                const int last = win->seen0[i] + (win->tok0[i + 1] - win->tok0[i]) - 1;
-                grp.g0[i + 1] = grp.g0[i] + (last - 1) / grp.per_group - (win->seen0[i] - 1) / grp.per_group + 1;
-            }
-            cfg.gridDim = dim3((unsigned)grp.g0[win->n], (unsigned)problems);
-        }
+        if (grp.cluster > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)grp.cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+        cfg.gridDim = dim3((unsigned)(grp.g0[win->n] * grp.cluster), (unsigned)problems);
         ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, *win, grp,
                                         cap, O, (float *)nullptr, status));
         count_launches(1);
@@ -684,17 +714,26 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     return cuda_status(cudaGetLastError());
 }
 
-template <typename Tin>
+template <typename Tin, int D>
 int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
                     const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
 {
     const int per_token = (p->q_heads / p->kv_heads) * p->n_q;
-    return with_groups(win && win->tok0[win->n] > 1 ? DEC_GMAX : per_token, [&](auto G) {
-        const Tin *q = (const Tin *)Q, *k = (const Tin *)K, *v = (const Tin *)V;
-        constexpr int g = decltype(G)::value;
-        return p->d == 64 ? launch_decode<Tin, 64, g>(q, k, v, idx, w, list_stride, n_core, win, p, (Tin *)O, part, part_room, status, per_token, st)
-                          : launch_decode<Tin, 128, g>(q, k, v, idx, w, list_stride, n_core, win, p, (Tin *)O, part, part_room, status, per_token, st);
+    DecodeForm form = {per_token, 1, 0};
+    if (win) form = decode_form<Tin, D>(*win, p->batch * p->kv_heads, per_token);
+    return with_groups(form.vectors, [&](auto G) {
+        return launch_decode<Tin, D, decltype(G)::value>((const Tin *)Q, (const Tin *)K, (const Tin *)V, idx, w, list_stride, n_core, win,
+                                                         form, p, (Tin *)O, part, part_room, status, per_token, st);
     });
+}
+int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
+                    const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
+{
+    if (p->dtype == ELM_F32)
+        return p->d == 64 ? dispatch_decode<float, 64>(Q, K, V, idx, w, list_stride, n_core, win, p, O, part, part_room, status, st)
+                          : dispatch_decode<float, 128>(Q, K, V, idx, w, list_stride, n_core, win, p, O, part, part_room, status, st);
+    return p->d == 64 ? dispatch_decode<__nv_bfloat16, 64>(Q, K, V, idx, w, list_stride, n_core, win, p, O, part, part_room, status, st)
+                      : dispatch_decode<__nv_bfloat16, 128>(Q, K, V, idx, w, list_stride, n_core, win, p, O, part, part_room, status, st);
 }
 
 }  // namespace
@@ -739,8 +778,7 @@ int attend_decode_windows(const void *Q, const void *K, const void *V, const int
 #ifdef ELM_BOUNDS_CHECK
     ELM_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
 #endif
-    return p->dtype == ELM_F32 ? dispatch_decode<float>(Q, K, V, idx, w, list_stride, 0, &win, p, O, nullptr, 0, status, st)
-                               : dispatch_decode<__nv_bfloat16>(Q, K, V, idx, w, list_stride, 0, &win, p, O, nullptr, 0, status, st);
+    return dispatch_decode(Q, K, V, idx, w, list_stride, 0, &win, p, O, nullptr, 0, status, st);
 }
 
 int attend_decode(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int n_core,
@@ -757,8 +795,7 @@ int attend_decode(const void *Q, const void *K, const void *V, const int32_t *id
     // bad row numbers are reported through the status word
     ELM_CUDA_TRY(cudaMemsetAsync(ws + L.flags, 0, sizeof(int) * (size_t)(problems + 1), st));
 #endif
-    return p->dtype == ELM_F32 ? dispatch_decode<float>(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st)
-                               : dispatch_decode<__nv_bfloat16>(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st);
+    return dispatch_decode(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st);
 }
 
 }  // namespace elm
