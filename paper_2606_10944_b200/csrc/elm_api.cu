@@ -284,7 +284,10 @@ extern "C" int elm_attend_status(const void *workspace, const elm_params *params
     return ELM_OK;
 }
 
-extern "C" int elm_debug_set(int32_t what, int64_t value) { return elm::debug_set_attend_tc(what, value); }
+extern "C" int elm_debug_set(int32_t what, int64_t value) 
+{
+    return what == ELM_DEBUG_DECODE_LARGEST_CLUSTER ? elm::debug_set_attend_decode(what, value) : elm::debug_set_attend_tc(what, value);
+}
 
 extern "C" int elm_profile_enable(int on)
 {

@@ -63,8 +63,9 @@ int attend_tc(const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat1
               const float *w, int n_core, const elm_params *p, __nv_bfloat16 *O, unsigned char *ws,
               cudaStream_t st, bool timed, const AttendWindow &win = AttendWindow());
 
-// elm_debug_set for the hooks that live with the tensor-core attention
+// elm_debug_set for the hooks that live with the tensor-core attention and with the decode attention
 int debug_set_attend_tc(int32_t what, int64_t value);
+int debug_set_attend_decode(int32_t what, int64_t value);
 
 // [count] E4M3 bytes -> bf16, exactly (every E4M3 value is a bf16 value)
 int widen_e4m3(const void *src, void *dst_bf16, int64_t count, cudaStream_t st);

@@ -24,6 +24,8 @@
 // in the same order as the cluster's, so a token's output is the same bit for bit whichever launch computes it.
 #include <math.h>
 
+#include <atomic>
+#include <mutex>
 #include <type_traits>
 
 #include "elm_attend.cuh"
@@ -579,6 +581,44 @@ template <typename F> auto with_groups(int groups, F f)
     return f(std::integral_constant<int, 8>());
 }
 
+// The largest cluster (a power of two, at most DEC_MAX_CLUSTER) of which the current device can hold one, asked once per
+// device: more than 8 CTAs need the opt-in and a GPC with that many SMs to give, which a partition of a GPU may not have.
+std::atomic<int> g_debug_largest_cluster{0};
+template <typename Tin, int D, int G> int decode_largest_cluster()
+{
+    static std::mutex mu;
+    static int cached[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    std::lock_guard<std::mutex> lock(mu);
+    if (cached[dev] == 0) {
+        using C = DecodeCfg<Tin, D, G>;
+        auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.blockDim = dim3(DEC_WARPS * 32);
+        cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int size = DEC_MAX_CLUSTER;
+        bool fits = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) == cudaSuccess &&
+                    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        for (; fits && size > 1; size >>= 1) {
+            int clusters = 0;
+            attr[0].val.clusterDim.x = (unsigned)size;
+            cfg.gridDim = dim3((unsigned)size);
+            if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1) break;
+        }
+        cudaGetLastError();
+        cached[dev] = fits ? size : 1;
+    }
+    const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
+    return limit && limit < cached[dev] ? limit : cached[dev];
+}
+
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
 // token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
 // most SMs idle is left to the form with partial results in the workspace.
@@ -586,7 +626,7 @@ template <typename Tin, int D> int decode_cap(int problems, int per_token)
 {
     const int ctas = with_groups(per_token, [](auto G) { return DecodeCfg<Tin, D, decltype(G)::value>::template ctas_per_sm<DEC_CLUSTER>(); });
     const int most = ctas * device_sm_count() / problems;
-    int cap = DEC_MAX_CLUSTER;
+    int cap = with_groups(per_token, [](auto G) { return decode_largest_cluster<Tin, D, decltype(G)::value>(); });
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
 }
@@ -796,6 +836,13 @@ int attend_decode(const void *Q, const void *K, const void *V, const int32_t *id
     ELM_CUDA_TRY(cudaMemsetAsync(ws + L.flags, 0, sizeof(int) * (size_t)(problems + 1), st));
 #endif
     return dispatch_decode(Q, K, V, idx, w, n_core, n_core, nullptr, p, O, part, room, status, st);
+}
+
+int debug_set_attend_decode(int32_t what, int64_t value)
+{
+    if (what != ELM_DEBUG_DECODE_LARGEST_CLUSTER || value < 0 || value > DEC_MAX_CLUSTER || (value & (value - 1))) return ELM_ERR_SHAPE;
+    g_debug_largest_cluster.store((int)value);
+    return ELM_OK;
 }
 
 }  // namespace elm

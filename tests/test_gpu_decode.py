@@ -21,13 +21,13 @@ def test_split_grid_is_resident_at_once(dtype_code, d, vectors):
 
 
 class _Exact:
-    """A stream inside its exact start, rewound to the same token before every call (what a call appends lies behind
-    the entries a rewound stream reads)."""
+    """A stream inside its exact start, rewound to the same token before every call: what a call appends lies behind
+    the entries a rewound stream reads, as long as it does not reach a multiple of 2**log2_nout tokens."""
 
     def __init__(self, dtype, d, rep, hkv, log2_nout, tokens, spare, batch=1):
         g = torch.Generator(device="cuda").manual_seed(3)
-        K = torch.randn(batch, hkv, 4 << log2_nout, d, device="cuda", generator=g).to(dtype)
-        V = torch.randn(batch, hkv, 4 << log2_nout, d, device="cuda", generator=g).to(dtype)
+        K = torch.randn(batch, hkv, tokens + spare, d, device="cuda", generator=g).to(dtype)
+        V = torch.randn(batch, hkv, tokens + spare, d, device="cuda", generator=g).to(dtype)
         self.Q = torch.randn(spare, batch, hkv * rep, 1, d, device="cuda", generator=g).to(dtype)
         self.s = elm.Stream(K, V, hkv * rep, log2_nout, 4)
         while self.s.state.n < tokens:
@@ -71,3 +71,35 @@ def test_short_stream_calls_over_long_lists(dtype, d, rep, hkv, log2_nout):
         assert torch.equal(x.one_call(T), x.single_steps(T))
         if T <= 8:
             assert _median_us(lambda: x.one_call(T)) <= 1.3 * _median_us(lambda: x.single_steps(T)) + 5
+
+
+@pytest.mark.parametrize("largest", [0, 8, 2, 1])
+@pytest.mark.parametrize("dtype,d,rep,hkv,batch,log2_nout,start", [
+    (torch.bfloat16, 128, 4, 2, 1, 10, 3072),       # sixteen parts: more than 2048 entries
+    (torch.float32, 128, 1, 3, 1, 9, 1536),         # sixteen parts: more than 1024 entries of 512 bytes
+    (torch.float32, 128, 4, 1, 1, 14, 8150),        # a window that grows past the longest list taken in clusters
+    (torch.bfloat16, 64, 2, 2, 32, 11, 1500),       # clusters of four: 64 problems
+])
+def test_streamed_tokens_over_long_lists_match_exact_attention(dtype, d, rep, hkv, batch, log2_nout, start, largest):
+    """Lists long enough for clusters of 16 CTAs, on devices that can place them and on devices that cannot: one call of
+    60 tokens and single steps agree bit for bit and equal exact causal attention in 64 bits (the exact start)."""
+    lib = binding.load_library()
+    assert lib.elm_debug_set(2, largest) == 0
+    try:
+        x = _Exact(dtype, d, rep, hkv, log2_nout, start, 256, batch)
+        got = x.one_call(60)
+        assert torch.equal(got, x.single_steps(60))
+    finally:
+        assert lib.elm_debug_set(2, 0) == 0
+    K, V = (t.double().repeat_interleave(rep, dim=1) for t in (x.s.K, x.s.V))
+    # fp32 sums of a few thousand positive terms; bf16 outputs are rounded to 8 bits
+    bound = 1e-5 if dtype == torch.float32 else 2.0 ** -8
+    for t in (0, 42, 43, 59):
+        p = torch.softmax(torch.einsum("bhqd,bhnd->bhqn", x.Q[t].double(), K[:, :, :start + t + 1]) / d ** 0.5, dim=-1)
+        want = p @ V[:, :, :start + t + 1]
+        assert ((got[t].double() - want).abs().amax(-1) / want.abs().amax(-1)).max() <= bound
+
+
+def test_debug_limit_of_clusters_refuses_other_sizes():
+    lib = binding.load_library()
+    assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
