@@ -5,7 +5,7 @@
 // in total, G <= 8) are processed together, so a row is read once for the whole group.  Rows are read through
 // the index list straight from K and V (no gathered copy).  fp32 arithmetic on fp32 or bf16 inputs.
 //
-// A warp takes a tile of 32 list entries (16 when a row is 512 bytes): the tile's K and V rows come to shared memory
+// A warp takes a tile of 32 list entries (16 when a row is 512 bytes, 8 of a short list): the tile's K and V rows come to shared memory
 // by asynchronous copies (the next tile's keys are requested as soon as this tile's logits are formed, its values
 // behind this tile's), eight lanes share a key row, and their partial dot products are reduced AND distributed in
 // one butterfly, so that a lane ends with finished logits of its own - 14 shuffles per 16 entries of four queries
@@ -57,16 +57,21 @@ constexpr int DEC_TOKENS = 2;
 // grid (groups, problems): the same for neighbouring tokens whose query vectors fit G together
 constexpr int DEC_NEIGHBOURS = 3;
 
-template <typename Tin, int D, int G> struct DecodeCfg {
+// entries of a warp's tile: 16 when a row is 512 bytes, else 32; 8 for lists so short that the SMs would have nothing else
+template <typename Tin, int D> constexpr int DEC_TILE = D * (int)sizeof(Tin) > 256 ? 16 : 32;
+constexpr int DEC_SHORT_TILE = 8;
+
+template <typename Tin, int D, int G, int TILE_ = DEC_TILE<Tin, D>> struct DecodeCfg {
     static constexpr int RB = D * (int)sizeof(Tin);              // bytes per row
     static constexpr int EPC = 16 / (int)sizeof(Tin);            // elements per 16-byte chunk
     static constexpr int NC = RB / 16;                           // chunks per row: 8, 16 or 32
     static constexpr int CH = NC / 8;                            // chunks of a key row per lane (eight lanes share a row)
-    static constexpr int TILE = RB > 256 ? 16 : 32;              // entries per warp tile
-    static constexpr int UB = G == 8 ? 2 : 4;                    // entries whose dot products a lane forms at a time
+    static constexpr int TILE = TILE_;                           // entries per warp tile
+    static constexpr int UB = G == 8 || TILE == DEC_SHORT_TILE ? 2 : 4;      // entries whose dot products a lane forms at a time
     static constexpr int NV = UB * G;                            // partial sums per lane: 4, 8 or 16
     static constexpr int EPI = 32 / NC;                          // entries a warp takes at a time in the value pass
     static constexpr int TILE_BYTES = TILE * RB;
+    static_assert(2 * TILE_BYTES >= G * D * 4, "a warp's partial results lie over its tiles");
     // shared memory: per warp a K tile, a V tile and the tile's logits; the scaled queries; what a form needs besides
     static constexpr int OFF_SC = DEC_WARPS * 2 * TILE_BYTES;
     static constexpr int OFF_Q = OFF_SC + DEC_WARPS * 32 * G * 4;
@@ -135,7 +140,7 @@ __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entrie
     chunk = ((len + parts - 1) / parts + tile - 1) / tile * tile;
 }
 
-template <typename Tin, int D, int G, int MODE>
+template <typename Tin, int D, int G, int MODE, int TILE = DEC_TILE<Tin, D>>
 __global__ void __launch_bounds__(DEC_WARPS * 32, DEC_CTAS)
 decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *__restrict__ V,
               const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int64_t list_stride, int q_heads,
@@ -143,8 +148,8 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
               const __grid_constant__ DecodeGroups grp, int cap, Tin *__restrict__ O, float *__restrict__ part,
               int *__restrict__ status)
 {
-    using C = DecodeCfg<Tin, D, G>;
-    constexpr int TILE = C::TILE, NC = C::NC, CH = C::CH, EPC = C::EPC, UB = C::UB, NV = C::NV, EPI = C::EPI;
+    using C = DecodeCfg<Tin, D, G, TILE>;
+    constexpr int NC = C::NC, CH = C::CH, EPC = C::EPC, UB = C::UB, NV = C::NV, EPI = C::EPI;
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned char *kt = smem + warp * 2 * C::TILE_BYTES, *vt = kt + C::TILE_BYTES;
@@ -400,7 +405,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         }
     }
 
-    // ---- the warp's partial result, over its own K tile ----
+    // ---- the warp's partial result, over its own tiles ----
     float *po = reinterpret_cast<float *>(kt);                     // [g][D]
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -632,24 +637,38 @@ template <typename Tin, int D> int decode_cap(int problems, int per_token)
 }
 template <typename Tin, int D> bool decode_clustered(int n_core, int problems, int per_token)
 {
-    // (a tile's entries do not depend on the number of query vectors)
-    const int cap = decode_cap<Tin, D>(problems, per_token), entries = DEC_WARPS * DecodeCfg<Tin, D, 1>::TILE;
+    const int cap = decode_cap<Tin, D>(problems, per_token), entries = DEC_WARPS * DEC_TILE<Tin, D>;
     return n_core <= 8 * entries * cap || problems * cap >= device_sm_count();
 }
 
-// How many CTAs per problem elm_attend's list is split over: as many as are resident at once, but at least one tile
-// per warp, and no more partial results than the workspace has room for.
-template <typename Tin, int D, int G> int decode_splits(int n_core, int problems, size_t part_room)
+// How elm_attend's list is split: CTAs per problem, and whether their warps take short tiles.
+struct DecodeSplits {
+    int n;
+    bool short_tiles;
+};
+template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int problems, size_t part_room)
 {
     using C = DecodeCfg<Tin, D, G>;
     static_assert(C::template ctas_per_sm<DEC_SPLIT>() == DEC_CTAS && C::template ctas_per_sm<DEC_TOKENS>() == DEC_CTAS,
                   "shared memory for as many CTAs as there are registers for");
-    int splits = (n_core + DEC_WARPS * C::TILE - 1) / (DEC_WARPS * C::TILE);
-    const int wanted = C::template ctas_per_sm<DEC_SPLIT>() * device_sm_count() / problems;
-    if (splits > wanted) splits = wanted < 1 ? 1 : wanted;
+    const int sms = device_sm_count();
+    auto ctas = [](int entries, int tile) { return (entries + DEC_WARPS * tile - 1) / (DEC_WARPS * tile); };
+    // A tile is a serial chain (rows, dot products, softmax, values), and a call with few of them is as long as that chain:
+    // lists of up to 512 entries take tiles of 8 while that makes no more than two CTAs per SM, or two per problem.
+    // 8 problems of 4 query vectors, bf16, d = 128: 32 entries 7.4 -> 5.9 us, 512 entries 7.8 -> 6.5 us, but 1024 entries
+    // 7.7 -> 8.0 us; 64 problems: 128 entries 8.0 -> 7.1 us, 200 entries 7.9 -> 8.9 us.
+    const int few = ctas(n_core, DEC_SHORT_TILE);
+    DecodeSplits s;
+    s.short_tiles = few <= 2 || (few <= 16 && few * problems <= 2 * sms);
+    // otherwise as many CTAs as are resident at once, but at least one tile per warp
+    const int wanted = C::template ctas_per_sm<DEC_SPLIT>() * sms / problems;
+    s.n = s.short_tiles ? few : ctas(n_core, C::TILE);
+    if (!s.short_tiles && s.n > wanted) s.n = wanted < 1 ? 1 : wanted;
+    // and no more partial results than the workspace has room for
     const size_t most = part_room / ((size_t)problems * G * (D + 2) * sizeof(float));
-    if ((size_t)splits > most) splits = (int)most;
-    return splits > DEC_MAX_SPLITS ? DEC_MAX_SPLITS : splits;
+    if ((size_t)s.n > most) s.n = (int)most;
+    if (s.n > DEC_MAX_SPLITS) s.n = DEC_MAX_SPLITS;
+    return s;
 }
 
 // How a launch of streaming tokens is laid out: query vectors per group, tokens per group, CTAs per group's cluster (0:
@@ -659,7 +678,7 @@ struct DecodeForm {
 };
 template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, int problems, int per_token)
 {
-    constexpr int TILE = DecodeCfg<Tin, D, 1>::TILE;               // (does not depend on the number of query vectors)
+    constexpr int TILE = DEC_TILE<Tin, D>;
     int longest = 0, parts, chunk, size = 1;
     for (int i = 0; i < win.n; ++i) {
         const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
@@ -737,10 +756,11 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     whole.n = 1;
     whole.tok0[1] = 1;
     whole.seen0[0] = n_core;
-    const int splits = decode_splits<Tin, D, G>(n_core, problems, part_room);
+    const DecodeSplits sp = decode_splits<Tin, D, G>(n_core, problems, part_room);
+    const int splits = sp.n;
     if (splits < 1) return ELM_ERR_WORKSPACE;
-    auto kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
-    cfg.dynamicSmemBytes = C::template total<DEC_SPLIT>();
+    auto kern = sp.short_tiles ? decode_kernel<Tin, D, G, DEC_SPLIT, DEC_SHORT_TILE> : decode_kernel<Tin, D, G, DEC_SPLIT>;
+    cfg.dynamicSmemBytes = sp.short_tiles ? DecodeCfg<Tin, D, G, DEC_SHORT_TILE>::template total<DEC_SPLIT>() : C::template total<DEC_SPLIT>();
     ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
     cfg.gridDim = dim3((unsigned)splits, (unsigned)problems);
     ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, whole, grp, 0, O,
@@ -798,14 +818,15 @@ bool attend_decode_windows_apply(const elm_params *p, int n_core)
 namespace {
 template <typename Tin, int D, int G> int decode_grid(const elm_params *p, int n_core, int32_t *ctas, int32_t *resident)
 {
-    using C = DecodeCfg<Tin, D, G>;
-    const int problems = p->batch * p->kv_heads, smem = C::template total<DEC_SPLIT>();
     const AttendLayout L = attend_layout(p, n_core);
-    auto kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
+    const int problems = p->batch * p->kv_heads;
+    const DecodeSplits sp = decode_splits<Tin, D, G>(n_core, problems, L.bias - L.Kc);
+    auto kern = sp.short_tiles ? decode_kernel<Tin, D, G, DEC_SPLIT, DEC_SHORT_TILE> : decode_kernel<Tin, D, G, DEC_SPLIT>;
+    const int smem = sp.short_tiles ? DecodeCfg<Tin, D, G, DEC_SHORT_TILE>::template total<DEC_SPLIT>() : DecodeCfg<Tin, D, G>::template total<DEC_SPLIT>();
     int per_sm = 0;
     ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     ELM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DEC_WARPS * 32, (size_t)smem));
-    *ctas = decode_splits<Tin, D, G>(n_core, problems, L.bias - L.Kc) * problems;
+    *ctas = sp.n * problems;
     *resident = per_sm * device_sm_count();
     return ELM_OK;
 }

@@ -103,3 +103,39 @@ def test_streamed_tokens_over_long_lists_match_exact_attention(dtype, d, rep, hk
 def test_debug_limit_of_clusters_refuses_other_sizes():
     lib = binding.load_library()
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_short_lists_are_spread_over_more_ctas(d):
+    """200 entries of 8 KV heads: a CTA for every 32 entries (128 per CTA left the SMs idle and its warps with a chain four
+    times as long)."""
+    for dtype_code in (binding.ELM_F32, binding.ELM_BF16):
+        ctas, _ = binding.debug_decode_grid(1, 32, 8, 200, d, 200, dtype_code=dtype_code)
+        assert ctas == 8 * 7
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("rep,n_q", [(1, 1), (2, 1), (4, 1), (1, 3), (8, 1)])
+def test_decode_of_short_lists(dtype, d, rep, n_q):
+    """Lists around the edges of the short tiles (8 per warp, 32 per CTA), of the CTAs (512 entries) and of the next form,
+    unequal weights, one of them zero, an infinite row that no list names."""
+    g = torch.Generator(device="cuda").manual_seed(7)
+    B, H, n = 2, 3, 700
+    K, V = (torch.randn(B, H, n, d, device="cuda", generator=g).to(dtype) for _ in range(2))
+    K[:, :, n - 1], V[:, :, n - 1] = float("inf"), float("inf")
+    Q = torch.randn(B, H * rep, n_q, d, device="cuda", generator=g).to(dtype)
+    # fp32 sums of positive terms; bf16 outputs are rounded to 8 bits
+    bound = 1e-5 if dtype == torch.float32 else 2.0 ** -8
+    for n_core in (1, 2, 7, 8, 9, 16, 31, 32, 33, 64, 65, 100, 128, 129, 511, 512, 513, 650):
+        idx = torch.randint(0, n - 1, (B, H, n_core), device="cuda", generator=g, dtype=torch.int32)
+        w = torch.rand(B, H, n_core, device="cuda", generator=g) + 0.05
+        if n_core > 1:
+            w[:, :, n_core // 2] = 0.0
+        got = elm.attend(Q, K, V, idx, w)
+        gather = idx.long().unsqueeze(-1).expand(-1, -1, -1, d)
+        Kc, Vc = (t.double().gather(2, gather).repeat_interleave(rep, dim=1) for t in (K, V))
+        s = torch.einsum("bhqd,bhnd->bhqn", Q.double(), Kc) / d ** 0.5 + w.double().log().repeat_interleave(rep, dim=1).unsqueeze(2)
+        want = torch.softmax(s, dim=-1) @ Vc
+        err = ((got - want).abs().amax(-1) / want.abs().amax(-1)).max()
+        assert err <= bound, (n_core, float(err))
