@@ -105,6 +105,14 @@ def test_debug_limit_of_clusters_refuses_other_sizes():
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
 
 
+@pytest.mark.parametrize("dtype_code", [binding.ELM_F32, binding.ELM_BF16])
+@pytest.mark.parametrize("vectors", [1, 4, 8])
+def test_more_problems_than_resident_ctas_fill_their_waves(dtype_code, vectors):
+    """512 problems of a long list: no wave that is nearly empty."""
+    ctas, resident = binding.debug_decode_grid(64, 8 * vectors, 8, 4096, 128, 4096, dtype_code=dtype_code)
+    assert ctas / (-(-ctas // resident) * resident) >= 0.75
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_short_lists_are_spread_over_more_ctas(d):
     """200 entries of 8 KV heads: a CTA for every 32 entries (128 per CTA left the SMs idle and its warps with a chain four
