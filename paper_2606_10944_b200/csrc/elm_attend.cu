@@ -229,8 +229,10 @@ __global__ void __launch_bounds__(128) attend_simt_kernel(const Tin *__restrict_
 }
 
 // ---------------------------------------------------------------------------------------------
-// Stage attend, fp32 inputs in fp32 mode: one CTA = 64 queries of one head, the coreset in blocks of 64 points.
-// Bound by FFMA issue.  A thread owns 8 rows x 4 columns of the logits and 8 rows x D / 16 columns of the output, both
+// Stage attend, fp32 inputs in fp32 mode: one CTA = 64 queries of one head, the coreset in blocks of BN = 64 points, or of
+// 32 when it has no more (12 heads x 200 queries x 32 points, with the gather: d = 128 25.6 us in a block of 64, 17.8 in
+// one of 32; d = 64 16.4 and 13.3).
+// Bound by FFMA issue.  A thread owns 8 rows x BN / 16 columns of the logits and 8 rows x D / 16 columns of the output, both
 // as packed pairs of rows, so that a step of either product is three or four 16-byte shared-memory reads and 16 or 32
 // packed fmas; its rows' maxima and denominators are finished by shuffles among the 16 threads that share them.  The
 // generic kernel (4 x 4 and scalar reads, softmax by half of the threads with the rest waiting) took 102 us for
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(128) attend_simt_kernel(const Tin *__restrict_
 // 16-byte chunks of a point's row exchanged by its column group (the threads that write a chunk at one time differ in
 // that group: no bank conflicts).
 // ---------------------------------------------------------------------------------------------
-template <int D>
+template <int D, int BN>
 __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict__ Q, const float *__restrict__ Kc,
                                                          const float *__restrict__ Vc, const float *__restrict__ bias,
                                                          float *__restrict__ O, int q_heads, int kv_heads, int64_t n_q, int n_core,
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
                                                          int n_pad, float *__restrict__ lse)
 {
     using namespace sm100;
-    constexpr int BM = 64, BN = 64, OC = D / 16;
+    constexpr int BM = 64, CN = BN / 16, OC = D / 16;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *Qt = reinterpret_cast<float *>(smem_raw);                // [D][BM]
     float *Kt = Qt + D * BM;                                        // [D][BN]
@@ -290,41 +292,47 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
                 c0 + rv < n_core ? __ldg(reinterpret_cast<const float4 *>(Vp + (int64_t)(c0 + rv) * D + kv)) : zero;
         }
         // the columns' weights and, where rows differ in what they see, lifetimes
-        float bc[4];
-        int32_t bt[4], dt[4];
+        float bc[CN];
+        int32_t bt[CN], dt[CN];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int col = c0 + 4 * tx + c;
+        for (int c = 0; c < CN; ++c) {
+            const int col = c0 + CN * tx + c;
             const bool in = col < n_core;
             bc[c] = in ? __ldg(bp + col) : 0.f;
             bt[c] = birth && in ? __ldg(birth + prob * n_pad + col) : 0;
             dt[c] = birth && in ? __ldg(death + prob * n_pad + col) : 0x7fffffff;
         }
         __syncthreads();
-        uint64_t s2[4][4];
+        uint64_t s2[4][CN];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) s2[r][c] = 0;
+            for (int c = 0; c < CN; ++c) s2[r][c] = 0;
 #pragma unroll 8
         for (int k = 0; k < D; ++k) {
             const ulonglong2 qa = *reinterpret_cast<const ulonglong2 *>(Qt + k * BM + 8 * ty);
             const ulonglong2 qb = *reinterpret_cast<const ulonglong2 *>(Qt + k * BM + 8 * ty + 4);
-            const float4 kv = *reinterpret_cast<const float4 *>(Kt + k * BN + 4 * tx);
             const uint64_t q2[4] = {qa.x, qa.y, qb.x, qb.y};
-            const uint64_t k2[4] = {pack2(kv.x, kv.x), pack2(kv.y, kv.y), pack2(kv.z, kv.z), pack2(kv.w, kv.w)};
+            uint64_t k2[CN];
+            if constexpr (CN == 4) {
+                const float4 kv = *reinterpret_cast<const float4 *>(Kt + k * BN + 4 * tx);
+                k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y); k2[2] = pack2(kv.z, kv.z); k2[3] = pack2(kv.w, kv.w);
+            } else {
+                const float2 kv = *reinterpret_cast<const float2 *>(Kt + k * BN + 2 * tx);
+                k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y);
+            }
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) s2[r][c] = fma2(q2[r], k2[c], s2[r][c]);
+                for (int c = 0; c < CN; ++c) s2[r][c] = fma2(q2[r], k2[c], s2[r][c]);
         }
         // a row sees the entries alive at its own position, or (tail rule) the list up to its own entry of the causal tail
         const bool all_seen = !birth && c0 + BN <= n_core && (int64_t)(c0 + BN) <= (int64_t)tail_start + q0 + 1;
-        float s[8][4];
+        float s[8][CN];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < CN; ++c) {
                 float x, y;
                 unpack2(s2[r][c], x, y);
                 s[2 * r][c] = x * scale + bc[c];
@@ -334,8 +342,8 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
 #pragma unroll
             for (int r = 0; r < 8; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int col = c0 + 4 * tx + c;
+                for (int c = 0; c < CN; ++c) {
+                    const int col = c0 + CN * tx + c;
                     const int64_t trow = q_row0 + q0 + 8 * ty + r;
                     const bool seen = col < n_core && (birth ? (bt[c] <= trow && trow < dt[c])
                                                              : (int64_t)col <= (int64_t)tail_start + q0 + 8 * ty + r);
@@ -345,7 +353,9 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
         float alpha[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            float mx = fmaxf(fmaxf(s[r][0], s[r][1]), fmaxf(s[r][2], s[r][3]));
+            float mx = s[r][0];
+#pragma unroll
+            for (int c = 1; c < CN; ++c) mx = fmaxf(mx, s[r][c]);
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
             mx = fmaxf(m[r], mx);
@@ -354,17 +364,17 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
             m[r] = mx;
             float sum = 0.f;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < CN; ++c) {
                 s[r][c] = s[r][c] == -INFINITY ? 0.f : exp2f(s[r][c] - ref);
                 sum += s[r][c];
             }
             l[r] = fmaf(l[r], alpha[r], sum);                      // (the 16 threads' shares are added at the end)
         }
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < CN; ++c)
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh)
-                *reinterpret_cast<float4 *>(Pt + (4 * tx + c) * BM + ((2 * ty + hh) ^ tx) * 4) =
+                *reinterpret_cast<float4 *>(Pt + (CN * tx + c) * BM + ((2 * ty + hh) ^ tx) * 4) =
                     make_float4(s[4 * hh][c], s[4 * hh + 1][c], s[4 * hh + 2][c], s[4 * hh + 3][c]);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -376,7 +386,7 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
         __syncwarp();
 #pragma unroll 4
         for (int c = 0; c < BN; ++c) {
-            const int g = c >> 2;
+            const int g = c / CN;
             const ulonglong2 pa = *reinterpret_cast<const ulonglong2 *>(Pt + c * BM + ((2 * ty) ^ g) * 4);
             const ulonglong2 pb = *reinterpret_cast<const ulonglong2 *>(Pt + c * BM + ((2 * ty + 1) ^ g) * 4);
             const uint64_t p2[4] = {pa.x, pa.y, pb.x, pb.y};
@@ -441,10 +451,12 @@ static int launch_attend_simt(const Tin *Q, const Tin *Kc, const Tin *Vc, const 
                               const elm_params *p, int n_core, cudaStream_t st, const AttendWindow &win = AttendWindow())
 {
     if constexpr (std::is_same<Tin, float>::value && std::is_same<T, float>::value) {
-        constexpr int BM = 64, BN = 64;
+        constexpr int BM = 64;
+        const int BN = n_core <= 32 ? 32 : 64;
         const size_t smem = sizeof(float) * (size_t)(D * BM + D * BN + BN * D + BN * BM);
-        ELM_CUDA_TRY(cudaFuncSetAttribute(attend_f32_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attend_f32_kernel<D><<<dim3((unsigned)((p->n_q + BM - 1) / BM), (unsigned)(p->batch * p->q_heads)), 128, smem, st>>>(
+        auto kern = BN == 32 ? attend_f32_kernel<D, 32> : attend_f32_kernel<D, 64>;
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<dim3((unsigned)((p->n_q + BM - 1) / BM), (unsigned)(p->batch * p->q_heads)), 128, smem, st>>>(
             Q, Kc, Vc, bias, O, p->q_heads, p->kv_heads, p->n_q, n_core, win.q_row0, win.n_q_total ? win.n_q_total : (int64_t)p->n_q,
             win.tail_start, win.birth, win.death, (n_core + 127) / 128 * 128, win.lse);
         count_launches(1);

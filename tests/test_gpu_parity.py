@@ -331,3 +331,42 @@ def test_compress_bf16_small_calls_select_what_the_fp64_mode_selects(d, kv_heads
     b, _ = elm.compress(K.cuda(), V.cuda(), log2_nout, m, seed=3, precision="fp64")
     torch.cuda.synchronize()
     assert (a != b).float().mean().item() <= 0.02
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_q", [9, 64, 130])
+def test_attention_of_short_fp32_coresets(d, n_q):
+    """fp32 coresets of up to 32 points (blocks of 32) and just beyond (blocks of 64), unequal weights, grouped queries."""
+    g = torch.Generator(device="cuda").manual_seed(11)
+    B, H, n = 2, 2, 80
+    K, V = (torch.randn(B, H, n, d, device="cuda", generator=g) for _ in range(2))
+    Q = torch.randn(B, 2 * H, n_q, d, device="cuda", generator=g)
+    for n_core in (1, 2, 15, 31, 32, 33, 64, 65):
+        idx = torch.randint(0, n, (B, H, n_core), device="cuda", generator=g, dtype=torch.int32)
+        w = torch.rand(B, H, n_core, device="cuda", generator=g) + 0.05
+        got = elm.attend(Q, K, V, idx, w)
+        gather = idx.long().unsqueeze(-1).expand(-1, -1, -1, d)
+        Kc, Vc = (t.double().gather(2, gather).repeat_interleave(2, dim=1) for t in (K, V))
+        s = torch.einsum("bhqd,bhnd->bhqn", Q.double(), Kc) / d ** 0.5 + w.double().log().repeat_interleave(2, dim=1).unsqueeze(2)
+        want = torch.softmax(s, dim=-1) @ Vc
+        # fp32 sums of a few dozen positive terms, logits of at most 10
+        assert ((got - want).abs().amax(-1) / want.abs().amax(-1)).max() <= 1e-5
+
+
+def test_short_fp32_coresets_are_not_padded_to_64_points():
+    """Attention over 32 points takes well under what it takes over 64."""
+    Q, K, V = (torch.randn(1, 48, n, 128, device="cuda") for n in (4096, 64, 64))
+    times = {}
+    for n_core in (32, 64):
+        idx = torch.arange(n_core, device="cuda", dtype=torch.int32).repeat(1, 48, 1)
+        w = torch.full((1, 48, n_core), 1.0 / n_core, device="cuda")
+        runs = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            elm.attend(Q, K, V, idx, w)
+            b.record()
+            b.synchronize()
+            runs.append(a.elapsed_time(b))
+        times[n_core] = sorted(runs)[4]
+    assert times[32] <= 0.8 * times[64]
