@@ -20,8 +20,9 @@
 // partial results (maximum, denominator, accumulator) in the workspace for decode_merge_kernel.  Tokens of a streaming
 // run (DecodeWindows: a token sees a prefix of its window's list): each over the CTAs of a thread-block cluster, which
 // hand each other their partial results through distributed shared memory, or, once there are tokens enough to fill the
-// SMs, by one CTA that walks the parts of the list one after the other (decode_form) - the same parts, tiles and merges
-// in the same order as the cluster's, so a token's output is the same bit for bit whichever launch computes it.
+// SMs, by one CTA that walks the parts of the list one after the other - the same parts, tiles and merges in the same
+// order as the cluster's, so a token's output is the same bit for bit whichever launch computes it.  How many of a
+// token's query vectors go together is free too (decode_form).
 #include <math.h>
 
 #include <atomic>
@@ -44,15 +45,15 @@ using sm100::unpack2;
 
 constexpr int DEC_WARPS = 4;
 constexpr int DEC_GMAX = 8;
-constexpr int DEC_GSERIAL = 4;         // fewest query vectors of a CTA that walks the parts of a list one after the other
+constexpr int DEC_GSTREAM = 4;         // most query vectors a CTA of a streaming token takes
 constexpr int DEC_MAX_CLUSTER = 16;
 constexpr int DEC_CTAS = 3;                                      // CTAs per SM the kernel is compiled for
 
 // grid (splits, problems); partial results part[problem][split][g][D + 2] = accumulator (D), maximum, denominator
 constexpr int DEC_SPLIT = 0;
-// grid (tokens x cluster size, problems): rank r of a token's cluster takes the r-th part of its list
+// grid (tokens x vec_groups x cluster size, problems): rank r of a cluster takes the r-th part of its token's list
 constexpr int DEC_CLUSTER = 1;
-// grid (tokens, problems): a token's parts one after the other
+// grid (tokens x vec_groups, problems): a token's parts one after the other
 constexpr int DEC_TOKENS = 2;
 // grid (groups, problems): the same for neighbouring tokens whose query vectors fit G together
 constexpr int DEC_NEIGHBOURS = 3;
@@ -84,13 +85,9 @@ template <typename Tin, int D, int G, int TILE_ = DEC_TILE<Tin, D>> struct Decod
     {
         return MODE == DEC_SPLIT ? OFF_RML : MODE == DEC_CLUSTER ? OFF_RECV + (G * D + DEC_MAX_CLUSTER) * 4 : OFF_RML + 2 * G * 2 * 4;
     }
-    // CTAs an SM holds: of 228 KB shared memory the system takes 1 KB per CTA; registers are kept to what three leave
-    // (launch bounds).  DEC_SPLIT and DEC_TOKENS always get three; DEC_CLUSTER two at G = 8 and D = 128 (79 KB), where
-    // two against three cost 1.2 times the time (8 problems x 5193 entries, split form: 24.0 against 20.0 us).
-    template <int MODE> static constexpr int ctas_per_sm()
-    {
-        return 228 * 1024 / (total<MODE>() + 1024) < DEC_CTAS ? 228 * 1024 / (total<MODE>() + 1024) : DEC_CTAS;
-    }
+    // DEC_CTAS to an SM: of its 228 KB the system takes 1 KB per CTA (at G = 8 and D = 128 two CTAs against three cost 1.2
+    // times the time, 8 problems x 5193 entries: 24.0 against 20.0 us)
+    template <int MODE> static constexpr bool fits = DEC_CTAS * (total<MODE>() + 1024) <= 228 * 1024;
 };
 
 __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool live)
@@ -123,19 +120,23 @@ __device__ __forceinline__ void merge_part(float &M, float &den, float &acc, flo
     M = Mn;
 }
 
-// The groups of tokens of a streaming launch
+// The groups of tokens of a streaming launch, and of a token's query vectors
 struct DecodeGroups {
     int32_t cluster;                               // CTAs per group
+    int32_t vec_groups;                            // groups a token's query vectors are dealt to, G to each
     int32_t per_group;                             // tokens per group: a power of two, 1 but in DEC_NEIGHBOURS
-    int32_t g0[DECODE_MAX_WINDOWS + 1];            // groups of the windows before
+    int32_t g0[DECODE_MAX_WINDOWS + 1];            // groups of tokens in the windows before
 };
 
-// How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp, at most `cap` parts.
-// Depends on n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
+// How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp (one in lists of up to 512
+// entries: 200 entries of one query vector 6.9 -> 5.7 us; longer ones gain less than the extra merges cost a CTA that
+// walks all parts, 1536 entries x 64 tokens 98 -> 114 us), at most `cap` parts.  Depends on n_core only through the next
+// multiple of 128, so that neighbouring tokens share their parts.
 __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entries, int tile, int cap, int &parts, int &chunk)
 {
     const int len = (n_core + 127) / 128 * 128;
-    const int t = (len + 2 * cta_entries - 1) / (2 * cta_entries);
+    const int least = len <= 512 ? cta_entries : 2 * cta_entries;
+    const int t = (len + least - 1) / least;
     parts = t < 1 ? 1 : (t < cap ? t : cap);
     chunk = ((len + parts - 1) / parts + tile - 1) / tile * tile;
 }
@@ -162,8 +163,16 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
     cudaGridDependencySynchronize();
     if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     constexpr bool SERIAL = MODE == DEC_TOKENS || MODE == DEC_NEIGHBOURS;
-    const int prob = blockIdx.y, group = MODE == DEC_SPLIT ? 0 : (int)blockIdx.x / grp.cluster;
+    static_assert(C::template fits<MODE>, "shared memory for as many CTAs as there are registers for");
+    const int prob = blockIdx.y;
+    int group = MODE == DEC_SPLIT ? 0 : (int)blockIdx.x / grp.cluster;
     const int rank = (int)blockIdx.x - group * grp.cluster;
+    // the group's query vectors of its token: vec0 .. vec0 + G - 1
+    int vec0 = 0;
+    if constexpr (MODE == DEC_CLUSTER || MODE == DEC_TOKENS) {
+        vec0 = group % grp.vec_groups * G;
+        group /= grp.vec_groups;
+    }
 #ifndef ELM_BOUNDS_CHECK
     // this path has no bounded waits and (in this build) no row checks: its status word reads 0 - written here
     // rather than by a memset of its own
@@ -182,7 +191,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
         z0 = win.tok0[wi] + (seen0 - win.seen0[wi]);
     }
     const int n_core = seen0 + tokens - 1;                         // what the last token sees
-    const int groups = tokens * per_token;                         // live query vectors
+    const int groups = tokens * per_token - vec0;                  // live query vectors (of G, if they are more)
     int parts, chunk;
     if constexpr (MODE == DEC_SPLIT) {
         // whole tiles per part, so that only the end of the list leaves a tile partly filled
@@ -197,8 +206,8 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
     const Tin *Kp = K + (int64_t)prob * n * D, *Vp = V + (int64_t)prob * n * D;
     // offset of query vector g's row in Q and O: token g / per_token, in it (head within the group) * n_q + row
     auto q_row = [&](int g) -> int64_t {
-        const int64_t z = z0 + g / per_token;
-        const int in = g % per_token;
+        const int64_t z = MODE == DEC_NEIGHBOURS ? z0 + g / per_token : z0;
+        const int in = MODE == DEC_NEIGHBOURS ? g % per_token : vec0 + g;
         return (((z * (gridDim.y / kv_heads) + b) * q_heads + kvh * rep + in / n_q) * n_q + in % n_q) * D;
     };
     int c0, c1 = 0;                                                // the part being worked on
@@ -502,7 +511,7 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
             const int i = tid + k * DEC_WARPS * 32;
-            if (i < groups * D) store_from(O, q_row(i / D) + i % D, run[k] / rml[((parts & 1) * G + i / D) * 2 + 1]);
+            if (i < G * D && i < groups * D) store_from(O, q_row(i / D) + i % D, run[k] / rml[((parts & 1) * G + i / D) * 2 + 1]);
         }
     }
 }
@@ -589,7 +598,7 @@ template <typename F> auto with_groups(int groups, F f)
 // The largest cluster (a power of two, at most DEC_MAX_CLUSTER) of which the current device can hold one, asked once per
 // device: more than 8 CTAs need the opt-in and a GPC with that many SMs to give, which a partition of a GPU may not have.
 std::atomic<int> g_debug_largest_cluster{0};
-template <typename Tin, int D, int G> int decode_largest_cluster()
+template <typename Tin, int D> int decode_largest_cluster()
 {
     static std::mutex mu;
     static int cached[64] = {0};
@@ -597,8 +606,8 @@ template <typename Tin, int D, int G> int decode_largest_cluster()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
     std::lock_guard<std::mutex> lock(mu);
     if (cached[dev] == 0) {
-        using C = DecodeCfg<Tin, D, G>;
-        auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
+        using C = DecodeCfg<Tin, D, DEC_GSTREAM>;
+        auto kern = decode_kernel<Tin, D, DEC_GSTREAM, DEC_CLUSTER>;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.y = 1;
@@ -626,12 +635,14 @@ template <typename Tin, int D, int G> int decode_largest_cluster()
 
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
 // token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
-// most SMs idle is left to the form with partial results in the workspace.
+// most SMs idle is left to the form with partial results in the workspace, token by token: over as many CTAs as fit the
+// device a single token gains from about 6000 entries on (8 KV heads of 4 query heads, bf16: 6144 entries 16.4 us in
+// clusters, 14.2 split; 12288 entries 25.2 and 18.6), but the tokens of a call can then no longer share a launch (64 tokens over
+// 12288 entries: 606 us together, 1190 one by one).
 template <typename Tin, int D> int decode_cap(int problems, int per_token)
 {
-    const int ctas = with_groups(per_token, [](auto G) { return DecodeCfg<Tin, D, decltype(G)::value>::template ctas_per_sm<DEC_CLUSTER>(); });
-    const int most = ctas * device_sm_count() / problems;
-    int cap = with_groups(per_token, [](auto G) { return decode_largest_cluster<Tin, D, decltype(G)::value>(); });
+    const int most = DEC_CTAS * device_sm_count() / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
+    int cap = decode_largest_cluster<Tin, D>();
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
 }
@@ -649,8 +660,6 @@ struct DecodeSplits {
 template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int problems, size_t part_room)
 {
     using C = DecodeCfg<Tin, D, G>;
-    static_assert(C::template ctas_per_sm<DEC_SPLIT>() == DEC_CTAS && C::template ctas_per_sm<DEC_TOKENS>() == DEC_CTAS,
-                  "shared memory for as many CTAs as there are registers for");
     const int sms = device_sm_count();
     auto ctas = [](int entries, int tile) { return (entries + DEC_WARPS * tile - 1) / (DEC_WARPS * tile); };
     // A tile is a serial chain (rows, dot products, softmax, values), and a call with few of them is as long as that chain:
@@ -664,7 +673,7 @@ template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int
     // as take the least time in waves of them, a CTA's start and merge counted as 3/4 round of tiles per query vector.
     // 512 problems on 444 CTAs, fp32, d = 128, one query vector: 2048 entries 173 -> 122 us (one CTA per problem: a second
     // wave that is nearly empty), 200 entries 16.9 -> 15.9 us; bf16, four query vectors, 2048 entries: 101 -> 91 us.
-    const int resident = C::template ctas_per_sm<DEC_SPLIT>() * sms, wanted = resident / problems;
+    const int resident = DEC_CTAS * sms, wanted = resident / problems;
     s.n = s.short_tiles ? few : ctas(n_core, C::TILE);
     if (!s.short_tiles && wanted < 1) {
         const int most_parts = s.n < 4 ? s.n : 4;
@@ -684,14 +693,15 @@ template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int
     return s;
 }
 
-// How a launch of streaming tokens is laid out: query vectors per group, tokens per group, CTAs per group's cluster (0:
-// one CTA per group, part after part).
+// How a launch of streaming tokens is laid out: query vectors per group, groups they make of a token's, tokens per group,
+// CTAs per group's cluster (0: one CTA per group, part after part).
 struct DecodeForm {
-    int32_t vectors, per_group, cluster;
+    int32_t G, vec_groups, per_group, cluster;
 };
 template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, int problems, int per_token)
 {
     constexpr int TILE = DEC_TILE<Tin, D>;
+    const int sms = device_sm_count();
     int longest = 0, parts, chunk, size = 1;
     for (int i = 0; i < win.n; ++i) {
         const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
@@ -700,19 +710,24 @@ template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, 
     decode_parts(longest, DEC_WARPS * TILE, TILE, decode_cap<Tin, D>(problems, per_token), parts, chunk);
     while (size < parts) size <<= 1;
     const int64_t tokens = win.tok0[win.n];
-    if (tokens == 1) return {per_token, 1, size};
-    // tokens that share a CTA when it walks the parts itself
-    int per_group = 1;
-    while (per_group * 2 * per_token <= DEC_GSERIAL) per_group *= 2;
-    const int vectors = per_token > DEC_GSERIAL ? DEC_GMAX : DEC_GSERIAL;
+    const int whole = (per_token + DEC_GSTREAM - 1) / DEC_GSTREAM;                // groups of DEC_GSTREAM vectors
     // Clusters spread a token over the SMs and are never slower than the tokens one by one (6144 entries, 8 KV heads of 4
     // query heads, bf16: 2 tokens 23 us, 8 tokens 68 us, one token 18 us).  Walking part after part saves their barriers
     // and merges but takes as long as one CTA needs for a whole list (137 us), so it pays from about one token per SM on
     // (16 tokens of 8 heads: 119 us in clusters, 137 walked; 32 tokens: 224 against 185; 64: 431 against 345), from two
     // on when its CTAs take several tokens (1 query head per KV head: 32 tokens 147 against 171, 64 tokens 282 against
     // 172).  A list of one part needs no merge at all.
-    const bool serial = tokens * problems >= (per_group > 1 ? 2 : 1) * device_sm_count() || (parts == 1 && per_group == 1);
-    return serial ? DecodeForm{vectors, per_group, 0} : DecodeForm{per_token, 1, size};
+    if (tokens > 1) {
+        int per_group = 1;
+        while (per_group * 2 * per_token <= DEC_GSTREAM) per_group *= 2;
+        if (tokens * problems * whole >= (per_group > 1 ? 2 : 1) * sms || (parts == 1 && per_group == 1)) return {DEC_GSTREAM, whole, per_group, 0};
+    }
+    // The chain of a tile grows with its query vectors, so clusters take as few as leave all their CTAs resident.
+    // 8 KV heads of 8 query heads, bf16: 200 entries 17.6 us with all eight together, 6.2 one by one, 6144 entries 29.7 and
+    // 22.1; of 4 query heads: 200 entries 11.0 and 6.0, 6144 entries 17.7 and 16.4.
+    int G = 1;
+    while (G < DEC_GSTREAM && G < per_token && tokens * problems * ((per_token + G - 1) / G) * size > DEC_CTAS * sms) G *= 2;
+    return {G, (per_token + G - 1) / G, 1, size};
 }
 
 // win set: streaming tokens, laid out as `form` says; else the list of elm_attend, n_core entries long
@@ -735,35 +750,38 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     const int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
     DecodeGroups grp = {};
     if (win) {
-        const int cap = decode_cap<Tin, D>(problems, per_token);
-        grp.per_group = form.per_group;
-        for (int i = 0; i < win->n; ++i) {
-            const int last = win->seen0[i] + (win->tok0[i + 1] - win->tok0[i]) - 1;
-            grp.g0[i + 1] = grp.g0[i] + (last - 1) / grp.per_group - (win->seen0[i] - 1) / grp.per_group + 1;
-        }
-        auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
-        cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
-        if constexpr (G >= DEC_GSERIAL) {
-            if (form.cluster == 0) {
-                kern = decode_kernel<Tin, D, G, DEC_TOKENS>;
-                if constexpr (G == DEC_GSERIAL)
-                    if (form.per_group > 1) kern = decode_kernel<Tin, D, G, DEC_NEIGHBOURS>;
-                cfg.dynamicSmemBytes = C::template total<DEC_TOKENS>();
+        if constexpr (G <= DEC_GSTREAM) {
+            const int cap = decode_cap<Tin, D>(problems, per_token);
+            grp.vec_groups = form.vec_groups;
+            grp.per_group = form.per_group;
+            for (int i = 0; i < win->n; ++i) {
+                const int last = win->seen0[i] + (win->tok0[i + 1] - win->tok0[i]) - 1;
+                grp.g0[i + 1] = grp.g0[i] + (last - 1) / grp.per_group - (win->seen0[i] - 1) / grp.per_group + 1;
             }
+            auto kern = decode_kernel<Tin, D, G, DEC_CLUSTER>;
+            cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
+            if constexpr (G == DEC_GSTREAM) {
+                if (form.cluster == 0) {
+                    kern = form.per_group > 1 ? decode_kernel<Tin, D, G, DEC_NEIGHBOURS> : decode_kernel<Tin, D, G, DEC_TOKENS>;
+                    cfg.dynamicSmemBytes = C::template total<DEC_TOKENS>();
+                }
+            }
+            grp.cluster = form.cluster ? form.cluster : 1;
+            ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+            if (grp.cluster > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            attr[1].id = cudaLaunchAttributeClusterDimension;
+            attr[1].val.clusterDim.x = (unsigned)grp.cluster;
+            attr[1].val.clusterDim.y = 1;
+            attr[1].val.clusterDim.z = 1;
+            cfg.numAttrs = 2;
+            cfg.gridDim = dim3((unsigned)(grp.g0[win->n] * grp.vec_groups * grp.cluster), (unsigned)problems);
+            ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, *win, grp,
+                                            cap, O, (float *)nullptr, status));
+            count_launches(1);
+            return cuda_status(cudaGetLastError());
+        } else {
+            return ELM_ERR_SHAPE;                                  // (decode_form gives no such G)
         }
-        grp.cluster = form.cluster ? form.cluster : 1;
-        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
-        if (grp.cluster > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)grp.cluster;
-        attr[1].val.clusterDim.y = 1;
-        attr[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
-        cfg.gridDim = dim3((unsigned)(grp.g0[win->n] * grp.cluster), (unsigned)problems);
-        ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, *win, grp,
-                                        cap, O, (float *)nullptr, status));
-        count_launches(1);
-        return cuda_status(cudaGetLastError());
     }
     DecodeWindows whole = {};
     whole.n = 1;
@@ -792,9 +810,9 @@ int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *
                     const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
 {
     const int per_token = (p->q_heads / p->kv_heads) * p->n_q;
-    DecodeForm form = {per_token, 1, 0};
+    DecodeForm form = {per_token, 1, 1, 0};
     if (win) form = decode_form<Tin, D>(*win, p->batch * p->kv_heads, per_token);
-    return with_groups(form.vectors, [&](auto G) {
+    return with_groups(form.G, [&](auto G) {
         return launch_decode<Tin, D, decltype(G)::value>((const Tin *)Q, (const Tin *)K, (const Tin *)V, idx, w, list_stride, n_core, win,
                                                          form, p, (Tin *)O, part, part_room, status, per_token, st);
     });

@@ -46,6 +46,17 @@ class _Exact:
         return torch.stack([self.s.step(self.Q[t]) for t in range(T)])
 
 
+def _graph_us(f, calls=10):
+    """Device time of a call: many of them replayed as one graph."""
+    f()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(calls):
+            f()
+    return _median_us(g.replay) / calls
+
+
 def _median_us(f, reps=15):
     times = []
     for i in range(reps + 3):
@@ -147,3 +158,22 @@ def test_decode_of_short_lists(dtype, d, rep, n_q):
         want = torch.softmax(s, dim=-1) @ Vc
         err = ((got - want).abs().amax(-1) / want.abs().amax(-1)).max()
         assert err <= bound, (n_core, float(err))
+
+
+@pytest.mark.parametrize("rep", [1, 4, 8])
+@pytest.mark.parametrize("entries", [100, 200, 400])
+def test_streamed_token_over_a_short_list_takes_no_longer_than_attend(rep, entries):
+    """One streaming token over a few hundred entries: two launches (its list, its attention) that take no longer than
+    elm_attend's two over the same list and a little for the list (a token of eight query vectors took twice as long)."""
+    x = _Exact(torch.bfloat16, 128, rep, 8, 9, entries, 64)
+    q, o = x.Q[0], torch.empty_like(x.Q[0])
+
+    def step():
+        x.rewind()
+        x.s.step(q, out=o)
+
+    idx = torch.arange(entries, device="cuda", dtype=torch.int32).repeat(1, 8, 1)
+    w = torch.ones(1, 8, entries, device="cuda")
+    ws = torch.empty(64 << 20, device="cuda", dtype=torch.uint8)
+    out = torch.empty_like(q)
+    assert _graph_us(step) <= 1.1 * _graph_us(lambda: elm.attend(q, x.s.K, x.s.V, idx, w, workspace=ws, out=out)) + 2.5
