@@ -523,10 +523,10 @@ extern "C" int elm_stream_steps(elm_stream *s, int32_t n_tokens, const void *Q_T
 {
     if (!s || !params) return ELM_ERR_NULL;
     if (n_tokens < 0) return ELM_ERR_SHAPE;
-    if (n_tokens == 0) return ELM_OK;
-    if (!Q_T || !O_T) return ELM_ERR_NULL;
+    if (n_tokens > 0 && (!Q_T || !O_T)) return ELM_ERR_NULL;
     const size_t per_token = (size_t)params->batch * params->q_heads * params->d * elm::elt_bytes(params->dtype);
     if (per_token & 15) return ELM_ERR_ALIGN;
+    if (n_tokens == 0) return ELM_OK;
     return elm::stream_steps_checked(s, n_tokens, Q_T, K, V, params, O_T, workspace, workspace_bytes, stream);
 }
 

@@ -162,3 +162,13 @@ def test_express_and_stream_argument_checks():
                                           ctypes.byref(need)) == -2
     assert lib.elm_stream_workspace_bytes(ctypes.byref(_params(n_kv=1024, n_q=1, log2_nout=4, m=0)), 2,
                                           ctypes.byref(need)) == 0 and need.value > 0
+
+
+def test_stream_steps_of_no_tokens_checks_its_arguments():
+    """Nothing to enqueue: fine, but rows that no token could have are refused as for any other count."""
+    lib = binding.load_library()
+    state = binding.ElmStream()
+    for d, code in ((64, 0), (3, -4)):
+        p = _params(n_q=1, d=d, q_heads=1, kv_heads=1)
+        assert lib.elm_stream_steps(ctypes.byref(state), 0, None, None, None, ctypes.byref(p), None, None, 0, None) == code
+    assert lib.elm_stream_steps(ctypes.byref(state), -1, None, None, None, ctypes.byref(p), None, None, 0, None) == -2
