@@ -137,8 +137,10 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _stream() -> int:
-    # the current device's current stream, without a torch.cuda.Stream object made for every call
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # the current device's current stream; torch's own accessor saves the torch.cuda.Stream object made for every call,
+    # but is not public, so a build of torch may lack it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
 
 
 def make_params(batch, q_heads, kv_heads, n_kv, n_q, d, log2_nout, m, dtype_code, precision="fp32",

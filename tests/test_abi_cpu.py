@@ -172,3 +172,12 @@ def test_stream_steps_of_no_tokens_checks_its_arguments():
         p = _params(n_q=1, d=d, q_heads=1, kv_heads=1)
         assert lib.elm_stream_steps(ctypes.byref(state), 0, None, None, None, ctypes.byref(p), None, None, 0, None) == code
     assert lib.elm_stream_steps(ctypes.byref(state), -1, None, None, None, ctypes.byref(p), None, None, 0, None) == -2
+
+
+def test_current_stream_without_the_private_accessor(monkeypatch):
+    """A torch that lacks the raw accessor: the public call is taken."""
+    class Stream:
+        cuda_stream = 1234
+    monkeypatch.delattr(binding.torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: Stream)
+    assert binding._stream() == 1234
