@@ -4,7 +4,6 @@
 #include <stdio.h>
 
 #include <atomic>
-#include <mutex>
 
 #include <vector>
 
@@ -243,17 +242,15 @@ extern "C" int elm_compress_attend_host(const void *Q_host, const void *K_host, 
 namespace elm {
 int device_sm_count()
 {
-    static std::mutex mu;
-    static int cached[64] = {0};
+    static std::atomic<int> cached[64];        // (threads that meet here first find the same answer)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    std::lock_guard<std::mutex> lock(mu);
-    if (cached[dev] == 0) {
-        int n = 0;
+    int n = cached[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        cached[dev] = n;
+        cached[dev].store(n, std::memory_order_relaxed);
     }
-    return cached[dev];
+    return n;
 }
 }  // namespace elm
 

