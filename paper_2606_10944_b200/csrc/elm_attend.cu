@@ -462,16 +462,16 @@ static int launch_attend_simt(const Tin *Q, const Tin *Kc, const Tin *Vc, const 
         count_launches(1);
         return cuda_status(cudaGetLastError());
     } else {
-    constexpr int BM = 64, BN = 32;
-    const size_t smem = sizeof(T) * (size_t)(D * BM + D * BN + BN * D + BM * (BN + 1) + 3 * BM + BN) + 2 * BN * sizeof(int32_t);
-    auto kern = attend_simt_kernel<Tin, T, D>;
-    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid((unsigned)((p->n_q + BM - 1) / BM), (unsigned)(p->batch * p->q_heads));
-    kern<<<grid, 128, smem, st>>>(Q, Kc, Vc, bias, O, p->q_heads, p->kv_heads, p->n_q, n_core, win.q_row0,
-                                  win.n_q_total ? win.n_q_total : (int64_t)p->n_q, win.tail_start, win.birth, win.death,
-                                  (n_core + 127) / 128 * 128, win.lse);
-    count_launches(1);
-    return cuda_status(cudaGetLastError());
+        constexpr int BM = 64, BN = 32;
+        const size_t smem = sizeof(T) * (size_t)(D * BM + D * BN + BN * D + BM * (BN + 1) + 3 * BM + BN) + 2 * BN * sizeof(int32_t);
+        auto kern = attend_simt_kernel<Tin, T, D>;
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        dim3 grid((unsigned)((p->n_q + BM - 1) / BM), (unsigned)(p->batch * p->q_heads));
+        kern<<<grid, 128, smem, st>>>(Q, Kc, Vc, bias, O, p->q_heads, p->kv_heads, p->n_q, n_core, win.q_row0,
+                                      win.n_q_total ? win.n_q_total : (int64_t)p->n_q, win.tail_start, win.birth, win.death,
+                                      (n_core + 127) / 128 * 128, win.lse);
+        count_launches(1);
+        return cuda_status(cudaGetLastError());
     }
 }
 

@@ -84,8 +84,9 @@ int attend_decode(const void *Q, const void *K, const void *V, const int32_t *id
 // The same for many tokens of a streaming run in one launch.  Window i holds the tokens tok0[i] .. tok0[i + 1] - 1 of
 // the launch (tok0[0] = 0); its list starts at entry off[i] of every problem's row of idx / w (row stride
 // list_stride), and its j-th token sees the first seen0[i] + j entries.  Q and O are [tokens][batch][q_heads][1][d].
-// Applies when the longest list a token sees has n_core entries and attend_decode_windows_apply says so; a token's
-// output is then the one attend_decode computes for it.
+// Applies when the longest list a token sees has n_core entries and attend_decode_windows_apply says so.  A token's
+// output is the same bit for bit whatever other tokens share its launch (attend_decode parts a list differently and
+// agrees to rounding).
 constexpr int DECODE_MAX_WINDOWS = 32;
 struct DecodeWindows {
     int32_t n;

@@ -255,254 +255,254 @@ decode_kernel(const Tin *__restrict__ Q, const Tin *__restrict__ K, const Tin *_
     const int gl = lane >> 3, sub = lane & 7;
 
     for (int pt = rank; pt < (SERIAL ? parts : rank + 1); ++pt) {
-    c0 = pt * chunk < n_core ? pt * chunk : n_core;
-    c1 = pt < parts ? (c0 + chunk < n_core ? c0 + chunk : n_core) : c0;
-    int t0 = c0 + warp * TILE;
-    fetch_entries(t0);
-    row = row_next;
-    lw = log2f(lw_next);
-    // (the queries are laid out / the merge of the part before has read the tiles)
-    __syncthreads();
-    if (t0 < c1) {
-        copy_rows(kt, Kp, row, t0);
-        copy_rows(vt, Vp, row, t0);
-        fetch_entries(t0 + DEC_WARPS * TILE);
-    }
-    float m[G], l[G];
-    uint64_t o[G][EPC / 2];
+        c0 = pt * chunk < n_core ? pt * chunk : n_core;
+        c1 = pt < parts ? (c0 + chunk < n_core ? c0 + chunk : n_core) : c0;
+        int t0 = c0 + warp * TILE;
+        fetch_entries(t0);
+        row = row_next;
+        lw = log2f(lw_next);
+        // (the queries are laid out / the merge of the part before has read the tiles)
+        __syncthreads();
+        if (t0 < c1) {
+            copy_rows(kt, Kp, row, t0);
+            copy_rows(vt, Vp, row, t0);
+            fetch_entries(t0 + DEC_WARPS * TILE);
+        }
+        float m[G], l[G];
+        uint64_t o[G][EPC / 2];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        m[g] = -INFINITY;
-        l[g] = 0.f;
+        for (int g = 0; g < G; ++g) {
+            m[g] = -INFINITY;
+            l[g] = 0.f;
 #pragma unroll
-        for (int i = 0; i < EPC / 2; ++i) o[g][i] = 0;
-    }
-    for (; t0 < c1; t0 += DEC_WARPS * TILE) {
-        const bool more = t0 + DEC_WARPS * TILE < c1;
-        // ---- logits: entry gl + 4 u of the tile by the eight lanes of group gl ----
-        cp_async_wait<1>();                                        // the keys (the values are the newer group)
-        __syncwarp();
+            for (int i = 0; i < EPC / 2; ++i) o[g][i] = 0;
+        }
+        for (; t0 < c1; t0 += DEC_WARPS * TILE) {
+            const bool more = t0 + DEC_WARPS * TILE < c1;
+            // ---- logits: entry gl + 4 u of the tile by the eight lanes of group gl ----
+            cp_async_wait<1>();                                        // the keys (the values are the newer group)
+            __syncwarp();
 #pragma unroll
-        for (int ub = 0; ub < TILE / 4 / UB; ++ub) {
-            uint64_t acc[UB][G];
+            for (int ub = 0; ub < TILE / 4 / UB; ++ub) {
+                uint64_t acc[UB][G];
 #pragma unroll
-            for (int u = 0; u < UB; ++u)
+                for (int u = 0; u < UB; ++u)
 #pragma unroll
-                for (int g = 0; g < G; ++g) acc[u][g] = 0;
+                    for (int g = 0; g < G; ++g) acc[u][g] = 0;
 #pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                uint64_t kf[UB][EPC / 2];
+                for (int c = 0; c < CH; ++c) {
+                    uint64_t kf[UB][EPC / 2];
 #pragma unroll
-                for (int u = 0; u < UB; ++u) {
-                    const int e = gl + 4 * (ub * UB + u);
-                    chunk_pairs(*reinterpret_cast<const uint4 *>(kt + (e * NC + c * 8 + sub) * 16), kf[u], (const Tin *)nullptr);
-                }
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-#pragma unroll
-                    for (int h = 0; h < EPC / 4; ++h) {
-                        const float4 q4 = *reinterpret_cast<const float4 *>(qs + (((g * CH + c) * (EPC / 4) + h) * 8 + sub) * 4);
-                        const uint64_t qa = pack2(q4.x, q4.y), qb = pack2(q4.z, q4.w);
-#pragma unroll
-                        for (int u = 0; u < UB; ++u) acc[u][g] = fma2(kf[u][2 * h + 1], qb, fma2(kf[u][2 * h], qa, acc[u][g]));
+                    for (int u = 0; u < UB; ++u) {
+                        const int e = gl + 4 * (ub * UB + u);
+                        chunk_pairs(*reinterpret_cast<const uint4 *>(kt + (e * NC + c * 8 + sub) * 16), kf[u], (const Tin *)nullptr);
                     }
-                }
-            }
-            // reduce over the eight lanes and leave each with its share of the NV sums
-            float v[NV];
 #pragma unroll
-            for (int u = 0; u < UB; ++u)
+                    for (int g = 0; g < G; ++g) {
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    float lo, hi;
-                    unpack2(acc[u][g], lo, hi);
-                    v[u * G + g] = lo + hi;
-                }
-            int base = 0;
-            {
-                int cnt = NV;
+                        for (int h = 0; h < EPC / 4; ++h) {
+                            const float4 q4 = *reinterpret_cast<const float4 *>(qs + (((g * CH + c) * (EPC / 4) + h) * 8 + sub) * 4);
+                            const uint64_t qa = pack2(q4.x, q4.y), qb = pack2(q4.z, q4.w);
 #pragma unroll
-                for (int off = 4; off > 0; off >>= 1) {
-                    if (cnt >= 2) {
-                        const bool up = (sub & off) != 0;
-                        cnt >>= 1;
-#pragma unroll
-                        for (int i = 0; i < NV / 2; ++i) {
-                            if (i < cnt) {
-                                const float send = up ? v[i] : v[i + cnt], keep = up ? v[i + cnt] : v[i];
-                                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-                            }
+                            for (int u = 0; u < UB; ++u) acc[u][g] = fma2(kf[u][2 * h + 1], qb, fma2(kf[u][2 * h], qa, acc[u][g]));
                         }
-                        base += up ? cnt : 0;
-                    } else {
-                        v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
                     }
                 }
-            }
-            constexpr int LEFT = NV >= 8 ? NV / 8 : 1;             // finished sums in this lane
+                // reduce over the eight lanes and leave each with its share of the NV sums
+                float v[NV];
 #pragma unroll
-            for (int i = 0; i < LEFT; ++i) {
-                const int j = base + i, u = j / G, g = j % G;
-                sc[(gl + 4 * (ub * UB + u)) * G + g] = v[i];
-            }
-        }
-        __syncwarp();
-        const int32_t row_ahead = row_next;
-        const float lw_ahead = lw_next;
-        if (more) copy_rows(kt, Kp, row_ahead, t0 + DEC_WARPS * TILE);
-        // ---- softmax of the tile, one entry per lane ----
-        float alpha[G];
+                for (int u = 0; u < UB; ++u)
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const bool live = lane < TILE && t0 + lane < (MODE == DEC_NEIGHBOURS ? min(c1, limit(g)) : c1);
-            const float s = live ? sc[lane * G + g] + lw : -INFINITY;            // base-2 logit
-            float mx = s;
+                    for (int g = 0; g < G; ++g) {
+                        float lo, hi;
+                        unpack2(acc[u][g], lo, hi);
+                        v[u * G + g] = lo + hi;
+                    }
+                int base = 0;
+                {
+                    int cnt = NV;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            mx = fmaxf(m[g], mx);
-            const float ref = mx == -INFINITY ? 0.f : mx;
-            alpha[g] = exp2f(m[g] - ref);                                        // exp2f(-inf) = 0 on the first tile
-            const float pw = live ? exp2f(s - ref) : 0.f;
-            l[g] = fmaf(l[g], alpha[g], pw);
-            m[g] = mx;
-            sc[lane * G + g] = pw;
-        }
+                    for (int off = 4; off > 0; off >>= 1) {
+                        if (cnt >= 2) {
+                            const bool up = (sub & off) != 0;
+                            cnt >>= 1;
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const uint64_t a2 = pack2(alpha[g], alpha[g]);
-#pragma unroll
-            for (int i = 0; i < EPC / 2; ++i) o[g][i] = mul2(o[g][i], a2);
-        }
-        // ---- values: lane owns chunk lane % NC of a row, EPI entries at a time ----
-        if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
-        else cp_async_wait<0>();
-        __syncwarp();
-        const int filled = c1 - t0 < TILE ? c1 - t0 : TILE;
-#pragma unroll 4
-        for (int i = 0; i < TILE / EPI; ++i) {
-            if (i * EPI >= filled) break;
-            const int e = i * EPI + lane / NC;
-            uint64_t vf[EPC / 2];
-            chunk_pairs(*reinterpret_cast<const uint4 *>(vt + (lane + 32 * i) * 16), vf, (const Tin *)nullptr);
-            float pe[G];
-            if constexpr (G >= 4) {
-#pragma unroll
-                for (int g = 0; g < G; g += 4) {
-                    const float4 p4 = *reinterpret_cast<const float4 *>(sc + e * G + g);
-                    pe[g] = p4.x; pe[g + 1] = p4.y; pe[g + 2] = p4.z; pe[g + 3] = p4.w;
+                            for (int i = 0; i < NV / 2; ++i) {
+                                if (i < cnt) {
+                                    const float send = up ? v[i] : v[i + cnt], keep = up ? v[i + cnt] : v[i];
+                                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                                }
+                            }
+                            base += up ? cnt : 0;
+                        } else {
+                            v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+                        }
+                    }
                 }
-            } else {
+                constexpr int LEFT = NV >= 8 ? NV / 8 : 1;             // finished sums in this lane
 #pragma unroll
-                for (int g = 0; g < G; ++g) pe[g] = sc[e * G + g];
+                for (int i = 0; i < LEFT; ++i) {
+                    const int j = base + i, u = j / G, g = j % G;
+                    sc[(gl + 4 * (ub * UB + u)) * G + g] = v[i];
+                }
+            }
+            __syncwarp();
+            const int32_t row_ahead = row_next;
+            const float lw_ahead = lw_next;
+            if (more) copy_rows(kt, Kp, row_ahead, t0 + DEC_WARPS * TILE);
+            // ---- softmax of the tile, one entry per lane ----
+            float alpha[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const bool live = lane < TILE && t0 + lane < (MODE == DEC_NEIGHBOURS ? min(c1, limit(g)) : c1);
+                const float s = live ? sc[lane * G + g] + lw : -INFINITY;            // base-2 logit
+                float mx = s;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                mx = fmaxf(m[g], mx);
+                const float ref = mx == -INFINITY ? 0.f : mx;
+                alpha[g] = exp2f(m[g] - ref);                                        // exp2f(-inf) = 0 on the first tile
+                const float pw = live ? exp2f(s - ref) : 0.f;
+                l[g] = fmaf(l[g], alpha[g], pw);
+                m[g] = mx;
+                sc[lane * G + g] = pw;
             }
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-                // (an entry behind the token's own must not meet its zero probability: it might be infinite)
-                if (MODE == DEC_NEIGHBOURS && t0 + TILE > seen0 && t0 + e >= limit(g)) continue;
-                const uint64_t p2 = pack2(pe[g], pe[g]);
+                const uint64_t a2 = pack2(alpha[g], alpha[g]);
 #pragma unroll
-                for (int j = 0; j < EPC / 2; ++j) o[g][j] = fma2(p2, vf[j], o[g][j]);
+                for (int i = 0; i < EPC / 2; ++i) o[g][i] = mul2(o[g][i], a2);
+            }
+            // ---- values: lane owns chunk lane % NC of a row, EPI entries at a time ----
+            if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
+            else cp_async_wait<0>();
+            __syncwarp();
+            const int filled = c1 - t0 < TILE ? c1 - t0 : TILE;
+#pragma unroll 4
+            for (int i = 0; i < TILE / EPI; ++i) {
+                if (i * EPI >= filled) break;
+                const int e = i * EPI + lane / NC;
+                uint64_t vf[EPC / 2];
+                chunk_pairs(*reinterpret_cast<const uint4 *>(vt + (lane + 32 * i) * 16), vf, (const Tin *)nullptr);
+                float pe[G];
+                if constexpr (G >= 4) {
+#pragma unroll
+                    for (int g = 0; g < G; g += 4) {
+                        const float4 p4 = *reinterpret_cast<const float4 *>(sc + e * G + g);
+                        pe[g] = p4.x; pe[g + 1] = p4.y; pe[g + 2] = p4.z; pe[g + 3] = p4.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int g = 0; g < G; ++g) pe[g] = sc[e * G + g];
+                }
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    // (an entry behind the token's own must not meet its zero probability: it might be infinite)
+                    if (MODE == DEC_NEIGHBOURS && t0 + TILE > seen0 && t0 + e >= limit(g)) continue;
+                    const uint64_t p2 = pack2(pe[g], pe[g]);
+#pragma unroll
+                    for (int j = 0; j < EPC / 2; ++j) o[g][j] = fma2(p2, vf[j], o[g][j]);
+                }
+            }
+            __syncwarp();
+            if (more) {
+                copy_rows(vt, Vp, row_ahead, t0 + DEC_WARPS * TILE);
+                lw = log2f(lw_ahead);
+                fetch_entries(t0 + 2 * DEC_WARPS * TILE);
             }
         }
-        __syncwarp();
-        if (more) {
-            copy_rows(vt, Vp, row_ahead, t0 + DEC_WARPS * TILE);
-            lw = log2f(lw_ahead);
-            fetch_entries(t0 + 2 * DEC_WARPS * TILE);
-        }
-    }
 
-    // ---- the warp's partial result, over its own tiles ----
-    float *po = reinterpret_cast<float *>(kt);                     // [g][D]
+        // ---- the warp's partial result, over its own tiles ----
+        float *po = reinterpret_cast<float *>(kt);                     // [g][D]
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        float ls = l[g];
+        for (int g = 0; g < G; ++g) {
+            float ls = l[g];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, off);
-        if (lane == 0) {
-            ml[(warp * G + g) * 2] = m[g];
-            ml[(warp * G + g) * 2 + 1] = ls;
-        }
-#pragma unroll
-        for (int i = 0; i < EPC / 2; ++i) {
-            float x, y;
-            unpack2(o[g][i], x, y);
-#pragma unroll
-            for (int off = NC; off < 32; off <<= 1) {
-                x += __shfl_xor_sync(0xffffffffu, x, off);
-                y += __shfl_xor_sync(0xffffffffu, y, off);
+            for (int off = 16; off > 0; off >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, off);
+            if (lane == 0) {
+                ml[(warp * G + g) * 2] = m[g];
+                ml[(warp * G + g) * 2 + 1] = ls;
             }
-            if (lane < NC) *reinterpret_cast<float2 *>(po + g * D + lane * EPC + 2 * i) = make_float2(x, y);
-        }
-    }
-    __syncthreads();
-    // ---- the part's result: to the workspace, to the cluster rank that finishes this slice of the output, or merged
-    // into what the parts before left ----
-    const int slice = (G * D + parts - 1) / parts;
-    // every CTA of the cluster is running (its shared memory may be written) once this wait is over
-    if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    auto remote = [&](const float *mine, int to) -> uint32_t {
-        uint32_t a;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(to));
-        return a;
-    };
-    if (pt < parts) {
 #pragma unroll
-        for (int k = 0; k < EPT; ++k) {
-            const int i = tid + k * DEC_WARPS * 32;
-            if (i >= G * D) break;
-            const int g = i / D;
-            float M = -INFINITY;
+            for (int i = 0; i < EPC / 2; ++i) {
+                float x, y;
+                unpack2(o[g][i], x, y);
 #pragma unroll
-            for (int wv = 0; wv < DEC_WARPS; ++wv) M = fmaxf(M, ml[(wv * G + g) * 2]);
-            float acc = 0.f, den = 0.f;
-#pragma unroll
-            for (int wv = 0; wv < DEC_WARPS; ++wv) {
-                const float mw = ml[(wv * G + g) * 2];
-                const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
-                acc = fmaf(f, reinterpret_cast<const float *>(smem + wv * 2 * C::TILE_BYTES)[i], acc);
-                den = fmaf(f, ml[(wv * G + g) * 2 + 1], den);
-            }
-            if constexpr (MODE == DEC_CLUSTER) {
-                const int to = i / slice;
-                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(recv + rank * slice + i - to * slice, to)), "f"(acc) : "memory");
-                if (i % D < parts) {                               // (parts <= 16 <= D: one thread per (g, rank))
-                    const uint32_t a = remote(rml + (rank * G + g) * 2, i % D);
-                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(M) : "memory");
-                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a + 4), "f"(den) : "memory");
+                for (int off = NC; off < 32; off <<= 1) {
+                    x += __shfl_xor_sync(0xffffffffu, x, off);
+                    y += __shfl_xor_sync(0xffffffffu, y, off);
                 }
-            } else if constexpr (SERIAL) {
-                // (running maximum and denominator in two buffers, part pt reading one and writing the other)
-                const float *was = rml + ((pt & 1) * G + g) * 2;
-                float Mr = was[0], dr = was[1];
-                merge_part(Mr, dr, run[k], M, den, acc);
-                if (i % D == 0) {
-                    float *now = rml + (((pt + 1) & 1) * G + g) * 2;
-                    now[0] = Mr;
-                    now[1] = dr;
-                }
-            } else {
-                float *out = part + (((int64_t)prob * gridDim.x + rank) * G + g) * (D + 2);
-                out[i % D] = acc;
-                if (i % D == 0) { out[D] = M; out[D + 1] = den; }
+                if (lane < NC) *reinterpret_cast<float2 *>(po + g * D + lane * EPC + 2 * i) = make_float2(x, y);
             }
         }
-    }
-    if constexpr (MODE == DEC_CLUSTER) {
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        const int i1 = (rank + 1) * slice < G * D ? (rank + 1) * slice : G * D;
-        if (rank < parts) {
-            for (int i = rank * slice + tid; i < i1; i += DEC_WARPS * 32) {
+        __syncthreads();
+        // ---- the part's result: to the workspace, to the cluster rank that finishes this slice of the output, or merged
+        // into what the parts before left ----
+        const int slice = (G * D + parts - 1) / parts;
+        // every CTA of the cluster is running (its shared memory may be written) once this wait is over
+        if constexpr (MODE == DEC_CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        auto remote = [&](const float *mine, int to) -> uint32_t {
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(to));
+            return a;
+        };
+        if (pt < parts) {
+#pragma unroll
+            for (int k = 0; k < EPT; ++k) {
+                const int i = tid + k * DEC_WARPS * 32;
+                if (i >= G * D) break;
                 const int g = i / D;
-                if (g >= groups) break;
-                float M = -INFINITY, den = 0.f, acc = 0.f;
-                for (int r = 0; r < parts; ++r)
-                    merge_part(M, den, acc, rml[(r * G + g) * 2], rml[(r * G + g) * 2 + 1], recv[r * slice + i - rank * slice]);
-                store_from(O, q_row(g) + i % D, acc / den);
+                float M = -INFINITY;
+#pragma unroll
+                for (int wv = 0; wv < DEC_WARPS; ++wv) M = fmaxf(M, ml[(wv * G + g) * 2]);
+                float acc = 0.f, den = 0.f;
+#pragma unroll
+                for (int wv = 0; wv < DEC_WARPS; ++wv) {
+                    const float mw = ml[(wv * G + g) * 2];
+                    const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
+                    acc = fmaf(f, reinterpret_cast<const float *>(smem + wv * 2 * C::TILE_BYTES)[i], acc);
+                    den = fmaf(f, ml[(wv * G + g) * 2 + 1], den);
+                }
+                if constexpr (MODE == DEC_CLUSTER) {
+                    const int to = i / slice;
+                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(recv + rank * slice + i - to * slice, to)), "f"(acc) : "memory");
+                    if (i % D < parts) {                               // (parts <= 16 <= D: one thread per (g, rank))
+                        const uint32_t a = remote(rml + (rank * G + g) * 2, i % D);
+                        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(M) : "memory");
+                        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a + 4), "f"(den) : "memory");
+                    }
+                } else if constexpr (SERIAL) {
+                    // (running maximum and denominator in two buffers, part pt reading one and writing the other)
+                    const float *was = rml + ((pt & 1) * G + g) * 2;
+                    float Mr = was[0], dr = was[1];
+                    merge_part(Mr, dr, run[k], M, den, acc);
+                    if (i % D == 0) {
+                        float *now = rml + (((pt + 1) & 1) * G + g) * 2;
+                        now[0] = Mr;
+                        now[1] = dr;
+                    }
+                } else {
+                    float *out = part + (((int64_t)prob * gridDim.x + rank) * G + g) * (D + 2);
+                    out[i % D] = acc;
+                    if (i % D == 0) { out[D] = M; out[D + 1] = den; }
+                }
             }
         }
-    }
+        if constexpr (MODE == DEC_CLUSTER) {
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            const int i1 = (rank + 1) * slice < G * D ? (rank + 1) * slice : G * D;
+            if (rank < parts) {
+                for (int i = rank * slice + tid; i < i1; i += DEC_WARPS * 32) {
+                    const int g = i / D;
+                    if (g >= groups) break;
+                    float M = -INFINITY, den = 0.f, acc = 0.f;
+                    for (int r = 0; r < parts; ++r)
+                        merge_part(M, den, acc, rml[(r * G + g) * 2], rml[(r * G + g) * 2 + 1], recv[r * slice + i - rank * slice]);
+                    store_from(O, q_row(g) + i % D, acc / den);
+                }
+            }
+        }
     }
     if constexpr (SERIAL) {
         __syncthreads();

@@ -15,8 +15,8 @@ struct CompressLayout {
     size_t cnorm;      // [BH][n]   c_t = ||k_t||^2 / sqrt(d)
     size_t cur;        // [BH][n]   current point sequence (row numbers)
     size_t nxt;        // [BH][n]   next level's sequence
-    size_t Mpair;      // [BH][n/2] running shift of each pair
-    size_t rdecay;     // [BH][n/2] exp(-(M_i - M_{i-1})/2)
+    size_t Mpair;      // [BH][pair_stride(n)] running shift of each pair
+    size_t rdecay;     // [BH][pair_stride(n)] exp(-(M_i - M_{i-1})/2)
     size_t F;          // [BH][n_out^2] pair Gram of the current level (all calls)
     size_t F_stride;   // elements per problem
     size_t wide;       // E4M3 inputs: K then V widened exactly to bf16, [BH][n][d] each
@@ -28,15 +28,15 @@ CompressLayout compress_layout(const elm_params *p);
 int compress_enqueue(const void *K, const void *V, const elm_params *params, uint64_t seed, int32_t *idx_out,
                      float *w_out, void *workspace, cudaStream_t st, uint32_t pbase);
 
-// What the Gram kernel needs to also run the halving walk of calls that fit one of its tiles
-// (at most 64 pairs): with `fused` set the pair Gram of the level never leaves shared memory and
+// What the Gram kernel needs to also run the halving walk of calls of which several fit one of its tiles
+// (fewer than 64 pairs): with `fused` set the pair Gram of the level never leaves shared memory and
 // the survivors go straight to `out`.
 struct WalkArgs {
     int fused;
     int64_t level;           // third counter word, first call and calls per sibling (pack_level in elm_common.cuh)
     uint64_t seed;
     float logfac;
-    const float *rdecay;     // [BH][n/2]
+    const float *rdecay;     // [BH][pair_stride(n)]
     int32_t *out;            // next level's sequence (or the final coreset)
     int64_t out_stride;
     uint32_t pbase;          // number of the first attention problem of this call (uniforms' counter)

@@ -53,9 +53,8 @@ struct Misc {
 static_assert(sizeof(Misc) <= 3072, "the misc block's share of shared memory");
 
 // Halving walk (Algorithm A.1) of the calls that lie inside one 64-pair tile, on the tile's pair
-// Gram in shared memory: warp w walks call w of the tile (P = 16, 32 or 64 pairs per call) in blocks
-// of 32 pairs with the warp-cooperative block walker; the first block of a 64-pair call folds its
-// decisions into the second block's scores as it goes.
+// Gram in shared memory: warp w walks call w of the tile (P = 16 or 32 pairs per call), one block of the
+// warp-cooperative block walker.
 __device__ __forceinline__ void walk_in_tile(const float *Fs, const float *rdec, const float *unif, int p,
                                              int64_t JR, int P, int64_t Ptotal, int64_t n,
                                              const int32_t *__restrict__ cur, const WalkArgs &wk, int warp, int lane)
@@ -66,21 +65,16 @@ __device__ __forceinline__ void walk_in_tile(const float *Fs, const float *rdec,
     if (J0 >= Ptotal) return;
     const float *Fc = Fs + (warp * P) * FS_LD + warp * P;      // the call's P x P block
     float bmax = 0.f, dn = 0.f;
-    for (int blk = 0; blk * 32 < P; ++blk) {
-        const int i = blk * 32 + lane;                         // pair within the call
-        const bool live = i < P;
-        const float dgn = live ? Fc[i * FS_LD + i] : 0.f;
-        const float a = walk_block_thresholds(sqrtf(dgn > 0.f ? dgn : 0.f), live ? rdec[warp * P + i] : 1.f, bmax,
-                                              wk.logfac, lane);
-        // the previous block already folded its decisions into this block's scores (dn); pairs
-        // past the end of a short call come after the live ones and decide nothing
-        const float d = walk_sign_score(dn, a, live ? unif[warp * P + i] : 1.f);
-        dn = 0.f;
-        const uint32_t swaps = walk_block_warp(Fc + (blk * 32) * FS_LD + blk * 32, FS_LD, d, dn, lane);
-        if (live) {
-            const uint32_t sw = (swaps >> lane) & 1u;
-            wk.out[(int64_t)p * wk.out_stride + J0 + i] = cur[(int64_t)p * n + 2 * (J0 + i) + sw];
-        }
+    const int i = lane;                                        // pair within the call
+    const bool live = i < P;
+    const float dgn = live ? Fc[i * FS_LD + i] : 0.f;
+    const float a = walk_block_thresholds(sqrtf(dgn > 0.f ? dgn : 0.f), live ? rdec[warp * P + i] : 1.f, bmax, wk.logfac, lane);
+    // pairs past the end of a short call come after the live ones and decide nothing
+    const float d = walk_sign_score(0.f, a, live ? unif[warp * P + i] : 1.f);
+    const uint32_t swaps = walk_block_warp(Fc, FS_LD, d, dn, lane);
+    if (live) {
+        const uint32_t sw = (swaps >> lane) & 1u;
+        wk.out[(int64_t)p * wk.out_stride + J0 + i] = cur[(int64_t)p * n + 2 * (J0 + i) + sw];
     }
 }
 

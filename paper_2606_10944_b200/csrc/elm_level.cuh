@@ -510,7 +510,7 @@ __device__ __forceinline__ void load4(const double *p, double (&f)[4])
 //   warp 1     copies the tiles the walker needs (asynchronous copies) AHEAD blocks before it needs them; DEEP: also
 //              the next block's thresholds.
 //   warps 2..  the updaters fold block c-1 into the scores of all columns from block c+1 on, one
-//              block behind the walker.  The rows of a block are streamed through two shared-memory
+//              block behind the walker.  The rows of a block are streamed through two (DEEP: three) shared-memory
 //              panels with asynchronous copies; F does not depend on the decisions, so the first
 //              panel of the next round is already in flight when its swap mask becomes known.
 // One __syncthreads per block separates the iterations.
@@ -529,7 +529,7 @@ static __global__ void __launch_bounds__(576) walk_cta_kernel(const T *__restric
                                                        T logfac, uint32_t pbase)
 {
     cudaGridDependencySynchronize();           // launched with programmatic stream serialization (launch_after)
-    constexpr int PW = 2048 / sizeof(T);                             // panel width in columns (64 KB / 2 buffers... per 32 rows)
+    constexpr int PW = 2048 / sizeof(T);                             // panel width in columns: 64 KB per panel of 32 rows
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int AHEAD = DEEP ? 3 : 1;                              // blocks between a tile's request and its use
     constexpr int TB = AHEAD + 1, PB = DEEP ? 3 : 2;                 // tile buffers, panel buffers
