@@ -96,4 +96,10 @@ bool attend_decode_windows_apply(const elm_params *p, int n_core);
 int attend_decode_windows(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
                           const DecodeWindows &win, const elm_params *p, void *O, int *status, cudaStream_t st);
 
+// Its launch for bf16 storage (elm_attend_tokens.cu): lists spread over at most `cap` CTAs, a power of two no larger than
+// tokens_largest_cluster(d), the largest cluster the current device can place.
+int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
+                       const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st);
+int tokens_largest_cluster(int d);
+
 }  // namespace elm

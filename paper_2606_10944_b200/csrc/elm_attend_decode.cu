@@ -128,7 +128,7 @@ struct DecodeGroups {
 };
 
 // How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp (with one, a single token over
-// 200 entries takes 5.8 us for 6.9, less than the host needs to enqueue it, but a CTA that walks all parts has twice the
+// 200 entries (figures here and in decode_form: bf16 rows, whose tokens took these forms when they were measured) takes 5.8 us for 6.9, less than the host needs to enqueue it, but a CTA that walks all parts has twice the
 // merges: 2000 tokens of 8 KV heads of 4 query heads, n_out = 128, 1010 us for 960), at most `cap` parts.  Depends on
 // n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
 __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entries, int tile, int cap, int &parts, int &chunk)
@@ -598,34 +598,19 @@ template <typename F> auto with_groups(int groups, F f)
 std::atomic<int> g_debug_largest_cluster{0};
 template <typename Tin, int D> int decode_largest_cluster()
 {
-    static std::atomic<int> cached[64];                            // (threads that meet here first find the same answer)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-    int largest = cached[dev].load(std::memory_order_relaxed);
-    if (largest == 0) {
-        using C = DecodeCfg<Tin, D, DEC_GSTREAM>;
-        auto kern = decode_kernel<Tin, D, DEC_GSTREAM, DEC_CLUSTER>;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.blockDim = dim3(DEC_WARPS * 32);
-        cfg.dynamicSmemBytes = C::template total<DEC_CLUSTER>();
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int size = DEC_MAX_CLUSTER;
-        bool fits = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) == cudaSuccess &&
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-        for (; fits && size > 1; size >>= 1) {
-            int clusters = 0;
-            attr[0].val.clusterDim.x = (unsigned)size;
-            cfg.gridDim = dim3((unsigned)size);
-            if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1) break;
+    int largest;
+    if constexpr (std::is_same<Tin, __nv_bfloat16>::value) {
+        largest = tokens_largest_cluster(D);
+    } else {
+        static std::atomic<int> cached[64];                        // (threads that meet here first find the same answer)
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+        largest = cached[dev].load(std::memory_order_relaxed);
+        if (largest == 0) {
+            largest = largest_cluster(decode_kernel<Tin, D, DEC_GSTREAM, DEC_CLUSTER>, DEC_WARPS * 32,
+                                      DecodeCfg<Tin, D, DEC_GSTREAM>::template total<DEC_CLUSTER>(), DEC_MAX_CLUSTER);
+            cached[dev].store(largest, std::memory_order_relaxed);
         }
-        cudaGetLastError();
-        largest = fits ? size : 1;
-        cached[dev].store(largest, std::memory_order_relaxed);
     }
     const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
     return limit && limit < largest ? limit : largest;
@@ -639,7 +624,9 @@ template <typename Tin, int D> int decode_largest_cluster()
 // 12288 entries: 606 us together, 1190 one by one).
 template <typename Tin, int D> int decode_cap(int problems, int per_token, int sms)
 {
-    const int most = DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
+    // (bf16: all query vectors of a token go together, two CTAs to an SM)
+    const int most = std::is_same<Tin, __nv_bfloat16>::value ? 2 * sms / problems
+                                                             : DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
     int cap = decode_largest_cluster<Tin, D>();
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
@@ -749,7 +736,7 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     const int q_heads = p->q_heads, kv_heads = p->kv_heads, n_q = p->n_q;
     DecodeGroups grp = {};
     if (win) {
-        if constexpr (G <= DEC_GSTREAM) {
+        if constexpr (G <= DEC_GSTREAM && std::is_same<Tin, float>::value) {
             grp.vec_groups = form.vec_groups;
             grp.per_group = form.per_group;
             for (int i = 0; i < win->n; ++i) {
@@ -778,7 +765,7 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
             count_launches(1);
             return cuda_status(cudaGetLastError());
         } else {
-            return ELM_ERR_SHAPE;                                  // (decode_form gives no such G)
+            return ELM_ERR_SHAPE;                                  // (decode_form gives no such G; bf16: attend_tokens_bf16)
         }
     }
     DecodeWindows whole = {};
@@ -809,7 +796,13 @@ int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *
 {
     const int per_token = (p->q_heads / p->kv_heads) * p->n_q;
     DecodeForm form = {per_token, 1, 1, 0, 0};
-    if (win) form = decode_form<Tin, D>(*win, p->batch * p->kv_heads, per_token);
+    if (win) {
+        const int problems = p->batch * p->kv_heads;
+        if constexpr (std::is_same<Tin, __nv_bfloat16>::value)
+            return attend_tokens_bf16(Q, K, V, idx, w, list_stride, *win, p, O, status, decode_cap<Tin, D>(problems, per_token, device_sm_count()), st);
+        else
+            form = decode_form<Tin, D>(*win, problems, per_token);
+    }
     return with_groups(form.G, [&](auto G) {
         return launch_decode<Tin, D, decltype(G)::value>((const Tin *)Q, (const Tin *)K, (const Tin *)V, idx, w, list_stride, n_core, win,
                                                          form, p, (Tin *)O, part, part_room, status, per_token, st);

@@ -1,0 +1,757 @@
+// Attention of the tokens of a streaming run, bf16 storage: every token attends over a prefix of its window's list
+//   O[t,:] = sum_c w_c exp(<q_t,k_c>/sqrt(d)) v_c / sum_c w_c exp(<q_t,k_c>/sqrt(d)),  c < seen(t)      Eq. (def:att_approx)
+//
+// Neighbouring tokens see all but a few of the same entries, and a token has one query vector per query head of its KV
+// head, so 16 rows of a matrix instruction hold the vectors of 16, 8, 4 or 2 neighbouring tokens (TokenGroups::per_group).
+// Both contractions are mma.sync m16n8k16 with fp32 accumulators: Q K^T on the stored bf16 values, P V with each fp32
+// probability as the sum of three bf16 values (split3: 24 bits, so nothing is rounded that fp32 arithmetic would keep).
+// tcgen05 takes 64 rows at least: a single token of four vectors would leave most of them empty, and the accumulators of
+// each 32-entry unit (below) would go through tensor memory and back.
+//
+// The work is cut the same way whatever tokens share a launch: the list in units of k tiles of 32 entries (token_units), a unit's softmax
+// by one warp from its own maximum, the units merged in the order of the list.  A row's arithmetic does not depend on
+// the other rows, so a token's output is the same bit for bit in every form:
+//   cluster  one thread-block cluster per group of neighbouring tokens, one unit per warp; the warps hand their results
+//            to the CTA that finishes the slice through distributed shared memory.
+//   serial   one CTA per four groups, a group's 16 rows per warp; the tiles come once for all four warps through a ring
+//            of asynchronous copies and every warp merges unit after unit in registers.
+//
+// Bound by the issue of mma.sync: 128 per tile and 16 rows, 32 for the logits and 96 for the values, at the 16 cycles that each
+// takes an SM sub-partition (measured: 2250 cycles per tile with two warps on each).  2496 tokens of 32 query / 8 KV heads,
+// n_out = 256: 1186 us with fp32 fma per token, 237 us here; a token over 6144 entries of 8 KV heads of 4 query heads 17.4 ->
+// 15.5 us, of 8 query heads 23.2 -> 16.9, over 500 entries 8.1 -> 8.2; of 1 query head over 4100 entries 9.3 -> 11.0 (its one
+// vector pays for eight).
+#include <math.h>
+
+#include <atomic>
+#include <type_traits>
+
+#include "elm_attend.cuh"
+#include "elm_common.cuh"
+#include "elm_sm100.cuh"
+
+namespace elm {
+namespace {
+
+using sm100::fma2;
+using sm100::mul2;
+using sm100::pack2;
+using sm100::pack_bf16x2;
+using sm100::smem_u32;
+using sm100::unpack2;
+
+constexpr int TOK_WARPS = 4;
+constexpr int TOK_THREADS = TOK_WARPS * 32;
+constexpr int TOK_ROWS = 16;                   // rows of the matrix instruction
+constexpr int TOK_TILE = 32;                   // entries per tile
+constexpr int TOK_MAX_CLUSTER = 16;
+constexpr int TOK_STAGES = 4;                  // ring of the serial form
+constexpr int TOK_CTAS = 2;                    // CTAs per SM the kernel is compiled for
+
+struct TokenGroups {
+    int32_t cluster;                           // CTAs per group (cluster form)
+    int32_t cap;                               // most CTAs a list is spread over
+    int32_t per_group;                         // neighbouring tokens of a warp: a power of two
+    int32_t span;                              // tokens per cluster or CTA: per_group, or four times as many
+    int32_t g0[DECODE_MAX_WINDOWS + 1];        // groups of `span` tokens in the windows before
+};
+
+// Tiles per unit of a list of n_core entries: at most 4 cap units.  Depends on n_core only through the next multiple of
+// 128, so that the (at most 64, aligned) tokens of a span agree.
+__host__ __device__ __forceinline__ int token_units(int n_core, int cap)
+{
+    const int tiles = (n_core + 127) / 128 * (128 / TOK_TILE);
+    return (tiles + TOK_WARPS * cap - 1) / (TOK_WARPS * cap);
+}
+
+template <int D> struct TokenCfg {
+    static constexpr int RB = D * 2;                               // bytes per row
+    static constexpr int NC = RB / 16;                             // 16-byte chunks per row
+    static constexpr int TILE_BYTES = TOK_TILE * RB;
+    static constexpr int MT = D / 16;                              // row tiles of the transposed output
+    static constexpr int MAX_UNITS = TOK_WARPS * TOK_MAX_CLUSTER;
+    // serial form: [stage][K, V], log2 weights, per warp the probabilities of the entries that are added by scalar code
+    static constexpr int P_STRIDE = TOK_ROWS + 1;                  // (a group of at most 16 tokens: at most 15 entries)
+    static constexpr int S_LW = TOK_STAGES * 2 * TILE_BYTES;
+    static constexpr int S_P = S_LW + TOK_STAGES * TOK_TILE * 4;
+    static constexpr int S_TOTAL = S_P + TOK_WARPS * TOK_ROWS * P_STRIDE * 4;
+    // cluster form: [warp][K, V], log2 weights, probabilities; maxima (then factors of the state) and denominators [row][unit],
+    // factors of the units (over the probabilities) likewise; the CTA's slice of every unit's result, [unit][column of the slice][row]
+    template <int ROWS> struct Cluster {
+        static constexpr int LW = TOK_WARPS * 2 * TILE_BYTES;
+        static constexpr int P = LW + TOK_WARPS * TOK_TILE * 4;
+        static constexpr int ML = P + TOK_WARPS * TOK_ROWS * P_STRIDE * 4;
+        static constexpr int RECV = ML + ROWS * MAX_UNITS * 8;
+        static constexpr int TOTAL = RECV + TOK_WARPS * D * (ROWS + 2) * 4;
+        static constexpr int FB = P;
+        static_assert(ROWS * MAX_UNITS * 4 <= ML - P, "the factors of the units lie over the probabilities");
+        static_assert(TOK_CTAS * (TOTAL + 1024) <= 228 * 1024, "shared memory for as many CTAs as there are registers for");
+    };
+};
+
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool live)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// chunk c of row e of a tile lies at chunk c ^ (e mod 8): the eight rows a matrix load reads fall into different banks
+template <int NC> __device__ __forceinline__ uint32_t chunk_at(int e, int c) { return (uint32_t)((e * NC + (c ^ (e & 7))) * 16); }
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Two probabilities as sums of three bf16 values each (low halves: p0, high halves: p1).  The first two parts are taken
+// just below what they stand for, so that all parts of a positive value are positive: an infinite value of V stays that
+// infinity instead of meeting a part that is zero or negative.
+__device__ __forceinline__ void split3(float p0, float p1, uint32_t &hi, uint32_t &mid, uint32_t &lo)
+{
+    const uint32_t h0 = (max(__float_as_uint(p0), 1u) - 1u) & 0xffff0000u, h1 = (max(__float_as_uint(p1), 1u) - 1u) & 0xffff0000u;
+    const float r0 = p0 - __uint_as_float(h0), r1 = p1 - __uint_as_float(h1);
+    const uint32_t m0 = (max(__float_as_uint(r0), 1u) - 1u) & 0xffff0000u, m1 = (max(__float_as_uint(r1), 1u) - 1u) & 0xffff0000u;
+    hi = __byte_perm(h0, h1, 0x7632);
+    mid = __byte_perm(m0, m1, 0x7632);
+    lo = pack_bf16x2(r0 - __uint_as_float(m0), r1 - __uint_as_float(m1));
+}
+
+// factors of a merge of a unit with maximum m into a state with maximum M
+__device__ __forceinline__ void merge_factors(float M, float m, float &Mn, float &a, float &b)
+{
+    Mn = fmaxf(M, m);
+    a = M == -INFINITY ? 0.f : exp2f(M - Mn);
+    b = m == -INFINITY ? 0.f : exp2f(m - Mn);
+}
+
+// The probabilities P [row][entry] as they leave Q K^T are the B operand of O^T = V^T P^T, whose columns are the query vectors,
+// eight at a time: a call of few vectors does not pay for sixteen in the larger of the two products.
+//
+// A unit's state.  o: of the rows 8 b + 2 (lane % 4) + {0, 1}, b < NB, the columns lane / 4 + 8 k; m, l: of the rows 8 b + lane / 4.
+template <int D, int NB> struct TokenUnit {
+    float o[D / 16][NB][4];
+    float m[NB], l[NB];
+    __device__ __forceinline__ void reset()
+    {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+#pragma unroll
+            for (int j = 0; j < D / 16; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) o[j][b][i] = 0.f;
+            m[b] = -INFINITY;
+            l[b] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void finish()
+    {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            l[b] += __shfl_xor_sync(0xffffffffu, l[b], 1);
+            l[b] += __shfl_xor_sync(0xffffffffu, l[b], 2);
+        }
+    }
+};
+// what the rows 2 (lane % 4) + {0, 1} of eight have of a value held by row
+__device__ __forceinline__ void of_columns(float x, float &x0, float &x1)
+{
+    const int quad = threadIdx.x & 3;
+    x0 = __shfl_sync(0xffffffffu, x, 8 * quad);
+    x1 = __shfl_sync(0xffffffffu, x, 8 * quad + 4);
+}
+
+// q k of one tile of 32 entries whose rows lie at kt: s[j][2 b + i], entry 8 j + 2 (lane % 4) + i of row 8 b + lane / 4
+template <int D, int NB>
+__device__ __forceinline__ void token_logits(float (&s)[4][4], const uint32_t (&qf)[D / 16][4], uint32_t kt)
+{
+    constexpr int NC = TokenCfg<D>::NC;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[j][i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) {
+        uint32_t b[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ldsm4(b[j], kt + chunk_at<NC>(8 * j + (lane & 7), 4 * i + (lane >> 3)));
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mma16816(s[j], qf[2 * i + h], b[j][2 * h], b[j][2 * h + 1]);
+    }
+}
+
+// The tile's softmax: logits to probabilities.  t0 is its first entry, lw its log2 weights; the thread's rows see the entries
+// below lim[.], all rows of the group those below `common`.
+template <int D, int NB>
+__device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, float (&s)[4][4], const float *lw, int t0,
+                                              const int (&lim)[NB], int common, float scale)
+{
+    const int quad = threadIdx.x & 3;
+    const bool tail = t0 + TOK_TILE > common;                      // (the same for the whole warp)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 w2 = *reinterpret_cast<const float2 *>(lw + 8 * j + 2 * quad);
+#pragma unroll
+        for (int i = 0; i < 2 * NB; ++i) s[j][i] = fmaf(s[j][i], scale, i & 1 ? w2.y : w2.x);
+    }
+    if (tail) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 2 * NB; ++i)
+                if (t0 + 8 * j + 2 * quad + (i & 1) >= lim[i >> 1]) s[j][i] = -INFINITY;
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mx = fmaxf(mx, fmaxf(s[j][2 * b], s[j][2 * b + 1]));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        mx = fmaxf(u.m[b], mx);
+        const float ref = mx == -INFINITY ? 0.f : mx;
+        if (!first) {
+            const float alpha = exp2f(u.m[b] - ref);
+            // (rounded on its own: whether a compiler fuses it with the sum below must not depend on the form)
+            u.l[b] = __fmul_rn(u.l[b], alpha);
+            float a0, a1;
+            of_columns(alpha, a0, a1);
+#pragma unroll
+            for (int j = 0; j < D / 16; ++j) {
+                u.o[j][b][0] *= a0; u.o[j][b][1] *= a1;
+                u.o[j][b][2] *= a0; u.o[j][b][3] *= a1;
+            }
+        }
+        u.m[b] = mx;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                s[j][2 * b + i] = exp2f(s[j][2 * b + i] - ref);
+                u.l[b] = __fadd_rn(u.l[b], s[j][2 * b + i]);
+            }
+    }
+}
+
+// The tile's values, whose rows lie at vrows; some row of the group sees the entries below `last`, and those below `loaded` are
+// there (what other warps of the CTA see)
+template <int D, int NB>
+__device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, const float (&s)[4][4], const unsigned char *vrows, float *sp,
+                                             int t0, const int (&lim)[NB], int common, int last, int loaded)
+{
+    using C = TokenCfg<D>;
+    constexpr int NC = C::NC;
+    const int lane = threadIdx.x & 31, quad = lane & 3;
+    const uint32_t vt = smem_u32(vrows);
+    // Entries that only some rows see, or none: one with an infinity or a NaN must not meet the zero probabilities of the others in the
+    // matrix instruction.  Its values are taken as zero there and added by scalar code to the rows that see it.
+    const int e0 = common > t0 ? common - t0 : 0, e1 = loaded - t0 < TOK_TILE ? loaded - t0 : TOK_TILE;
+    uint32_t bad = 0;
+    if (e0 < e1) {
+        for (int i = lane; i < (e1 - e0) * NC; i += 32) {
+            const uint4 x = *reinterpret_cast<const uint4 *>(vrows + chunk_at<NC>(e0 + i / NC, i % NC));
+            // an exponent of all ones carries into the sign's place
+            const uint32_t y = ((x.x & 0x7f807f80u) + 0x00800080u) | ((x.y & 0x7f807f80u) + 0x00800080u) |
+                               ((x.z & 0x7f807f80u) + 0x00800080u) | ((x.w & 0x7f807f80u) + 0x00800080u);
+            if (y & 0x80008000u) bad |= 1u << (e0 + i / NC);
+        }
+        bad = __reduce_or_sync(0xffffffffu, bad);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        uint32_t p[NB][3][2];                                          // entries 16 k + {0, 8} + 2 (lane % 4) + {0, 1} of row 8 b + lane / 4
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                split3(s[2 * k + h][2 * b], s[2 * k + h][2 * b + 1], p[b][0][h], p[b][1][h], p[b][2][h]);
+        auto mask_of = [&](int e) { return (bad >> e & 1 ? 0u : 0xffffu) | (bad >> (e + 1) & 1 ? 0u : 0xffff0000u); };
+        const uint32_t k0 = mask_of(16 * k + 2 * quad), k1 = mask_of(16 * k + 8 + 2 * quad);
+        // matrices of a load: entries 16 k + {0, 0, 8, 8} + 0..7, chunks {0, 1, 0, 1} of the 16 columns
+        const uint32_t va = vt + (uint32_t)((16 * k + (lane >> 4) * 8 + (lane & 7)) * C::RB);
+        const int sw = lane & 7, half = (lane >> 3) & 1;
+#pragma unroll
+        for (int j = 0; j < D / 16; j += 2) {
+            uint32_t a[2][4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                ldsm4_t(a[h], va + (uint32_t)(((2 * (j + h) + half) ^ sw) * 16));
+                if (bad) {
+                    a[h][0] &= k0; a[h][1] &= k0;
+                    a[h][2] &= k1; a[h][3] &= k1;
+                }
+            }
+#pragma unroll
+            for (int part = 0; part < 3; ++part)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) mma16816(u.o[j + h][b], a[h], p[b][part][0], p[b][part][1]);
+        }
+    }
+    if (bad) {
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 2 * NB; ++i) {
+                const int e = 8 * j + 2 * quad + (i & 1);
+                if (e >= e0 && t0 + e < last) sp[((lane >> 2) + 8 * (i >> 1)) * C::P_STRIDE + e - e0] = s[j][i];
+            }
+        __syncwarp();
+        for (int e = e0; e < e1 && t0 + e < last; ++e) {
+            if (!(bad >> e & 1)) continue;
+            float v[D / 8];
+#pragma unroll
+            for (int j = 0; j < D / 8; ++j)
+                v[j] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(vrows + chunk_at<NC>(e, j) + 2 * (lane >> 2)));
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                int lim2[2];
+                lim2[0] = __shfl_sync(0xffffffffu, lim[b], 8 * quad);
+                lim2[1] = __shfl_sync(0xffffffffu, lim[b], 8 * quad + 4);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float pe = sp[(8 * b + 2 * quad + i) * C::P_STRIDE + e - e0];
+                    if (t0 + e < lim2[i]) {
+#pragma unroll
+                        for (int j = 0; j < D / 16; ++j) {
+                            u.o[j][b][i] = fmaf(pe, v[2 * j], u.o[j][b][i]);
+                            u.o[j][b][2 + i] = fmaf(pe, v[2 * j + 1], u.o[j][b][2 + i]);
+                        }
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// NB: query vectors of a warp, in eights (the serial form takes two)
+template <int D, bool CLUSTER, int NB>
+__global__ void __launch_bounds__(TOK_THREADS, TOK_CTAS)
+tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
+              const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int64_t list_stride, int q_heads, int kv_heads,
+              int per_token, const __grid_constant__ DecodeWindows win, const __grid_constant__ TokenGroups grp,
+              __nv_bfloat16 *__restrict__ O, int *__restrict__ status)
+{
+    using C = TokenCfg<D>;
+    using CC = typename C::template Cluster<8 * NB>;
+    constexpr int NC = C::NC, MT = C::MT;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, quad = lane & 3;
+    // (launched with programmatic stream serialization: nothing is read or written before this point)
+    cudaGridDependencySynchronize();
+    if constexpr (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const int prob = blockIdx.y;
+    const int rank = CLUSTER ? (int)blockIdx.x % grp.cluster : 0;
+    // (serial form: the longest lists, those of the last tokens, start first)
+    const int group = CLUSTER ? (int)blockIdx.x / grp.cluster : (int)(gridDim.x - 1 - blockIdx.x);
+#ifndef ELM_BOUNDS_CHECK
+    // this path has no bounded waits and (in this build) no row checks: its status word reads 0
+    if (tid == 0 && prob == 0 && blockIdx.x == 0) *status = 0;
+#endif
+    int wi = 0;
+    while (wi + 1 < win.n && group >= grp.g0[wi + 1]) ++wi;
+    // the tokens of the span see lo + 1 .. lo + span entries, as far as the window has them
+    const int lo = ((win.seen0[wi] - 1) / grp.span + (group - grp.g0[wi])) * grp.span;
+    const int last_seen = win.seen0[wi] + (win.tok0[wi + 1] - win.tok0[wi]) - 1;
+    const int n_span = min(last_seen, lo + grp.span);              // what the last of them sees
+    // this warp's group: first entry count that is aligned, first that is in the launch, last
+    const int aligned = lo + (CLUSTER ? 0 : warp * grp.per_group) + 1;
+    const int first = max(aligned, win.seen0[wi]);
+    const int rows = max(min(n_span, aligned + grp.per_group - 1) - first + 1, 0) * per_token;
+    const int last = rows ? min(n_span, aligned + grp.per_group - 1) : 0;
+    const int b = prob / kv_heads, kvh = prob % kv_heads, rep = q_heads / kv_heads;
+    const int32_t *ip = idx + (int64_t)prob * list_stride + win.off[wi];
+    const float *wp = w + (int64_t)prob * list_stride + win.off[wi];
+    const __nv_bfloat16 *Kp = K + (int64_t)prob * n * D, *Vp = V + (int64_t)prob * n * D;
+    // offset of row r in Q and O
+    auto q_row = [&](int r) -> int64_t {
+        const int64_t z = win.tok0[wi] + (first - win.seen0[wi]) + r / per_token;
+        return ((z * (gridDim.y / kv_heads) + b) * q_heads + kvh * rep + r % per_token) * D;
+    };
+    int lim[NB];
+    // the query vectors as operands, scaled by 1/8: exactly, and close enough to 1/sqrt(d) that no product is larger than
+    // the logit's
+    uint32_t qf[D / 16][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = 8 * h + (lane >> 2);
+        const bool live = h < NB && r < rows;
+        if (h < NB) lim[h < NB ? h : 0] = live ? first + r / per_token : 0;
+        const __nv_bfloat16 *q = Q + (live ? q_row(r) : 0) + 2 * quad;
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                __nv_bfloat162 x = __floats2bfloat162_rn(0.f, 0.f);
+                if (live) x = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(q + 16 * i + 8 * c), __floats2bfloat162_rn(0.125f, 0.125f));
+                qf[i][2 * c + h] = *reinterpret_cast<const uint32_t *>(&x);
+            }
+    }
+    const float scale = 8.f * 1.4426950408889634f / sqrtf((float)D);
+    const int unit_tiles = token_units(n_span, grp.cap);
+    const int tiles = (n_span + TOK_TILE - 1) / TOK_TILE;
+    float *sp = reinterpret_cast<float *>(smem + (CLUSTER ? CC::P : C::S_P)) + warp * TOK_ROWS * C::P_STRIDE;
+    TokenUnit<D, NB> u;
+
+    if constexpr (CLUSTER) {
+        // ---- one unit per warp ----
+        const int units = (tiles + unit_tiles - 1) / unit_tiles;
+        const int unit = rank * TOK_WARPS + warp;
+        unsigned char *kt = smem + warp * 2 * C::TILE_BYTES, *vt = kt + C::TILE_BYTES;
+        float *lw = reinterpret_cast<float *>(smem + CC::LW) + warp * TOK_TILE;
+        int32_t row = 0;
+        float wt = 0.f;
+        auto fetch_entries = [&](int t) {
+            const int e = t * TOK_TILE + lane;
+            row = 0;
+            wt = 0.f;
+            if (e < n_span) {
+                row = (int32_t)checked_row(__ldg(ip + e), n, status);
+                wt = __ldg(wp + e);
+            }
+        };
+        auto copy_rows = [&](unsigned char *dst, const __nv_bfloat16 *X, int32_t from, int t) {
+            const uint32_t d0 = smem_u32(dst);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) {
+                const int e = (lane + 32 * i) / NC, c = lane % NC;
+                const int64_t r = __shfl_sync(0xffffffffu, from, e);
+                cp_async16_zfill(d0 + chunk_at<NC>(e, c), X + r * D + c * 8, t * TOK_TILE + e < n_span);
+            }
+            cp_async_commit();
+        };
+        const int t_end = min((unit + 1) * unit_tiles, tiles);
+        int t = unit * unit_tiles;
+        u.reset();
+        if (t < t_end) {
+            fetch_entries(t);
+            copy_rows(kt, Kp, row, t);
+            copy_rows(vt, Vp, row, t);
+        }
+        for (bool head = true; t < t_end; ++t, head = false) {
+            const bool more = t + 1 < t_end;
+            float s[4][4];
+            lw[lane] = log2f(wt);
+            if (more) fetch_entries(t + 1);
+            cp_async_wait<1>();                                        // the keys (the values are the newer group)
+            __syncwarp();
+            token_logits<D, NB>(s, qf, smem_u32(kt));
+            __syncwarp();
+            if (more) copy_rows(kt, Kp, row, t + 1);
+            token_softmax<D, NB>(u, head, s, lw, t * TOK_TILE, lim, aligned, scale);
+            if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
+            else cp_async_wait<0>();
+            __syncwarp();
+            token_values<D, NB>(u, s, vt, sp, t * TOK_TILE, lim, aligned, last, n_span);
+            __syncwarp();
+            if (more) copy_rows(vt, Vp, row, t + 1);
+        }
+        u.finish();
+        // ---- to the CTA that finishes the slice: columns of all rows, as many to each of `parts` (a power of two) CTAs ----
+        int parts_log = 0;
+        while ((1 << parts_log) < (units + TOK_WARPS - 1) / TOK_WARPS) ++parts_log;
+        constexpr int D_LOG = D == 64 ? 6 : 7;
+        const int cols_log = D_LOG - parts_log;
+        // (rows go in pairs, and 18 floats from column to column spread 16 rows over the banks)
+        const int col_stride = ((rows + 1) & ~1) + 2, slice = col_stride << cols_log;
+        float2 *ml = reinterpret_cast<float2 *>(smem + CC::ML);
+        float *fb = reinterpret_cast<float *>(smem + CC::FB), *recv = reinterpret_cast<float *>(smem + CC::RECV);
+        auto remote = [&](const void *mine, int to) -> uint32_t {
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(to));
+            return a;
+        };
+        auto send2 = [&](uint32_t a, float x, float y) {
+            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+        };
+        // every CTA of the cluster is running (its shared memory may be written) once this wait is over
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (unit < units) {
+#pragma unroll
+            for (int h = 0; h < NB; ++h) {
+                const int r = 8 * h + 2 * quad;
+                if (r < rows) {
+#pragma unroll
+                    for (int j = 0; j < 2 * MT; ++j) {
+                        const int c = 8 * j + (lane >> 2);
+                        send2(remote(recv + unit * slice + (c & ((1 << cols_log) - 1)) * col_stride + r, c >> cols_log), u.o[j >> 1][h][2 * (j & 1)],
+                              u.o[j >> 1][h][2 * (j & 1) + 1]);
+                    }
+                }
+                if (8 * h + (lane >> 2) < rows)
+                    for (int to = quad; to < 1 << parts_log; to += 4)
+                        send2(remote(ml + (8 * h + (lane >> 2)) * C::MAX_UNITS + unit, to), u.m[h], u.l[h]);
+            }
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank < 1 << parts_log) {
+            // factors of the merges: running maxima of the rows' units, by a warp per row or, for short lists, four rows to a warp
+            auto factors = [&](auto lanes) {
+                constexpr int W = decltype(lanes)::value;
+                const int li = lane & (W - 1);
+                for (int r = warp * (32 / W) + lane / W; r - lane / W < rows; r += TOK_WARPS * (32 / W)) {
+                    float carry = -INFINITY;
+                    for (int u0 = 0; u0 < units; u0 += W) {
+                        const bool live = r < rows && u0 + li < units;
+                        const float m = live ? ml[r * C::MAX_UNITS + u0 + li].x : -INFINITY;
+                        float mx = m;
+#pragma unroll
+                        for (int off = 1; off < W; off <<= 1) {
+                            const float y = __shfl_up_sync(0xffffffffu, mx, off, W);
+                            if (li >= off) mx = fmaxf(mx, y);
+                        }
+                        float before = __shfl_up_sync(0xffffffffu, mx, 1, W);
+                        before = li == 0 ? carry : fmaxf(before, carry);
+                        float Mn, a, b;
+                        merge_factors(before, m, Mn, a, b);
+                        if (live) {
+                            ml[r * C::MAX_UNITS + u0 + li].x = a;
+                            fb[r * C::MAX_UNITS + u0 + li] = b;
+                        }
+                        carry = fmaxf(carry, __shfl_sync(0xffffffffu, mx, W - 1, W));
+                    }
+                }
+            };
+            if (units <= 8) factors(std::integral_constant<int, 8>());
+            else factors(std::integral_constant<int, 32>());
+            __syncthreads();
+            const int c0 = rank << cols_log;
+            for (int i = tid; i < rows << cols_log; i += TOK_THREADS) {
+                const int c = i & ((1 << cols_log) - 1), r = i >> cols_log;
+                float den = 0.f, acc = 0.f;
+#pragma unroll 4
+                for (int k = 0; k < units; ++k) {
+                    const float2 f = ml[r * C::MAX_UNITS + k];
+                    const float b = fb[r * C::MAX_UNITS + k];
+                    den = fmaf(b, f.y, __fmul_rn(den, f.x));
+                    acc = fmaf(b, recv[k * slice + c * col_stride + r], __fmul_rn(acc, f.x));
+                }
+                store_from(O, q_row(r) + c0 + c, acc / den);
+            }
+        }
+    } else {
+        // ---- the tiles one after the other, for the four groups of the CTA ----
+        constexpr int RPP = TOK_THREADS / NC, PASSES = TOK_TILE / RPP;
+        const int my_row = tid / NC, my_chunk = tid % NC;
+        const uint32_t ring = smem_u32(smem);
+        float *lw = reinterpret_cast<float *>(smem + C::S_LW);
+        int32_t rowno[PASSES];
+        float wt = 0.f;
+        auto fetch_entries = [&](int t) {
+#pragma unroll
+            for (int i = 0; i < PASSES; ++i) {
+                const int e = t * TOK_TILE + my_row + i * RPP;
+                rowno[i] = e < n_span ? (int32_t)checked_row(__ldg(ip + e), n, status) : 0;
+            }
+            if (tid < TOK_TILE) wt = t * TOK_TILE + tid < n_span ? __ldg(wp + t * TOK_TILE + tid) : 0.f;
+        };
+        auto fill = [&](int t) {
+            if (t < tiles) {
+                const int stage = t % TOK_STAGES;
+                const uint32_t kd = ring + (uint32_t)(stage * 2 * C::TILE_BYTES), vd = kd + C::TILE_BYTES;
+#pragma unroll
+                for (int i = 0; i < PASSES; ++i) {
+                    const int e = my_row + i * RPP;
+                    const bool live = t * TOK_TILE + e < n_span;
+                    const int64_t at = (int64_t)rowno[i] * D + my_chunk * 8;
+                    cp_async16_zfill(kd + chunk_at<NC>(e, my_chunk), Kp + at, live);
+                    cp_async16_zfill(vd + chunk_at<NC>(e, my_chunk), Vp + at, live);
+                }
+                if (tid < TOK_TILE) lw[stage * TOK_TILE + tid] = log2f(wt);
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int t = 0; t < TOK_STAGES - 1; ++t) {
+            if (t < tiles) fetch_entries(t);
+            fill(t);
+        }
+        if (TOK_STAGES - 1 < tiles) fetch_entries(TOK_STAGES - 1);
+        uint64_t run[MT][NB][2];                                       // pairs of rows
+        float M[NB], den[NB];
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            M[h] = -INFINITY;
+            den[h] = 0.f;
+#pragma unroll
+            for (int j = 0; j < MT; ++j) run[j][h][0] = run[j][h][1] = 0;
+        }
+        int in_unit = 0;
+        for (int t = 0; t < tiles; ++t) {
+            cp_async_wait<TOK_STAGES - 2>();
+            __syncthreads();
+            fill(t + TOK_STAGES - 1);                                  // (into the stage of the tile before)
+            if (t + TOK_STAGES < tiles) fetch_entries(t + TOK_STAGES);
+            const int stage = t % TOK_STAGES;
+            const unsigned char *kt = smem + stage * 2 * C::TILE_BYTES;
+            if (in_unit == 0) u.reset();
+            if (t * TOK_TILE < last) {                                 // (behind what the group sees there is nothing to add)
+                float s[4][4];
+                token_logits<D, NB>(s, qf, smem_u32(kt));
+                token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale);
+                token_values<D, NB>(u, s, kt + C::TILE_BYTES, sp, t * TOK_TILE, lim, aligned, last, n_span);
+            }
+            if (++in_unit == unit_tiles || t + 1 == tiles) {
+                in_unit = 0;
+                u.finish();
+#pragma unroll
+                for (int h = 0; h < NB; ++h) {
+                    float fa, fb, x0, x1;
+                    merge_factors(M[h], u.m[h], M[h], fa, fb);
+                    den[h] = fmaf(fb, u.l[h], __fmul_rn(den[h], fa));
+                    of_columns(fa, x0, x1);
+                    const uint64_t a2 = pack2(x0, x1);
+                    of_columns(fb, x0, x1);
+                    const uint64_t b2 = pack2(x0, x1);
+#pragma unroll
+                    for (int j = 0; j < MT; ++j)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+                            run[j][h][i] = fma2(b2, pack2(u.o[j][h][2 * i], u.o[j][h][2 * i + 1]), mul2(run[j][h][i], a2));
+                }
+            }
+        }
+        cp_async_wait<0>();
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            float den2[2];
+            of_columns(den[h], den2[0], den2[1]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int r = 8 * h + 2 * quad + i;
+                if (r >= rows) continue;
+                __nv_bfloat16 *o = O + q_row(r) + (lane >> 2);
+#pragma unroll
+                for (int j = 0; j < 2 * MT; ++j) {
+                    float x[2];
+                    unpack2(run[j >> 1][h][j & 1], x[0], x[1]);
+                    o[8 * j] = __float2bfloat16_rn(x[i] / den2[i]);
+                }
+            }
+        }
+    }
+}
+
+int tokens_per_group(int per_token)
+{
+    int t = 1;
+    while (2 * t * per_token <= TOK_ROWS) t *= 2;
+    return t;
+}
+template <int D>
+int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
+                  const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st)
+{
+    using C = TokenCfg<D>;
+    const int problems = p->batch * p->kv_heads, per_token = p->q_heads / p->kv_heads;
+    const int sms = device_sm_count();
+    TokenGroups grp = {};
+    grp.cap = cap;
+    grp.per_group = tokens_per_group(per_token);
+    auto count = [&](int span) {
+        grp.span = span;
+        for (int i = 0; i < win.n; ++i) {
+            const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
+            grp.g0[i + 1] = grp.g0[i] + (last - 1) / span - (win.seen0[i] - 1) / span + 1;
+        }
+        return grp.g0[win.n];
+    };
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(TOK_THREADS);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    // The serial form takes as long as one CTA needs for the longest list, about 1.5 us a tile, whatever few tokens there are;
+    // clusters finish one after the other, 0.2 us each for a list of 200 entries and 1.5 for 6144.  Measured, bf16, d = 128, 8 KV heads
+    // of 4 query heads (8 clusters per 4 tokens), clusters against serial: 200 entries 32 tokens 12 / 20 us, 64 tokens 29 / 26;
+    // 2053 entries 32 tokens 82 / 106, 64 tokens 154 / 113; 6144 entries 64 tokens 204 / 303, 128 tokens 390 / 306.
+    int longest = 0;
+    for (int i = 0; i < win.n; ++i) {
+        const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
+        longest = last > longest ? last : longest;
+    }
+    const int64_t clusters = (int64_t)count(grp.per_group) * problems;
+    const bool serial = clusters > 2 * sms / 5 + (longest + TOK_TILE - 1) / TOK_TILE / 2;
+    auto kern = tokens_kernel<D, false, 2>;
+    if (serial) {
+        grp.cluster = 1;
+        cfg.dynamicSmemBytes = C::S_TOTAL;
+        cfg.gridDim = dim3((unsigned)count(TOK_WARPS * grp.per_group), (unsigned)problems);
+    } else {
+        int units = 1, most = 1;
+        for (int i = 0; i < win.n; ++i) {
+            const int tokens = win.tok0[i + 1] - win.tok0[i], last = win.seen0[i] + tokens - 1;
+            const int per_unit = token_units(last, cap), tiles = (last + TOK_TILE - 1) / TOK_TILE;
+            // (a window that grows past a list of `cap` full CTAs: the units are longer from there on, and fewer)
+            const int u = token_units(win.seen0[i], cap) < per_unit ? TOK_WARPS * cap : (tiles + per_unit - 1) / per_unit;
+            units = u > units ? u : units;
+            most = tokens > most ? tokens : most;
+        }
+        grp.cluster = 1;
+        while (grp.cluster * TOK_WARPS < units) grp.cluster *= 2;
+        const bool few = (most < grp.per_group ? most : grp.per_group) * per_token <= 8;
+        kern = few ? tokens_kernel<D, true, 1> : tokens_kernel<D, true, 2>;
+        cfg.dynamicSmemBytes = few ? C::template Cluster<8>::TOTAL : C::template Cluster<16>::TOTAL;
+        if (grp.cluster > 8) ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)grp.cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+        cfg.gridDim = dim3((unsigned)(grp.g0[win.n] * grp.cluster), (unsigned)problems);
+    }
+    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+    typedef __nv_bfloat16 bf;
+    ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const bf *)Q, (const bf *)K, (const bf *)V, idx, w, (int64_t)p->n_kv, list_stride,
+                                    (int)p->q_heads, (int)p->kv_heads, per_token, win, grp, (bf *)O, status));
+    count_launches(1);
+    return cuda_status(cudaGetLastError());
+}
+
+}  // namespace
+
+int tokens_largest_cluster(int d)
+{
+    static std::atomic<int> cached[64][2];                         // (threads that meet here first find the same answer)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    std::atomic<int> &slot = cached[dev][d == 64 ? 0 : 1];
+    int largest = slot.load(std::memory_order_relaxed);
+    if (largest == 0) {
+        largest = d == 64 ? largest_cluster(tokens_kernel<64, true, 2>, TOK_THREADS, TokenCfg<64>::Cluster<16>::TOTAL, TOK_MAX_CLUSTER)
+                          : largest_cluster(tokens_kernel<128, true, 2>, TOK_THREADS, TokenCfg<128>::Cluster<16>::TOTAL, TOK_MAX_CLUSTER);
+        slot.store(largest, std::memory_order_relaxed);
+    }
+    return largest;
+}
+
+int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
+                       const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st)
+{
+    return p->d == 64 ? launch_tokens<64>(Q, K, V, idx, w, list_stride, win, p, O, status, cap, st)
+                      : launch_tokens<128>(Q, K, V, idx, w, list_stride, win, p, O, status, cap, st);
+}
+
+}  // namespace elm

@@ -111,6 +111,36 @@ def test_streamed_tokens_over_long_lists_match_exact_attention(dtype, d, rep, hk
         assert ((got[t].double() - want).abs().amax(-1) / want.abs().amax(-1)).max() <= bound
 
 
+@pytest.mark.parametrize("d,rep,hkv,log2_nout", [(128, 1, 2, 10), (128, 2, 1, 8), (64, 3, 2, 9), (128, 4, 8, 9), (64, 5, 1, 8), (128, 8, 3, 10)])
+@pytest.mark.parametrize("start", [1, 30, 127, 500, 2046])
+def test_bf16_tokens_match_exact_attention(d, rep, hkv, log2_nout, start):
+    """Calls of 1 ... 600 tokens (eight and sixteen query vectors per warp, clusters and CTAs that walk the list) whose lists
+    cross the edges of tiles, groups and units, against exact causal attention in 64 bits; an infinite value reaches
+    the tokens that see it, in its column, as an infinity."""
+    if start + 600 > 4 << log2_nout:
+        start = (4 << log2_nout) - 602                 # (the exact start ends there)
+    x = _Exact(torch.bfloat16, d, rep, hkv, log2_nout, start, 600)
+    K, V = (t.double().repeat_interleave(rep, dim=1) for t in (x.s.K, x.s.V))
+    seen = torch.arange(start + 600, device="cuda")
+    for T in (1, 2, 7, 33, 600):
+        if T > (1 << log2_nout) - start % (1 << log2_nout):
+            continue                                   # (what a call appends must lie behind what a rewound stream reads)
+        got = x.one_call(T).double()
+        s = torch.einsum("tbhqd,bhnd->tbhqn", x.Q[:T].double(), K) / d ** 0.5
+        s = s.masked_fill(seen > start + torch.arange(T, device="cuda")[:, None, None, None, None], -torch.inf)
+        want = torch.einsum("tbhqn,bhnd->tbhqd", torch.softmax(s, dim=-1), V)
+        assert ((got - want).abs().amax(-1) / want.abs().amax(-1)).max() <= 2.0 ** -8          # rounded to 8 bits
+        inf_at = start + T // 2                        # seen by the tokens from T // 2 on
+        keep = x.s.V[:, :, inf_at, 3].clone()
+        x.s.V[:, :, inf_at, 3] = torch.inf
+        after = x.one_call(T).double()
+        x.s.V[:, :, inf_at, 3] = keep
+        assert (after[T // 2:, ..., 3] == torch.inf).all()
+        after[T // 2:, ..., 3] = got[T // 2:, ..., 3]
+        # (sums in another order: neighbouring values of 8 bits are up to 2^-7 of the larger apart)
+        assert ((after - got).abs() <= 2.0 ** -7 * got.abs().amax(-1, keepdim=True)).all()
+
+
 def test_debug_limit_of_clusters_refuses_other_sizes():
     lib = binding.load_library()
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
