@@ -54,6 +54,12 @@ constexpr int STAGES = 2;
 constexpr int NTHREADS = 608;          // 16 softmax warps + TMA producer + two MMA issuers (one per query tile)
 constexpr int TMA_WARP = 16, MMA_WARP = 17;
 constexpr uint32_t TMEM_COLS = 512;
+// What bounds it: per block and tile the chain softmax (1600 cycles), hand-over, O += P V (610), S = Q K^T (650), hand-over: 3600 cycles, of which
+// the pipe works 2800 for the two tiles (2048 at its nominal rate: Q K^T reads both operands from shared memory), and 2900
+// cycles per item around it.  32 heads x 131072 queries x 2048 points: 6.95 -> 6.66 million cycles per launch, 32768 x 1024: 0.945 ->
+// 0.857, 64 heads x 8192 x 256: 0.190 -> 0.140 (535 -> 490 us, 106 -> 80 us; the longest at the power cap, where fewer cycles
+// lower the clock: 4.20 -> 4.07 ms) with the stores of an item's rows coalesced (store_rows), its queries reloaded tile by tile and
+// the tiles' MMAs in turn (below).
 constexpr float RESCALE_TAU = 8.0f;      // rescale the accumulator only if the max grew by > 2^8
 // Of every 16 column pairs, how many take 2^x from the FMA pipe (a cubic for 2^f, relative error 1e-4 - below the
 // bf16 rounding of the probabilities) instead of the special-function unit.  Launches with a mask only: there all
@@ -67,9 +73,10 @@ constexpr int EMU_PAIRS = 4;
 using namespace sm100;
 
 struct __align__(8) Barriers {
-    uint64_t q_full, q_free;
-    uint64_t k_full[STAGES], v_full[STAGES], kv_free[STAGES];
+    uint64_t q_full[2], q_free[2];
+    uint64_t k_full[STAGES], v_full[STAGES], k_free[STAGES], v_free[STAGES];
     uint64_t s_full[2], p_ready[2], o_done[2], o_free[2];
+    uint64_t turn[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
     float xchg[2][4][BM];        // per tile, per column quarter: row maxima / denominators being exchanged
@@ -348,6 +355,42 @@ __device__ __forceinline__ float exp_pass_keep(uint32_t tP, float scale_log2, fl
     return s_lo + s_hi;
 }
 
+// Writes a warp's 32 rows of 8 NC finished columns (a row per lane, `inv` its normalisation) to rows of D at dst, of which `rows`
+// exist.  A lane that stored its own row would send every 16 bytes of a store instruction to a line of its own: 256
+// passes of the load/store unit per warp and item, 3000 cycles of an item in which the exchanges and barriers of the other
+// tile's warps queued behind them.  So NC neighbouring lanes first exchange their 16-byte chunks (a transposition in registers,
+// log2 NC steps), after which each of their stores covers 16 NC contiguous bytes.
+template <int D, int NC>
+__device__ __forceinline__ void store_rows(const uint32_t (&o)[32], float inv, __nv_bfloat16 *dst, int64_t rows)
+{
+    const int lane = threadIdx.x & 31, a = lane & (NC - 1);
+    uint32_t v[NC][4];
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            v[c][i] = pack_bf16x2(__uint_as_float(o[8 * c + 2 * i]) * inv, __uint_as_float(o[8 * c + 2 * i + 1]) * inv);
+#pragma unroll
+    for (int s = 1; s < NC; s *= 2) {
+        const bool up = (a & s) != 0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (c & s) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? v[c][i] : v[c + s][i], s);
+                v[c][i] = up ? got : v[c][i];
+                v[c + s][i] = up ? v[c + s][i] : got;
+            }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NC; ++b) {
+        const int r = lane - a + b;                                // chunk a of the row of lane r
+        if (r < rows) *reinterpret_cast<uint4 *>(dst + (int64_t)r * D + 8 * a) = make_uint4(v[b][0], v[b][1], v[b][2], v[b][3]);
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // TMA producer of a launch with block lists (one thread): the queries of each pair, and the K / V^T / bias blocks
 // of each pair's own list through the 2-stage ring.  Same protocol as the producer inside the kernel; kept out of
@@ -399,12 +442,16 @@ __device__ __noinline__ bool produce_block_lists(const ProducerArgs *a)
         if (++c.j == c.nb) { c.j = 0; ++c.k; enter(c, want_bias); }
         else fetch_blk(c);
     };
-    auto load_q = [&](int id) {
+    auto load_q = [&](int id, int t) {
         const int bh = id / tiles_x, q0 = (id % tiles_x) * (2 * BM);
-        mbar_expect_tx(&bar->q_full, 2 * SM::Q_TILE);
+        mbar_expect_tx(&bar->q_full[t], SM::Q_TILE);
+        for (int kh = 0; kh < KH; ++kh)
+            tma_load_3d(smem + SM::OFF_Q + t * SM::Q_TILE + kh * (BM * 128), a->mapQ, &bar->q_full[t], kh * ROW_ELTS, a->q_row0 + q0 + t * BM, bh);
+    };
+    auto prefetch_q = [&](int id) {
+        const int bh = id / tiles_x, q0 = (id % tiles_x) * (2 * BM);
         for (int t = 0; t < 2; ++t)
-            for (int kh = 0; kh < KH; ++kh)
-                tma_load_3d(smem + SM::OFF_Q + t * SM::Q_TILE + kh * (BM * 128), a->mapQ, &bar->q_full, kh * ROW_ELTS, a->q_row0 + q0 + t * BM, bh);
+            for (int kh = 0; kh < KH; ++kh) tma_prefetch_3d(a->mapQ, kh * ROW_ELTS, a->q_row0 + q0 + t * BM, bh);
     };
     int total = 0;
     if (a->tile_cnt)
@@ -430,36 +477,33 @@ __device__ __noinline__ bool produce_block_lists(const ProducerArgs *a)
         cursor_next(vc, false);
     };
     bool ok = true;
-    // The queries of item k may replace those of item k - 1 once every S = Q K^T of item k - 1 has been computed
-    // (q_free); they are fetched right after the keys of the item's first block (the key cursor then stands
-    // behind that block).
+    // A tile's queries of item k may replace those of item k - 1 once every S = Q K^T of the tile in item k - 1 has been
+    // computed (q_free); they are fetched right after the keys of the item's first block (the key cursor then stands
+    // behind that block), from L2, where they were sent for when item k - 1 began.
     int next_q = 1;
     auto feed_q = [&]() {
         while (ok && next_q < n_items && (kc.k > next_q || (kc.k == next_q && kc.j > 0))) {
-            ok = sm100::mbar_wait(&bar->q_free, (uint32_t)(next_q - 1) & 1u, limit);
-            if (ok) load_q(item_id(next_q));
+            for (int t = 0; t < 2 && ok; ++t) {
+                ok = sm100::mbar_wait(&bar->q_free[t], (uint32_t)(next_q - 1) & 1u, limit);
+                if (ok) load_q(item_id(next_q), t);
+            }
             ++next_q;
+            if (ok && next_q < n_items) prefetch_q(item_id(next_q));
         }
     };
-    if (n_items > 0) load_q(item_id(0));
-    // The issuer commits "event" i to kv_free[i % 2] after the prologue (i = 0: S = Q K^T of block 0 issued) and
-    // after iteration i - 1 (O += P V of block i - 1 and S = Q K^T of block i issued).  Once event i is complete,
-    // K's stage i % 2 (block i) and V's stage (i + 1) % 2 (block i - 1) have been read, so K(i + 2) and V(i + 1)
-    // may overwrite them.
+    if (n_items > 0) { load_q(item_id(0), 0); load_q(item_id(0), 1); }
+    // A stage is free once both tiles' MMAs have read it: K's when S = Q K^T of its block is complete, V's with the S = Q K^T
+    // that was issued behind its O += P V.
     for (int G = 0; G < STAGES && G < total; ++G) { load_k(G); load_v(G); }
+    if (n_items > 1) prefetch_q(item_id(1));
     feed_q();
-    for (int i = 0; i + 2 < total && ok; ++i) {
-        ok = sm100::mbar_wait(&bar->kv_free[i % STAGES], (uint32_t)(i / STAGES) & 1u, limit);
+    for (int i = 0; i + STAGES < total && ok; ++i) {
+        ok = sm100::mbar_wait(&bar->k_free[i % STAGES], (uint32_t)(i / STAGES) & 1u, limit);
         if (!ok) break;
-        load_k(i + 2);
-        if (i >= 1) load_v(i + 1);
+        load_k(i + STAGES);
         feed_q();
-    }
-    // the last V block: freed by event total - 1
-    if (ok && total > STAGES) {
-        const int i = total - 2;
-        ok = sm100::mbar_wait(&bar->kv_free[i % STAGES], (uint32_t)(i / STAGES) & 1u, limit);
-        if (ok) load_v(i + 1);
+        ok = ok && sm100::mbar_wait(&bar->v_free[i % STAGES], (uint32_t)(i / STAGES) & 1u, limit);
+        if (ok) load_v(i + STAGES);
     }
     return ok;
 }
@@ -542,14 +586,16 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     if (*reinterpret_cast<volatile int *>(status) != 0) return;
 
     if (threadIdx.x == 0) {
-        mbar_init(&bar->q_full, 1);
-        mbar_init(&bar->q_free, 2);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&bar->k_full[s], 1);
             mbar_init(&bar->v_full[s], 1);
-            mbar_init(&bar->kv_free[s], 2);
+            mbar_init(&bar->k_free[s], 2);
+            mbar_init(&bar->v_free[s], 2);
         }
         for (int t = 0; t < 2; ++t) {
+            mbar_init(&bar->q_full[t], 1);
+            mbar_init(&bar->q_free[t], 1);
+            mbar_init(&bar->turn[t], 1);
             mbar_init(&bar->s_full[t], 1);
             // (extra_arrivals is 0 except in the test that lets a wait run out: arrivals that nobody makes)
             mbar_init(&bar->p_ready[t], (MASKED ? 512 : 256) + extra_arrivals);
@@ -573,12 +619,16 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     if (warp == TMA_WARP) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            auto load_q = [&](int k) {
+            auto load_q = [&](int k, int t) {
                 const int bh = item_bh(k), q0 = item_q0(k);
-                mbar_expect_tx(&bar->q_full, 2 * SM::Q_TILE);
+                mbar_expect_tx(&bar->q_full[t], SM::Q_TILE);
+                for (int kh = 0; kh < KH; ++kh)
+                    tma_load_3d(smem + SM::OFF_Q + t * SM::Q_TILE + kh * (BM * 128), &mapQ, &bar->q_full[t], kh * ROW_ELTS, q_row0 + q0 + t * BM, bh);
+            };
+            auto prefetch_q = [&](int k) {
+                const int bh = item_bh(k), q0 = item_q0(k);
                 for (int t = 0; t < 2; ++t)
-                    for (int kh = 0; kh < KH; ++kh)
-                        tma_load_3d(smem + SM::OFF_Q + t * SM::Q_TILE + kh * (BM * 128), &mapQ, &bar->q_full, kh * ROW_ELTS, q_row0 + q0 + t * BM, bh);
+                    for (int kh = 0; kh < KH; ++kh) tma_prefetch_3d(&mapQ, kh * ROW_ELTS, q_row0 + q0 + t * BM, bh);
             };
             bool ok = true;
             if (!MASKED || !tile_cnt) {
@@ -607,36 +657,36 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     for (int hh = 0; hh < 2; ++hh)
                         tma_load_3d(smem + SM::OFF_V + s * SM::V_BLOCK + hh * (D * 128), &mapV, &bar->v_full[s], hh * 64, 0, prob * nblk + G % nblk);
                 };
-                // The queries of item k may replace those of item k - 1 once every S = Q K^T of item k - 1
-                // has been computed (q_free); they are fetched right after the keys of the item's first block.
+                // A tile's queries of item k may replace those of item k - 1 once every S = Q K^T of the tile in
+                // item k - 1 has been computed (q_free); they are fetched right after the keys of the item's first
+                // block, from L2: all CTAs come to the ends of their items at about the same time, so the queries are
+                // sent for when item k - 1 begins.
                 int next_q = 1, k_loaded = -1;
                 auto feed_q = [&]() {
                     while (ok && next_q < n_items && next_q * nblk <= k_loaded) {
-                        ok = mbar_wait(&bar->q_free, (uint32_t)(next_q - 1) & 1u);
-                        if (ok) load_q(next_q);
+                        for (int t = 0; t < 2 && ok; ++t) {
+                            ok = mbar_wait(&bar->q_free[t], (uint32_t)(next_q - 1) & 1u);
+                            if (ok) load_q(next_q, t);
+                        }
                         ++next_q;
+                        if (ok && next_q < n_items) prefetch_q(next_q);
                     }
                 };
-                load_q(0);
-                // The issuer commits "event" i to kv_free[i % 2] after the prologue (i = 0: S = Q K^T of block
-                // 0 issued) and after iteration i - 1 (O += P V of block i - 1 and S = Q K^T of block i issued).
-                // Once event i is complete, K's stage i % 2 (block i) and V's stage (i + 1) % 2 (block i - 1)
-                // have been read, so K(i + 2) and V(i + 1) may overwrite them.
+                load_q(0, 0);
+                load_q(0, 1);
+                // A stage is free once both tiles' MMAs have read it: K's when S = Q K^T of its block is complete, V's
+                // with the S = Q K^T that was issued behind its O += P V.
                 for (int G = 0; G < STAGES && G < total; ++G) { load_k(G); load_v(G); k_loaded = G; }
+                if (n_items > 1) prefetch_q(1);
                 feed_q();
-                for (int i = 0; i + 2 < total && ok; ++i) {
-                    ok = mbar_wait(&bar->kv_free[i % STAGES], (uint32_t)(i / STAGES) & 1u);
+                for (int i = 0; i + STAGES < total && ok; ++i) {
+                    ok = mbar_wait(&bar->k_free[i % STAGES], (uint32_t)(i / STAGES) & 1u);
                     if (!ok) break;
-                    load_k(i + 2);
-                    k_loaded = i + 2;
-                    if (i >= 1) load_v(i + 1);
+                    load_k(i + STAGES);
+                    k_loaded = i + STAGES;
                     feed_q();
-                }
-                // the last V block: freed by event total - 1
-                if (ok && total > STAGES) {
-                    const int i = total - 2;
-                    ok = mbar_wait(&bar->kv_free[i % STAGES], (uint32_t)(i / STAGES) & 1u);
-                    if (ok) load_v(i + 1);
+                    ok = ok && mbar_wait(&bar->v_free[i % STAGES], (uint32_t)(i / STAGES) & 1u);
+                    if (ok) load_v(i + STAGES);
                 }
             } else {
                 // (launch with block lists: the producer that walks them is a function of its own, not inlined - the
@@ -697,14 +747,14 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             };
             const int total = count_blocks();
             int nb = n_items > 0 ? item_nblk(0) : 0;                           // blocks of item k
-            bool ok = mbar_wait(&bar->q_full, 0) && mbar_wait(&bar->k_full[0], 0);
+            bool ok = mbar_wait(&bar->q_full[t], 0) && mbar_wait(&bar->k_full[0], 0);
             if (ok) {
                 tc_fence_after();
                 const bool b0 = item_bias(0);
                 issue_qk(t, 0, b0);
                 tc_commit(&bar->s_full[t]);
-                if (nb == 1) tc_commit(&bar->q_free);                          // item 0 needs its queries no more
-                tc_commit(&bar->kv_free[0]);                                   // event 0
+                if (nb == 1) tc_commit(&bar->q_free[t]);                       // item 0 needs its queries no more
+                tc_commit(&bar->k_free[0]);
             }
             // Iteration G: O += P V of block G, then S = Q K^T of block G + 1 - which may be the first
             // block of the next item: the tensor pipe runs on while the softmax warps finish an item.
@@ -724,6 +774,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 if (last) bias_next = bias_after;
                 if (more) ok = mbar_wait(&bar->k_full[sn], (uint32_t)((G + 1) / STAGES) & 1u);
                 ok = ok && mbar_wait(&bar->v_full[s], (uint32_t)(G / STAGES) & 1u);
+                // The tiles' MMAs take turns (without a mask, where a softmax group serves each tile).  Left to themselves the
+                // two issuers interleave: both tiles' logits are then ready at the same time, their exponentials share the
+                // special-function unit, and both tiles wait for the tensor pipe again - 5100 cycles per block, a state the
+                // kernel falls into once nothing else sets the tiles apart; one after the other 3600.
+                if (!MASKED && ok && (t == 1 || G > 0)) ok = mbar_wait(&bar->turn[t], (uint32_t)(t == 1 ? G : G - 1) & 1u);
                 ok = ok && mbar_wait(&bar->p_ready[t], (uint32_t)G & 1u);
                 // a new item overwrites the accumulator: the epilogue of the previous one must have read it
                 if (ok && j == 0 && k > 0) ok = mbar_wait(&bar->o_free[t], (uint32_t)(k - 1) & 1u);
@@ -735,16 +790,18 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 if (last) tc_commit(&bar->o_done[t]);
                 if (more) {
                     // the next item's queries are needed only now, after this item's last O += P V went out
-                    if (last) ok = mbar_wait(&bar->q_full, (uint32_t)(k + 1) & 1u);
+                    if (last) ok = mbar_wait(&bar->q_full[t], (uint32_t)(k + 1) & 1u);
                     if (!ok) break;
                     issue_qk(t, sn, bias_next);
                     tc_commit(&bar->s_full[t]);
                 }
                 if (!ok) break;
+                if (!MASKED) mbar_arrive(&bar->turn[t ^ 1]);
+                tc_commit(&bar->v_free[s]);
                 // the logits just issued belong to block j + 1 of item k, or to block 0 of item k + 1
                 const int jn = last ? 0 : j + 1;
-                if (more && jn == (last ? nb_after : nb) - 1) tc_commit(&bar->q_free);
-                tc_commit(&bar->kv_free[(G + 1) % STAGES]);                    // event G + 1
+                if (more && jn == (last ? nb_after : nb) - 1) tc_commit(&bar->q_free[t]);
+                if (more) tc_commit(&bar->k_free[sn]);
                 j = jn;
                 if (last) { ++k; nb = nb_after; }
             }
@@ -856,7 +913,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             const float inv = 1.f / l_all;
             const int64_t qrow = (int64_t)q0 + t * BM + row;
             if (lse && ch == 0 && qrow < n_q) lse[(int64_t)bh * n_q_total + q_row0 + qrow] = m_ref + log2f(l_all);
-            __nv_bfloat16 *dst = O + ((int64_t)bh * n_q_total + q_row0 + qrow) * D + ch * (D / 2);
+            const int64_t warp_row = qrow - lane;
+            __nv_bfloat16 *dst = O + ((int64_t)bh * n_q_total + q_row0 + warp_row) * D + ch * (D / 2);
 #pragma unroll 1
             for (int c0 = 0; c0 < D / 2; c0 += 32) {
                 uint32_t o[32];
@@ -868,17 +926,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bar->o_free[t]);
                 }
-                if (qrow < n_q) {
-#pragma unroll
-                    for (int c = 0; c < 32; c += 8) {
-                        uint4 v;
-                        v.x = pack_bf16x2(__uint_as_float(o[c]) * inv, __uint_as_float(o[c + 1]) * inv);
-                        v.y = pack_bf16x2(__uint_as_float(o[c + 2]) * inv, __uint_as_float(o[c + 3]) * inv);
-                        v.z = pack_bf16x2(__uint_as_float(o[c + 4]) * inv, __uint_as_float(o[c + 5]) * inv);
-                        v.w = pack_bf16x2(__uint_as_float(o[c + 6]) * inv, __uint_as_float(o[c + 7]) * inv);
-                        *reinterpret_cast<uint4 *>(dst + c0 + c) = v;
-                    }
-                }
+                store_rows<D, 4>(o, inv, dst + c0, n_q - warp_row);
             }
         }
         if (!ok && lane == 0) atomicExch(status, 3);
@@ -1026,7 +1074,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 const float inv = 1.f / l_all;
                 const int64_t qrow = (int64_t)q0 + t * BM + row;
                 if (lse && cq == 0 && qrow < n_q) lse[(int64_t)bh * n_q_total + q_row0 + qrow] = m_ref[t] + log2f(l_all);
-                __nv_bfloat16 *dst = O + ((int64_t)bh * n_q_total + q_row0 + qrow) * D + cq * (D / 4);
                 uint32_t o[32];
                 if (D == 128) tmem_ld32(tO, o);
                 else tmem_ld16(tO, o);
@@ -1035,17 +1082,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bar->o_free[t]);
-                if (qrow < n_q) {
-#pragma unroll
-                    for (int c = 0; c < D / 4; c += 8) {
-                        uint4 v;
-                        v.x = pack_bf16x2(__uint_as_float(o[c]) * inv, __uint_as_float(o[c + 1]) * inv);
-                        v.y = pack_bf16x2(__uint_as_float(o[c + 2]) * inv, __uint_as_float(o[c + 3]) * inv);
-                        v.z = pack_bf16x2(__uint_as_float(o[c + 4]) * inv, __uint_as_float(o[c + 5]) * inv);
-                        v.w = pack_bf16x2(__uint_as_float(o[c + 6]) * inv, __uint_as_float(o[c + 7]) * inv);
-                        *reinterpret_cast<uint4 *>(dst + c) = v;
-                    }
-                }
+                const int64_t warp_row = qrow - lane;
+                store_rows<D, D / 32>(o, inv, O + ((int64_t)bh * n_q_total + q_row0 + warp_row) * D + cq * (D / 4), n_q - warp_row);
             }
         }
         if (!ok && lane == 0) atomicExch(status, 3);
