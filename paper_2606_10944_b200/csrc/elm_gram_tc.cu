@@ -253,6 +253,11 @@ gram_walk_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__res
 //               (K K^T | V V^T, 256 columns each); its commits free the operand buffers
 //   warps 5-12  epilogue of the previous tile (exp2, product, pair combination, stores) while the
 //               next tile is gathered and multiplied
+// Bound by the gathers: 128 KB per tile off the diagonal at about 64 bytes per cycle into an SM, and the row numbers
+// that queue behind them; about 3500 cycles per tile, of which the MMAs take 1400.  32 problems, d = 128, 128-KB tiles of calls of
+// 1024 pairs 67.5 -> 63.2 us per level, of calls of 64 pairs (64 KB from HBM) 128 -> 126, 128 pairs 94 -> 89, 256 pairs 78 -> 71:
+// descriptors by adding to one of them (the MMAs' issue took 1175 cycles per operand, now 700), row numbers of the next tile fetched
+// behind this tile's copies, pair rows stored as 128 contiguous bytes.
 // ---------------------------------------------------------------------------------------------
 constexpr int PNS = 3;                       // operand ring depth (jobs)
 constexpr int PLOAD = 4;                      // loader warps (8 were slower: 0.76 against 0.71 ms per cfg5 step)
@@ -336,23 +341,30 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
 
     if (warp < PLOAD) {
         // ------------------------------ loaders ------------------------------
-        int job = 0, lk = 0;
-        for (int it = blockIdx.x; it < total_items && ok; it += gridDim.x, ++lk) {
-            int p;
+        // chunk q = tid + NL i of a 128-row tile lies in row tid / CHUNKS + (NL / CHUNKS) i, NL loader threads
+        constexpr int NL = PLOAD * 32;
+        constexpr int RPT = TR * CHUNKS / NL;                // chunks (= distinct rows) per thread and tile
+        int32_t ra[RPT], rb[RPT];
+        int p_next = 0;
+        bool diagonal_next = false;
+        // row numbers of item k: fetched while the copies of the item before are on their way
+        auto fetch_rows = [&](int k, int it) {
             int64_t JR, JC;
-            item(lk, it, p, JR, JC);
-            const bool diagonal = JR == JC;
-            const int32_t *curp = cur + (int64_t)p * n;
-            // chunk q = tid + NL i of a 128-row tile lies in row tid / CHUNKS + (NL / CHUNKS) i, NL loader threads
-            constexpr int NL = PLOAD * 32;
-            constexpr int RPT = TR * CHUNKS / NL;            // chunks (= distinct rows) per thread and tile
-            int32_t ra[RPT], rb[RPT];
+            item(k, it, p_next, JR, JC);
+            diagonal_next = JR == JC;
+            const int32_t *curp = cur + (int64_t)p_next * n;
 #pragma unroll
             for (int i = 0; i < RPT; ++i) {
                 const int r = tid / CHUNKS + (NL / CHUNKS) * i;
                 ra[i] = __ldg(curp + 2 * JR + r);
-                rb[i] = diagonal ? 0 : __ldg(curp + 2 * JC + r);
+                rb[i] = diagonal_next ? 0 : __ldg(curp + 2 * JC + r);
             }
+        };
+        int job = 0, lk = 0;
+        if ((int)blockIdx.x < total_items) fetch_rows(0, blockIdx.x);
+        for (int it = blockIdx.x; it < total_items && ok; it += gridDim.x, ++lk) {
+            const int p = p_next;
+            const bool diagonal = diagonal_next;
             const int ch = tid % CHUNKS, kh = ch >> 3, c = ch & 7;
             for (int op = 0; op < 2 && ok; ++op, ++job) {     // 0: keys, 1: values
                 const int b = job % PNS;
@@ -371,6 +383,7 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
                 // the job's barrier completes when every loader thread's copies have landed
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&bar->full[b])) : "memory");
             }
+            if (it + (int)gridDim.x < total_items) fetch_rows(lk + 1, it + gridDim.x);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (!ok && lane == 0) atomicExch(status, 5);
@@ -378,6 +391,11 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
             constexpr uint32_t IDESC = umma_idesc_bf16(TR, TR);
+            // descriptors differ only in the start address (address / 16, in their low word): a lone thread that builds each
+            // from its address issues a tile's sixteen MMAs at half the tensor pipe's rate
+            const uint64_t d0 = umma_desc_k128(smem_u32(smem));
+            const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
+            auto desc = [&](uint32_t lo) { uint64_t d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(d_hi)); return d; };
             int job = 0, k = 0;
             for (int it = blockIdx.x; it < total_items && ok; it += gridDim.x, ++k) {
                 int p;
@@ -394,13 +412,13 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
                     if (!ok) break;
                     fence_proxy_async();                       // the gathered bytes were written by generic-proxy copies
                     tc_fence_after();
-                    const uint32_t sA = smem_u32(smem + b * SM::JOB), sB = diagonal ? sA : sA + TR * D * 2;
+                    const uint32_t dA = d_lo + b * (SM::JOB >> 4), dB = diagonal ? dA : dA + (TR * D * 2 >> 4);
 #pragma unroll
                     for (int kh = 0; kh < KH; ++kh)
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_ss(tmem + slot * 256 + op * 128, umma_desc_k128(sA + kh * (TR * 128) + ks * 32),
-                                   umma_desc_k128(sB + kh * (TR * 128) + ks * 32), IDESC, (kh | ks) != 0);
+                            mma_ss(tmem + slot * 256 + op * 128, desc(dA + ((kh * (TR * 128) + ks * 32) >> 4)),
+                                   desc(dB + ((kh * (TR * 128) + ks * 32) >> 4)), IDESC, (kh | ks) != 0);
                     tc_commit(&bar->empty[b]);
                 }
                 if (ok) tc_commit(&bar->accfull[slot]);
@@ -466,16 +484,30 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
                 const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
                 f[i] = odd ? recv - h[i + 16] : h[i] - recv;
             }
-            const int64_t jr = JR + (r >> 1);
-            const int64_t jc0 = JC + ch * 32 + (odd ? 16 : 0);
-            const int64_t gr = jr / P;
-            float *Fp = F + (int64_t)p * F_stride + jr * P - gr * P;
-            // 64 contiguous bytes per thread.  On a diagonal tile half of them lie below the diagonal of the
-            // call's P x P block, which nothing reads: written all the same, four vector stores being
-            // cheaper than sixteen predicated ones.
+            // A lane pair holds a pair row's 32 columns, 64 bytes each: stored as they are, every 16 bytes of a store instruction
+            // would go to a place of their own.  Four lane pairs exchange 16-byte chunks (lane bits 2 and 1 against chunk
+            // bits 1 and 0), after which eight lanes hold one pair row per store: 128 contiguous bytes.  On a diagonal tile
+            // half of them lie below the diagonal of the call's P x P block, which nothing reads.
 #pragma unroll
-            for (int i = 0; i < 16; i += 4)
-                *reinterpret_cast<float4 *>(Fp + jc0 + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+            for (int s = 1; s <= 2; s *= 2) {
+                const bool up = (lane & (2 * s)) != 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (c & s) continue;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float got = __shfl_xor_sync(0xffffffffu, up ? f[4 * c + i] : f[4 * (c + s) + i], 2 * s);
+                        f[4 * c + i] = up ? got : f[4 * c + i];
+                        f[4 * (c + s) + i] = up ? f[4 * (c + s) + i] : got;
+                    }
+                }
+            }
+            const int64_t jr0 = JR + (q4 * 32 + (lane & ~7)) / 2;           // the first of the four pair rows
+            const int64_t gr = jr0 / P;                                     // (calls begin at multiples of 64 pairs)
+            float *Fp = F + (int64_t)p * F_stride + (jr0 - gr) * P + JC + ch * 32 + (odd ? 16 : 0) + 4 * ((lane >> 1) & 3);
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                *reinterpret_cast<float4 *>(Fp + (int64_t)b * P) = make_float4(f[4 * b], f[4 * b + 1], f[4 * b + 2], f[4 * b + 3]);
         }
         if (!ok && lane == 0) atomicExch(status, 7);
     }
