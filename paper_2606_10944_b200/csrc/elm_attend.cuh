@@ -85,7 +85,7 @@ int attend_decode(const void *Q, const void *K, const void *V, const int32_t *id
 // the launch (tok0[0] = 0); its list starts at entry off[i] of every problem's row of idx / w (row stride
 // list_stride), and its j-th token sees the first seen0[i] + j entries.  Q and O are [tokens][batch][q_heads][1][d].
 // Applies when the longest list a token sees has n_core entries and attend_decode_windows_apply says so.  A token's
-// output is the same bit for bit whatever other tokens share its launch (attend_decode parts a list differently and
+// output is the same bit for bit whatever other tokens share its launch (attend_decode may part a list differently and
 // agrees to rounding).
 constexpr int DECODE_MAX_WINDOWS = 32;
 struct DecodeWindows {
@@ -96,10 +96,20 @@ bool attend_decode_windows_apply(const elm_params *p, int n_core);
 int attend_decode_windows(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
                           const DecodeWindows &win, const elm_params *p, void *O, int *status, cudaStream_t st);
 
-// Its launch for bf16 storage (elm_attend_tokens.cu): lists spread over at most `cap` CTAs, a power of two no larger than
-// tokens_largest_cluster(d), the largest cluster the current device can place.
+// Its launch for bf16 storage (elm_attend_tokens.cu).  Lists of up to TOKENS_SHORT_LIST entries are spread over at most `of_short`
+// CTAs, longer ones over `of_long`: powers of two that tokens_caps chose for the device and the number of problems.
+constexpr int TOKENS_SHORT_LIST = 4096;
+struct TokenCaps {
+    int32_t of_short, of_long;
+};
+TokenCaps tokens_caps(int d, int problems, int limit /* largest cluster to use */);
 int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
-                       const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st);
-int tokens_largest_cluster(int d);
+                       const DecodeWindows &win, const elm_params *p, void *O, int *status, TokenCaps caps, cudaStream_t st);
+
+// The first launch of elm_attend's split form on bf16 storage with the matrix instructions: every problem's list over `splits`
+// CTAs, which leave part[problem][split][G][d + 2] for attend_decode's merge; up to 8 query vectors, n_q rows of every head.
+int launch_tokens_split(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int n_core, int splits, int G,
+                        const elm_params *p, float *part, int *status, cudaStream_t st);
+cudaError_t tokens_split_occupancy(int d, int *ctas_per_sm);
 
 }  // namespace elm

@@ -594,26 +594,27 @@ template <typename F> auto with_groups(int groups, F f)
 }
 
 // The largest cluster (a power of two, at most DEC_MAX_CLUSTER) of which the current device can hold one, asked once per
-// device: more than 8 CTAs need the opt-in and a GPC with that many SMs to give, which a partition of a GPU may not have.
+// device.
 std::atomic<int> g_debug_largest_cluster{0};
-template <typename Tin, int D> int decode_largest_cluster()
+template <int D> int decode_largest_cluster()
 {
-    int largest;
-    if constexpr (std::is_same<Tin, __nv_bfloat16>::value) {
-        largest = tokens_largest_cluster(D);
-    } else {
-        static std::atomic<int> cached[64];                        // (threads that meet here first find the same answer)
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-        largest = cached[dev].load(std::memory_order_relaxed);
-        if (largest == 0) {
-            largest = largest_cluster(decode_kernel<Tin, D, DEC_GSTREAM, DEC_CLUSTER>, DEC_WARPS * 32,
-                                      DecodeCfg<Tin, D, DEC_GSTREAM>::template total<DEC_CLUSTER>(), DEC_MAX_CLUSTER);
-            cached[dev].store(largest, std::memory_order_relaxed);
-        }
+    static std::atomic<int> cached[64];                            // (threads that meet here first find the same answer)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    int largest = cached[dev].load(std::memory_order_relaxed);
+    if (largest == 0) {
+        using C = DecodeCfg<float, D, DEC_GSTREAM>;
+        for (largest = DEC_MAX_CLUSTER; largest > 1; largest >>= 1)
+            if (resident_clusters(decode_kernel<float, D, DEC_GSTREAM, DEC_CLUSTER>, DEC_WARPS * 32, C::template total<DEC_CLUSTER>(), largest)) break;
+        cached[dev].store(largest, std::memory_order_relaxed);
     }
     const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
     return limit && limit < largest ? limit : largest;
+}
+TokenCaps decode_token_caps(const elm_params *p)
+{
+    const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
+    return tokens_caps(p->d, p->batch * p->kv_heads, limit ? limit : DEC_MAX_CLUSTER);
 }
 
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
@@ -622,20 +623,23 @@ template <typename Tin, int D> int decode_largest_cluster()
 // device a single token gains from about 6000 entries on (8 KV heads of 4 query heads, bf16: 6144 entries 16.4 us in
 // clusters, 14.2 split; 12288 entries 25.2 and 18.6), but the tokens of a call can then no longer share a launch (64 tokens over
 // 12288 entries: 606 us together, 1190 one by one).
-template <typename Tin, int D> int decode_cap(int problems, int per_token, int sms)
+template <int D> int decode_cap(int problems, int per_token, int sms)
 {
-    // (bf16: all query vectors of a token go together, two CTAs to an SM)
-    const int most = std::is_same<Tin, __nv_bfloat16>::value ? 2 * sms / problems
-                                                             : DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
-    int cap = decode_largest_cluster<Tin, D>();
+    const int most = DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
+    int cap = decode_largest_cluster<D>();
     while (cap > 1 && cap > most) cap >>= 1;
     return cap;
 }
-template <typename Tin, int D> bool decode_clustered(int n_core, int problems, int per_token)
+bool decode_clustered(int n_core, int problems, int cap, int entries)
 {
-    const int sms = device_sm_count(), cap = decode_cap<Tin, D>(problems, per_token, sms), entries = DEC_WARPS * DEC_TILE<Tin, D>;
-    return n_core <= 8 * entries * cap || problems * cap >= sms;
+    return n_core <= 8 * entries * cap || problems * cap >= device_sm_count();
 }
+
+// The split form of three query vectors and more on bf16 storage is a contraction for the matrix instructions (tokens_split_kernel,
+// elm_attend_tokens.cu): 4 vectors, 8 problems of 2048 entries 8.4 -> 6.9 us, 32 of 5193 25.5 -> 22.1 us; 8 vectors 12.2 -> 7.6 and
+// 41.6 -> 24.2 us; d = 64 alike.  One or two vectors would pay for eight (they are within 10 % of it from 64 problems on).
+template <typename Tin, int G> constexpr bool DECODE_MMA = std::is_same<Tin, __nv_bfloat16>::value && G >= 4;
+template <typename Tin, int G> constexpr bool DECODE_SHORT = !DECODE_MMA<Tin, G> || G < 8;
 
 // How elm_attend's list is split: CTAs per problem, and whether their warps take short tiles.
 struct DecodeSplits {
@@ -644,27 +648,29 @@ struct DecodeSplits {
 };
 template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int problems, size_t part_room)
 {
-    using C = DecodeCfg<Tin, D, G>;
     const int sms = device_sm_count();
     auto ctas = [](int entries, int tile) { return (entries + DEC_WARPS * tile - 1) / (DEC_WARPS * tile); };
     // A tile is a serial chain (rows, dot products, softmax, values), and a call with few of them is as long as that chain:
     // lists of up to 512 entries take tiles of 8 while that makes no more than two CTAs per SM, or two per problem.
     // 8 problems of 4 query vectors, bf16, d = 128: 32 entries 7.4 -> 5.9 us, 512 entries 7.8 -> 6.5 us, but 1024 entries
     // 7.7 -> 8.0 us; 64 problems: 128 entries 8.0 -> 7.1 us, 200 entries 7.9 -> 8.9 us.
+    // (Eight vectors on bf16 storage go to the matrix instructions whatever the length: 8 problems
+    // of 130 entries 9.1 -> 6.6 us.)
     const int few = ctas(n_core, DEC_SHORT_TILE);
     DecodeSplits s;
-    s.short_tiles = few <= 2 || (few <= 16 && few * problems <= 2 * sms);
+    s.short_tiles = false;
+    if constexpr (DECODE_SHORT<Tin, G>) s.short_tiles = few <= 2 || (few <= 16 && few * problems <= 2 * sms);
     // otherwise as many CTAs as are resident at once, but at least one tile per warp; with more problems than that, as many
     // as take the least time in waves of them, a CTA's start and merge counted as 3/4 round of tiles per query vector.
     // 512 problems on 444 CTAs, fp32, d = 128, one query vector: 2048 entries 173 -> 122 us (one CTA per problem: a second
     // wave that is nearly empty), 200 entries 16.9 -> 15.9 us; bf16, four query vectors, 2048 entries: 101 -> 91 us.
     const int resident = DEC_CTAS * sms, wanted = resident / problems;
-    s.n = s.short_tiles ? few : ctas(n_core, C::TILE);
+    s.n = s.short_tiles ? few : ctas(n_core, DEC_TILE<Tin, D>);
     if (!s.short_tiles && wanted < 1) {
         const int most_parts = s.n < 4 ? s.n : 4;
         int64_t least = INT64_MAX;
         for (int n = 1; n <= most_parts; ++n) {
-            const int rounds = ctas((n_core + n - 1) / n, C::TILE);
+            const int rounds = ctas((n_core + n - 1) / n, DEC_TILE<Tin, D>);
             const int64_t time = (((int64_t)n * problems + resident - 1) / resident) * (4 * rounds + (G == 1 ? 4 : 3 * G));
             if (time < least) { least = time; s.n = n; }
         }
@@ -687,7 +693,7 @@ template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, 
 {
     constexpr int TILE = DEC_TILE<Tin, D>;
     const int sms = device_sm_count();
-    const int cap = decode_cap<Tin, D>(problems, per_token, sms);
+    const int cap = decode_cap<D>(problems, per_token, sms);
     int longest = 0, parts, chunk, size = 1;
     for (int i = 0; i < win.n; ++i) {
         const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
@@ -716,13 +722,25 @@ template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, 
     return {G, (per_token + G - 1) / G, 1, size, cap};
 }
 
+template <typename Tin, int D, int G> auto decode_split_kernel(bool short_tiles, int &smem)
+{
+    auto kern = decode_kernel<Tin, D, G, DEC_SPLIT, DEC_SHORT_TILE>;
+    smem = DecodeCfg<Tin, D, G, DEC_SHORT_TILE>::template total<DEC_SPLIT>();
+    if constexpr (!DECODE_MMA<Tin, G>) {
+        if (!short_tiles) {
+            kern = decode_kernel<Tin, D, G, DEC_SPLIT>;
+            smem = DecodeCfg<Tin, D, G>::template total<DEC_SPLIT>();
+        }
+    }
+    return kern;
+}
+
 // win set: streaming tokens, laid out as `form` says; else the list of elm_attend, n_core entries long
 template <typename Tin, int D, int G>
 int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, const float *w, int64_t list_stride, int n_core,
                   const DecodeWindows *win, DecodeForm form, const elm_params *p, Tin *O, float *part, size_t part_room, int *status,
                   int per_token, cudaStream_t st)
 {
-    using C = DecodeCfg<Tin, D, G>;
     const int problems = p->batch * p->kv_heads;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -737,6 +755,7 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     DecodeGroups grp = {};
     if (win) {
         if constexpr (G <= DEC_GSTREAM && std::is_same<Tin, float>::value) {
+            using C = DecodeCfg<Tin, D, G>;
             grp.vec_groups = form.vec_groups;
             grp.per_group = form.per_group;
             for (int i = 0; i < win->n; ++i) {
@@ -775,12 +794,18 @@ int launch_decode(const Tin *Q, const Tin *K, const Tin *V, const int32_t *idx, 
     const DecodeSplits sp = decode_splits<Tin, D, G>(n_core, problems, part_room);
     const int splits = sp.n;
     if (splits < 1) return ELM_ERR_WORKSPACE;
-    auto kern = sp.short_tiles ? decode_kernel<Tin, D, G, DEC_SPLIT, DEC_SHORT_TILE> : decode_kernel<Tin, D, G, DEC_SPLIT>;
-    cfg.dynamicSmemBytes = sp.short_tiles ? DecodeCfg<Tin, D, G, DEC_SHORT_TILE>::template total<DEC_SPLIT>() : C::template total<DEC_SPLIT>();
-    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
     cfg.gridDim = dim3((unsigned)splits, (unsigned)problems);
-    ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, whole, grp, 0, O,
-                                    part, status));
+    if (DECODE_MMA<Tin, G> && !sp.short_tiles) {
+        const int rc = launch_tokens_split(Q, K, V, idx, w, n_core, splits, G, p, part, status, st);
+        if (rc != ELM_OK) return rc;
+    } else if constexpr (DECODE_SHORT<Tin, G>) {
+        int smem;
+        auto kern = decode_split_kernel<Tin, D, G>(sp.short_tiles, smem);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+        ELM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, Q, K, V, idx, w, n_kv, list_stride, q_heads, kv_heads, n_q, per_token, whole, grp, 0, O,
+                                        part, status));
+    }
     cfg.gridDim = dim3((unsigned)per_token, (unsigned)problems);
     cfg.blockDim = dim3(D);
     cfg.dynamicSmemBytes = 0;
@@ -799,7 +824,7 @@ int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *
     if (win) {
         const int problems = p->batch * p->kv_heads;
         if constexpr (std::is_same<Tin, __nv_bfloat16>::value)
-            return attend_tokens_bf16(Q, K, V, idx, w, list_stride, *win, p, O, status, decode_cap<Tin, D>(problems, per_token, device_sm_count()), st);
+            return attend_tokens_bf16(Q, K, V, idx, w, list_stride, *win, p, O, status, decode_token_caps(p), st);
         else
             form = decode_form<Tin, D>(*win, problems, per_token);
     }
@@ -831,10 +856,12 @@ bool attend_decode_windows_apply(const elm_params *p, int n_core)
 {
     if (!attend_decode_applies(p) || p->n_q != 1 || (p->dtype != ELM_F32 && p->dtype != ELM_BF16)) return false;
     const int problems = p->batch * p->kv_heads, per_token = p->q_heads / p->kv_heads;
-    if (p->dtype == ELM_F32)
-        return p->d == 64 ? decode_clustered<float, 64>(n_core, problems, per_token) : decode_clustered<float, 128>(n_core, problems, per_token);
-    return p->d == 64 ? decode_clustered<__nv_bfloat16, 64>(n_core, problems, per_token)
-                      : decode_clustered<__nv_bfloat16, 128>(n_core, problems, per_token);
+    if (p->dtype == ELM_F32) {
+        const int sms = device_sm_count();
+        return p->d == 64 ? decode_clustered(n_core, problems, decode_cap<64>(problems, per_token, sms), DEC_WARPS * DEC_TILE<float, 64>)
+                          : decode_clustered(n_core, problems, decode_cap<128>(problems, per_token, sms), DEC_WARPS * DEC_TILE<float, 128>);
+    }
+    return decode_clustered(n_core, problems, decode_token_caps(p).of_long, 128);
 }
 
 namespace {
@@ -843,13 +870,21 @@ template <typename Tin, int D, int G> int decode_grid(const elm_params *p, int n
     const AttendLayout L = attend_layout(p, n_core);
     const int problems = p->batch * p->kv_heads;
     const DecodeSplits sp = decode_splits<Tin, D, G>(n_core, problems, L.bias - L.Kc);
-    auto kern = sp.short_tiles ? decode_kernel<Tin, D, G, DEC_SPLIT, DEC_SHORT_TILE> : decode_kernel<Tin, D, G, DEC_SPLIT>;
-    const int smem = sp.short_tiles ? DecodeCfg<Tin, D, G, DEC_SHORT_TILE>::template total<DEC_SPLIT>() : DecodeCfg<Tin, D, G>::template total<DEC_SPLIT>();
     int per_sm = 0;
-    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ELM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DEC_WARPS * 32, (size_t)smem));
-    *ctas = sp.n * problems;
-    *resident = per_sm * device_sm_count();
+    if (DECODE_MMA<Tin, G> && !sp.short_tiles) {
+        ELM_CUDA_TRY(tokens_split_occupancy(D, &per_sm));
+        *ctas = sp.n * problems;
+        *resident = per_sm * device_sm_count();
+        return ELM_OK;
+    }
+    if constexpr (DECODE_SHORT<Tin, G>) {
+        int smem;
+        auto kern = decode_split_kernel<Tin, D, G>(sp.short_tiles, smem);
+        ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        ELM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DEC_WARPS * 32, (size_t)smem));
+        *ctas = sp.n * problems;
+        *resident = per_sm * device_sm_count();
+    }
     return ELM_OK;
 }
 }  // namespace

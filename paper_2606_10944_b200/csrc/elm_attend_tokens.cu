@@ -1,4 +1,5 @@
 // Attention of the tokens of a streaming run, bf16 storage: every token attends over a prefix of its window's list
+// (and, in tokens_split_kernel, the first launch of elm_attend's split form: one list per problem)
 //   O[t,:] = sum_c w_c exp(<q_t,k_c>/sqrt(d)) v_c / sum_c w_c exp(<q_t,k_c>/sqrt(d)),  c < seen(t)      Eq. (def:att_approx)
 //
 // Neighbouring tokens see all but a few of the same entries, and a token has one query vector per query head of its KV
@@ -50,18 +51,30 @@ constexpr int TOK_CTAS = 2;                    // CTAs per SM the kernel is comp
 
 struct TokenGroups {
     int32_t cluster;                           // CTAs per group (cluster form)
-    int32_t cap;                               // most CTAs a list is spread over
+    TokenCaps caps;                            // most CTAs a list is spread over
     int32_t per_group;                         // neighbouring tokens of a warp: a power of two
     int32_t span;                              // tokens per cluster or CTA: per_group, or four times as many
     int32_t g0[DECODE_MAX_WINDOWS + 1];        // groups of `span` tokens in the windows before
 };
 
-// Tiles per unit of a list of n_core entries: at most 4 cap units.  Depends on n_core only through the next multiple of
+// Tiles per unit of a list of n_core entries: at most 4 units per CTA.  Depends on n_core only through the next multiple of
 // 128, so that the (at most 64, aligned) tokens of a span agree.
-__host__ __device__ __forceinline__ int token_units(int n_core, int cap)
+__host__ __device__ __forceinline__ int token_units(int n_core, TokenCaps caps)
 {
-    const int tiles = (n_core + 127) / 128 * (128 / TOK_TILE);
-    return (tiles + TOK_WARPS * cap - 1) / (TOK_WARPS * cap);
+    const int tiles = (n_core + 127) / 128 * (128 / TOK_TILE), most = TOK_WARPS * (n_core <= TOKENS_SHORT_LIST ? caps.of_short : caps.of_long);
+    return (tiles + most - 1) / most;
+}
+
+// CTAs of a cluster for lists of n0 .. n1 entries
+int tokens_cluster(int n0, int n1, TokenCaps caps)
+{
+    auto units = [&](int n) { const int k = token_units(n, caps), tiles = (n + TOK_TILE - 1) / TOK_TILE; return (tiles + k - 1) / k; };
+    // (where the units grow longer there are fewer of them: the most are at an end, or just below a step)
+    int most = units(n1);
+    for (int n = (n0 + 127) / 128 * 128; n < n1; n += 128) most = units(n) > most ? units(n) : most;
+    int size = 1;
+    while (size * TOK_WARPS < most) size *= 2;
+    return size;
 }
 
 template <int D> struct TokenCfg {
@@ -75,6 +88,10 @@ template <int D> struct TokenCfg {
     static constexpr int S_LW = TOK_STAGES * 2 * TILE_BYTES;
     static constexpr int S_P = S_LW + TOK_STAGES * TOK_TILE * 4;
     static constexpr int S_TOTAL = S_P + TOK_WARPS * TOK_ROWS * P_STRIDE * 4;
+    // split form: [warp][K, V], log2 weights, (maximum, denominator) [warp][row]
+    static constexpr int P_LW = TOK_WARPS * 2 * TILE_BYTES;
+    static constexpr int P_ML = P_LW + TOK_WARPS * TOK_TILE * 4;
+    static constexpr int P_TOTAL = P_ML + TOK_WARPS * 8 * 8;
     // cluster form: [warp][K, V], log2 weights, probabilities; maxima (then factors of the state) and denominators [row][unit],
     // factors of the units (over the probabilities) likewise; the CTA's slice of every unit's result, [unit][column of the slice][row]
     template <int ROWS> struct Cluster {
@@ -406,7 +423,7 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             }
     }
     const float scale = 8.f * 1.4426950408889634f / sqrtf((float)D);
-    const int unit_tiles = token_units(n_span, grp.cap);
+    const int unit_tiles = token_units(n_span, grp.caps);
     const int tiles = (n_span + TOK_TILE - 1) / TOK_TILE;
     float *sp = reinterpret_cast<float *>(smem + (CLUSTER ? CC::P : C::S_P)) + warp * TOK_ROWS * C::P_STRIDE;
     TokenUnit<D, NB> u;
@@ -651,6 +668,124 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
     }
 }
 
+// elm_attend's lists: CTA (split, problem) takes its split's tiles, a warp every fourth of them, and leaves the merged result of its
+// warps in part[problem][split][G][D + 2] (accumulator, maximum, denominator).  Bound by HBM latency and issue: three CTAs to an SM.
+template <int D>
+__global__ void __launch_bounds__(TOK_THREADS, 3)
+tokens_split_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
+                    const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t n, int n_core, int q_heads, int kv_heads,
+                    int n_q, int G, float *__restrict__ part, int *__restrict__ status)
+{
+    using C = TokenCfg<D>;
+    constexpr int NC = C::NC;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, quad = lane & 3;
+    // (launched with programmatic stream serialization: nothing is read or written before this point)
+    cudaGridDependencySynchronize();
+#ifndef ELM_BOUNDS_CHECK
+    if (tid == 0 && blockIdx.y == 0 && blockIdx.x == 0) *status = 0;
+#endif
+    const int prob = blockIdx.y, rep = q_heads / kv_heads, rows = rep * n_q;
+    const int b = prob / kv_heads, kvh = prob % kv_heads;
+    const int32_t *ip = idx + (int64_t)prob * n_core;
+    const float *wp = w + (int64_t)prob * n_core;
+    const __nv_bfloat16 *Kp = K + (int64_t)prob * n * D, *Vp = V + (int64_t)prob * n * D;
+    const int tiles = (n_core + TOK_TILE - 1) / TOK_TILE, per = (tiles + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int t_end = min(((int)blockIdx.x + 1) * per, tiles);
+    int t = (int)blockIdx.x * per + warp;
+    unsigned char *kt = smem + warp * 2 * C::TILE_BYTES, *vt = kt + C::TILE_BYTES;
+    float *lw = reinterpret_cast<float *>(smem + C::P_LW) + warp * TOK_TILE;
+    int32_t row = 0;
+    float wt = 0.f;
+    auto fetch_entries = [&](int tile) {
+        const int e = tile * TOK_TILE + lane;
+        row = 0;
+        wt = 0.f;
+        if (e < n_core) {
+            row = (int32_t)checked_row(__ldg(ip + e), n, status);
+            wt = __ldg(wp + e);
+        }
+    };
+    auto copy_rows = [&](unsigned char *dst, const __nv_bfloat16 *X, int32_t from, int tile) {
+        const uint32_t d0 = smem_u32(dst);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            const int e = (lane + 32 * i) / NC, c = lane % NC;
+            const int64_t r = __shfl_sync(0xffffffffu, from, e);
+            cp_async16_zfill(d0 + chunk_at<NC>(e, c), X + r * D + c * 8, tile * TOK_TILE + e < n_core);
+        }
+        cp_async_commit();
+    };
+    TokenUnit<D, 1> u;
+    u.reset();
+    if (t < t_end) {
+        fetch_entries(t);
+        copy_rows(kt, Kp, row, t);
+        copy_rows(vt, Vp, row, t);
+    }
+    // the query vectors as operands, scaled by 1/8: exactly
+    uint32_t qf[D / 16][4];
+    {
+        const int r = lane >> 2;
+        const __nv_bfloat16 *q = Q + (r < rows ? (((int64_t)b * q_heads + kvh * rep + r / n_q) * n_q + r % n_q) * D : 0) + 2 * quad;
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                __nv_bfloat162 x = __floats2bfloat162_rn(0.f, 0.f);
+                if (r < rows) x = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(q + 16 * i + 8 * c), __floats2bfloat162_rn(0.125f, 0.125f));
+                qf[i][2 * c] = *reinterpret_cast<const uint32_t *>(&x);
+                qf[i][2 * c + 1] = 0u;
+            }
+    }
+    const float scale = 8.f * 1.4426950408889634f / sqrtf((float)D);
+    const int lim[1] = {n_core};
+    for (bool head = true; t < t_end; t += TOK_WARPS, head = false) {
+        const bool more = t + TOK_WARPS < t_end;
+        float s[4][4];
+        lw[lane] = log2f(wt);
+        if (more) fetch_entries(t + TOK_WARPS);
+        cp_async_wait<1>();                                        // the keys (the values are the newer group)
+        __syncwarp();
+        token_logits<D, 1>(s, qf, smem_u32(kt));
+        __syncwarp();
+        if (more) copy_rows(kt, Kp, row, t + TOK_WARPS);
+        token_softmax<D, 1>(u, head, s, lw, t * TOK_TILE, lim, n_core, scale);
+        if (more) cp_async_wait<1>();
+        else cp_async_wait<0>();
+        __syncwarp();
+        token_values<D, 1>(u, s, vt, nullptr, t * TOK_TILE, lim, n_core, n_core, n_core);
+        __syncwarp();
+        if (more) copy_rows(vt, Vp, row, t + TOK_WARPS);
+    }
+    u.finish();
+    // the warps' results over their own tiles, then their merge
+    float *po = reinterpret_cast<float *>(kt);
+    float2 *ml = reinterpret_cast<float2 *>(smem + C::P_ML);
+    if (quad == 0) ml[warp * 8 + (lane >> 2)] = make_float2(u.m[0], u.l[0]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < D / 8; ++j) po[(2 * quad + i) * D + 8 * j + (lane >> 2)] = u.o[j >> 1][0][2 * (j & 1) + i];
+    __syncthreads();
+    for (int i = tid; i < rows * D; i += TOK_THREADS) {
+        const int g = i / D;
+        float M = -INFINITY, acc = 0.f, den = 0.f;
+#pragma unroll
+        for (int v = 0; v < TOK_WARPS; ++v) M = fmaxf(M, ml[v * 8 + g].x);
+#pragma unroll
+        for (int v = 0; v < TOK_WARPS; ++v) {
+            const float2 x = ml[v * 8 + g];
+            const float f = x.x == -INFINITY ? 0.f : exp2f(x.x - M);
+            acc = fmaf(f, reinterpret_cast<const float *>(smem + v * 2 * C::TILE_BYTES)[i], acc);
+            den = fmaf(f, x.y, den);
+        }
+        float *out = part + (((int64_t)prob * gridDim.x + blockIdx.x) * G + g) * (D + 2);
+        out[i % D] = acc;
+        if (i % D == 0) { out[D] = M; out[D + 1] = den; }
+    }
+}
+
 int tokens_per_group(int per_token)
 {
     int t = 1;
@@ -659,13 +794,13 @@ int tokens_per_group(int per_token)
 }
 template <int D>
 int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
-                  const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st)
+                  const DecodeWindows &win, const elm_params *p, void *O, int *status, TokenCaps caps, cudaStream_t st)
 {
     using C = TokenCfg<D>;
     const int problems = p->batch * p->kv_heads, per_token = p->q_heads / p->kv_heads;
     const int sms = device_sm_count();
     TokenGroups grp = {};
-    grp.cap = cap;
+    grp.caps = caps;
     grp.per_group = tokens_per_group(per_token);
     auto count = [&](int span) {
         grp.span = span;
@@ -686,31 +821,28 @@ int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *id
     // The serial form takes as long as one CTA needs for the longest list, about 1.5 us a tile, whatever few tokens there are;
     // clusters finish one after the other, 0.2 us each for a list of 200 entries and 1.5 for 6144.  Measured, bf16, d = 128, 8 KV heads
     // of 4 query heads (8 clusters per 4 tokens), clusters against serial: 200 entries 32 tokens 12 / 20 us, 64 tokens 29 / 26;
-    // 2053 entries 32 tokens 82 / 106, 64 tokens 154 / 113; 6144 entries 64 tokens 204 / 303, 128 tokens 390 / 306.
+    // 2053 entries 32 tokens 47 / 106, 64 tokens 81 / 113; 6144 entries 64 tokens 203 / 303, 128 tokens 390 / 306.
     int longest = 0;
     for (int i = 0; i < win.n; ++i) {
         const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
         longest = last > longest ? last : longest;
     }
     const int64_t clusters = (int64_t)count(grp.per_group) * problems;
-    const bool serial = clusters > 2 * sms / 5 + (longest + TOK_TILE - 1) / TOK_TILE / 2;
+    // (calls of no more tokens than share a warp would leave three of the CTA's four idle)
+    const bool serial = win.tok0[win.n] > grp.per_group && clusters > 3 * sms / 5 + 3 * ((longest + TOK_TILE - 1) / TOK_TILE) / 4;
     auto kern = tokens_kernel<D, false, 2>;
     if (serial) {
         grp.cluster = 1;
         cfg.dynamicSmemBytes = C::S_TOTAL;
         cfg.gridDim = dim3((unsigned)count(TOK_WARPS * grp.per_group), (unsigned)problems);
     } else {
-        int units = 1, most = 1;
+        int most = 1;
+        grp.cluster = 1;
         for (int i = 0; i < win.n; ++i) {
-            const int tokens = win.tok0[i + 1] - win.tok0[i], last = win.seen0[i] + tokens - 1;
-            const int per_unit = token_units(last, cap), tiles = (last + TOK_TILE - 1) / TOK_TILE;
-            // (a window that grows past a list of `cap` full CTAs: the units are longer from there on, and fewer)
-            const int u = token_units(win.seen0[i], cap) < per_unit ? TOK_WARPS * cap : (tiles + per_unit - 1) / per_unit;
-            units = u > units ? u : units;
+            const int tokens = win.tok0[i + 1] - win.tok0[i], size = tokens_cluster(win.seen0[i], win.seen0[i] + tokens - 1, caps);
+            grp.cluster = size > grp.cluster ? size : grp.cluster;
             most = tokens > most ? tokens : most;
         }
-        grp.cluster = 1;
-        while (grp.cluster * TOK_WARPS < units) grp.cluster *= 2;
         const bool few = (most < grp.per_group ? most : grp.per_group) * per_token <= 8;
         kern = few ? tokens_kernel<D, true, 1> : tokens_kernel<D, true, 2>;
         cfg.dynamicSmemBytes = few ? C::template Cluster<8>::TOTAL : C::template Cluster<16>::TOTAL;
@@ -732,26 +864,59 @@ int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *id
 
 }  // namespace
 
-int tokens_largest_cluster(int d)
+// Clusters of `size` CTAs that the current device holds at once, asked once per device (0: the size cannot be placed at all)
+static int tokens_clusters(int d, int size)
 {
-    static std::atomic<int> cached[64][2];                         // (threads that meet here first find the same answer)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-    std::atomic<int> &slot = cached[dev][d == 64 ? 0 : 1];
-    int largest = slot.load(std::memory_order_relaxed);
-    if (largest == 0) {
-        largest = d == 64 ? largest_cluster(tokens_kernel<64, true, 2>, TOK_THREADS, TokenCfg<64>::Cluster<16>::TOTAL, TOK_MAX_CLUSTER)
-                          : largest_cluster(tokens_kernel<128, true, 2>, TOK_THREADS, TokenCfg<128>::Cluster<16>::TOTAL, TOK_MAX_CLUSTER);
-        slot.store(largest, std::memory_order_relaxed);
+    static std::atomic<int> cached[64][2][5];                      // answer + 1 (threads that meet here first find the same)
+    int dev = 0, log = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return size == 1 ? 1 : 0;
+    while (1 << log < size) ++log;
+    std::atomic<int> &slot = cached[dev][d == 64 ? 0 : 1][log];
+    int n = slot.load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+        n = d == 64 ? resident_clusters(tokens_kernel<64, true, 2>, TOK_THREADS, TokenCfg<64>::Cluster<16>::TOTAL, size)
+                    : resident_clusters(tokens_kernel<128, true, 2>, TOK_THREADS, TokenCfg<128>::Cluster<16>::TOTAL, size);
+        slot.store(n + 1, std::memory_order_relaxed);
     }
-    return largest;
+    return n;
+}
+
+TokenCaps tokens_caps(int d, int problems, int limit)
+{
+    // as many CTAs as leave all problems' clusters resident
+    int cap = limit < TOK_MAX_CLUSTER ? limit : TOK_MAX_CLUSTER;
+    while (cap > 1 && tokens_clusters(d, cap) < problems) cap >>= 1;
+    // Up to 4096 entries clusters of 16 gain nothing over 8 with twice the tiles per warp (8 problems of 4 query vectors: 2048 entries
+    // 9.2 against 8.0 us, 4000 entries 10.8 / 10.6, 5193 entries 12.3 / 14.0).
+    return {cap < 8 ? cap : 8, cap};
 }
 
 int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
-                       const DecodeWindows &win, const elm_params *p, void *O, int *status, int cap, cudaStream_t st)
+                       const DecodeWindows &win, const elm_params *p, void *O, int *status, TokenCaps caps, cudaStream_t st)
 {
-    return p->d == 64 ? launch_tokens<64>(Q, K, V, idx, w, list_stride, win, p, O, status, cap, st)
-                      : launch_tokens<128>(Q, K, V, idx, w, list_stride, win, p, O, status, cap, st);
+    return p->d == 64 ? launch_tokens<64>(Q, K, V, idx, w, list_stride, win, p, O, status, caps, st)
+                      : launch_tokens<128>(Q, K, V, idx, w, list_stride, win, p, O, status, caps, st);
+}
+
+cudaError_t tokens_split_occupancy(int d, int *ctas_per_sm)
+{
+    if (d == 64) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, tokens_split_kernel<64>, TOK_THREADS, TokenCfg<64>::P_TOTAL);
+    const cudaError_t e = cudaFuncSetAttribute(tokens_split_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, TokenCfg<128>::P_TOTAL);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, tokens_split_kernel<128>, TOK_THREADS, TokenCfg<128>::P_TOTAL);
+}
+
+int launch_tokens_split(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int n_core, int splits, int G,
+                        const elm_params *p, float *part, int *status, cudaStream_t st)
+{
+    typedef __nv_bfloat16 bf;
+    auto kern = p->d == 64 ? tokens_split_kernel<64> : tokens_split_kernel<128>;
+    const int smem = p->d == 64 ? TokenCfg<64>::P_TOTAL : TokenCfg<128>::P_TOTAL;
+    ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ELM_CUDA_TRY(launch_after(kern, dim3((unsigned)splits, (unsigned)(p->batch * p->kv_heads)), dim3(TOK_THREADS), (size_t)smem, st, (const bf *)Q,
+                              (const bf *)K, (const bf *)V, idx, w, (int64_t)p->n_kv, n_core, (int)p->q_heads, (int)p->kv_heads, (int)p->n_q, G,
+                              part, status));
+    return ELM_OK;
 }
 
 }  // namespace elm

@@ -64,30 +64,27 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// The largest cluster (a power of two, at most `most`) of `kernel` of which the current device can hold one: more than 8 CTAs
-// need the opt-in and a GPC with that many SMs to give, which a partition of a GPU may not have.
-template <typename... KArgs> inline int largest_cluster(void (*kernel)(KArgs...), int threads, int smem, int most)
+// Clusters of `size` CTAs of `kernel` that the current device holds at once: more than 8 CTAs need the opt-in and a GPC with that
+// many SMs to give, which a partition of a GPU may not have.
+template <typename... KArgs> inline int resident_clusters(void (*kernel)(KArgs...), int threads, int smem, int size)
 {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-                      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-    int size = fits ? most : 1;
-    for (; size > 1; size >>= 1) {
-        int clusters = 0;
-        attr[0].val.clusterDim.x = (unsigned)size;
-        cfg.gridDim = dim3((unsigned)size);
-        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1) break;
-    }
+    int clusters = 0;
+    const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess;
     cudaGetLastError();
-    return size;
+    return ok && clusters > 0 ? clusters : 0;
 }
 
 // Multiprocessors of the current device (looked up once per device ordinal; 148 if the query fails).

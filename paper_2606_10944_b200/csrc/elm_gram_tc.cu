@@ -430,7 +430,6 @@ gram_tc_persistent_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat
         const int e = warp - (PLOAD + 1);                     // 0..7
         const int q4 = warp & 3;                              // TMEM lane quarter this warp may access
         const int ch = e >> 2;                                // column half
-        const int r = q4 * 32 + lane;                         // point row in the tile
         const float LOG2E = 1.4426950408889634f;
         const float qscale = LOG2E / sqrtf((float)D);
         int k = 0;

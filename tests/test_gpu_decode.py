@@ -190,6 +190,29 @@ def test_decode_of_short_lists(dtype, d, rep, n_q):
         assert err <= bound, (n_core, float(err))
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,rep,n_q", [(1, 1, 3, 1), (2, 4, 4, 1), (1, 3, 2, 2), (1, 2, 1, 5), (3, 1, 8, 1), (8, 8, 6, 1), (160, 1, 1, 3)])
+def test_decode_on_matrix_instructions(d, B, H, rep, n_q):
+    """Lists around the lengths where elm_attend's route, the clusters and the warps' tiles change, three to eight query
+    vectors per KV head (heads and rows), unequal weights, one of them zero, against 64 bits."""
+    g = torch.Generator(device="cuda").manual_seed(11)
+    n = 5300
+    K, V = (torch.randn(B, H, n, d, device="cuda", generator=g).bfloat16() for _ in range(2))
+    Q = torch.randn(B, H * rep, n_q, d, device="cuda", generator=g).bfloat16()
+    for n_core in (1, 31, 33, 129, 513, 1025, 2048, 2049, 4096, 4097, 5250) if B * H < 60 else (33, 600, 4097):
+        idx = torch.randint(0, n, (B, H, n_core), device="cuda", generator=g, dtype=torch.int32)
+        w = torch.rand(B, H, n_core, device="cuda", generator=g) + 0.05
+        if n_core > 1:
+            w[:, :, n_core // 2] = 0.0
+        got = elm.attend(Q, K, V, idx, w)
+        gather = idx.long().unsqueeze(-1).expand(-1, -1, -1, d)
+        Kc, Vc = (t.double().gather(2, gather).repeat_interleave(rep, dim=1) for t in (K, V))
+        s = torch.einsum("bhqd,bhnd->bhqn", Q.double(), Kc) / d ** 0.5 + w.double().log().repeat_interleave(rep, dim=1).unsqueeze(2)
+        want = torch.softmax(s, dim=-1) @ Vc
+        err = ((got - want).abs().amax(-1) / want.abs().amax(-1)).max()
+        assert err <= 2.0 ** -8, (n_core, float(err))                    # rounded to 8 bits
+
+
 @pytest.mark.parametrize("rep", [1, 4, 8])
 @pytest.mark.parametrize("entries", [100, 200, 400])
 def test_streamed_token_over_a_short_list_takes_no_longer_than_attend(rep, entries):
