@@ -160,7 +160,10 @@ gram_walk_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__res
     if ((int)blockIdx.x < total_tiles) gather(blockIdx.x, misc->tile[0]);
 
     constexpr uint32_t IDESC = umma_idesc_bf16(TR, TR);
-    const uint32_t sK = smem_u32(smem + SM::OFF_K), sV = smem_u32(smem + SM::OFF_V);
+    // (descriptors differ only in the start address, in their low word; see the persistent kernel)
+    const uint64_t desc0 = umma_desc_k128(smem_u32(smem));
+    const uint32_t d_hi = (uint32_t)(desc0 >> 32), dK = (uint32_t)desc0 + (SM::OFF_K >> 4), dV = (uint32_t)desc0 + (SM::OFF_V >> 4);
+    auto desc = [&](uint32_t lo) { uint64_t d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(d_hi)); return d; };
     const int r = (warp & 3) * 32 + lane;                     // epilogue: point row in the tile = TMEM lane
     const int ch = warp >> 2;                                 // and column half
     const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch * 64;
@@ -184,7 +187,7 @@ gram_walk_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__res
                 for (int kh = 0; kh < KH; ++kh)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t d = umma_desc_k128((op == 0 ? sK : sV) + kh * (TR * 128) + ks * 32);
+                        const uint64_t d = desc((op == 0 ? dK : dV) + ((kh * (TR * 128) + ks * 32) >> 4));
                         mma_ss(tmem + op * 128, d, d, IDESC, (kh | ks) != 0);
                     }
             tc_commit(&misc->mma_done);
