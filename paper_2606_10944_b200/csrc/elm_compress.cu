@@ -58,8 +58,9 @@ static int compress_impl(const Tin *K, const Tin *V, const elm_params *p, uint64
     if (m > 0) {
         StageTimer t(ELM_STAGE_PREPASS, st, 1);
         ELM_CUDA_TRY(cudaMemsetAsync(c.vmax_bits, 0, (size_t)(BH + 1) * 4, st));
-        dim3 grid((unsigned)((n + 255) / 256), (unsigned)BH);
-        ELM_CUDA_TRY(launch_after(prepass_kernel<Tin, T>, grid, dim3(256), 0, st, K, V, n, p->d, c.cnorm, c.vmax_bits, cur, (int64_t)0, (int64_t)-1));
+        const int cta_rows = prepass_rows(n, BH, (int)sizeof(Tin), p->d);
+        ELM_CUDA_TRY(launch_after(prepass_kernel<Tin, T>, prepass_grid(n, BH, cta_rows), dim3(256), 0, st, K, V, n, p->d, c.cnorm, c.vmax_bits, cur,
+                                  cta_rows, (int64_t)0, (int64_t)-1));
         count_launches(1);
         ELM_CUDA_TRY(cudaGetLastError());
     }

@@ -379,7 +379,8 @@ static int express_impl(const Tin *K, const Tin *V, const elm_params *p, int mba
     {
         StageTimer t(ELM_STAGE_PREPASS, st, 2);
         ELM_CUDA_TRY(cudaMemsetAsync(c.vmax_bits, 0, (size_t)(BH + 1) * 4, st));
-        prepass_kernel<Tin, T><<<dim3(blocks(n), (unsigned)BH), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, listA);
+        const int cta_rows = prepass_rows(n, BH, (int)sizeof(Tin), p->d);
+        prepass_kernel<Tin, T><<<prepass_grid(n, BH, cta_rows), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, listA, cta_rows);
         range_kernel<<<dim3(blocks(n_out), (unsigned)BH), 256, 0, st>>>(E, n, 0, 0, n_out);      // exact phase
         count_launches(2);
         ELM_CUDA_TRY(cudaGetLastError());

@@ -14,6 +14,8 @@
 #include <type_traits>
 
 #include "elm_attend.cuh"
+#include <type_traits>
+
 #include "elm_common.cuh"
 #include "elm_compress.cuh"
 #include "elm_walk.cuh"
@@ -45,6 +47,19 @@ template <typename T> __device__ __forceinline__ void chunk_sq_absmax(const uint
     }
 }
 
+// Rows per CTA of the prepass: one pass of its loads, two or four.  A pass is a round trip to HBM, so a call of a few
+// thousand rows takes as many CTAs as there are passes (8 problems of 256 rows: one pass 3.3 us, four 7.5); from four CTAs per SM
+// on longer CTAs cost less (0.54 GB: one pass 144 us, two 100, four 94).
+constexpr int PREPASS_UNROLL = 4;
+inline int prepass_rows(int64_t rows, int problems, int item, int d)
+{
+    const int pass = PREPASS_UNROLL * 256 * 16 / (d * item);
+    for (int k = 4; k > 1; k /= 2)
+        if ((rows + k * pass - 1) / (k * pass) * problems >= 4 * device_sm_count()) return k * pass;
+    return pass;
+}
+inline dim3 prepass_grid(int64_t rows, int problems, int cta_rows) { return dim3((unsigned)((rows + cta_rows - 1) / cta_rows), (unsigned)problems); }
+
 // One pass over K and V with 16-byte loads: a group of (row bytes / 16) lanes owns a row.  Bound by HBM: four rows of
 // each are requested before the first is used.  0.54 GB: 95 us, 0.27 GB: 57 us (one
 // at a time: 103 and 61).
@@ -53,7 +68,7 @@ static __global__ void __launch_bounds__(256) prepass_kernel(const Tin *__restri
                                                       const Tin *__restrict__ V, int64_t n, int d,
                                                       T *__restrict__ cnorm,
                                                       unsigned *__restrict__ vmax_bits,
-                                                      int32_t *__restrict__ cur, int64_t first = 0,
+                                                      int32_t *__restrict__ cur, int cta_rows, int64_t first = 0,
                                                       int64_t last = -1 /* rows [first, last); -1: n */)
 {
     cudaGridDependencySynchronize();           // launched with programmatic stream serialization (launch_after)
@@ -63,13 +78,13 @@ static __global__ void __launch_bounds__(256) prepass_kernel(const Tin *__restri
     const int lpr = d / EPC;                              // lanes per row: 8, 16 or 32
     const int rows_per_pass = 256 / lpr;
     const int sub = threadIdx.x % lpr, rloc = threadIdx.x / lpr;
-    const int64_t row0 = first + (int64_t)blockIdx.x * 256;   // 256 rows per CTA
+    const int64_t row0 = first + (int64_t)blockIdx.x * cta_rows;
     const Tin *Kp = K + (int64_t)p * n * d;
     const Tin *Vp = V + (int64_t)p * n * d;
     const T rsd = sqrt((T)d);
     float vm = 0.f;
-    constexpr int U = 4;                                      // (256 rows are a multiple of U passes of 8, 16 or 32 rows)
-    for (int r = rloc; r < 256 && row0 + r - rloc < last; r += U * rows_per_pass) {
+    constexpr int U = PREPASS_UNROLL;
+    for (int r = rloc; r < cta_rows && row0 + r - rloc < last; r += U * rows_per_pass) {
         uint4 kq[U], vq[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -312,7 +327,10 @@ static __global__ void __launch_bounds__(256) gram_simt_kernel(const Tin *__rest
 // a thread multiplies packed pairs of dimensions: 8 reads of 16 bytes per 32 packed fmas, nothing transposed.  The
 // generic kernel (scalar gathers of 16 dimensions between two barriers each) took 31 us per level for 48 problems of
 // 1024 points, d = 64 (10.9 us for one problem); this one 27 us (7.6).
-template <int D>
+// SKIP: where every tile is on the diagonal (calls of 32 pairs: 1), the products of row pair ty + 16 with column pair tx are not of
+// use, and of calls of up to 16 pairs (2) those of row pair ty with column pair tx + 16 neither: 48 problems, 32 pairs
+// a call 33.3 -> 28.6 us, one problem, up to 16 pairs 8.2 -> 7.0 us.
+template <int D, int SKIP>
 static __global__ void __launch_bounds__(256, 3) gram_f32_kernel(const float *__restrict__ K, const float *__restrict__ V,
                                                        const int32_t *__restrict__ cur, const float *__restrict__ Mpair,
                                                        const unsigned *__restrict__ vmax_bits, int64_t n, int P, int64_t Ptotal,
@@ -387,7 +405,10 @@ static __global__ void __launch_bounds__(256, 3) gram_f32_kernel(const float *__
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = fma2(a[r].y, b[c].y, fma2(a[r].x, b[c].x, acc[r][c]));
+                for (int c = 0; c < 4; ++c) {
+                    if ((SKIP >= 1 && r >= 2 && c < 2) || (SKIP == 2 && r < 2 && c >= 2)) continue;
+                    acc[r][c] = fma2(a[r].y, b[c].y, fma2(a[r].x, b[c].x, acc[r][c]));
+                }
         }
         __syncthreads();
         if (ph + 2 < PH) issue(ph + 2);
@@ -792,7 +813,9 @@ static int run_gram_simt(const Tin *K, const Tin *V, const elm_params *p, const 
     }
     dim3 grid((unsigned)tiles, (unsigned)BH);
     if constexpr (std::is_same<Tin, float>::value && std::is_same<T, float>::value) {
-        auto kern = p->d == 64 ? gram_f32_kernel<64> : gram_f32_kernel<128>;
+        auto kern = P > 32 ? (p->d == 64 ? gram_f32_kernel<64, 0> : gram_f32_kernel<128, 0>)
+                           : P == 32 ? (p->d == 64 ? gram_f32_kernel<64, 1> : gram_f32_kernel<128, 1>)
+                                     : (p->d == 64 ? gram_f32_kernel<64, 2> : gram_f32_kernel<128, 2>);
         const size_t smem = 2 * 2 * 64 * 64 * sizeof(float);
         ELM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         ELM_CUDA_TRY(launch_after(kern, grid, dim3(256), smem, st, K, V, cur, Mpair, vmax_bits, p->n_kv, P, Ptotal, F, F_stride));

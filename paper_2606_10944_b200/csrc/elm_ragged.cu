@@ -75,7 +75,8 @@ static int ragged_impl(const Tin *K, const Tin *V, const elm_params *p, const Ra
         // key norms and v_max over every row of the problem; level 0 starts as the middle rows in order
         StageTimer t(ELM_STAGE_PREPASS, st, 2);
         ELM_CUDA_TRY(cudaMemsetAsync(c.vmax_bits, 0, (size_t)(BH + 1) * 4, st));
-        prepass_kernel<Tin, T><<<dim3(blocks(n), (unsigned)BH), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, list[1]);
+        const int cta_rows = prepass_rows(n, BH, (int)sizeof(Tin), p->d);
+        prepass_kernel<Tin, T><<<prepass_grid(n, BH, cta_rows), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, list[1], cta_rows);
         count_launches(1);
         if (pl.n_mid > 0) {
             range_kernel<<<dim3(blocks(pl.n_mid), (unsigned)BH), 256, 0, st>>>(list[0], n, 0, n_sink, pl.n_mid);

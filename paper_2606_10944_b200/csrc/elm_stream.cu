@@ -215,7 +215,8 @@ static int stream_step_impl(elm_stream *s, const Tin *Q, const Tin *K, const Tin
         // tokens that were not there at init: their key norms, and v_max grows with them (it is read by the Halve
         // calls alone, which come behind the last token of a window)
         const int64_t from = t > s->n_known ? t : s->n_known;
-        prepass_kernel<Tin, T><<<dim3(blocks(t + W - from), (unsigned)BH), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, T1, from, t + W);
+        const int cta_rows = prepass_rows(t + W - from, BH, (int)sizeof(Tin), p->d);
+        prepass_kernel<Tin, T><<<prepass_grid(t + W - from, BH, cta_rows), 256, 0, st>>>(K, V, n, p->d, c.cnorm, c.vmax_bits, T1, cta_rows, from, t + W);
         count_launches(1);
         ELM_CUDA_TRY(cudaGetLastError());
     }
@@ -466,21 +467,22 @@ extern "C" int elm_stream_init(elm_stream *s, const void *K, const void *V, int6
     s->n_known = n_known;
     ELM_CUDA_TRY(cudaMemsetAsync(ws + L.vmax_bits, 0, (size_t)(BH + 1) * 4, st));
     if (n_known > 0) {
-        const dim3 grid((unsigned)((n_known + 255) / 256), (unsigned)BH);
+        const int cta_rows = prepass_rows(n_known, BH, (int)elt_bytes(params->dtype), params->d);
+        const dim3 grid = prepass_grid(n_known, BH, cta_rows);
         unsigned *vb = reinterpret_cast<unsigned *>(ws + L.vmax_bits);
         int32_t *scratch = reinterpret_cast<int32_t *>(ws + L.T1);
         const int64_t n = params->n_kv;
         typedef __nv_bfloat16 bf;
         if (params->dtype == ELM_F32) {
             if (params->precision == ELM_PREC_FP64_DET)
-                prepass_kernel<float, double><<<grid, 256, 0, st>>>((const float *)K, (const float *)V, n, params->d, reinterpret_cast<double *>(ws + L.cnorm), vb, scratch, 0, n_known);
+                prepass_kernel<float, double><<<grid, 256, 0, st>>>((const float *)K, (const float *)V, n, params->d, reinterpret_cast<double *>(ws + L.cnorm), vb, scratch, cta_rows, 0, n_known);
             else
-                prepass_kernel<float, float><<<grid, 256, 0, st>>>((const float *)K, (const float *)V, n, params->d, reinterpret_cast<float *>(ws + L.cnorm), vb, scratch, 0, n_known);
+                prepass_kernel<float, float><<<grid, 256, 0, st>>>((const float *)K, (const float *)V, n, params->d, reinterpret_cast<float *>(ws + L.cnorm), vb, scratch, cta_rows, 0, n_known);
         } else {
             if (params->precision == ELM_PREC_FP64_DET)
-                prepass_kernel<bf, double><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, n, params->d, reinterpret_cast<double *>(ws + L.cnorm), vb, scratch, 0, n_known);
+                prepass_kernel<bf, double><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, n, params->d, reinterpret_cast<double *>(ws + L.cnorm), vb, scratch, cta_rows, 0, n_known);
             else
-                prepass_kernel<bf, float><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, n, params->d, reinterpret_cast<float *>(ws + L.cnorm), vb, scratch, 0, n_known);
+                prepass_kernel<bf, float><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, n, params->d, reinterpret_cast<float *>(ws + L.cnorm), vb, scratch, cta_rows, 0, n_known);
         }
         count_launches(1);
         ELM_CUDA_TRY(cudaGetLastError());
