@@ -236,10 +236,11 @@ __global__ void __launch_bounds__(128) attend_simt_kernel(const Tin *__restrict_
 // as packed pairs of rows, so that a step of either product is three or four 16-byte shared-memory reads and 16 or 32
 // packed fmas; its rows' maxima and denominators are finished by shuffles among the 16 threads that share them.  The
 // generic kernel (4 x 4 and scalar reads, softmax by half of the threads with the rest waiting) took 102 us for
-// 48 heads x 1024 queries x 128 points, d = 64; this one 57 us (28 TFLOP/s).
-// Shared memory: queries and keys as [dimension][row], values [point][dimension], probabilities [point][row] with the
-// 16-byte chunks of a point's row exchanged by its column group (the threads that write a chunk at one time differ in
-// that group: no bank conflicts).
+// 48 heads x 1024 queries x 128 points, d = 64; this one 57 us, 55 with whole lines read (d = 128: 126 -> 107, 12 heads x 200 x 32 points
+// with the gather 13.0 -> 11.0 and 19.0 -> 16.5).
+// Shared memory: queries and keys as [dimension][row], values [point][dimension], probabilities [point][row]; the 16-byte
+// chunks of a row exchanged by the dimension (queries, keys) or the column group (probabilities), so that the threads that
+// write a chunk at one time meet no bank conflicts.
 // ---------------------------------------------------------------------------------------------
 template <int D, int BN>
 __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict__ Q, const float *__restrict__ Kc,
@@ -266,11 +267,24 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
     const float scale = (float)(1.4426950408889634 / sqrt((double)D));
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
 
-    // consecutive threads take consecutive rows, so that the transposed writes do not conflict
+    // A warp reads eight chunks of four rows at a time, whole lines (a lane per row had each of its 32 lanes in a line of its
+    // own); the transposed rows of dimension k have their 16-byte chunks exchanged by k / 4, so that its writes fall into
+    // different banks.
+    auto chunk_of = [](int e, int &r, int &k) {
+        const int lane = e & 31, i = e >> 5;
+        r = i / (D / 32) * 4 + (lane >> 3);
+        k = (i % (D / 32) * 8 + (lane & 7)) * 4;
+    };
+    auto at = [](int k, int row, int rows) { return k * rows + ((((row >> 2) ^ (k >> 2)) & (rows / 4 - 1)) << 2) + (row & 3); };
+    auto put = [&](float *X, int k, int row, int rows, const float4 &v) {
+        float *x = X + at(k, row, rows);                            // (dimensions k .. k + 3, k a multiple of 4)
+        x[0] = v.x; x[rows] = v.y; x[2 * rows] = v.z; x[3 * rows] = v.w;
+    };
+#pragma unroll 4
     for (int e = tid; e < BM * D / 4; e += 128) {
-        const int r = e % BM, k = e / BM * 4;
-        const float4 v = q0 + r < n_q ? __ldg(reinterpret_cast<const float4 *>(Qp + (q0 + r) * D + k)) : zero;
-        Qt[k * BM + r] = v.x; Qt[(k + 1) * BM + r] = v.y; Qt[(k + 2) * BM + r] = v.z; Qt[(k + 3) * BM + r] = v.w;
+        int r, k;
+        chunk_of(e, r, k);
+        put(Qt, k, r, BM, q0 + r < n_q ? __ldg(reinterpret_cast<const float4 *>(Qp + (q0 + r) * D + k)) : zero);
     }
     float m[8], l[8];
     uint64_t o[4][OC];
@@ -283,13 +297,13 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
 
     for (int c0 = 0; c0 < n_core; c0 += BN) {
         __syncthreads();
+#pragma unroll 4
         for (int e = tid; e < BN * D / 4; e += 128) {
-            const int r = e % BN, k = e / BN * 4;
-            const float4 v = c0 + r < n_core ? __ldg(reinterpret_cast<const float4 *>(Kp + (int64_t)(c0 + r) * D + k)) : zero;
-            Kt[k * BN + r] = v.x; Kt[(k + 1) * BN + r] = v.y; Kt[(k + 2) * BN + r] = v.z; Kt[(k + 3) * BN + r] = v.w;
-            const int rv = e / (D / 4), kv = e % (D / 4) * 4;
-            *reinterpret_cast<float4 *>(Vs + rv * D + kv) =
-                c0 + rv < n_core ? __ldg(reinterpret_cast<const float4 *>(Vp + (int64_t)(c0 + rv) * D + kv)) : zero;
+            int r, k;
+            chunk_of(e, r, k);
+            const bool in = c0 + r < n_core;
+            put(Kt, k, r, BN, in ? __ldg(reinterpret_cast<const float4 *>(Kp + (int64_t)(c0 + r) * D + k)) : zero);
+            *reinterpret_cast<float4 *>(Vs + r * D + k) = in ? __ldg(reinterpret_cast<const float4 *>(Vp + (int64_t)(c0 + r) * D + k)) : zero;
         }
         // the columns' weights and, where rows differ in what they see, lifetimes
         float bc[CN];
@@ -308,23 +322,27 @@ __global__ void __launch_bounds__(128) attend_f32_kernel(const float *__restrict
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int c = 0; c < CN; ++c) s2[r][c] = 0;
-#pragma unroll 8
-        for (int k = 0; k < D; ++k) {
-            const ulonglong2 qa = *reinterpret_cast<const ulonglong2 *>(Qt + k * BM + 8 * ty);
-            const ulonglong2 qb = *reinterpret_cast<const ulonglong2 *>(Qt + k * BM + 8 * ty + 4);
-            const uint64_t q2[4] = {qa.x, qa.y, qb.x, qb.y};
-            uint64_t k2[CN];
-            if constexpr (CN == 4) {
-                const float4 kv = *reinterpret_cast<const float4 *>(Kt + k * BN + 4 * tx);
-                k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y); k2[2] = pack2(kv.z, kv.z); k2[3] = pack2(kv.w, kv.w);
-            } else {
-                const float2 kv = *reinterpret_cast<const float2 *>(Kt + k * BN + 2 * tx);
-                k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y);
+#pragma unroll 2
+        for (int k4 = 0; k4 < D; k4 += 4) {
+            const float *qx = Qt + at(k4, 8 * ty, BM), *qy = Qt + at(k4, 8 * ty + 4, BM), *kx = Kt + at(k4, CN * tx, BN);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const ulonglong2 qa = *reinterpret_cast<const ulonglong2 *>(qx + kk * BM);
+                const ulonglong2 qb = *reinterpret_cast<const ulonglong2 *>(qy + kk * BM);
+                const uint64_t q2[4] = {qa.x, qa.y, qb.x, qb.y};
+                uint64_t k2[CN];
+                if constexpr (CN == 4) {
+                    const float4 kv = *reinterpret_cast<const float4 *>(kx + kk * BN);
+                    k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y); k2[2] = pack2(kv.z, kv.z); k2[3] = pack2(kv.w, kv.w);
+                } else {
+                    const float2 kv = *reinterpret_cast<const float2 *>(kx + kk * BN);
+                    k2[0] = pack2(kv.x, kv.x); k2[1] = pack2(kv.y, kv.y);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < CN; ++c) s2[r][c] = fma2(q2[r], k2[c], s2[r][c]);
             }
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < CN; ++c) s2[r][c] = fma2(q2[r], k2[c], s2[r][c]);
         }
         // a row sees the entries alive at its own position, or (tail rule) the list up to its own entry of the causal tail
         const bool all_seen = !birth && c0 + BN <= n_core && (int64_t)(c0 + BN) <= (int64_t)tail_start + q0 + 1;
