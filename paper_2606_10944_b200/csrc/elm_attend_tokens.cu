@@ -83,25 +83,23 @@ template <int D> struct TokenCfg {
     static constexpr int TILE_BYTES = TOK_TILE * RB;
     static constexpr int MT = D / 16;                              // row tiles of the transposed output
     static constexpr int MAX_UNITS = TOK_WARPS * TOK_MAX_CLUSTER;
-    // serial form: [stage][K, V], log2 weights, per warp the probabilities of the entries that are added by scalar code
-    static constexpr int P_STRIDE = TOK_ROWS + 1;                  // (a group of at most 16 tokens: at most 15 entries)
+    // serial form: [stage][K, V], log2 weights, queries by warp
     static constexpr int S_LW = TOK_STAGES * 2 * TILE_BYTES;
-    static constexpr int S_P = S_LW + TOK_STAGES * TOK_TILE * 4;
-    static constexpr int S_TOTAL = S_P + TOK_WARPS * TOK_ROWS * P_STRIDE * 4;
-    // split form: [warp][K, V], log2 weights, (maximum, denominator) [warp][row]
+    static constexpr int S_Q = S_LW + TOK_STAGES * TOK_TILE * 4;
+    static constexpr int S_TOTAL = S_Q + TOK_WARPS * TOK_ROWS * RB;
+    // split form: [warp][K, V], log2 weights, (maximum, denominator) [warp][row], queries by warp
     static constexpr int P_LW = TOK_WARPS * 2 * TILE_BYTES;
     static constexpr int P_ML = P_LW + TOK_WARPS * TOK_TILE * 4;
-    static constexpr int P_TOTAL = P_ML + TOK_WARPS * 8 * 8;
-    // cluster form: [warp][K, V], log2 weights, probabilities; maxima (then factors of the state) and denominators [row][unit],
-    // factors of the units (over the probabilities) likewise; the CTA's slice of every unit's result, [unit][column of the slice][row]
+    static constexpr int P_Q = P_ML + TOK_WARPS * 8 * 8;
+    static constexpr int P_TOTAL = P_Q + TOK_WARPS * 8 * RB;
+    // cluster form: [warp][K, V], log2 weights; factors of the units, maxima (then factors of the state) and denominators [row][unit];
+    // the CTA's slice of every unit's result, [unit][column of the slice][row]
     template <int ROWS> struct Cluster {
         static constexpr int LW = TOK_WARPS * 2 * TILE_BYTES;
-        static constexpr int P = LW + TOK_WARPS * TOK_TILE * 4;
-        static constexpr int ML = P + TOK_WARPS * TOK_ROWS * P_STRIDE * 4;
+        static constexpr int FB = LW + TOK_WARPS * TOK_TILE * 4;
+        static constexpr int ML = FB + ROWS * MAX_UNITS * 4;
         static constexpr int RECV = ML + ROWS * MAX_UNITS * 8;
         static constexpr int TOTAL = RECV + TOK_WARPS * D * (ROWS + 2) * 4;
-        static constexpr int FB = P;
-        static_assert(ROWS * MAX_UNITS * 4 <= ML - P, "the factors of the units lie over the probabilities");
         static_assert(TOK_CTAS * (TOTAL + 1024) <= 228 * 1024, "shared memory for as many CTAs as there are registers for");
     };
 };
@@ -121,6 +119,10 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a)
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
 }
+__device__ __forceinline__ void ldsm2(uint32_t &r0, uint32_t &r1, uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
+}
 __device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t a)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -131,6 +133,14 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// the same with c = 0
+__device__ __forceinline__ void mma16816_new(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // Two probabilities as sums of three bf16 values each (low halves: p0, high halves: p1).  The first two parts are taken
@@ -190,33 +200,103 @@ __device__ __forceinline__ void of_columns(float x, float &x0, float &x1)
     x1 = __shfl_sync(0xffffffffu, x, 8 * quad + 4);
 }
 
-// q k of one tile of 32 entries whose rows lie at kt: s[j][2 b + i], entry 8 j + 2 (lane % 4) + i of row 8 b + lane / 4
-template <int D, int NB>
-__device__ __forceinline__ void token_logits(float (&s)[4][4], const uint32_t (&qf)[D / 16][4], uint32_t kt)
+// A warp's query vectors, scaled by 1/8 - exactly, and close enough to 1/sqrt(d) that no product is larger than the logit's: as operands
+// in registers, or as rows in shared memory that are read again for every tile (where the accumulators need the registers).
+template <int D, int NB, bool SHARED> struct TokenQueries;
+template <int D, int NB> struct TokenQueries<D, NB, false> {
+    uint32_t f[D / 16][4];
+    __device__ __forceinline__ void put(int i, int c, int h, uint32_t x) { f[i][2 * c + h] = x; }
+    __device__ __forceinline__ void get(int i, uint32_t (&a)[4]) const
+    {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = f[i][k];
+    }
+};
+template <int D, int NB> struct TokenQueries<D, NB, true> {
+    static constexpr int BYTES = 8 * NB * D * 2;
+    uint32_t at;                                                   // [row][chunk ^ row % 8]
+    __device__ __forceinline__ void put(int i, int c, int h, uint32_t x)
+    {
+        const int lane = threadIdx.x & 31;
+        if (h < NB)
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(at + chunk_at<TokenCfg<D>::NC>(8 * h + (lane >> 2), 2 * i + c) + 4 * (lane & 3)), "r"(x) : "memory");
+    }
+    __device__ __forceinline__ void get(int i, uint32_t (&a)[4]) const
+    {
+        const int lane = threadIdx.x & 31;
+        if constexpr (NB == 2) {
+            ldsm4(a, at + chunk_at<TokenCfg<D>::NC>(lane & 15, 2 * i + (lane >> 4)));
+        } else {
+            ldsm2(a[0], a[2], at + chunk_at<TokenCfg<D>::NC>(lane & 7, 2 * i + ((lane >> 3) & 1)));
+            a[1] = a[3] = 0;
+        }
+    }
+};
+// The loads and what is made of them, apart: their round trip goes by in between.  row(r): where vector r lies in Q; `rows` of the 8 NB exist.
+template <int D, int NB> struct TokenRawQueries { uint32_t x[NB][D / 16][2]; };
+template <int D, int NB, typename Row>
+__device__ __forceinline__ void load_queries(TokenRawQueries<D, NB> &raw, const __nv_bfloat16 *Q, int rows, Row row)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 0; h < NB; ++h) {
+        const int r = 8 * h + (lane >> 2);
+        const __nv_bfloat16 *q = Q + (r < rows ? row(r) : 0) + 2 * (lane & 3);
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) raw.x[h][i][c] = r < rows ? *reinterpret_cast<const uint32_t *>(q + 16 * i + 8 * c) : 0u;
+    }
+}
+template <int D, int NB, bool SHARED> __device__ __forceinline__ void put_queries(TokenQueries<D, NB, SHARED> &qs, const TokenRawQueries<D, NB> &raw)
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                uint32_t x = 0;
+                if (h < NB) {
+                    const __nv_bfloat162 y = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x[h < NB ? h : 0][i][c]), __floats2bfloat162_rn(0.125f, 0.125f));
+                    x = *reinterpret_cast<const uint32_t *>(&y);
+                }
+                qs.put(i, c, h, x);
+            }
+}
+
+// q k of one tile of 32 entries whose rows lie at kt: s[j][2 b + i], entry 8 j + 2 (lane % 4) + i of row 8 b + lane / 4.  32 dimensions
+// at a time by the matrix instruction, their sums by fp32 additions (see token_contract).
+template <int D, int NB, bool SHARED>
+__device__ __forceinline__ void token_logits(float (&s)[4][4], const TokenQueries<D, NB, SHARED> &qs, uint32_t kt)
 {
     constexpr int NC = TokenCfg<D>::NC;
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) s[j][i] = 0.f;
-#pragma unroll
     for (int i = 0; i < D / 32; ++i) {
-        uint32_t b[4][4];
+        uint32_t b[4][4], qa[4], qb[4];
+        float t[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) ldsm4(b[j], kt + chunk_at<NC>(8 * j + (lane & 7), 4 * i + (lane >> 3)));
+        qs.get(2 * i, qa);
+        qs.get(2 * i + 1, qb);
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int j = 0; j < 4; ++j) mma16816_new(t[j], qa, b[j][0], b[j][1]);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) mma16816(s[j], qf[2 * i + h], b[j][2 * h], b[j][2 * h + 1]);
+        for (int j = 0; j < 4; ++j) mma16816(t[j], qb, b[j][2], b[j][3]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int k = 0; k < 2 * NB; ++k) s[j][k] = i == 0 ? t[j][k] : __fadd_rn(s[j][k], t[j][k]);
     }
 }
 
 // The tile's softmax: logits to probabilities.  t0 is its first entry, lw its log2 weights; the thread's rows see the entries
-// below lim[.], all rows of the group those below `common`.
+// below lim[.], all rows of the group those below `common`.  alpha: by what token_values scales the accumulators of rows
+// 8 b + 2 (lane % 4) + {0, 1}, unless the tile is the unit's first.
 template <int D, int NB>
 __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, float (&s)[4][4], const float *lw, int t0,
-                                              const int (&lim)[NB], int common, float scale)
+                                              const int (&lim)[NB], int common, float scale, uint64_t (&alpha)[NB])
 {
     const int quad = threadIdx.x & 3;
     const bool tail = t0 + TOK_TILE > common;                      // (the same for the whole warp)
@@ -243,16 +323,12 @@ __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, f
         mx = fmaxf(u.m[b], mx);
         const float ref = mx == -INFINITY ? 0.f : mx;
         if (!first) {
-            const float alpha = exp2f(u.m[b] - ref);
+            const float f = exp2f(u.m[b] - ref);
             // (rounded on its own: whether a compiler fuses it with the sum below must not depend on the form)
-            u.l[b] = __fmul_rn(u.l[b], alpha);
+            u.l[b] = __fmul_rn(u.l[b], f);
             float a0, a1;
-            of_columns(alpha, a0, a1);
-#pragma unroll
-            for (int j = 0; j < D / 16; ++j) {
-                u.o[j][b][0] *= a0; u.o[j][b][1] *= a1;
-                u.o[j][b][2] *= a0; u.o[j][b][3] *= a1;
-            }
+            of_columns(f, a0, a1);
+            alpha[b] = pack2(a0, a1);
         }
         u.m[b] = mx;
 #pragma unroll
@@ -265,97 +341,143 @@ __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, f
     }
 }
 
-// The tile's values, whose rows lie at vrows; some row of the group sees the entries below `last`, and those below `loaded` are
-// there (what other warps of the CTA see)
-template <int D, int NB>
-__device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, const float (&s)[4][4], const unsigned char *vrows, float *sp,
-                                             int t0, const int (&lim)[NB], int common, int last, int loaded)
+// The halves of x that are infinite or NaN as masks of ones: an exponent of all ones carries into the sign's place
+__device__ __forceinline__ uint32_t not_finite(uint32_t x) { return (((x & 0x7f807f80u) + 0x00800080u) >> 15 & 0x00010001u) * 0xffffu; }
+
+// O^T += V^T P^T of a tile: the unit's accumulators times alpha (not if the tile is the first) plus the tile's products.
+// The matrix instruction rounds toward zero, every time by up to a bit of what it has accumulated so far.  So a tile's sums start
+// at zero, take the small parts first, and go to the unit's accumulators by fp32 fma (one accumulator through a warp's whole share of a
+// list: relative error 5.0e-7 over 5193 entries, 1.9e-6 over 12288; fp32 fma alone 2.1e-7 and 3.6e-7; so 1.8e-7 and 2.3e-7).
+// `odd`: entries of which the values that are not finite are taken as zeros.
+template <int D, int NB, bool ODD>
+__device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], const float (&s)[4][4],
+                                               uint32_t vt, uint32_t odd)
 {
     using C = TokenCfg<D>;
-    constexpr int NC = C::NC;
     const int lane = threadIdx.x & 31, quad = lane & 3;
-    const uint32_t vt = smem_u32(vrows);
-    // Entries that only some rows see, or none: one with an infinity or a NaN must not meet the zero probabilities of the others in the
-    // matrix instruction.  Its values are taken as zero there and added by scalar code to the rows that see it.
-    const int e0 = common > t0 ? common - t0 : 0, e1 = loaded - t0 < TOK_TILE ? loaded - t0 : TOK_TILE;
-    uint32_t bad = 0;
-    if (e0 < e1) {
-        for (int i = lane; i < (e1 - e0) * NC; i += 32) {
-            const uint4 x = *reinterpret_cast<const uint4 *>(vrows + chunk_at<NC>(e0 + i / NC, i % NC));
-            // an exponent of all ones carries into the sign's place
-            const uint32_t y = ((x.x & 0x7f807f80u) + 0x00800080u) | ((x.y & 0x7f807f80u) + 0x00800080u) |
-                               ((x.z & 0x7f807f80u) + 0x00800080u) | ((x.w & 0x7f807f80u) + 0x00800080u);
-            if (y & 0x80008000u) bad |= 1u << (e0 + i / NC);
-        }
-        bad = __reduce_or_sync(0xffffffffu, bad);
-    }
+    uint32_t p[2][NB][3][2];                                           // [k]: entries 16 k + {0, 8} + 2 (lane % 4) + {0, 1} of row 8 b + lane / 4
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        uint32_t p[NB][3][2];                                          // entries 16 k + {0, 8} + 2 (lane % 4) + {0, 1} of row 8 b + lane / 4
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int b = 0; b < NB; ++b)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-                split3(s[2 * k + h][2 * b], s[2 * k + h][2 * b + 1], p[b][0][h], p[b][1][h], p[b][2][h]);
-        auto mask_of = [&](int e) { return (bad >> e & 1 ? 0u : 0xffffu) | (bad >> (e + 1) & 1 ? 0u : 0xffff0000u); };
-        const uint32_t k0 = mask_of(16 * k + 2 * quad), k1 = mask_of(16 * k + 8 + 2 * quad);
-        // matrices of a load: entries 16 k + {0, 0, 8, 8} + 0..7, chunks {0, 1, 0, 1} of the 16 columns
-        const uint32_t va = vt + (uint32_t)((16 * k + (lane >> 4) * 8 + (lane & 7)) * C::RB);
-        const int sw = lane & 7, half = (lane >> 3) & 1;
-#pragma unroll
-        for (int j = 0; j < D / 16; j += 2) {
-            uint32_t a[2][4];
-#pragma unroll
             for (int h = 0; h < 2; ++h) {
-                ldsm4_t(a[h], va + (uint32_t)(((2 * (j + h) + half) ^ sw) * 16));
-                if (bad) {
-                    a[h][0] &= k0; a[h][1] &= k0;
-                    a[h][2] &= k1; a[h][3] &= k1;
+                split3(s[2 * k + h][2 * b], s[2 * k + h][2 * b + 1], p[k][b][0][h], p[k][b][1][h], p[k][b][2][h]);
+            }
+    constexpr int JG = 4;                                              // output tiles at a time
+    const int sw = lane & 7, half = (lane >> 3) & 1;
+#pragma unroll
+    for (int j = 0; j < D / 16; j += JG) {
+        uint32_t a[2][JG][4];
+        float t[JG][NB][4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            // matrices of a load: entries 16 k + {0, 0, 8, 8} + 0..7, chunks {0, 1, 0, 1} of the 16 columns
+            const uint32_t va = vt + (uint32_t)((16 * k + (lane >> 4) * 8 + (lane & 7)) * C::RB);
+#pragma unroll
+            for (int h = 0; h < JG; ++h) {
+                ldsm4_t(a[k][h], va + (uint32_t)(((2 * (j + h) + half) ^ sw) * 16));
+                if constexpr (ODD) {
+                    auto mask_of = [&](int e) { return (odd >> e & 1 ? 0xffffu : 0u) | (odd >> (e + 1) & 1 ? 0xffff0000u : 0u); };
+                    const uint32_t k0 = mask_of(16 * k + 2 * quad), k1 = mask_of(16 * k + 8 + 2 * quad);
+                    a[k][h][0] &= ~(not_finite(a[k][h][0]) & k0); a[k][h][1] &= ~(not_finite(a[k][h][1]) & k0);
+                    a[k][h][2] &= ~(not_finite(a[k][h][2]) & k1); a[k][h][3] &= ~(not_finite(a[k][h][3]) & k1);
                 }
             }
-#pragma unroll
-            for (int part = 0; part < 3; ++part)
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) mma16816(u.o[j + h][b], a[h], p[b][part][0], p[b][part][1]);
         }
-    }
-    if (bad) {
-        __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int part = 2; part >= 0; --part)
 #pragma unroll
-            for (int i = 0; i < 2 * NB; ++i) {
-                const int e = 8 * j + 2 * quad + (i & 1);
-                if (e >= e0 && t0 + e < last) sp[((lane >> 2) + 8 * (i >> 1)) * C::P_STRIDE + e - e0] = s[j][i];
-            }
-        __syncwarp();
-        for (int e = e0; e < e1 && t0 + e < last; ++e) {
-            if (!(bad >> e & 1)) continue;
-            float v[D / 8];
+            for (int k = 0; k < 2; ++k)
 #pragma unroll
-            for (int j = 0; j < D / 8; ++j)
-                v[j] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(vrows + chunk_at<NC>(e, j) + 2 * (lane >> 2)));
+                for (int h = 0; h < JG; ++h)
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        if (part == 2 && k == 0) mma16816_new(t[h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
+                        else mma16816(t[h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
+                    }
+#pragma unroll
+        for (int h = 0; h < JG; ++h)
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-                int lim2[2];
-                lim2[0] = __shfl_sync(0xffffffffu, lim[b], 8 * quad);
-                lim2[1] = __shfl_sync(0xffffffffu, lim[b], 8 * quad + 4);
+                float (&o)[4] = u.o[j + h][b];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const float pe = sp[(8 * b + 2 * quad + i) * C::P_STRIDE + e - e0];
-                    if (t0 + e < lim2[i]) {
-#pragma unroll
-                        for (int j = 0; j < D / 16; ++j) {
-                            u.o[j][b][i] = fmaf(pe, v[2 * j], u.o[j][b][i]);
-                            u.o[j][b][2 + i] = fmaf(pe, v[2 * j + 1], u.o[j][b][2 + i]);
-                        }
+                for (int i = 0; i < 4; i += 2) {
+                    if (first) {
+                        o[i] = t[h][b][i];
+                        o[i + 1] = t[h][b][i + 1];
+                    } else {
+                        unpack2(fma2(pack2(o[i], o[i + 1]), alpha[b], pack2(t[h][b][i], t[h][b][i + 1])), o[i], o[i + 1]);
                     }
                 }
             }
+    }
+}
+
+// A tile with entries that do not go through the matrix instruction alone (rare, so on a copy of the accumulators in local memory and
+// out of line): the values that are not finite are added by scalar code to the rows that see the entry.
+template <int D, int NB> struct TokenOdd {
+    TokenUnit<D, NB> u;
+    uint64_t alpha[NB];
+    float s[4][4];
+    int lim[NB];
+};
+template <int D, int NB> __device__ __noinline__ void token_values_odd(TokenOdd<D, NB> *x, bool first, const unsigned char *vrows, int t0, uint32_t odd)
+{
+    using C = TokenCfg<D>;
+    const int lane = threadIdx.x & 31, quad = lane & 3;
+    token_contract<D, NB, true>(x->u, first, x->alpha, x->s, smem_u32(vrows), odd);
+    for (uint32_t left = odd; left; left &= left - 1) {
+        const int e = __ffs(left) - 1;
+        for (int b = 0; b < NB; ++b)
+            for (int i = 0; i < 2; ++i) {
+                const int from = 8 * quad + 4 * i;                     // the first lane that holds the row's probabilities
+                const float pe = __shfl_sync(0xffffffffu, x->s[e >> 3][2 * b + (e & 1)], from + ((e & 7) >> 1));
+                const bool sees = t0 + e < __shfl_sync(0xffffffffu, x->lim[b], from);
+                for (int j = 0; j < D / 8; ++j) {                      // column lane / 4 + 8 j
+                    const uint32_t v = (uint32_t)*reinterpret_cast<const uint16_t *>(vrows + chunk_at<C::NC>(e, j) + 2 * (lane >> 2)) << 16;
+                    float &o = x->u.o[j >> 1][b][2 * (j & 1) + i];
+                    if (sees && not_finite(v)) o = fmaf(pe, __uint_as_float(v), o);
+                }
+            }
+    }
+}
+
+// The tile's values, whose rows lie at vrows; the thread's rows see the entries below lim[.], all rows of the group those
+// below `common`, and those below `loaded` are there (what other warps of the CTA see).
+template <int D, int NB>
+__device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], const float (&s)[4][4],
+                                             const unsigned char *vrows, int t0, const int (&lim)[NB], int common, int loaded)
+{
+    constexpr int NC = TokenCfg<D>::NC;
+    const int lane = threadIdx.x & 31;
+    // Entries whose values do not go through the matrix instruction alone.  One that only some rows see, or none, and that holds an infinity
+    // or a NaN must not meet the zero probabilities of the others.  No row's arithmetic depends on another's.
+    uint32_t odd = 0;
+    const int e0 = common > t0 ? common - t0 : 0, e1 = loaded - t0 < TOK_TILE ? loaded - t0 : TOK_TILE;
+    if (e0 < e1) {
+        for (int i = lane; i < (e1 - e0) * NC; i += 32) {
+            const uint4 x = *reinterpret_cast<const uint4 *>(vrows + chunk_at<NC>(e0 + i / NC, i % NC));
+            if (not_finite(x.x) | not_finite(x.y) | not_finite(x.z) | not_finite(x.w)) odd |= 1u << (e0 + i / NC);
         }
-        __syncwarp();
+        odd = __reduce_or_sync(0xffffffffu, odd);
+    }
+    if (odd) {
+        TokenOdd<D, NB> x;
+        x.u = u;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            x.alpha[b] = first ? 0 : alpha[b];
+            x.lim[b] = lim[b];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 2 * NB; ++i) x.s[j][i] = s[j][i];
+        token_values_odd(&x, first, vrows, t0, odd);
+        u = x.u;
+    } else {
+        token_contract<D, NB, false>(u, first, alpha, s, smem_u32(vrows), 0);
     }
 }
 
@@ -404,28 +526,13 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
         return ((z * (gridDim.y / kv_heads) + b) * q_heads + kvh * rep + r % per_token) * D;
     };
     int lim[NB];
-    // the query vectors as operands, scaled by 1/8: exactly, and close enough to 1/sqrt(d) that no product is larger than
-    // the logit's
-    uint32_t qf[D / 16][4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int r = 8 * h + (lane >> 2);
-        const bool live = h < NB && r < rows;
-        if (h < NB) lim[h < NB ? h : 0] = live ? first + r / per_token : 0;
-        const __nv_bfloat16 *q = Q + (live ? q_row(r) : 0) + 2 * quad;
-#pragma unroll
-        for (int i = 0; i < D / 16; ++i)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                __nv_bfloat162 x = __floats2bfloat162_rn(0.f, 0.f);
-                if (live) x = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(q + 16 * i + 8 * c), __floats2bfloat162_rn(0.125f, 0.125f));
-                qf[i][2 * c + h] = *reinterpret_cast<const uint32_t *>(&x);
-            }
-    }
+    for (int h = 0; h < NB; ++h) lim[h] = 8 * h + (lane >> 2) < rows ? first + (8 * h + (lane >> 2)) / per_token : 0;
+    TokenRawQueries<D, NB> raw;
+    TokenQueries<D, NB, !CLUSTER> qs;
     const float scale = 8.f * 1.4426950408889634f / sqrtf((float)D);
     const int unit_tiles = token_units(n_span, grp.caps);
     const int tiles = (n_span + TOK_TILE - 1) / TOK_TILE;
-    float *sp = reinterpret_cast<float *>(smem + (CLUSTER ? CC::P : C::S_P)) + warp * TOK_ROWS * C::P_STRIDE;
     TokenUnit<D, NB> u;
 
     if constexpr (CLUSTER) {
@@ -458,26 +565,29 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
         const int t_end = min((unit + 1) * unit_tiles, tiles);
         int t = unit * unit_tiles;
         u.reset();
+        if (t < t_end) fetch_entries(t);
+        load_queries(raw, Q, rows, q_row);
         if (t < t_end) {
-            fetch_entries(t);
             copy_rows(kt, Kp, row, t);
             copy_rows(vt, Vp, row, t);
         }
+        put_queries(qs, raw);
         for (bool head = true; t < t_end; ++t, head = false) {
             const bool more = t + 1 < t_end;
             float s[4][4];
+            uint64_t alpha[NB];
             lw[lane] = log2f(wt);
             if (more) fetch_entries(t + 1);
             cp_async_wait<1>();                                        // the keys (the values are the newer group)
             __syncwarp();
-            token_logits<D, NB>(s, qf, smem_u32(kt));
+            token_logits(s, qs, smem_u32(kt));
             __syncwarp();
             if (more) copy_rows(kt, Kp, row, t + 1);
-            token_softmax<D, NB>(u, head, s, lw, t * TOK_TILE, lim, aligned, scale);
+            token_softmax<D, NB>(u, head, s, lw, t * TOK_TILE, lim, aligned, scale, alpha);
             if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
             else cp_async_wait<0>();
             __syncwarp();
-            token_values<D, NB>(u, s, vt, sp, t * TOK_TILE, lim, aligned, last, n_span);
+            token_values<D, NB>(u, head, alpha, s, vt, t * TOK_TILE, lim, aligned, n_span);
             __syncwarp();
             if (more) copy_rows(vt, Vp, row, t + 1);
         }
@@ -567,6 +677,10 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
         }
     } else {
         // ---- the tiles one after the other, for the four groups of the CTA ----
+        qs.at = smem_u32(smem + C::S_Q + warp * TokenQueries<D, NB, true>::BYTES);
+        load_queries(raw, Q, rows, q_row);
+        put_queries(qs, raw);
+        __syncwarp();
         constexpr int RPP = TOK_THREADS / NC, PASSES = TOK_TILE / RPP;
         const int my_row = tid / NC, my_chunk = tid % NC;
         const uint32_t ring = smem_u32(smem);
@@ -623,9 +737,10 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             if (in_unit == 0) u.reset();
             if (t * TOK_TILE < last) {                                 // (behind what the group sees there is nothing to add)
                 float s[4][4];
-                token_logits<D, NB>(s, qf, smem_u32(kt));
-                token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale);
-                token_values<D, NB>(u, s, kt + C::TILE_BYTES, sp, t * TOK_TILE, lim, aligned, last, n_span);
+                uint64_t alpha[NB];
+                token_logits(s, qs, smem_u32(kt));
+                token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale, alpha);
+                token_values<D, NB>(u, in_unit == 0, alpha, s, kt + C::TILE_BYTES, t * TOK_TILE, lim, aligned, n_span);
             }
             if (++in_unit == unit_tiles || t + 1 == tiles) {
                 in_unit = 0;
@@ -718,43 +833,35 @@ tokens_split_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
     };
     TokenUnit<D, 1> u;
     u.reset();
+    if (t < t_end) fetch_entries(t);
+    TokenRawQueries<D, 1> raw;
+    load_queries(raw, Q, rows, [&](int r) -> int64_t { return (((int64_t)b * q_heads + kvh * rep + r / n_q) * n_q + r % n_q) * D; });
     if (t < t_end) {
-        fetch_entries(t);
         copy_rows(kt, Kp, row, t);
         copy_rows(vt, Vp, row, t);
     }
-    // the query vectors as operands, scaled by 1/8: exactly
-    uint32_t qf[D / 16][4];
-    {
-        const int r = lane >> 2;
-        const __nv_bfloat16 *q = Q + (r < rows ? (((int64_t)b * q_heads + kvh * rep + r / n_q) * n_q + r % n_q) * D : 0) + 2 * quad;
-#pragma unroll
-        for (int i = 0; i < D / 16; ++i)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                __nv_bfloat162 x = __floats2bfloat162_rn(0.f, 0.f);
-                if (r < rows) x = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(q + 16 * i + 8 * c), __floats2bfloat162_rn(0.125f, 0.125f));
-                qf[i][2 * c] = *reinterpret_cast<const uint32_t *>(&x);
-                qf[i][2 * c + 1] = 0u;
-            }
-    }
+    TokenQueries<D, 1, true> qs;
+    qs.at = smem_u32(smem + C::P_Q + warp * TokenQueries<D, 1, true>::BYTES);
+    put_queries(qs, raw);
+    __syncwarp();
     const float scale = 8.f * 1.4426950408889634f / sqrtf((float)D);
     const int lim[1] = {n_core};
     for (bool head = true; t < t_end; t += TOK_WARPS, head = false) {
         const bool more = t + TOK_WARPS < t_end;
         float s[4][4];
+        uint64_t alpha[1];
         lw[lane] = log2f(wt);
         if (more) fetch_entries(t + TOK_WARPS);
         cp_async_wait<1>();                                        // the keys (the values are the newer group)
         __syncwarp();
-        token_logits<D, 1>(s, qf, smem_u32(kt));
+        token_logits(s, qs, smem_u32(kt));
         __syncwarp();
         if (more) copy_rows(kt, Kp, row, t + TOK_WARPS);
-        token_softmax<D, 1>(u, head, s, lw, t * TOK_TILE, lim, n_core, scale);
+        token_softmax<D, 1>(u, head, s, lw, t * TOK_TILE, lim, n_core, scale, alpha);
         if (more) cp_async_wait<1>();
         else cp_async_wait<0>();
         __syncwarp();
-        token_values<D, 1>(u, s, vt, nullptr, t * TOK_TILE, lim, n_core, n_core, n_core);
+        token_values<D, 1>(u, head, alpha, s, vt, t * TOK_TILE, lim, n_core, n_core);
         __syncwarp();
         if (more) copy_rows(vt, Vp, row, t + TOK_WARPS);
     }

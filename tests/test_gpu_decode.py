@@ -141,6 +141,43 @@ def test_bf16_tokens_match_exact_attention(d, rep, hkv, log2_nout, start):
         assert ((after - got).abs() <= 2.0 ** -7 * got.abs().amax(-1, keepdim=True)).all()
 
 
+@pytest.mark.parametrize("d,B,H,rep,n_core", [(128, 4, 8, 4, 5193), (128, 8, 8, 4, 12288), (64, 8, 8, 8, 12288), (128, 1, 8, 5, 2048)])
+def test_partial_results_of_decode_are_as_precise_as_fp32_fma(d, B, H, rep, n_core):
+    """The partial results that the split form leaves at the front of the workspace ([problem][split][vector][accumulator, maximum,
+    denominator]), put together in 64 bits, against attention in 64 bits."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    K, V, Q = (torch.randn(s, device="cuda", generator=g).bfloat16() for s in ((B, H, n_core, d), (B, H, n_core, d), (B, H * rep, 1, d)))
+    idx = torch.arange(n_core, device="cuda", dtype=torch.int32).repeat(B, H, 1)
+    w = torch.rand(B, H, n_core, device="cuda", generator=g) + 0.05
+    ws = torch.zeros(1 << 30, device="cuda", dtype=torch.uint8)
+    elm.attend(Q, K, V, idx, w, workspace=ws)
+    ctas, _ = binding.debug_decode_grid(B, H * rep, H, n_core, d, n_core)
+    splits, vectors = ctas // (B * H), 4 if rep <= 4 else 8
+    part = ws.view(torch.float32)[:ctas * vectors * (d + 2)].view(B, H, splits, vectors, d + 2)[:, :, :, :rep].double()
+    f = torch.exp2(part[..., d] - part[..., d].amax(2, keepdim=True))
+    got = (f.unsqueeze(-1) * part[..., :d]).sum(2) / (f * part[..., d + 1]).sum(2).unsqueeze(-1)
+    s = Q.double().view(B, H, rep, d) @ K.double().transpose(-1, -2) / d ** 0.5 + w.double().log().unsqueeze(2)
+    want = torch.softmax(s, dim=-1) @ V.double()
+    # fp32 sums of terms that mostly cancel: 8 roundings to 24 bits (fp32 fma: 2.1e-7 and, over 12288 entries, 3.6e-7)
+    assert (got - want).norm() / want.norm() <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("d,rep", [(128, 4), (128, 1), (64, 4)])
+def test_streamed_bf16_outputs_are_mostly_the_rounded_exact_value(d, rep):
+    """Neighbouring bf16 values are 2^-8 to 2^-7 of themselves apart, and outputs are many times smaller than what fp32 sums: errors of 2^-22
+    of an output put about one in 2^12 on the other side of a rounding."""
+    x = _Exact(torch.bfloat16, d, rep, 8, 11, 6000, 512)
+    got = x.one_call(144)
+    K, V = (t.double().repeat_interleave(rep, dim=1) for t in (x.s.K, x.s.V))
+    wrong = 0
+    for t in range(0, 144, 16):
+        s = torch.einsum("tbhqd,bhnd->tbhqn", x.Q[t:t + 16].double(), K) / d ** 0.5
+        s = s.masked_fill(torch.arange(6512, device="cuda") > 6000 + t + torch.arange(16, device="cuda")[:, None, None, None, None], -torch.inf)
+        want = torch.einsum("tbhqn,bhnd->tbhqd", torch.softmax(s, dim=-1), V).bfloat16()
+        wrong += (got[t:t + 16] != want).sum().item()
+    assert wrong / got.numel() <= 1.2 * 2.0 ** -12
+
+
 def test_debug_limit_of_clusters_refuses_other_sizes():
     lib = binding.load_library()
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
