@@ -145,7 +145,9 @@ __device__ __forceinline__ void mma16816_new(float (&c)[4], const uint32_t (&a)[
 
 // Two probabilities as sums of three bf16 values each (low halves: p0, high halves: p1).  The first two parts are taken
 // just below what they stand for, so that all parts of a positive value are positive: an infinite value of V stays that
-// infinity instead of meeting a part that is zero or negative.
+// infinity instead of meeting a part that is zero or negative.  So it is for values of 2^-100 and more, whose last bit and with it
+// the smallest part is a normal bf16 value; smaller ones do not come here (token_values).
+constexpr uint32_t SMALLEST_SPLIT = 27u << 23;                     // the bits of 2^-100
 __device__ __forceinline__ void split3(float p0, float p1, uint32_t &hi, uint32_t &mid, uint32_t &lo)
 {
     const uint32_t h0 = (max(__float_as_uint(p0), 1u) - 1u) & 0xffff0000u, h1 = (max(__float_as_uint(p1), 1u) - 1u) & 0xffff0000u;
@@ -343,12 +345,14 @@ __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, f
 
 // The halves of x that are infinite or NaN as masks of ones: an exponent of all ones carries into the sign's place
 __device__ __forceinline__ uint32_t not_finite(uint32_t x) { return (((x & 0x7f807f80u) + 0x00800080u) >> 15 & 0x00010001u) * 0xffffu; }
+// Probabilities that are too small to be split, and not zero
+__device__ __forceinline__ bool too_small(float p) { return __float_as_uint(p) - 1u < SMALLEST_SPLIT - 1u; }
 
 // O^T += V^T P^T of a tile: the unit's accumulators times alpha (not if the tile is the first) plus the tile's products.
 // The matrix instruction rounds toward zero, every time by up to a bit of what it has accumulated so far.  So a tile's sums start
 // at zero, take the small parts first, and go to the unit's accumulators by fp32 fma (one accumulator through a warp's whole share of a
 // list: relative error 5.0e-7 over 5193 entries, 1.9e-6 over 12288; fp32 fma alone 2.1e-7 and 3.6e-7; so 1.8e-7 and 2.3e-7).
-// `odd`: entries of which the values that are not finite are taken as zeros.
+// `odd`: entries of which the values that are not finite are taken as zeros, and so are probabilities that cannot be split.
 template <int D, int NB, bool ODD>
 __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], const float (&s)[4][4],
                                                uint32_t vt, uint32_t odd)
@@ -362,7 +366,12 @@ __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, 
         for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                split3(s[2 * k + h][2 * b], s[2 * k + h][2 * b + 1], p[k][b][0][h], p[k][b][1][h], p[k][b][2][h]);
+                float x = s[2 * k + h][2 * b], y = s[2 * k + h][2 * b + 1];
+                if constexpr (ODD) {
+                    x = too_small(x) ? 0.f : x;
+                    y = too_small(y) ? 0.f : y;
+                }
+                split3(x, y, p[k][b][0][h], p[k][b][1][h], p[k][b][2][h]);
             }
     constexpr int JG = 4;                                              // output tiles at a time
     const int sw = lane & 7, half = (lane >> 3) & 1;
@@ -415,7 +424,8 @@ __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, 
 }
 
 // A tile with entries that do not go through the matrix instruction alone (rare, so on a copy of the accumulators in local memory and
-// out of line): the values that are not finite are added by scalar code to the rows that see the entry.
+// out of line).  What such an entry needs is added by scalar code: to the rows whose probability is too small to be split all its
+// values, to the other rows that see it the values that are not finite.
 template <int D, int NB> struct TokenOdd {
     TokenUnit<D, NB> u;
     uint64_t alpha[NB];
@@ -433,11 +443,11 @@ template <int D, int NB> __device__ __noinline__ void token_values_odd(TokenOdd<
             for (int i = 0; i < 2; ++i) {
                 const int from = 8 * quad + 4 * i;                     // the first lane that holds the row's probabilities
                 const float pe = __shfl_sync(0xffffffffu, x->s[e >> 3][2 * b + (e & 1)], from + ((e & 7) >> 1));
-                const bool sees = t0 + e < __shfl_sync(0xffffffffu, x->lim[b], from);
+                const bool sees = t0 + e < __shfl_sync(0xffffffffu, x->lim[b], from), all = too_small(pe);
                 for (int j = 0; j < D / 8; ++j) {                      // column lane / 4 + 8 j
                     const uint32_t v = (uint32_t)*reinterpret_cast<const uint16_t *>(vrows + chunk_at<C::NC>(e, j) + 2 * (lane >> 2)) << 16;
                     float &o = x->u.o[j >> 1][b][2 * (j & 1) + i];
-                    if (sees && not_finite(v)) o = fmaf(pe, __uint_as_float(v), o);
+                    if (sees && (all || not_finite(v))) o = fmaf(pe, __uint_as_float(v), o);
                 }
             }
     }
@@ -450,10 +460,11 @@ __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, co
                                              const unsigned char *vrows, int t0, const int (&lim)[NB], int common, int loaded)
 {
     constexpr int NC = TokenCfg<D>::NC;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, quad = lane & 3;
     // Entries whose values do not go through the matrix instruction alone.  One that only some rows see, or none, and that holds an infinity
-    // or a NaN must not meet the zero probabilities of the others.  No row's arithmetic depends on another's.
-    uint32_t odd = 0;
+    // or a NaN must not meet the zero probabilities of the others; a probability that three bf16 parts cannot hold (below 2^-100, for
+    // which a logit has to lie 69 below the largest of its unit) must meet its values in fp32.  No row's arithmetic depends on another's.
+    uint32_t odd = 0, least = 0xffffffffu;
     const int e0 = common > t0 ? common - t0 : 0, e1 = loaded - t0 < TOK_TILE ? loaded - t0 : TOK_TILE;
     if (e0 < e1) {
         for (int i = lane; i < (e1 - e0) * NC; i += 32) {
@@ -461,6 +472,19 @@ __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, co
             if (not_finite(x.x) | not_finite(x.y) | not_finite(x.z) | not_finite(x.w)) odd |= 1u << (e0 + i / NC);
         }
         odd = __reduce_or_sync(0xffffffffu, odd);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 2 * NB; ++i) least = min(least, __float_as_uint(s[j][i]) - 1u);
+    if (__any_sync(0xffffffffu, least < SMALLEST_SPLIT - 1u)) {
+        uint32_t small = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 2 * NB; ++i)
+                if (too_small(s[j][i])) small |= 1u << (8 * j + 2 * quad + (i & 1));
+        odd |= __reduce_or_sync(0xffffffffu, small);
     }
     if (odd) {
         TokenOdd<D, NB> x;

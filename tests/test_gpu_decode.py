@@ -178,6 +178,40 @@ def test_streamed_bf16_outputs_are_mostly_the_rounded_exact_value(d, rep):
     assert wrong / got.numel() <= 1.2 * 2.0 ** -12
 
 
+@pytest.mark.parametrize("gap", [6.0, 7.0, 8.0, 8.75])             # the entry's probability: about 2^-101, 2^-117, 2^-134, 2^-146
+@pytest.mark.parametrize("d,rep", [(64, 1), (128, 3), (128, 8)])
+def test_infinite_values_at_vanishing_probabilities(d, rep, gap):
+    """An entry far below the others: its infinite values reach the output as infinities as long as fp32 holds its probability, a value
+    of 1e38 with its share, and the other columns as always - in decode, in single tokens and beside tokens that see the entry with
+    an ordinary probability."""
+    H, at, n = 2, 70, 700
+    x = _Exact(torch.bfloat16, d, rep, H, 8, n, 70)
+    K, V, Q = x.s.K, x.s.V, x.Q
+    K *= 0.125
+    K[:, :, at] = -gap * (128 / d) ** 0.5
+    V[:, :, at, 3], V[:, :, at, 5], V[:, :, at, 7] = torch.inf, -torch.inf, 1e38
+    ordinary = torch.arange(70, device="cuda") % 5 == 2
+    Q[~ordinary] = 1.0
+    Q[ordinary] *= 0.125
+    Kd, Vd = (t.double().repeat_interleave(rep, dim=1) for t in (K, V))
+    Vd[..., at, 3] = Vd[..., at, 5] = 0
+
+    def check(got, q, seen):
+        s = q.double() @ Kd[:, :, :seen].transpose(-1, -2) / d ** 0.5
+        want = torch.softmax(s, dim=-1) @ Vd[:, :, :seen]
+        assert (got[..., 3] == torch.inf).all() and (got[..., 5] == -torch.inf).all()
+        for c in (slice(0, 3), slice(4, 5), slice(6, 7), slice(7, 8), slice(8, d)):
+            # rounded to 8 bits; 2^-20: columns that come out near zero
+            assert ((got[..., c].double() - want[..., c]).abs().amax(-1) <= 2.0 ** -8 * want[..., c].abs().amax(-1) + 2.0 ** -20).all()
+
+    together = x.one_call(60)
+    assert torch.equal(together, x.single_steps(60))
+    for t in (0, 1, 2, 37, 59):
+        check(together[t], Q[t], n + t + 1)
+    idx = torch.arange(n, device="cuda", dtype=torch.int32).repeat(1, H, 1)
+    check(elm.attend(Q[0], K, V, idx, torch.ones(1, H, n, device="cuda")), Q[0], n)
+
+
 def test_debug_limit_of_clusters_refuses_other_sizes():
     lib = binding.load_library()
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
