@@ -611,10 +611,10 @@ template <int D> int decode_largest_cluster()
     const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
     return limit && limit < largest ? limit : largest;
 }
-TokenCaps decode_token_caps(const elm_params *p)
+TokenCaps decode_token_caps(const elm_params *p, int problems)
 {
     const int limit = g_debug_largest_cluster.load(std::memory_order_relaxed);
-    return tokens_caps(p->d, p->batch * p->kv_heads, limit ? limit : DEC_MAX_CLUSTER);
+    return tokens_caps(p->d, problems, limit ? limit : DEC_MAX_CLUSTER);
 }
 
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
@@ -824,7 +824,7 @@ int dispatch_decode(const void *Q, const void *K, const void *V, const int32_t *
     if (win) {
         const int problems = p->batch * p->kv_heads;
         if constexpr (std::is_same<Tin, __nv_bfloat16>::value)
-            return attend_tokens_bf16(Q, K, V, idx, w, list_stride, *win, p, O, status, decode_token_caps(p), st);
+            return attend_tokens_bf16(Q, K, V, idx, w, list_stride, *win, p, O, status, decode_token_caps(p, problems), st);
         else
             form = decode_form<Tin, D>(*win, problems, per_token);
     }
@@ -861,7 +861,11 @@ bool attend_decode_windows_apply(const elm_params *p, int n_core)
         return p->d == 64 ? decode_clustered(n_core, problems, decode_cap<64>(problems, per_token, sms), DEC_WARPS * DEC_TILE<float, 64>)
                           : decode_clustered(n_core, problems, decode_cap<128>(problems, per_token, sms), DEC_WARPS * DEC_TILE<float, 128>);
     }
-    return decode_clustered(n_core, problems, decode_token_caps(p).of_long, 128);
+    // Clusters cut short because the device cannot hold all problems' longer ones at once leave few SMs idle, although their CTAs may be
+    // fewer than the SMs.  16 problems (clusters of 8) of 4 query vectors, 9000 entries: one token 23.6 us for 16.9 token by token, but
+    // two 25.0 for 33.2 and 128 554 for 2088; 36 problems (clusters of 4), 4100 entries: 23.4 / 16.7, 24.7 / 32.5, 680 / 2060.
+    const int cap = decode_token_caps(p, problems).of_long;
+    return decode_clustered(n_core, problems, cap, 128) || cap < decode_token_caps(p, 1).of_long;
 }
 
 namespace {

@@ -212,6 +212,17 @@ def test_infinite_values_at_vanishing_probabilities(d, rep, gap):
     check(elm.attend(Q[0], K, V, idx, torch.ones(1, H, n, device="cuda")), Q[0], n)
 
 
+@pytest.mark.parametrize("B,H,rep,log2_nout,start", [(2, 8, 4, 12, 9000), (2, 9, 1, 12, 8300), (9, 4, 2, 11, 4500), (2, 8, 8, 12, 9000)])
+def test_streams_of_many_problems_share_their_launches(B, H, rep, log2_nout, start):
+    """Problems whose longer clusters the device cannot hold all at once, lists beyond eight rounds of the shorter ones: the tokens
+    of a call still take two launches, the list and the attention, and agree with single steps."""
+    x = _Exact(torch.bfloat16, 128, rep, H, log2_nout, start, 64, B)
+    before = elm.launch_count()
+    got = x.one_call(60)
+    assert elm.launch_count() - before == 2
+    assert torch.equal(got, x.single_steps(60))
+
+
 def test_debug_limit_of_clusters_refuses_other_sizes():
     lib = binding.load_library()
     assert all(lib.elm_debug_set(2, v) != 0 for v in (-1, 3, 12, 32))
