@@ -34,6 +34,7 @@
 namespace elm {
 namespace {
 
+using sm100::add2;
 using sm100::fma2;
 using sm100::mul2;
 using sm100::pack2;
@@ -274,7 +275,14 @@ __device__ __forceinline__ void token_logits(float (&s)[4][4], const TokenQuerie
 {
     constexpr int NC = TokenCfg<D>::NC;
     const int lane = threadIdx.x & 31;
+    // The split form leaves this loop one: unrolled, its loads are all moved to the front, where they push accumulators out of the registers
+    // (64 problems of 5193 entries 40.0 us, so 32.8; the serial form 258 unrolled, 267 not: 128 tokens over 4100 entries).
+    constexpr bool ONE_LOOP = SHARED && NB == 1;
+    if constexpr (ONE_LOOP) {
 #pragma unroll
+        for (int j = 0; j < 4; ++j) s[j][0] = s[j][1] = 0.f;
+    }
+#pragma unroll(ONE_LOOP ? 1 : D / 32)
     for (int i = 0; i < D / 32; ++i) {
         uint32_t b[4][4], qa[4], qb[4];
         float t[4][4];
@@ -289,19 +297,23 @@ __device__ __forceinline__ void token_logits(float (&s)[4][4], const TokenQuerie
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int k = 0; k < 2 * NB; ++k) s[j][k] = i == 0 ? t[j][k] : __fadd_rn(s[j][k], t[j][k]);
+            for (int k = 0; k < 2 * NB; k += 2) {
+                const uint64_t x = pack2(t[j][k], t[j][k + 1]);
+                unpack2(!ONE_LOOP && i == 0 ? x : add2(pack2(s[j][k], s[j][k + 1]), x), s[j][k], s[j][k + 1]);
+            }
     }
 }
 
 // The tile's softmax: logits to probabilities.  t0 is its first entry, lw its log2 weights; the thread's rows see the entries
 // below lim[.], all rows of the group those below `common`.  alpha: by what token_values scales the accumulators of rows
-// 8 b + 2 (lane % 4) + {0, 1}, unless the tile is the unit's first.
+// 8 b + 2 (lane % 4) + {0, 1}, unless the tile is the unit's first.  low: the smallest log2 of the thread's probabilities.
 template <int D, int NB>
 __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, float (&s)[4][4], const float *lw, int t0,
-                                              const int (&lim)[NB], int common, float scale, uint64_t (&alpha)[NB])
+                                              const int (&lim)[NB], int common, float scale, uint64_t (&alpha)[NB], float &low)
 {
     const int quad = threadIdx.x & 3;
     const bool tail = t0 + TOK_TILE > common;                      // (the same for the whole warp)
+    low = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const float2 w2 = *reinterpret_cast<const float2 *>(lw + 8 * j + 2 * quad);
@@ -337,7 +349,9 @@ __device__ __forceinline__ void token_softmax(TokenUnit<D, NB> &u, bool first, f
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                s[j][2 * b + i] = exp2f(s[j][2 * b + i] - ref);
+                const float x = s[j][2 * b + i] - ref;
+                low = fminf(low, x);
+                s[j][2 * b + i] = exp2f(x);
                 u.l[b] = __fadd_rn(u.l[b], s[j][2 * b + i]);
             }
     }
@@ -456,7 +470,7 @@ template <int D, int NB> __device__ __noinline__ void token_values_odd(TokenOdd<
 // The tile's values, whose rows lie at vrows; the thread's rows see the entries below lim[.], all rows of the group those
 // below `common`, and those below `loaded` are there (what other warps of the CTA see).
 template <int D, int NB>
-__device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], const float (&s)[4][4],
+__device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], float low, const float (&s)[4][4],
                                              const unsigned char *vrows, int t0, const int (&lim)[NB], int common, int loaded)
 {
     constexpr int NC = TokenCfg<D>::NC;
@@ -464,7 +478,7 @@ __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, co
     // Entries whose values do not go through the matrix instruction alone.  One that only some rows see, or none, and that holds an infinity
     // or a NaN must not meet the zero probabilities of the others; a probability that three bf16 parts cannot hold (below 2^-100, for
     // which a logit has to lie 69 below the largest of its unit) must meet its values in fp32.  No row's arithmetic depends on another's.
-    uint32_t odd = 0, least = 0xffffffffu;
+    uint32_t odd = 0;
     const int e0 = common > t0 ? common - t0 : 0, e1 = loaded - t0 < TOK_TILE ? loaded - t0 : TOK_TILE;
     if (e0 < e1) {
         for (int i = lane; i < (e1 - e0) * NC; i += 32) {
@@ -473,11 +487,7 @@ __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, co
         }
         odd = __reduce_or_sync(0xffffffffu, odd);
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int i = 0; i < 2 * NB; ++i) least = min(least, __float_as_uint(s[j][i]) - 1u);
-    if (__any_sync(0xffffffffu, least < SMALLEST_SPLIT - 1u)) {
+    if (__any_sync(0xffffffffu, low < -100.f)) {
         uint32_t small = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -600,6 +610,7 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             const bool more = t + 1 < t_end;
             float s[4][4];
             uint64_t alpha[NB];
+            float low;
             lw[lane] = log2f(wt);
             if (more) fetch_entries(t + 1);
             cp_async_wait<1>();                                        // the keys (the values are the newer group)
@@ -607,11 +618,11 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             token_logits(s, qs, smem_u32(kt));
             __syncwarp();
             if (more) copy_rows(kt, Kp, row, t + 1);
-            token_softmax<D, NB>(u, head, s, lw, t * TOK_TILE, lim, aligned, scale, alpha);
+            token_softmax<D, NB>(u, head, s, lw, t * TOK_TILE, lim, aligned, scale, alpha, low);
             if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
             else cp_async_wait<0>();
             __syncwarp();
-            token_values<D, NB>(u, head, alpha, s, vt, t * TOK_TILE, lim, aligned, n_span);
+            token_values<D, NB>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, aligned, n_span);
             __syncwarp();
             if (more) copy_rows(vt, Vp, row, t + 1);
         }
@@ -762,9 +773,10 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             if (t * TOK_TILE < last) {                                 // (behind what the group sees there is nothing to add)
                 float s[4][4];
                 uint64_t alpha[NB];
+                float low;
                 token_logits(s, qs, smem_u32(kt));
-                token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale, alpha);
-                token_values<D, NB>(u, in_unit == 0, alpha, s, kt + C::TILE_BYTES, t * TOK_TILE, lim, aligned, n_span);
+                token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale, alpha, low);
+                token_values<D, NB>(u, in_unit == 0, alpha, low, s, kt + C::TILE_BYTES, t * TOK_TILE, lim, aligned, n_span);
             }
             if (++in_unit == unit_tiles || t + 1 == tiles) {
                 in_unit = 0;
@@ -874,6 +886,7 @@ tokens_split_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
         const bool more = t + TOK_WARPS < t_end;
         float s[4][4];
         uint64_t alpha[1];
+        float low;
         lw[lane] = log2f(wt);
         if (more) fetch_entries(t + TOK_WARPS);
         cp_async_wait<1>();                                        // the keys (the values are the newer group)
@@ -881,11 +894,11 @@ tokens_split_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
         token_logits(s, qs, smem_u32(kt));
         __syncwarp();
         if (more) copy_rows(kt, Kp, row, t + TOK_WARPS);
-        token_softmax<D, 1>(u, head, s, lw, t * TOK_TILE, lim, n_core, scale, alpha);
+        token_softmax<D, 1>(u, head, s, lw, t * TOK_TILE, lim, n_core, scale, alpha, low);
         if (more) cp_async_wait<1>();
         else cp_async_wait<0>();
         __syncwarp();
-        token_values<D, 1>(u, head, alpha, s, vt, t * TOK_TILE, lim, n_core, n_core);
+        token_values<D, 1>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, n_core, n_core);
         __syncwarp();
         if (more) copy_rows(vt, Vp, row, t + TOK_WARPS);
     }
