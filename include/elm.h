@@ -389,6 +389,10 @@ int elm_debug_round_check(const elm_params *params, int32_t mbar, int32_t r, uin
  * once.  For tests. */
 int elm_debug_decode_grid(const elm_params *params, int32_t n_core, int32_t *ctas, int32_t *resident);
 
+/* How elm_stream_steps attends `tokens` tokens of one window, the first of which sees `seen` entries, bf16 storage (else
+ * ELM_ERR_SHAPE): *form = 0 one token at a time, 1 in clusters, 2 by CTAs that walk the list.  For tests. */
+int elm_debug_stream_form(const elm_params *params, int32_t seen, int32_t tokens, int32_t *form);
+
 /* Kernels launched by this library since it was loaded (all calls, all stages). */
 int64_t elm_launch_count(void);
 

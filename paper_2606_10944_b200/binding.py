@@ -24,7 +24,7 @@ EXPORTED_SYMBOLS = [
     "elm_express_prefill_workspace_bytes", "elm_express_prefill",
     "elm_stream_workspace_bytes", "elm_stream_init", "elm_stream_step", "elm_stream_steps", "elm_stream_cache",
     "elm_host_call_scratch_bytes", "elm_compress_attend_host",
-    "elm_compress_status", "elm_attend_status", "elm_debug_set", "elm_debug_round_check", "elm_debug_decode_grid", "elm_profile_enable", "elm_profile_read", "elm_launch_count", "elm_strerror", "elm_version",
+    "elm_compress_status", "elm_attend_status", "elm_debug_set", "elm_debug_round_check", "elm_debug_decode_grid", "elm_debug_stream_form", "elm_profile_enable", "elm_profile_read", "elm_launch_count", "elm_strerror", "elm_version",
 ]
 
 
@@ -95,6 +95,7 @@ def load_library():
     lib.elm_attend_status.argtypes = [vp, pp, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), vp]
     lib.elm_debug_set.argtypes = [ctypes.c_int32, ctypes.c_int64]
     lib.elm_debug_decode_grid.argtypes = [pp, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
+    lib.elm_debug_stream_form.argtypes = [pp, ctypes.c_int32, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]
     lib.elm_debug_round_check.argtypes = [ctypes.POINTER(ElmParams), ctypes.c_int32, ctypes.c_int32, ctypes.c_uint64,
                                           ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64),
                                           ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
@@ -457,6 +458,14 @@ def debug_decode_grid(B, Hq, Hkv, n, d, n_core, n_q=1, dtype_code=None):
     ctas, resident = ctypes.c_int32(0), ctypes.c_int32(0)
     _check(lib.elm_debug_decode_grid(ctypes.byref(p), n_core, ctypes.byref(ctas), ctypes.byref(resident)), "elm_debug_decode_grid")
     return int(ctas.value), int(resident.value)
+
+
+def debug_stream_form(B, Hq, Hkv, n, d, seen, tokens) -> int:
+    """elm_debug_stream_form: how a stream's call over bf16 rows attends these tokens (0 one by one, 1 clusters, 2 CTAs that walk)."""
+    p, _ = make_params(B, Hq, Hkv, n, 1, d, n.bit_length() - 1, 0, ELM_BF16)
+    form = ctypes.c_int32(-1)
+    _check(load_library().elm_debug_stream_form(ctypes.byref(p), seen, tokens, ctypes.byref(form)), "elm_debug_stream_form")
+    return int(form.value)
 
 
 def profile_enable(on=True):

@@ -944,3 +944,20 @@ extern "C" int elm_debug_decode_grid(const elm_params *params, int32_t n_core, i
                                : decode_grid<__nv_bfloat16, 128, g>(params, n_core, ctas, resident);
     });
 }
+
+extern "C" int elm_debug_stream_form(const elm_params *params, int32_t seen, int32_t tokens, int32_t *form)
+{
+    using namespace elm;
+    if (!params || !form) return ELM_ERR_NULL;
+    const int rc = validate_attend_params(params);
+    if (rc != ELM_OK) return rc;
+    if (seen < 1 || tokens < 1 || (int64_t)seen + tokens - 1 > params->n_kv || params->n_q != 1 || params->dtype != ELM_BF16 ||
+        !attend_decode_applies(params))
+        return ELM_ERR_SHAPE;
+    DecodeWindows win = {};
+    win.n = 1;
+    win.tok0[1] = tokens;
+    win.seen0[0] = seen;
+    *form = !attend_decode_windows_apply(params, seen + tokens - 1) ? 0 : attend_tokens_serial(win, params) ? 2 : 1;
+    return ELM_OK;
+}

@@ -936,22 +936,39 @@ int tokens_per_group(int per_token)
     while (2 * t * per_token <= TOK_ROWS) t *= 2;
     return t;
 }
+// what the last token of window i sees, and the groups of `span` neighbouring tokens that its tokens fall into
+int last_seen(const DecodeWindows &win, int i) { return win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1; }
+int token_groups(const DecodeWindows &win, int i, int span) { return (last_seen(win, i) - 1) / span - (win.seen0[i] - 1) / span + 1; }
+
+bool tokens_serial(const DecodeWindows &win, int per_group, int problems)
+{
+    // The serial form takes as long as one CTA needs for the longest list, about 1.5 us a tile, whatever few tokens there are;
+    // clusters finish one after the other, 0.2 us each for a list of 200 entries and 1.5 for 6144.  Measured, bf16, d = 128, 8 KV heads
+    // of 4 query heads (8 clusters per 4 tokens), clusters against serial: 200 entries 32 tokens 12 / 20 us, 64 tokens 29 / 26;
+    // 2053 entries 32 tokens 47 / 106, 64 tokens 81 / 113; 6144 entries 64 tokens 203 / 303, 128 tokens 390 / 306.
+    int longest = 0;
+    int64_t clusters = 0;
+    for (int i = 0; i < win.n; ++i) {
+        const int last = last_seen(win, i);
+        longest = last > longest ? last : longest;
+        clusters += (int64_t)token_groups(win, i, per_group) * problems;
+    }
+    // (calls of no more tokens than share a warp would leave three of the CTA's four idle)
+    return win.tok0[win.n] > per_group && clusters > 3 * device_sm_count() / 5 + 3 * ((longest + TOK_TILE - 1) / TOK_TILE) / 4;
+}
+
 template <int D>
 int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
                   const DecodeWindows &win, const elm_params *p, void *O, int *status, TokenCaps caps, cudaStream_t st)
 {
     using C = TokenCfg<D>;
     const int problems = p->batch * p->kv_heads, per_token = p->q_heads / p->kv_heads;
-    const int sms = device_sm_count();
     TokenGroups grp = {};
     grp.caps = caps;
     grp.per_group = tokens_per_group(per_token);
     auto count = [&](int span) {
         grp.span = span;
-        for (int i = 0; i < win.n; ++i) {
-            const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
-            grp.g0[i + 1] = grp.g0[i] + (last - 1) / span - (win.seen0[i] - 1) / span + 1;
-        }
+        for (int i = 0; i < win.n; ++i) grp.g0[i + 1] = grp.g0[i] + token_groups(win, i, span);
         return grp.g0[win.n];
     };
     cudaLaunchAttribute attr[2];
@@ -962,18 +979,7 @@ int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *id
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // The serial form takes as long as one CTA needs for the longest list, about 1.5 us a tile, whatever few tokens there are;
-    // clusters finish one after the other, 0.2 us each for a list of 200 entries and 1.5 for 6144.  Measured, bf16, d = 128, 8 KV heads
-    // of 4 query heads (8 clusters per 4 tokens), clusters against serial: 200 entries 32 tokens 12 / 20 us, 64 tokens 29 / 26;
-    // 2053 entries 32 tokens 47 / 106, 64 tokens 81 / 113; 6144 entries 64 tokens 203 / 303, 128 tokens 390 / 306.
-    int longest = 0;
-    for (int i = 0; i < win.n; ++i) {
-        const int last = win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1;
-        longest = last > longest ? last : longest;
-    }
-    const int64_t clusters = (int64_t)count(grp.per_group) * problems;
-    // (calls of no more tokens than share a warp would leave three of the CTA's four idle)
-    const bool serial = win.tok0[win.n] > grp.per_group && clusters > 3 * sms / 5 + 3 * ((longest + TOK_TILE - 1) / TOK_TILE) / 4;
+    const bool serial = tokens_serial(win, grp.per_group, problems);
     auto kern = tokens_kernel<D, false, 2>;
     if (serial) {
         grp.cluster = 1;
@@ -981,6 +987,7 @@ int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *id
         cfg.gridDim = dim3((unsigned)count(TOK_WARPS * grp.per_group), (unsigned)problems);
     } else {
         int most = 1;
+        count(grp.per_group);
         grp.cluster = 1;
         for (int i = 0; i < win.n; ++i) {
             const int tokens = win.tok0[i + 1] - win.tok0[i], size = tokens_cluster(win.seen0[i], win.seen0[i] + tokens - 1, caps);
@@ -1033,6 +1040,11 @@ TokenCaps tokens_caps(int d, int problems, int limit)
     // Up to 4096 entries clusters of 16 gain nothing over 8 with twice the tiles per warp (8 problems of 4 query vectors: 2048 entries
     // 9.2 against 8.0 us, 4000 entries 10.8 / 10.6, 5193 entries 12.3 / 14.0).
     return {cap < 8 ? cap : 8, cap};
+}
+
+bool attend_tokens_serial(const DecodeWindows &win, const elm_params *p)
+{
+    return tokens_serial(win, tokens_per_group(p->q_heads / p->kv_heads), p->batch * p->kv_heads);
 }
 
 int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
