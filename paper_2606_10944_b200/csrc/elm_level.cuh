@@ -14,8 +14,6 @@
 #include <type_traits>
 
 #include "elm_attend.cuh"
-#include <type_traits>
-
 #include "elm_common.cuh"
 #include "elm_compress.cuh"
 #include "elm_walk.cuh"
