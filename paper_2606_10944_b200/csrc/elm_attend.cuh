@@ -106,7 +106,7 @@ TokenCaps tokens_caps(int d, int problems, int limit /* largest cluster to use *
 int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
                        const DecodeWindows &win, const elm_params *p, void *O, int *status, TokenCaps caps, cudaStream_t st);
 
-bool attend_tokens_serial(const DecodeWindows &win, const elm_params *p);       // by CTAs that walk the list, not in clusters
+bool attend_tokens_serial(const DecodeWindows &win, const elm_params *p, TokenCaps caps);       // by CTAs that walk the list, not in clusters
 
 // The first launch of elm_attend's split form on bf16 storage with the matrix instructions: every problem's list over `splits`
 // CTAs, which leave part[problem][split][G][d + 2] for attend_decode's merge; up to 8 query vectors, n_q rows of every head.

@@ -3,7 +3,8 @@
 // With so few queries the work is reading each coreset row of K and V once: HBM-bound, and far too
 // small for the tile kernels.  All query heads that share the KV head (and all their query rows: G vectors
 // in total, G <= 8) are processed together, so a row is read once for the whole group.  Rows are read through
-// the index list straight from K and V (no gathered copy).  fp32 arithmetic on fp32 or bf16 inputs.
+// the index list straight from K and V (no gathered copy).  fp32 arithmetic on fp32 or bf16 inputs.  On bf16 inputs streaming
+// tokens, and lists of three query vectors and more that are not short, go to the kernels of elm_attend_tokens.cu instead.
 //
 // A warp takes a tile of 32 list entries (16 when a row is 512 bytes, 8 of a short list): the tile's K and V rows come to shared memory
 // by asynchronous copies (the next tile's keys are requested as soon as this tile's logits are formed, its values
@@ -11,10 +12,8 @@
 // one butterfly, so that a lane ends with finished logits of its own - 14 shuffles per 16 entries of four queries
 // where a butterfly that leaves every sum in every lane needs 20 per entry.  The softmax of a tile is one entry per
 // lane; for the values a lane owns one 16-byte chunk of the row.  The instruction count per entry is what decides
-// here: the version with one entry per warp at a time and the softmax repeated in every lane issued about 120
-// instructions per entry of four bf16 queries (this one about 45) and took 68.0 us for 4 x 8 problems of 5193 entries
-// (86 MB), bound by issue; now 20.0 us (4.3 TB/s).  8 problems of 2048 entries: 8.0 -> 6.6 us, latency of the chain row
-// number -> row -> softmax -> merge.
+// here: a version with one entry per warp at a time and the softmax repeated in every lane issued about 120
+// instructions per entry of four queries, this one about 45.
 //
 // The list of an attention problem is split over CTAs.  elm_attend: over as many as the SMs can hold, which leave
 // partial results (maximum, denominator, accumulator) in the workspace for decode_merge_kernel.  Tokens of a streaming
@@ -128,9 +127,9 @@ struct DecodeGroups {
 };
 
 // How a list of n_core entries is parted: parts of whole tiles, at least two tiles per warp (with one, a single token over
-// 200 entries (figures here and in decode_form: bf16 rows, whose tokens took these forms when they were measured) takes 5.8 us for 6.9, less than the host needs to enqueue it, but a CTA that walks all parts has twice the
-// merges: 2000 tokens of 8 KV heads of 4 query heads, n_out = 128, 1010 us for 960), at most `cap` parts.  Depends on
-// n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
+// 200 entries takes 5.8 us for 6.9, less than the host needs to enqueue it, but a CTA that walks all parts has twice the
+// merges: 2000 tokens of 8 KV heads of 4 query heads, n_out = 128, 1010 us for 960; measured on bf16 rows, which took this form then),
+// at most `cap` parts.  Depends on n_core only through the next multiple of 128, so that neighbouring tokens share their parts.
 __host__ __device__ __forceinline__ void decode_parts(int n_core, int cta_entries, int tile, int cap, int &parts, int &chunk)
 {
     const int len = (n_core + 127) / 128 * 128;
@@ -620,9 +619,9 @@ TokenCaps decode_token_caps(const elm_params *p, int problems)
 // Streaming tokens of `per_token` query vectors: most parts of a list - a power of two, so that the SMs hold one
 // token's clusters at once.  A list that would give each CTA of its cluster more than eight rounds of tiles while
 // most SMs idle is left to the form with partial results in the workspace, token by token: over as many CTAs as fit the
-// device a single token gains from about 6000 entries on (8 KV heads of 4 query heads, bf16: 6144 entries 16.4 us in
-// clusters, 14.2 split; 12288 entries 25.2 and 18.6), but the tokens of a call can then no longer share a launch (64 tokens over
-// 12288 entries: 606 us together, 1190 one by one).
+// device a single token gains (8 KV heads of 4 query heads: fp32, 4500 entries 16.4 us in clusters, 14.5 split, 9000 26.6 and
+// 18.3, 24000 57.5 and 43.3; bf16, 9000 17.2 and 14.6, 17000 24.8 and 18.1), but the tokens of a call can then no longer share a launch (32
+// tokens together and one by one: fp32, 9000 entries 297 and 563 us; bf16, 17000 177 and 567).
 template <int D> int decode_cap(int problems, int per_token, int sms)
 {
     const int most = DEC_CTAS * sms / (problems * ((per_token + DEC_GSTREAM - 1) / DEC_GSTREAM));
@@ -636,8 +635,8 @@ bool decode_clustered(int n_core, int problems, int cap, int entries)
 }
 
 // The split form of three query vectors and more on bf16 storage is a contraction for the matrix instructions (tokens_split_kernel,
-// elm_attend_tokens.cu): 4 vectors, 8 problems of 2048 entries 8.4 -> 6.9 us, 32 of 5193 25.5 -> 22.1 us; 8 vectors 12.2 -> 7.6 and
-// 41.6 -> 24.2 us; d = 64 alike.  One or two vectors would pay for eight (they are within 10 % of it from 64 problems on).
+// elm_attend_tokens.cu): a loop of calls of 4 vectors, 8 problems of 2048 entries, 8.4 -> 7.2 us, 32 of 5193 25.5 -> 22.4 us; 8 vectors 12.2 -> 7.8
+// and 41.6 -> 24.4 us; d = 64 alike.  One or two vectors would pay for eight (they are within 10 % of it from 64 problems on).
 template <typename Tin, int G> constexpr bool DECODE_MMA = std::is_same<Tin, __nv_bfloat16>::value && G >= 4;
 template <typename Tin, int G> constexpr bool DECODE_SHORT = !DECODE_MMA<Tin, G> || G < 8;
 
@@ -661,9 +660,11 @@ template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int
     s.short_tiles = false;
     if constexpr (DECODE_SHORT<Tin, G>) s.short_tiles = few <= 2 || (few <= 16 && few * problems <= 2 * sms);
     // otherwise as many CTAs as are resident at once, but at least one tile per warp; with more problems than that, as many
-    // as take the least time in waves of them, a CTA's start and merge counted as 3/4 round of tiles per query vector.
+    // as take the least time in waves of them, a CTA's start and merge counted as 3/4 round of tiles per query vector, on matrix instructions as
+    // 3/2 round whatever the vectors (450 problems of 2048 entries, 4 vectors, parts 1 / 2 / 3 / 4: 95.6 / 85.4 / 82.7 / 81.5 us, 8 vectors
+    // 98.6 / 89.0 / 87.6 / 86.7; 600 problems 116.8 / 102.1 / 106.0 / 105.0; 300 problems 56.6 / 63.3 / 61.6 / 57.3).
     // 512 problems on 444 CTAs, fp32, d = 128, one query vector: 2048 entries 173 -> 122 us (one CTA per problem: a second
-    // wave that is nearly empty), 200 entries 16.9 -> 15.9 us; bf16, four query vectors, 2048 entries: 101 -> 91 us.
+    // wave that is nearly empty), 200 entries 16.9 -> 15.9 us.
     const int resident = DEC_CTAS * sms, wanted = resident / problems;
     s.n = s.short_tiles ? few : ctas(n_core, DEC_TILE<Tin, D>);
     if (!s.short_tiles && wanted < 1) {
@@ -671,7 +672,7 @@ template <typename Tin, int D, int G> DecodeSplits decode_splits(int n_core, int
         int64_t least = INT64_MAX;
         for (int n = 1; n <= most_parts; ++n) {
             const int rounds = ctas((n_core + n - 1) / n, DEC_TILE<Tin, D>);
-            const int64_t time = (((int64_t)n * problems + resident - 1) / resident) * (4 * rounds + (G == 1 ? 4 : 3 * G));
+            const int64_t time = (((int64_t)n * problems + resident - 1) / resident) * (4 * rounds + (DECODE_MMA<Tin, G> ? 6 : G == 1 ? 4 : 3 * G));
             if (time < least) { least = time; s.n = n; }
         }
     } else if (!s.short_tiles && s.n > wanted) {
@@ -703,20 +704,20 @@ template <typename Tin, int D> DecodeForm decode_form(const DecodeWindows &win, 
     while (size < parts) size <<= 1;
     const int64_t tokens = win.tok0[win.n];
     const int whole = (per_token + DEC_GSTREAM - 1) / DEC_GSTREAM;                // groups of DEC_GSTREAM vectors
-    // Clusters spread a token over the SMs and are never slower than the tokens one by one (6144 entries, 8 KV heads of 4
-    // query heads, bf16: 2 tokens 23 us, 8 tokens 68 us, one token 18 us).  Walking part after part saves their barriers
-    // and merges but takes as long as one CTA needs for a whole list (137 us), so it pays from about one token per SM on
-    // (16 tokens of 8 heads: 119 us in clusters, 137 walked; 32 tokens: 224 against 185; 64: 431 against 345), from two
-    // on when its CTAs take several tokens (1 query head per KV head: 32 tokens 147 against 171, 64 tokens 282 against
-    // 172).  A list of one part needs no merge at all.
+    // Clusters spread a token over the SMs and are never slower than the tokens one by one (fp32, 6144 entries, 8 KV heads of 4
+    // query heads: 2 tokens 25 us, 8 tokens 80 us, one token 20 us).  Walking part after part saves their barriers
+    // and merges but takes as long as one CTA needs for a whole list (161 us), so it pays from about one token per SM on
+    // (16 tokens of 8 heads: 141 us in clusters, 163 walked; 32 tokens: 264 against 221; 64: 505 against 424), from two
+    // on when its CTAs take several tokens (1 query head per KV head: 32 tokens 199 against 307, 64 tokens 379 against
+    // 311).  A list of one part needs no merge at all.
     if (tokens > 1) {
         int per_group = 1;
         while (per_group * 2 * per_token <= DEC_GSTREAM) per_group *= 2;
         if (tokens * problems * whole >= (per_group > 1 ? 2 : 1) * sms || (parts == 1 && per_group == 1)) return {DEC_GSTREAM, whole, per_group, 0, cap};
     }
     // The chain of a tile grows with its query vectors, so clusters take as few as leave all their CTAs resident.
-    // 8 KV heads of 8 query heads, bf16: 200 entries 17.6 us with all eight together, 6.2 one by one, 6144 entries 29.7 and
-    // 22.1; of 4 query heads: 200 entries 11.0 and 6.0, 6144 entries 17.7 and 16.4.
+    // fp32, 8 KV heads of 8 query heads, vectors one by one, in twos, in fours: 200 entries 6.9 / 7.7 / 9.3 us, 2000 entries 28.7 / 18.9 / 13.0; of 4
+    // query heads: 200 entries 6.6 / 7.7 / 9.2, 2000 entries 16.6 / 10.7 / 10.9, 6144 entries 32.7 / 19.9 / 19.7.
     int G = 1;
     while (G < DEC_GSTREAM && G < per_token && tokens * problems * ((per_token + G - 1) / G) * size > DEC_CTAS * sms) G *= 2;
     return {G, (per_token + G - 1) / G, 1, size, cap};
@@ -958,6 +959,6 @@ extern "C" int elm_debug_stream_form(const elm_params *params, int32_t seen, int
     win.n = 1;
     win.tok0[1] = tokens;
     win.seen0[0] = seen;
-    *form = !attend_decode_windows_apply(params, seen + tokens - 1) ? 0 : attend_tokens_serial(win, params) ? 2 : 1;
+    *form = !attend_decode_windows_apply(params, seen + tokens - 1) ? 0 : attend_tokens_serial(win, params, decode_token_caps(params, params->batch * params->kv_heads)) ? 2 : 1;
     return ELM_OK;
 }

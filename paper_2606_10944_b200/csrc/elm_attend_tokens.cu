@@ -5,7 +5,8 @@
 // Neighbouring tokens see all but a few of the same entries, and a token has one query vector per query head of its KV
 // head, so 16 rows of a matrix instruction hold the vectors of 16, 8, 4 or 2 neighbouring tokens (TokenGroups::per_group).
 // Both contractions are mma.sync m16n8k16 with fp32 accumulators: Q K^T on the stored bf16 values, P V with each fp32
-// probability as the sum of three bf16 values (split3: 24 bits, so nothing is rounded that fp32 arithmetic would keep).
+// probability as the sum of three bf16 values (split3: 24 bits).  How the instruction rounds inside is not documented; against 64 bits it rounds
+// toward zero, so its chains are short and their sums go on in fp32 (token_contract has the errors).
 // tcgen05 takes 64 rows at least: a single token of four vectors would leave most of them empty, and the accumulators of
 // each 32-entry unit (below) would go through tensor memory and back.
 //
@@ -940,12 +941,15 @@ int tokens_per_group(int per_token)
 int last_seen(const DecodeWindows &win, int i) { return win.seen0[i] + (win.tok0[i + 1] - win.tok0[i]) - 1; }
 int token_groups(const DecodeWindows &win, int i, int span) { return (last_seen(win, i) - 1) / span - (win.seen0[i] - 1) / span + 1; }
 
-bool tokens_serial(const DecodeWindows &win, int per_group, int problems)
+bool tokens_serial(const DecodeWindows &win, int per_group, int problems, TokenCaps caps)
 {
-    // The serial form takes as long as one CTA needs for the longest list, about 1.5 us a tile, whatever few tokens there are;
-    // clusters finish one after the other, 0.2 us each for a list of 200 entries and 1.5 for 6144.  Measured, bf16, d = 128, 8 KV heads
-    // of 4 query heads (8 clusters per 4 tokens), clusters against serial: 200 entries 32 tokens 12 / 20 us, 64 tokens 29 / 26;
-    // 2053 entries 32 tokens 47 / 106, 64 tokens 81 / 113; 6144 entries 64 tokens 203 / 303, 128 tokens 390 / 306.
+    // The serial form takes as long as one CTA needs for the longest list, 1.9 us a tile (2.5 where two CTAs share an SM), whatever few tokens
+    // there are.  Clusters take 0.05 to 0.1 us per CTA, and the larger they are the fewer the device holds at once.  Measured, clusters
+    // against serial, us (d = 64 has the same crossings at about 0.7 of the times):
+    //   8 problems of 4 vectors, 64 tokens (136 clusters): 200 entries 26 / 27, 1000 61 / 73, 4100 184 / 254, 9000 238 / 540
+    //   128 tokens (264 clusters): 200 entries 48 / 31, 1000 116 / 77, 4100 355 / 257, 9000 459 / 541; of 8 vectors (520): 9000 895 / 544
+    //   32 problems of 4 vectors, 32 tokens (288 clusters): 1000 entries 113 / 71, 4100 188 / 252; 64 tokens (544): 4100 371 / 333, 9000 543 / 714
+    //   32 problems of 1 vector, 64 tokens (160 clusters): 1000 entries 69 / 74; 128 tokens (288): 1000 122 / 78, 4100 206 / 259, 9000 300 / 544
     int longest = 0;
     int64_t clusters = 0;
     for (int i = 0; i < win.n; ++i) {
@@ -953,8 +957,9 @@ bool tokens_serial(const DecodeWindows &win, int per_group, int problems)
         longest = last > longest ? last : longest;
         clusters += (int64_t)token_groups(win, i, per_group) * problems;
     }
+    const int tiles = (longest + TOK_TILE - 1) / TOK_TILE, cap = longest <= TOKENS_SHORT_LIST ? caps.of_short : caps.of_long;
     // (calls of no more tokens than share a warp would leave three of the CTA's four idle)
-    return win.tok0[win.n] > per_group && clusters > 3 * device_sm_count() / 5 + 3 * ((longest + TOK_TILE - 1) / TOK_TILE) / 4;
+    return win.tok0[win.n] > per_group && clusters > 9 * device_sm_count() / 10 + 12 * tiles / cap;
 }
 
 template <int D>
@@ -979,7 +984,7 @@ int launch_tokens(const void *Q, const void *K, const void *V, const int32_t *id
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool serial = tokens_serial(win, grp.per_group, problems);
+    const bool serial = tokens_serial(win, grp.per_group, problems, caps);
     auto kern = tokens_kernel<D, false, 2>;
     if (serial) {
         grp.cluster = 1;
@@ -1037,14 +1042,15 @@ TokenCaps tokens_caps(int d, int problems, int limit)
     // as many CTAs as leave all problems' clusters resident
     int cap = limit < TOK_MAX_CLUSTER ? limit : TOK_MAX_CLUSTER;
     while (cap > 1 && tokens_clusters(d, cap) < problems) cap >>= 1;
-    // Up to 4096 entries clusters of 16 gain nothing over 8 with twice the tiles per warp (8 problems of 4 query vectors: 2048 entries
-    // 9.2 against 8.0 us, 4000 entries 10.8 / 10.6, 5193 entries 12.3 / 14.0).
+    // Up to 4096 entries clusters of 16 gain nothing over 8 with twice the tiles per warp (8 problems of 4 query vectors, one token: 2000 entries
+    // 10.3 against 9.2 us, 4000 12.1 / 11.9, 5000 13.7 / 13.4; 8 tokens: 4000 entries 32.8 / 22.5; 8 problems of one vector: 4000 11.1 / 11.6, 5000
+    // 12.6 / 13.2; d = 64, 4 vectors: 4000 9.6 / 9.8).
     return {cap < 8 ? cap : 8, cap};
 }
 
-bool attend_tokens_serial(const DecodeWindows &win, const elm_params *p)
+bool attend_tokens_serial(const DecodeWindows &win, const elm_params *p, TokenCaps caps)
 {
-    return tokens_serial(win, tokens_per_group(p->q_heads / p->kv_heads), p->batch * p->kv_heads);
+    return tokens_serial(win, tokens_per_group(p->q_heads / p->kv_heads), p->batch * p->kv_heads, caps);
 }
 
 int attend_tokens_bf16(const void *Q, const void *K, const void *V, const int32_t *idx, const float *w, int64_t list_stride,
