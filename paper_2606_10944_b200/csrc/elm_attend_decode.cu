@@ -635,8 +635,8 @@ bool decode_clustered(int n_core, int problems, int cap, int entries)
 }
 
 // The split form of three query vectors and more on bf16 storage is a contraction for the matrix instructions (tokens_split_kernel,
-// elm_attend_tokens.cu): a loop of calls of 4 vectors, 8 problems of 2048 entries, 8.4 -> 7.2 us, 32 of 5193 25.5 -> 22.4 us; 8 vectors 12.2 -> 7.8
-// and 41.6 -> 24.4 us; d = 64 alike.  One or two vectors would pay for eight (they are within 10 % of it from 64 problems on).
+// elm_attend_tokens.cu): both launches, replayed as a graph, 4 vectors, 8 problems of 2048 entries 7.9 -> 6.9 us, 32 of 5193 21.4 -> 16.8 us, 64 of 12288
+// 74.8 -> 66.9; 8 vectors, 8 problems of 2048 11.9 -> 7.4, 64 of 12288 136 -> 68.9; d = 64 alike.  One or two vectors would pay for eight.
 template <typename Tin, int G> constexpr bool DECODE_MMA = std::is_same<Tin, __nv_bfloat16>::value && G >= 4;
 template <typename Tin, int G> constexpr bool DECODE_SHORT = !DECODE_MMA<Tin, G> || G < 8;
 

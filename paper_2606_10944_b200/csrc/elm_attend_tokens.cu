@@ -19,10 +19,10 @@
 //            of asynchronous copies and every warp merges unit after unit in registers.
 //
 // Bound by the issue of mma.sync: 128 per tile and 16 rows, 32 for the logits and 96 for the values, at the 16 cycles that each
-// takes an SM sub-partition (measured: 2250 cycles per tile with two warps on each).  2496 tokens of 32 query / 8 KV heads,
-// n_out = 256: 1186 us with fp32 fma per token, 237 us here; a token over 6144 entries of 8 KV heads of 4 query heads 17.4 ->
-// 15.5 us, of 8 query heads 23.2 -> 16.9, over 500 entries 8.1 -> 8.2; of 1 query head over 4100 entries 9.3 -> 11.0 (its one
-// vector pays for eight).
+// takes an SM sub-partition (about 2500 cycles per tile with two warps on each; 2250 with the sums of the list left to the instruction).
+// With fp32 fma per token and here: a generation of 2496 tokens of 32 query / 8 KV heads, n_out = 256, 1443 -> 486 us; 512 tokens over 6144
+// entries 2145 -> 522, over 200 218 -> 65; one token over 6144 entries of 8 KV heads of 4 query heads 16.6 -> 15.2 us, of 8 query heads 22.3 -> 17.3,
+// over 200 entries 7.1 -> 7.6; of 1 query head over 4100 entries 10.2 -> 12.5 (its one vector pays for eight), but 8 of them 36.5 -> 14.9.
 #include <math.h>
 
 #include <atomic>
@@ -368,7 +368,7 @@ __device__ __forceinline__ bool too_small(float p) { return __float_as_uint(p) -
 // at zero, take the small parts first, and go to the unit's accumulators by fp32 fma (one accumulator through a warp's whole share of a
 // list: relative error 5.0e-7 over 5193 entries, 1.9e-6 over 12288; fp32 fma alone 2.1e-7 and 3.6e-7; so 1.8e-7 and 2.3e-7).
 // `odd`: entries of which the values that are not finite are taken as zeros, and so are probabilities that cannot be split.
-template <int D, int NB, bool ODD>
+template <int D, int NB, bool ODD, bool SERIAL>
 __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], const float (&s)[4][4],
                                                uint32_t vt, uint32_t odd)
 {
@@ -388,12 +388,31 @@ __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, 
                 }
                 split3(x, y, p[k][b][0][h], p[k][b][1][h], p[k][b][2][h]);
             }
-    constexpr int JG = 4;                                              // output tiles at a time
+    // Output tiles at a time: four, or, where eight warps of an SM leave the tensor cores little time between them (serial form), two and two of
+    // them on their way while the two before are added (512 tokens over 4100 entries, 4 vectors: 366 us with four, 358 so).
+    constexpr int JG = SERIAL ? 2 : 4;
     const int sw = lane & 7, half = (lane >> 3) & 1;
+    float t[SERIAL ? 2 : 1][JG][NB][4];
+    auto add = [&](int j) {
+#pragma unroll
+        for (int h = 0; h < JG; ++h)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                float (&o)[4] = u.o[j + h][b], (&x)[4] = t[SERIAL ? j / JG & 1 : 0][h][b];
+#pragma unroll
+                for (int i = 0; i < 4; i += 2) {
+                    if (first) {
+                        o[i] = x[i];
+                        o[i + 1] = x[i + 1];
+                    } else {
+                        unpack2(fma2(pack2(o[i], o[i + 1]), alpha[b], pack2(x[i], x[i + 1])), o[i], o[i + 1]);
+                    }
+                }
+            }
+    };
 #pragma unroll
     for (int j = 0; j < D / 16; j += JG) {
         uint32_t a[2][JG][4];
-        float t[JG][NB][4];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             // matrices of a load: entries 16 k + {0, 0, 8, 8} + 0..7, chunks {0, 1, 0, 1} of the 16 columns
@@ -417,25 +436,13 @@ __device__ __forceinline__ void token_contract(TokenUnit<D, NB> &u, bool first, 
                 for (int h = 0; h < JG; ++h)
 #pragma unroll
                     for (int b = 0; b < NB; ++b) {
-                        if (part == 2 && k == 0) mma16816_new(t[h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
-                        else mma16816(t[h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
+                        if (part == 2 && k == 0) mma16816_new(t[SERIAL ? j / JG & 1 : 0][h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
+                        else mma16816(t[SERIAL ? j / JG & 1 : 0][h][b], a[k][h], p[k][b][part][0], p[k][b][part][1]);
                     }
-#pragma unroll
-        for (int h = 0; h < JG; ++h)
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                float (&o)[4] = u.o[j + h][b];
-#pragma unroll
-                for (int i = 0; i < 4; i += 2) {
-                    if (first) {
-                        o[i] = t[h][b][i];
-                        o[i + 1] = t[h][b][i + 1];
-                    } else {
-                        unpack2(fma2(pack2(o[i], o[i + 1]), alpha[b], pack2(t[h][b][i], t[h][b][i + 1])), o[i], o[i + 1]);
-                    }
-                }
-            }
+        if (!SERIAL) add(j);
+        else if (j > 0) add(j - JG);
     }
+    if (SERIAL) add(D / 16 - JG);
 }
 
 // A tile with entries that do not go through the matrix instruction alone (rare, so on a copy of the accumulators in local memory and
@@ -451,7 +458,7 @@ template <int D, int NB> __device__ __noinline__ void token_values_odd(TokenOdd<
 {
     using C = TokenCfg<D>;
     const int lane = threadIdx.x & 31, quad = lane & 3;
-    token_contract<D, NB, true>(x->u, first, x->alpha, x->s, smem_u32(vrows), odd);
+    token_contract<D, NB, true, false>(x->u, first, x->alpha, x->s, smem_u32(vrows), odd);
     for (uint32_t left = odd; left; left &= left - 1) {
         const int e = __ffs(left) - 1;
         for (int b = 0; b < NB; ++b)
@@ -470,7 +477,7 @@ template <int D, int NB> __device__ __noinline__ void token_values_odd(TokenOdd<
 
 // The tile's values, whose rows lie at vrows; the thread's rows see the entries below lim[.], all rows of the group those
 // below `common`, and those below `loaded` are there (what other warps of the CTA see).
-template <int D, int NB>
+template <bool SERIAL, int D, int NB>
 __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, const uint64_t (&alpha)[NB], float low, const float (&s)[4][4],
                                              const unsigned char *vrows, int t0, const int (&lim)[NB], int common, int loaded)
 {
@@ -512,7 +519,7 @@ __device__ __forceinline__ void token_values(TokenUnit<D, NB> &u, bool first, co
         token_values_odd(&x, first, vrows, t0, odd);
         u = x.u;
     } else {
-        token_contract<D, NB, false>(u, first, alpha, s, smem_u32(vrows), 0);
+        token_contract<D, NB, false, SERIAL>(u, first, alpha, s, smem_u32(vrows), 0);
     }
 }
 
@@ -623,7 +630,7 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
             if (more) cp_async_wait<1>();                              // (the next tile's keys may still be on their way)
             else cp_async_wait<0>();
             __syncwarp();
-            token_values<D, NB>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, aligned, n_span);
+            token_values<false>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, aligned, n_span);
             __syncwarp();
             if (more) copy_rows(vt, Vp, row, t + 1);
         }
@@ -777,7 +784,7 @@ tokens_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restri
                 float low;
                 token_logits(s, qs, smem_u32(kt));
                 token_softmax<D, NB>(u, in_unit == 0, s, lw + stage * TOK_TILE, t * TOK_TILE, lim, aligned, scale, alpha, low);
-                token_values<D, NB>(u, in_unit == 0, alpha, low, s, kt + C::TILE_BYTES, t * TOK_TILE, lim, aligned, n_span);
+                token_values<true>(u, in_unit == 0, alpha, low, s, kt + C::TILE_BYTES, t * TOK_TILE, lim, aligned, n_span);
             }
             if (++in_unit == unit_tiles || t + 1 == tiles) {
                 in_unit = 0;
@@ -899,7 +906,7 @@ tokens_split_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
         if (more) cp_async_wait<1>();
         else cp_async_wait<0>();
         __syncwarp();
-        token_values<D, 1>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, n_core, n_core);
+        token_values<false>(u, head, alpha, low, s, vt, t * TOK_TILE, lim, n_core, n_core);
         __syncwarp();
         if (more) copy_rows(vt, Vp, row, t + TOK_WARPS);
     }

@@ -393,8 +393,8 @@ static int64_t stream_window(const elm_stream *s, const elm_params *p, int64_t l
 
 // n_tokens tokens, window by window: the list, the prepass and the Halve calls of a window are enqueued as its tokens
 // would have them, and the attention of many windows' tokens is one launch - a list built for a window is
-// not touched by what comes behind it, so the launch may wait.  2496 tokens of 32 query / 8 KV heads, n_out = 256, bf16: 0.50 ms
-// (attention 0.24 in one launch, the chain of 8 Halve calls and 10 lists 0.27) against 27 ms token by token, two launches
+// not touched by what comes behind it, so the launch may wait.  2496 tokens of 32 query / 8 KV heads, n_out = 256, bf16: 0.49 ms
+// (more than half of it the one launch of the attention, the rest the chain of 8 Halve calls and 10 lists) against 27 ms token by token, two launches
 // and the host's part of a step each.
 template <typename Tin, typename T>
 static int stream_steps_impl(elm_stream *s, int64_t n_tokens, const Tin *Q, const Tin *K, const Tin *V, const elm_params *p, Tin *O,
