@@ -959,6 +959,7 @@ extern "C" int elm_debug_stream_form(const elm_params *params, int32_t seen, int
     win.n = 1;
     win.tok0[1] = tokens;
     win.seen0[0] = seen;
-    *form = !attend_decode_windows_apply(params, seen + tokens - 1) ? 0 : attend_tokens_serial(win, params, decode_token_caps(params, params->batch * params->kv_heads)) ? 2 : 1;
+    const TokenCaps caps = decode_token_caps(params, params->batch * params->kv_heads);
+    *form = !attend_decode_windows_apply(params, seen + tokens - 1) ? 0 : attend_tokens_serial(win, params, caps) ? 2 : 1;
     return ELM_OK;
 }

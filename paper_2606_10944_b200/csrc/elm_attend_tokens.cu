@@ -20,7 +20,7 @@
 //
 // Bound by the issue of mma.sync: 128 per tile and 16 rows, 32 for the logits and 96 for the values, at the 16 cycles that each
 // takes an SM sub-partition (about 2500 cycles per tile with two warps on each; 2250 with the sums of the list left to the instruction).
-// With fp32 fma per token and here: a generation of 2496 tokens of 32 query / 8 KV heads, n_out = 256, 1443 -> 486 us; 512 tokens over 6144
+// With fp32 fma per token and here: a generation of 2496 tokens of 32 query / 8 KV heads, n_out = 256, 1443 -> 490 us; 512 tokens over 6144
 // entries 2145 -> 522, over 200 218 -> 65; one token over 6144 entries of 8 KV heads of 4 query heads 16.6 -> 15.2 us, of 8 query heads 22.3 -> 17.3,
 // over 200 entries 7.1 -> 7.6; of 1 query head over 4100 entries 10.2 -> 12.5 (its one vector pays for eight), but 8 of them 36.5 -> 14.9.
 #include <math.h>
